@@ -285,6 +285,22 @@ cudaError_t mirror_copy(cudaStream_t st, int32_t* x, int64_t per, const int2* pa
 // out[b][I][J] = a[b][J][I] * c[b][I][J] for nb blocks of n x n.
 cudaError_t hadamard_t(cudaStream_t st, const double2* a, const double2* c, int n, int nb, double2* out);
 
+// FP64-accurate complex GEMM on the tensor cores (k_ztc.cu): C_b = alpha op(A_b) op(B_b),
+// any K, eight exact slices per operand (36 fp16 products), no less accurate than an FP64
+// FMA chain.  lowerA and brow as in ztrmm_gather.  work: zgemm_tc_work_bytes for the batch
+// entries of one chunk (one at least); err: device word set on a bounded-wait timeout.
+// zgemm_tc_same: op(A) op(A)^T or ^H of one array, whose slices serve both sides.
+inline bool zgemm_tc_same(char opA, char opB, int m, int n, const double2* A, int64_t lda, int64_t sA,
+                          const double2* B, int64_t ldb, int64_t sB) {
+  const bool aT = opA == 'T' || opA == 'C', bT = opB == 'T' || opB == 'C';
+  return A == B && lda == ldb && sA == sB && m == n && aT != bT;
+}
+size_t zgemm_tc_work_bytes(int m, int n, int k, int nb, bool same);
+cudaError_t zgemm_tc(cudaStream_t st, char opA, char opB, int m, int n, int k, double alpha, const double2* A,
+                     int64_t lda, int64_t sA, const double2* B, int64_t ldb, int64_t sB, double2* C, int64_t ldc,
+                     int64_t sC, int batch, int lowerA, const int32_t* brow, int64_t sIdx, void* work,
+                     size_t work_bytes, int* err);
+
 // FP64-accurate complex GEMM on the tensor cores for 2K <= 128 (k_emu.cu):
 // C_b = op(A_b) B_b, op 'N' or 'R' (conjugate), seven exact 7-bit slices per
 // operand.  work: zgemm_emu_work_bytes(M, N, K, batch) bytes; err: device word

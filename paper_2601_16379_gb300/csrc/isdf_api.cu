@@ -167,7 +167,7 @@ struct isdf_handle {
   // them, or isdf_coulomb_metric_eta, then needs a new isdf_fit_zeta).
   static bool in_frag_group(const std::string& n) { return n.rfind("frag_", 0) == 0 || n.rfind("tc_", 0) == 0; }
   static bool in_fit_group(const std::string& n) {
-    return n == "eta" || n == "xi" || n == "grid_work" || n == "grid_work_emu" || n == "grid_work_v";
+    return n == "eta" || n == "xi" || n == "grid_work" || n == "grid_work_z" || n == "grid_work_v";
   }
   bool evict_other(const char* name) {
     const std::string n(name);
@@ -358,10 +358,62 @@ int upload_basis(isdf_handle* h) {
   b.prim_cn = nullptr;
   if (!b.ao_shell || !b.ao_lxyz || !b.sh_atom || !b.sh_off || !b.prim_exp || !b.prim_norm || !b.coords)
     return fail(h, ISDF_ERR_OOM, "uploading the basis failed");
+  const int words[4] = {0, 0, 0, 0};
+  if (!up("err_words", words, sizeof(words))) return fail(h, ISDF_ERR_OOM, "allocating the error words failed");
   double2 tw[192];
   grid_twiddles(h->cell.mesh, tw);
   if (!up("grid_tw", tw, sizeof(tw))) return fail(h, ISDF_ERR_OOM, "uploading twiddles failed");
   return ISDF_OK;
+}
+
+// C_b = alpha op(A_b) op(B_b) in complex128 (FP64-accurate): on the tensor cores with its slices
+// in the buffer `wname` (batch entries in chunks of kSliceBytes), on the FP64 pipe where the
+// inner dimension is too short to pay for the slicing or the workspace cannot be had.
+// lowerA / brow as in ztrmm_gather.  A bounded wait that expires sets the handle's error
+// word, read by tc_status at the next synchronisation point.
+// wname NULL keeps the FP64 pipe.
+//
+// kMinTcK: a 64 x 64 tile of the SIMT kernel takes 4.3 us per unit of K however few tiles there
+// are, the tensor path ~23 us for the smallest product (three launches): measured 43 against
+// 23 us at 64 x 64 x 8 (batch 8), 282 against 27 at K = 64, 33.7 against 1.5 ms at
+// 1600 x 1600 x 1680, so that the line lies below K = 8.
+constexpr size_t kSliceBytes = (size_t)512 << 20;
+constexpr int kMinTcK = 6;
+int zmul(isdf_handle* h, const char* wname, char opA, char opB, int m, int n, int k, double alpha, const double2* A,
+         int64_t lda, int64_t sA, const double2* B, int64_t ldb, int64_t sB, double2* C, int64_t ldc, int64_t sC,
+         int batch, int lowerA = 0, const int32_t* brow = nullptr, int64_t sIdx = 0) {
+  void* w = nullptr;
+  size_t bytes = 0;
+  if (wname && k >= kMinTcK) {
+    const bool same = !brow && zgemm_tc_same(opA, opB, m, n, A, lda, sA, B, ldb, sB);
+    bytes = std::min(zgemm_tc_work_bytes(m, n, k, batch, same),
+                     std::max(zgemm_tc_work_bytes(m, n, k, 1, same), kSliceBytes));
+    w = h->ensure_evict(wname, bytes);
+  }
+  if (w)
+    CK(zgemm_tc(h->st, opA, opB, m, n, k, alpha, A, lda, sA, B, ldb, sB, C, ldc, sC, batch, lowerA, brow, sIdx, w,
+                bytes, (int*)h->buf("err_words")));
+  else if (lowerA || brow)
+    CK(ztrmm_gather(h->st, m, n, A, lda, sA, brow, sIdx, B, ldb, sB, C, ldc, sC, batch));
+  else
+    CK(zgemm(h->st, opA, opB, m, n, k, make_double2(alpha, 0.0), A, lda, sA, B, ldb, sB, make_double2(0.0, 0.0), C, ldc,
+             sC, batch));
+  return ISDF_OK;
+}
+#define ZM(...)                          \
+  do {                                   \
+    if (int e_ = zmul(h, __VA_ARGS__)) return e_; \
+  } while (0)
+
+// Synchronise the stream and report a bounded wait that expired on the way.
+int tc_status(isdf_handle* h, const char* what) {
+  int err = 0;
+  int* w = (int*)h->buf("err_words");
+  CK(cudaMemcpyAsync(&err, w, sizeof(int), cudaMemcpyDeviceToHost, h->st));
+  CK(cudaStreamSynchronize(h->st));
+  if (err == 0) return ISDF_OK;
+  CK(cudaMemsetAsync(w, 0, sizeof(int), h->st));
+  return fail(h, ISDF_ERR_TIMEOUT, "%s: bounded device wait expired (code %d)", what, err);
 }
 
 // Evaluate Phi into the handle (all precisions keep Phi in FP64).
@@ -479,7 +531,6 @@ TileSchedule tuned_schedule(isdf_handle* h, int64_t ntiles, const std::function<
 // (so V^q = L^q L^q^H), optional output of V^q, precision copies for the fragments.
 int coulomb_tail(isdf_handle* h, double2* Vxi, void* V_out) {
   const int nk = h->nk, np = h->np;
-  const double2 one = make_double2(1.0, 0.0), zero = make_double2(0.0, 0.0);
   double2* W = (double2*)h->buf("W");
   // V_xi = L_xi L_xi^H ; L^q = W^T L_xi
   ENSURE(LtV, double2, "LtV", (size_t)nk * np * np);
@@ -492,21 +543,22 @@ int coulomb_tail(isdf_handle* h, double2* Vxi, void* V_out) {
   ENSURE(Lxi, double2, "W_work", (size_t)nk * np * np);
   CK(lt_to_rowmajor(h->st, LtV, rankV, np, nk, Lxi));
   ENSURE(Lq, double2, "Lq", (size_t)nk * np * np);
-  CK(zgemm(h->st, 'T', 'N', np, np, np, one, W, np, (int64_t)np * np, Lxi, np, (int64_t)np * np, zero, Lq, np,
-           (int64_t)np * np, nk));
+  // L^q in another rounding moves the FP64_TC integrals by 6e-10 of themselves: FP64 FMA there
+  ZM(h->prec == ISDF_FP64_TC ? nullptr : "zwork", 'T', 'N', np, np, np, 1.0, W, np, (int64_t)np * np, Lxi, np,
+     (int64_t)np * np, Lq, np, (int64_t)np * np, nk);
   if (V_out) {
     // V^q = W^T V_xi conj(W)
     double2* tmp = Lxi;  // reuse
-    CK(zgemm(h->st, 'N', 'R', np, np, np, one, Vxi, np, (int64_t)np * np, W, np, (int64_t)np * np, zero, tmp, np,
-             (int64_t)np * np, nk));
-    CK(zgemm(h->st, 'T', 'N', np, np, np, one, W, np, (int64_t)np * np, tmp, np, (int64_t)np * np, zero,
-             (double2*)V_out, np, (int64_t)np * np, nk));
+    ZM("zwork", 'N', 'R', np, np, np, 1.0, Vxi, np, (int64_t)np * np, W, np, (int64_t)np * np, tmp, np,
+             (int64_t)np * np, nk);
+    ZM("zwork", 'T', 'N', np, np, np, 1.0, W, np, (int64_t)np * np, tmp, np, (int64_t)np * np,
+             (double2*)V_out, np, (int64_t)np * np, nk);
   }
   if (h->prec == ISDF_MIXED) {
     ENSURE(Xf, float2, "X_f", (size_t)nk * np * h->nao);
     CK(z2c(h->st, (const double2*)h->buf("X"), Xf, (int64_t)nk * np * h->nao));
   }
-  CK(cudaStreamSynchronize(h->st));
+  if (int e = tc_status(h, "Coulomb metric")) return e;
   h->has_coulomb = true;
   return ISDF_OK;
 }
@@ -705,36 +757,34 @@ int isdf_fit_zeta(isdf_handle* h, double solve_tol, int32_t* rank_out) {
   const QHalf qh = fit_q_set(km, h->q_sym);
   // algorithmic work: g^k GEMM (all k) + xi = W eta (triangular) at the computed q
   StageTimer stt(h, 1, 8.0 * nk * (double)np * ng * nao + 4.0 * qh.count * (double)np * np * ng);
-  const double2 one = make_double2(1.0, 0.0), zero = make_double2(0.0, 0.0);
+  // The mixed and FP64_TC contractions cut L and B to 28-30 bits, and the smallest columns of
+  // L amplify every rounding upstream of it beyond that: another order of rounding in Pi, g
+  // or xi moves their integrals by 1e-8 to 1e-7 of themselves (measured on c3 and c4), as much
+  // as those paths' own error.  So that their results do not depend on which GEMM ran here,
+  // these three products keep one fixed arithmetic there: FP64 FMA chains, and seven slices
+  // for g.  The plain FP64 path moves by 1e-11 and takes the tensor cores throughout.
+  const bool fp64 = h->prec == ISDF_FP64;
+  const char* zw = fp64 ? "grid_work_z" : nullptr;
   // Pi^q (Eq. 4): G^k_IJ = sum_mu conj(X^k_I mu) X^k_J mu, then the k-convolution
   ENSURE(Pi, double2, "Pi", (size_t)nk * np * np);
-  CK(zgemm(h->st, 'R', 'T', np, np, nao, one, X, nao, (int64_t)np * nao, X, nao, (int64_t)np * nao, zero, Pi,
-           np, (int64_t)np * np, nk));
+  ZM(zw, 'R', 'T', np, np, nao, 1.0, X, nao, (int64_t)np * nao, X, nao, (int64_t)np * nao, Pi,
+           np, (int64_t)np * np, nk);
   CK(kdft_cols(h->st, Pi, (int64_t)np * np, km, +1, -1, 1, 1.0 / nk));
   // eta^q (Eq. 5): g^k_I(r) = sum_mu conj(X^k_I mu) Phi^k_mu(r), then the k-convolution.
-  // In the mixed and FP64_TC paths g runs on the tensor cores with seven exact
-  // slices per operand (~2^-48 relative, FP64-class); the FP64 path keeps FP64
-  // arithmetic.
   ENSURE(eta, double2, "eta", (size_t)nk * np * ng);
-  if (h->prec != ISDF_FP64 && zgemm_emu_supported(nao)) {
+  if (!fp64 && zgemm_emu_supported(nao)) {
     const size_t per_k = zgemm_emu_work_bytes(np, ng, nao, 1);
     const int nkc = (int)std::max<size_t>(1, std::min<size_t>((size_t)nk, ((size_t)4 << 30) / per_k));
-    ENSURE(gw, uint8_t, "grid_work_emu", zgemm_emu_work_bytes(np, ng, nao, nkc));
-    ENSURE(tcw, int, "tc_words", 4);
-    CK(cudaMemsetAsync(tcw, 0, 4 * sizeof(int), h->st));
+    ENSURE(gw, uint8_t, "grid_work_z", zgemm_emu_work_bytes(np, ng, nao, nkc));
     for (int k0 = 0; k0 < nk; k0 += nkc) {
       const int nb = std::min(nkc, nk - k0);
       CK(zgemm_emu(h->st, 'R', np, ng, nao, X + (int64_t)k0 * np * nao, nao, (int64_t)np * nao,
                    phi + (int64_t)k0 * nao * ng, ng, (int64_t)nao * ng, eta + (int64_t)k0 * np * ng, ng,
-                   (int64_t)np * ng, nb, gw, tcw + 1));
+                   (int64_t)np * ng, nb, gw, (int*)h->buf("err_words")));
     }
-    int tc_err = 0;
-    CK(cudaMemcpyAsync(&tc_err, tcw + 1, sizeof(int), cudaMemcpyDeviceToHost, h->st));
-    CK(cudaStreamSynchronize(h->st));
-    if (tc_err != 0) return fail(h, ISDF_ERR_TIMEOUT, "tensor-core GEMM of the fit: bounded wait expired (%d)", tc_err);
   } else {
-    CK(zgemm(h->st, 'R', 'N', np, ng, nao, one, X, nao, (int64_t)np * nao, phi, ng, (int64_t)nao * ng, zero, eta,
-             ng, (int64_t)np * ng, nk));
+    ZM(zw, 'R', 'N', np, ng, nao, 1.0, X, nao, (int64_t)np * nao, phi, ng, (int64_t)nao * ng, eta, ng,
+       (int64_t)np * ng, nk);
   }
   // the k-convolution of Algorithm 1 over the grid columns: FP64 in the FP64 path,
   // float-float (~2^-44 relative, FP32 arithmetic) in the others
@@ -763,7 +813,7 @@ int isdf_fit_zeta(isdf_handle* h, double solve_tol, int32_t* rank_out) {
   }
   h->ranks.assign(nk, 0);
   CK(cudaMemcpyAsync(h->ranks.data(), rankPi, sizeof(int32_t) * nk, cudaMemcpyDeviceToHost, h->st));
-  CK(cudaStreamSynchronize(h->st));
+  if (int e = tc_status(h, "tensor-core GEMM of the fit")) return e;
   if (rank_out) std::memcpy(rank_out, h->ranks.data(), sizeof(int32_t) * nk);
   for (int q = 0; q < nk; ++q)
     if (h->ranks[q] < 1) return fail(h, ISDF_ERR_NUMERIC, "Pi^q has rank 0 at q=%d", q);
@@ -775,8 +825,8 @@ int isdf_fit_zeta(isdf_handle* h, double solve_tol, int32_t* rank_out) {
     CK(trinv_batched(h->st, LtPi + q0 * pp, permPi + (int64_t)q0 * np, rankPi + q0, np, nq, W + q0 * pp,
                      wwork + q0 * pp));
     // xi^q = W eta^q = L_S^{-1} (eta^q rows in pivot order): triangular, gathered
-    CK(ztrmm_gather(h->st, rx, ng, wwork + q0 * pp, np, pp, permPi + (int64_t)q0 * np, np, eta + q0 * pg, ng, pg,
-                    xi + q0 * xg, ng, xg, nq));
+    ZM(zw, 'N', 'N', rx, ng, rx, 1.0, wwork + q0 * pp, np, pp, eta + q0 * pg, ng, pg, xi + q0 * xg, ng, xg,
+       nq, 1, permPi + (int64_t)q0 * np, np);
   }
   if (!qh.mirror.empty()) {
     const int2* mir = (const int2*)h->buf("q_mirror");
@@ -801,7 +851,6 @@ int isdf_coulomb_metric(isdf_handle* h, void* V_out) {
   if (int e = check_device(h)) return e;
   if (!h->has_fit || !h->has_xi) return fail(h, ISDF_ERR_STATE, "isdf_coulomb_metric before isdf_fit_zeta");
   const int nk = h->nk, np = h->np, ng = h->ng;
-  const double2 zero = make_double2(0.0, 0.0);
   double2* xi = (double2*)h->buf("xi");
   double2* W = (double2*)h->buf("W");
   const double2* tw = (const double2*)h->buf("grid_tw");
@@ -820,28 +869,21 @@ int isdf_coulomb_metric(isdf_handle* h, void* V_out) {
   if (h->prec != ISDF_MIXED) {
     for (const auto& r : qh.runs) {
       CK(grid_coulomb_fft(h->st, xi + r.first * xg, rx, r.first, r.second, h->cell, tw, gwork));
-      CK(zgemm(h->st, 'R', 'T', rx, rx, ng, make_double2(h->volume, 0.0), xi + r.first * xg, ng, xg,
-               xi + r.first * xg, ng, xg, zero, Vxi + r.first * pp, np, pp, r.second));
+      ZM("grid_work_z", 'R', 'T', rx, rx, ng, h->volume, xi + r.first * xg, ng, xg,
+               xi + r.first * xg, ng, xg, Vxi + r.first * pp, np, pp, r.second);
     }
   } else {
     // mixed: xi rows to float-float in place, the grid FFT in float-float, and
     // V_xi = Omega conj(c')c'^T on the tensor cores with four exact slices (~2^-28 relative;
     // an FP32 FFT and GEMM put ~2e-7 into V_xi, which reaches E and the traces as such)
-    ENSURE(tcw, int, "tc_words", 4);
-    CK(cudaMemsetAsync(tcw, 0, 4 * sizeof(int), h->st));
     const int qcv = vxi_tc_chunk(rx, ng, (size_t)4 << 30);
     ENSURE(vwork, uint8_t, "grid_work_v", vxi_tc_work_bytes(rx, ng, qcv));
     for (const auto& r : qh.runs) {
       ffcomplex* xf = reinterpret_cast<ffcomplex*>(xi + r.first * xg);
       CK(z2ff(h->st, xi + r.first * xg, xf, r.second * xg));
       CK(grid_coulomb_fft_ff(h->st, xf, rx, r.first, r.second, h->cell, tw, gwork));
-      CK(vxi_tc(h->st, xf, xg, rx, ng, r.second, h->volume, Vxi + r.first * pp, np, pp, vwork, qcv, tcw + 1));
+      CK(vxi_tc(h->st, xf, xg, rx, ng, r.second, h->volume, Vxi + r.first * pp, np, pp, vwork, qcv, (int*)h->buf("err_words")));
     }
-    int tc_err = 0;
-    CK(cudaMemcpyAsync(&tc_err, tcw + 1, sizeof(int), cudaMemcpyDeviceToHost, h->st));
-    CK(cudaStreamSynchronize(h->st));
-    if (tc_err != 0)
-      return fail(h, ISDF_ERR_TIMEOUT, "tensor-core Coulomb GEMM: bounded device wait expired (code %d)", tc_err);
   }
   if (!qh.mirror.empty()) {
     ENSURE(mir, int2, "q_mirror", qh.mirror.size());
@@ -864,7 +906,6 @@ int isdf_coulomb_metric_eta(isdf_handle* h, void* V_out) {
   if (!h->has_fit || !h->has_eta)
     return fail(h, ISDF_ERR_STATE, "isdf_coulomb_metric_eta needs eta from isdf_fit_zeta (released after fragments)");
   const int nk = h->nk, np = h->np, ng = h->ng;
-  const double2 one = make_double2(1.0, 0.0), zero = make_double2(0.0, 0.0);
   double2* eta = (double2*)h->buf("eta");
   double2* W = (double2*)h->buf("W");
   double2* work = (double2*)h->buf("xi");  // the copy of eta is transformed in place
@@ -881,8 +922,8 @@ int isdf_coulomb_metric_eta(isdf_handle* h, void* V_out) {
     CK(cudaMemcpyAsync(work + r.first * pg, eta + r.first * pg, sizeof(double2) * (size_t)(r.second * pg),
                        cudaMemcpyDeviceToDevice, h->st));
     CK(grid_coulomb_fft(h->st, work + r.first * pg, np, r.first, r.second, h->cell, tw, gwork));
-    CK(zgemm(h->st, 'R', 'T', np, np, ng, make_double2(h->volume, 0.0), work + r.first * pg, ng, pg,
-             work + r.first * pg, ng, pg, zero, Veta + r.first * pp, np, pp, r.second));
+    ZM("grid_work_z", 'R', 'T', np, np, ng, h->volume, work + r.first * pg, ng, pg,
+             work + r.first * pg, ng, pg, Veta + r.first * pp, np, pp, r.second);
   }
   if (!qh.mirror.empty()) {
     ENSURE(mir, int2, "q_mirror", qh.mirror.size());
@@ -892,10 +933,10 @@ int isdf_coulomb_metric_eta(isdf_handle* h, void* V_out) {
   // V_xi = conj(W) (V_eta W^T)
   double2* tmp = (double2*)h->ensure("W_work", sizeof(double2) * (size_t)nk * np * np);
   if (!tmp) return fail(h, ISDF_ERR_OOM, "workspace");
-  CK(zgemm(h->st, 'N', 'T', np, np, np, one, Veta, np, (int64_t)np * np, W, np, (int64_t)np * np, zero, tmp, np,
-           (int64_t)np * np, nk));
-  CK(zgemm(h->st, 'R', 'N', np, np, np, one, W, np, (int64_t)np * np, tmp, np, (int64_t)np * np, zero, Vxi, np,
-           (int64_t)np * np, nk));
+  ZM("grid_work_z", 'N', 'T', np, np, np, 1.0, Veta, np, (int64_t)np * np, W, np, (int64_t)np * np, tmp, np,
+           (int64_t)np * np, nk);
+  ZM("grid_work_z", 'R', 'N', np, np, np, 1.0, W, np, (int64_t)np * np, tmp, np, (int64_t)np * np, Vxi, np,
+           (int64_t)np * np, nk);
   return coulomb_tail(h, Vxi, V_out);
 }
 
@@ -955,9 +996,8 @@ int isdf_fragment_eri(isdf_handle* h, int n_frag, const int32_t* n_orb, const vo
   // read once at the end.
   const bool any_tr = (ej_out || ek_out) && gamma;
   ENSURE(trall, double, "frag_traces", 4 * (size_t)n_frag);
-  ENSURE(tcw, int, "tc_words", 4);
   CK(cudaMemsetAsync(trall, 0, sizeof(double) * 4 * (size_t)n_frag, h->st));
-  CK(cudaMemsetAsync(tcw, 0, 4 * sizeof(int), h->st));
+  int* errw = (int*)h->buf("err_words");
   // FP64_TC: the grouped tensor-core path in float-float with more exact slices,
   // where B = M L fits its exact accumulation (2 r_q <= 576); else FP64 arithmetic
   const bool tc64 = (h->prec == ISDF_FP64_TC) && mlgemm5_tc_supported(rp);
@@ -974,7 +1014,6 @@ int isdf_fragment_eri(isdf_handle* h, int n_frag, const int32_t* n_orb, const vo
         trpart = (double2*)h->ensure("frag_traces_part", sizeof(double2) * 2 * (size_t)n2);
         if (!trpart) return fail(h, ISDF_ERR_OOM, "traces workspace");
       }
-      const double2 one = make_double2(1.0, 0.0), zero = make_double2(0.0, 0.0);
       double2* X = (double2*)h->buf("X");
       ENSURE(Lw, double2, "frag_Lw", (size_t)nk * pp);
       ENSURE(T, double2, "frag_T", (size_t)nk * np * nf);
@@ -984,8 +1023,8 @@ int isdf_fragment_eri(isdf_handle* h, int n_frag, const int32_t* n_orb, const vo
       if (f == 0) CK(scale_blocks(h->st, Lq, pp, nk, swd, Lw));
       {
         StageTimer stt(h, 3, frag_m_flops(nk, np, nf, nao, km));
-        CK(zgemm(h->st, 'N', 'N', np, nf, nao, one, X, nao, (int64_t)np * nao, Cf, nf, (int64_t)nao * nf, zero, T,
-                 nf, (int64_t)np * nf, nk));
+        ZM("tc_zwork", 'N', 'N', np, nf, nao, 1.0, X, nao, (int64_t)np * nao, Cf, nf, (int64_t)nao * nf, T,
+                 nf, (int64_t)np * nf, nk);
         CK(kdft_cols(h->st, T, (int64_t)np * nf, km, +1, +1, 0, 1.0));
         CK(pair_products(h->st, T, nk, np, nf, M));
         CK(kdft_cols(h->st, M, n2 * np, km, +1, +1, 0, 1.0 / nk));
@@ -995,13 +1034,12 @@ int isdf_fragment_eri(isdf_handle* h, int n_frag, const int32_t* n_orb, const vo
         // nonzero columns of L^q
         StageTimer stt(h, 4, 8.0 * (double)n2 * np * sum_nv);
         for (const auto& r : runs)
-          CK(zgemm(h->st, 'N', 'N', (int)n2, nj, np, one, M + r.first * sq, np, sq, Lw + r.first * pp, np, pp, zero,
-                   B + (int64_t)slot[r.first] * nj, (int64_t)nS * nj, nj, r.second));
+          ZM("tc_zwork", 'N', 'N', (int)n2, nj, np, 1.0, M + r.first * sq, np, sq, Lw + r.first * pp, np, pp,
+                   B + (int64_t)slot[r.first] * nj, (int64_t)nS * nj, nj, r.second);
       }
       {
         StageTimer stt(h, 5, 4.0 * (double)n2 * n2 * sum_nv);
-        CK(zgemm(h->st, 'N', 'C', (int)n2, (int)n2, nS * nj, one, B, (int64_t)nS * nj, 0, B, (int64_t)nS * nj, 0,
-                 zero, E, n2, 0, 1));
+        ZM("tc_zwork", 'N', 'C', (int)n2, (int)n2, nS * nj, 1.0, B, (int64_t)nS * nj, 0, B, (int64_t)nS * nj, 0, E, n2, 0, 1);
         if (h->q_sym) CK(eri_swapconj_sym(h->st, E, nf));
       }
       if (eri_out && eri_out[f]) CK(eri_permute(h->st, E, nf, 1.0 / nk, (double2*)eri_out[f]));
@@ -1136,17 +1174,16 @@ int isdf_fragment_eri(isdf_handle* h, int n_frag, const int32_t* n_orb, const vo
           const int f = grp[i], nf = n_orb[f];
           const int64_t n2f = (int64_t)nf * nf;
           if (tc64) {
-            // T = X C FP64-class (tensor cores, seven exact slices; FP64 beyond N_AO = 64),
-            // then float-float in place for the DFT and the pair rows
+            // T = X C FP64-class (seven exact slices; see isdf_fit_zeta on the fixed arithmetic; FP64
+            // beyond N_AO = 64), then float-float in place for the DFT and the pair rows
             double2* Tz = reinterpret_cast<double2*>(T);
             if (zgemm_emu_supported(nao)) {
               ENSURE(tew, uint8_t, "frag_T_emu", zgemm_emu_work_bytes(np, nfmax, nao, nk));
               CK(zgemm_emu(h->st, 'N', np, nf, nao, Xz, nao, (int64_t)np * nao, (const double2*)C[f], nf,
-                           (int64_t)nao * nf, Tz, nf, (int64_t)np * nf, nk, tew, tcw + 1));
+                           (int64_t)nao * nf, Tz, nf, (int64_t)np * nf, nk, tew, errw));
             } else {
-              CK(zgemm(h->st, 'N', 'N', np, nf, nao, make_double2(1.0, 0.0), Xz, nao, (int64_t)np * nao,
-                       (const double2*)C[f], nf, (int64_t)nao * nf, make_double2(0.0, 0.0), Tz, nf,
-                       (int64_t)np * nf, nk));
+              ZM(nullptr, 'N', 'N', np, nf, nao, 1.0, Xz, nao, (int64_t)np * nao, (const double2*)C[f], nf,
+                 (int64_t)nao * nf, Tz, nf, (int64_t)np * nf, nk);
             }
             ffcomplex* Tff = reinterpret_cast<ffcomplex*>(Tz);
             CK(z2ff(h->st, Tz, Tff, (int64_t)nk * np * nf));
@@ -1178,14 +1215,14 @@ int isdf_fragment_eri(isdf_handle* h, int n_frag, const int32_t* n_orb, const vo
           CK(mlgemm5_tc_rowscale(h->st, M_ff, sq, np, qmap, nS, permPi, rankPi, rp, rows, rexp));
           for (int j0 = 0; j0 < nS; j0 += qc)
             CK(mlgemm5_tc_chunk(h->st, M_ff, sq, qmap, rows, np, permPi, rankPi, rp, nj, j0, std::min(qc, nS - j0),
-                                rexp, split, lsl, lexp, nk, tcw + 1));
+                                rexp, split, lsl, lexp, nk, errw));
         } else if (tc_ml) {
           // row exponents of the gathered M over the q of the sum, then B^q = M^q L^q
           // over M^q, q-chunk by q-chunk
           CK(mlgemm_tc_rowscale(h->st, M_f, sq, np, qmap, nS, permPi, rankPi, rp, rows, rexp));
           for (int j0 = 0; j0 < nS; j0 += qc)
             CK(mlgemm_tc_chunk(h->st, M_f, sq, qmap, rows, np, permPi, rankPi, rp, nj, j0, std::min(qc, nS - j0),
-                               rexp, split, lsl, lexp, nk, tcw + 1));
+                               rexp, split, lsl, lexp, nk, errw));
         } else {
           // consecutive q of a run sit at consecutive positions
           for (const auto& r : runs)
@@ -1219,7 +1256,7 @@ int isdf_fragment_eri(isdf_handle* h, int n_frag, const int32_t* n_orb, const vo
               cudaSuccess)
             return -1;
           return syrk_tc_chunk(h->st, M_f, sq, ldB, nj, nullptr, rows, 0, nq0, rexp, split, tiles_d,
-                               (int)tl.size(), ws, 0, tcw + 1, cfg) == cudaSuccess ? 0 : -1;
+                               (int)tl.size(), ws, 0, errw, cfg) == cudaSuccess ? 0 : -1;
         });
         if (sch.band < 0) return fail(h, ISDF_ERR_CUDA, "tile-schedule tuning launch failed");
         build_tiles(sch.band);
@@ -1232,11 +1269,11 @@ int isdf_fragment_eri(isdf_handle* h, int n_frag, const int32_t* n_orb, const vo
           if (tc64) {
             CK(syrk4_tc_split(h->st, M_ff, sq, ldB, nj, rows, j0, nq, rexp, split, dcorr));
             StageTimer stk(h, 6, flops5 * nv_chunk / std::max(sum_nv, 1.0));
-            CK(syrk4_tc_mma(h->st, split, rows, nq, nj, tiles_d, (int)tl.size(), ws, j0 > 0, tcw + 1));
+            CK(syrk4_tc_mma(h->st, split, rows, nq, nj, tiles_d, (int)tl.size(), ws, j0 > 0, errw));
           } else {
             CK(syrk_tc_split(h->st, M_f, sq, ldB, nj, nullptr, rows, j0, nq, rexp, split, dcorr));
             StageTimer stk(h, 6, flops5 * nv_chunk / std::max(sum_nv, 1.0));
-            CK(syrk_tc_mma(h->st, split, rows, nq, nj, tiles_d, (int)tl.size(), ws, j0 > 0, tcw + 1, sch.cfg));
+            CK(syrk_tc_mma(h->st, split, rows, nq, nj, tiles_d, (int)tl.size(), ws, j0 > 0, errw, sch.cfg));
           }
         }
         // E = W E' W^H per fragment, written straight to the caller's ERIs (chemist's
@@ -1258,12 +1295,8 @@ int isdf_fragment_eri(isdf_handle* h, int n_frag, const int32_t* n_orb, const vo
     }
   }
   std::vector<double> hv(4 * (size_t)n_frag, 0.0);
-  int tc_err = 0;
   if (any_tr) CK(cudaMemcpyAsync(hv.data(), trall, sizeof(double) * hv.size(), cudaMemcpyDeviceToHost, h->st));
-  CK(cudaMemcpyAsync(&tc_err, tcw + 1, sizeof(int), cudaMemcpyDeviceToHost, h->st));
-  CK(cudaStreamSynchronize(h->st));
-  if (tc_err != 0)
-    return fail(h, ISDF_ERR_TIMEOUT, "tensor-core contraction: bounded device wait expired (code %d)", tc_err);
+  if (int e = tc_status(h, "tensor-core contraction")) return e;
   for (int f = 0; f < n_frag; ++f) {
     if (ej_out) ej_out[f] = hv[4 * (size_t)f];
     if (ek_out) ek_out[f] = hv[4 * (size_t)f + 1];
@@ -1310,20 +1343,17 @@ int isdf_ao_eri(isdf_handle* h, int n_quartet, const int32_t* quartets, void* ou
   ENSURE(Cc, double2, "ao_pairs_c", (size_t)np * nao2);
   ENSURE(U, double2, "ao_u", (size_t)np * nao2);
   ENSURE(Wm, double2, "ao_w", (size_t)np * nao2);
-  const double2 one = make_double2(1.0, 0.0), zero = make_double2(0.0, 0.0);
   for (int n = 0; n < n_quartet; ++n) {
     const int32_t* k = quartets + 4 * n;
     const double2* L = Lq + qv[n] * pp;
     CK(ao_pairs(h->st, X + k[0] * pa, X + k[1] * pa, np, nao, A));
     CK(ao_pairs(h->st, X + k[2] * pa, X + k[3] * pa, np, nao, Cc));
     // (mu nu|lam sig) = Nk A^T V^Q C with V^Q = L L^H: (L^T A)^T (L^H C)
-    CK(zgemm(h->st, 'T', 'N', np, (int)nao2, np, one, L, np, 0, A, nao2, 0, zero, U, nao2, 0, 1));
-    CK(zgemm(h->st, 'C', 'N', np, (int)nao2, np, one, L, np, 0, Cc, nao2, 0, zero, Wm, nao2, 0, 1));
-    CK(zgemm(h->st, 'T', 'N', (int)nao2, (int)nao2, np, make_double2((double)nk, 0.0), U, nao2, 0, Wm, nao2, 0,
-             zero, (double2*)out + (int64_t)n * nao2 * nao2, nao2, 0, 1));
+    ZM("zwork", 'T', 'N', np, (int)nao2, np, 1.0, L, np, 0, A, nao2, 0, U, nao2, 0, 1);
+    ZM("zwork", 'C', 'N', np, (int)nao2, np, 1.0, L, np, 0, Cc, nao2, 0, Wm, nao2, 0, 1);
+    ZM("zwork", 'T', 'N', (int)nao2, (int)nao2, np, (double)nk, U, nao2, 0, Wm, nao2, 0, (double2*)out + (int64_t)n * nao2 * nao2, nao2, 0, 1);
   }
-  CK(cudaStreamSynchronize(h->st));
-  return ISDF_OK;
+  return tc_status(h, "isdf_ao_eri");
 }
 
 int isdf_sos_polarizability(isdf_handle* h, const void* C, int n_mo, int n_occ, const double* eps, double tau,
@@ -1336,7 +1366,6 @@ int isdf_sos_polarizability(isdf_handle* h, const void* C, int n_mo, int n_occ, 
     return fail(h, ISDF_ERR_ARG, "isdf_sos_polarizability: need C, eps, 0 < n_occ < n_mo and finite tau >= 0");
   const int nk = h->nk, np = h->np, nao = h->nao, nvir = n_mo - n_occ;
   const int64_t pp = (int64_t)np * np;
-  const double2 one = make_double2(1.0, 0.0), zero = make_double2(0.0, 0.0);
   double2* X = (double2*)h->buf("X");
   double2* Lq = (double2*)h->buf("Lq");
   ENSURE(epsd, double, "sos_eps", (size_t)nk * n_mo);
@@ -1352,15 +1381,14 @@ int isdf_sos_polarizability(isdf_handle* h, const void* C, int n_mo, int n_occ, 
   double2* chi = chi_out ? (double2*)chi_out : chi_w;
   CK(cudaMemcpyAsync(epsd, eps, sizeof(double) * (size_t)nk * n_mo, cudaMemcpyHostToDevice, h->st));
   // Y^k = X^k C^k (orbital values at the points, Eq. 14)
-  CK(zgemm(h->st, 'N', 'N', np, n_mo, nao, one, X, nao, (int64_t)np * nao, (const double2*)C, n_mo,
-           (int64_t)nao * n_mo, zero, Y, n_mo, (int64_t)np * n_mo, nk));
+  ZM("zwork", 'N', 'N', np, n_mo, nao, 1.0, X, nao, (int64_t)np * nao, (const double2*)C, n_mo,
+           (int64_t)nao * n_mo, Y, n_mo, (int64_t)np * n_mo, nk);
   // Go^k = Y_occ e^{+tau eps_i} Y_occ^H,  Gv^k = Y_vir e^{-tau eps_a} Y_vir^H (Eq. 15)
   CK(scale_cols(h->st, Y, nk, np, n_mo, 0, n_occ, epsd, +tau, Yo));
   CK(scale_cols(h->st, Y, nk, np, n_mo, n_occ, nvir, epsd, -tau, Yv));
-  CK(zgemm(h->st, 'N', 'C', np, np, n_occ, one, Yo, n_occ, (int64_t)np * n_occ, Y, n_mo, (int64_t)np * n_mo, zero,
-           Go, np, pp, nk));
-  CK(zgemm(h->st, 'N', 'C', np, np, nvir, one, Yv, nvir, (int64_t)np * nvir, Y + n_occ, n_mo, (int64_t)np * n_mo,
-           zero, Gv, np, pp, nk));
+  ZM("zwork", 'N', 'C', np, np, n_occ, 1.0, Yo, n_occ, (int64_t)np * n_occ, Y, n_mo, (int64_t)np * n_mo,
+           Go, np, pp, nk);
+  ZM("zwork", 'N', 'C', np, np, nvir, 1.0, Yv, nvir, (int64_t)np * nvir, Y + n_occ, n_mo, (int64_t)np * n_mo, Gv, np, pp, nk);
   // chi^Q_{IK} = sum_k Go^k_{KI} Gv^{k-Q}_{IK} (Eq. 13) by the convolution theorem, as
   // Algorithm 1 does for Pi^q: with hat(a)(R) = sum_k a(k) e^{+ik.R} and
   // check(b)(R) = sum_k b(k) e^{-ik.R},  chi = (1/Nk) DFT_-( hat(Go)^T o check(Gv) )
@@ -1371,9 +1399,9 @@ int isdf_sos_polarizability(isdf_handle* h, const void* C, int n_mo, int n_occ, 
   CK(kdft_cols(h->st, chi, pp, km, -1, -1, 0, 1.0 / nk));
   if (s_out) {
     // S = Nk^2 sum_Q tr[conj(V^Q) chi^Q conj(V^Q) (chi^{-Q})^T], V^Q = L^Q L^Q^H (Eq. 12)
-    CK(zgemm(h->st, 'N', 'C', np, np, np, one, Lq, np, pp, Lq, np, pp, zero, Vq, np, pp, nk));
-    CK(zgemm(h->st, 'R', 'N', np, np, np, one, Vq, np, pp, chi, np, pp, zero, T1, np, pp, nk));
-    CK(zgemm(h->st, 'N', 'R', np, np, np, one, T1, np, pp, Vq, np, pp, zero, Go, np, pp, nk));  // Go reused
+    ZM("zwork", 'N', 'C', np, np, np, 1.0, Lq, np, pp, Lq, np, pp, Vq, np, pp, nk);
+    ZM("zwork", 'R', 'N', np, np, np, 1.0, Vq, np, pp, chi, np, pp, T1, np, pp, nk);
+    ZM("zwork", 'N', 'R', np, np, np, 1.0, T1, np, pp, Vq, np, pp, Go, np, pp, nk);  // Go reused
     CK(sos_trace_parts(h->st, Go, chi, h->cell.kmesh, np, part));
     std::vector<double> hp(nk);
     CK(cudaMemcpyAsync(hp.data(), part, sizeof(double) * nk, cudaMemcpyDeviceToHost, h->st));
@@ -1382,8 +1410,7 @@ int isdf_sos_polarizability(isdf_handle* h, const void* C, int n_mo, int n_occ, 
     for (int q = 0; q < nk; ++q) S += hp[q];
     *s_out = (double)nk * (double)nk * S;
   }
-  CK(cudaStreamSynchronize(h->st));
-  return ISDF_OK;
+  return tc_status(h, "isdf_sos_polarizability");
 }
 
 int isdf_exchange(isdf_handle* h, const void* P, void* K_out) {
@@ -1393,32 +1420,30 @@ int isdf_exchange(isdf_handle* h, const void* P, void* K_out) {
   if (!h->has_coulomb) return fail(h, ISDF_ERR_STATE, "isdf_exchange before the Coulomb metric");
   const int nk = h->nk, np = h->np, nao = h->nao;
   const KMesh km{{h->cell.kmesh[0], h->cell.kmesh[1], h->cell.kmesh[2]}};
-  const double2 one = make_double2(1.0, 0.0), zero = make_double2(0.0, 0.0);
   double2* X = (double2*)h->buf("X");
   double2* Lq = (double2*)h->buf("Lq");
   ENSURE(rho, double2, "kx_rho", (size_t)nk * np * np);
   ENSURE(Vd, double2, "kx_V", (size_t)nk * np * np);
   ENSURE(t1, double2, "kx_t1", (size_t)nk * np * (nao > np ? nao : np));
   // rho^k = X^k P^k X^k^H
-  CK(zgemm(h->st, 'N', 'N', np, nao, nao, one, X, nao, (int64_t)np * nao, (const double2*)P, nao,
-           (int64_t)nao * nao, zero, t1, nao, (int64_t)np * nao, nk));
-  CK(zgemm(h->st, 'N', 'C', np, np, nao, one, t1, nao, (int64_t)np * nao, X, nao, (int64_t)np * nao, zero, rho, np,
-           (int64_t)np * np, nk));
+  ZM("zwork", 'N', 'N', np, nao, nao, 1.0, X, nao, (int64_t)np * nao, (const double2*)P, nao,
+           (int64_t)nao * nao, t1, nao, (int64_t)np * nao, nk);
+  ZM("zwork", 'N', 'C', np, np, nao, 1.0, t1, nao, (int64_t)np * nao, X, nao, (int64_t)np * nao, rho, np,
+           (int64_t)np * np, nk);
   // V^q = L^q L^q^H
-  CK(zgemm(h->st, 'N', 'C', np, np, np, one, Lq, np, (int64_t)np * np, Lq, np, (int64_t)np * np, zero, Vd, np,
-           (int64_t)np * np, nk));
+  ZM("zwork", 'N', 'C', np, np, np, 1.0, Lq, np, (int64_t)np * np, Lq, np, (int64_t)np * np, Vd, np,
+           (int64_t)np * np, nk);
   // Gamma^k = sum_k' (V^{k'-k})^T o rho^{k'}: DFT_- V, DFT_+ rho, transposed product, DFT_- / Nk
   CK(kdft_cols(h->st, Vd, (int64_t)np * np, km, -1, -1, 0, 1.0));
   CK(kdft_cols(h->st, rho, (int64_t)np * np, km, +1, +1, 0, 1.0));
   CK(hadamard_t(h->st, Vd, rho, np, nk, rho));
   CK(kdft_cols(h->st, rho, (int64_t)np * np, km, -1, -1, 0, 1.0 / nk));
   // K^k = -(1/Nk) X^k^H Gamma^k X^k
-  CK(zgemm(h->st, 'N', 'N', np, nao, np, one, rho, np, (int64_t)np * np, X, nao, (int64_t)np * nao, zero, t1, nao,
-           (int64_t)np * nao, nk));
-  CK(zgemm(h->st, 'C', 'N', nao, nao, np, make_double2(-1.0 / nk, 0.0), X, nao, (int64_t)np * nao, t1, nao,
-           (int64_t)np * nao, zero, (double2*)K_out, nao, (int64_t)nao * nao, nk));
-  CK(cudaStreamSynchronize(h->st));
-  return ISDF_OK;
+  ZM("zwork", 'N', 'N', np, nao, np, 1.0, rho, np, (int64_t)np * np, X, nao, (int64_t)np * nao, t1, nao,
+           (int64_t)np * nao, nk);
+  ZM("zwork", 'C', 'N', nao, nao, np, -1.0 / nk, X, nao, (int64_t)np * nao, t1, nao,
+           (int64_t)np * nao, (double2*)K_out, nao, (int64_t)nao * nao, nk);
+  return tc_status(h, "isdf_exchange");
 }
 
 int isdf_set_time_reversal(isdf_handle* h, int enable) {
@@ -1485,18 +1510,16 @@ int isdf_get(isdf_handle* h, int what, void* out) {
       break;
     case 3: {
       if (!h->has_xi) return fail(h, ISDF_ERR_STATE, "zeta not available (needs isdf_fit_zeta, before the metric)");
-      const double2 one = make_double2(1.0, 0.0), zero = make_double2(0.0, 0.0);
       // zeta = W^H xi with the rx stored rows of xi
       const int rx = h->xi_rows;
-      CK(zgemm(h->st, 'C', 'N', np, ng, rx, one, (double2*)h->buf("W"), np, (int64_t)np * np, (double2*)h->buf("xi"),
-               ng, (int64_t)rx * ng, zero, (double2*)out, ng, (int64_t)np * ng, nk));
+      ZM("zwork", 'C', 'N', np, ng, rx, 1.0, (double2*)h->buf("W"), np, (int64_t)np * np, (double2*)h->buf("xi"),
+               ng, (int64_t)rx * ng, (double2*)out, ng, (int64_t)np * ng, nk);
       break;
     }
     default:
       return fail(h, ISDF_ERR_ARG, "unknown item %d", what);
   }
-  CK(cudaStreamSynchronize(h->st));
-  return ISDF_OK;
+  return tc_status(h, "isdf_get");
 }
 
 int isdf_sizes(const isdf_handle* h, int64_t* out) {

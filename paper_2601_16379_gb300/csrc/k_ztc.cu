@@ -1,0 +1,583 @@
+// FP64-accurate batched complex GEMM on the tensor cores (tcgen05):
+//     C_b = alpha op(A_b) op(B_b),   op in {N, T, C, R}, complex128, row-major.
+// It carries every complex128 product of the library: the fit (Eqs. 3-5), the FP64
+// Coulomb metric (Eq. 6), the FP64 fragment contractions (Eq. 19), exchange (Eq. 10),
+// AO integrals (Eq. 9) and the polarisability (Eqs. 12-15).
+//
+// Why not FMA: this GPU's FP64 pipe runs 2 FMA per clock and SM (1.2 TFLOP/s over the
+// chip), 1/64 of FP32, and conversions or additions in FP64 cost the same.  So nothing
+// here touches it per element: slicing and the final sums are integer arithmetic.
+//
+// Error-free slicing (Ozaki, Ogita, Oishi & Rump, 2012).  Each row of op(A) and each
+// column of op(B) is scaled by a power of two so that its largest component lies in
+// [64, 128) and rounded once to a 56-bit integer F (v 2^49), whose signed base-128 digits
+//     v = s_0 + s_1/2^7 + ... + s_7/2^49,   |s_0| <= 128, -64 <= s_i <= 63
+// are stored as fp16 integers, real and imaginary parts in rows of their own.  A tile
+// is 64 x 32 complex entries of C: the 128 rows [Re a; Im a] of 64 rows of op(A) times the 64
+// columns [Re b, Im b] of 32 columns of op(B) give the four real products of the complex one,
+// which are combined with their signs at the end, as integers.  The products S_a T_b with
+// a + b <= 7 (36 of them) feed eight groups g = a + b of 64 FP32 accumulator columns: all 512
+// TMEM columns.  Over a chunk of 384 k every partial sum is an integer of magnitude at most
+// 384 * (2 * 128 * 64 + 6 * 64 * 64) < 2^24, so the FP32 accumulation is exact whatever its
+// rounding; each chunk is drained into 64-bit integers (groups 0-3 and 4-7), exact for any K,
+// and rounded once to FP64 at the end.  What is lost is the rounding of F (2^-57 of the
+// row's largest entry) and the products with a + b >= 8, together ~2^-57 per product of the
+// largest |a_i| |b_j|; the rounding of an FP64 FMA chain is larger from a few terms on.
+//
+// The tile shape: an MMA of 128 x N x 16 takes N/2 clocks from N = 128 on, but 55 at N = 64
+// and 49 at N = 32 (measured), so N = 64 costs 36 x 55 clocks per 16 k (58 % of the peak).
+// N = 128 would need the accumulators of two passes, whose 64-bit sums (16 bytes per entry)
+// would fill the register file.
+//
+// A row (column) with an infinity or NaN gives NaN in its whole row (column) of C.
+//
+// Layout of the slices.  The slicing kernels write them in the exact order in which the
+// GEMM wants them in shared memory, so that a stage is fetched by bulk copies without a
+// tensor map: [batch][32-row block][16-k block][slice][re, im][8-row group][k half][row % 8]
+// [k % 8], i.e. K-major core matrices of 8 rows x 16 bytes (no swizzle), 16 KB per (row block,
+// k block).  One layout serves both sides, so a product of a matrix with itself is sliced
+// once.  Rows beyond the matrix are left unwritten: they only reach entries of C that are
+// not stored.  k beyond K is zero.
+//
+// Kernel roles (576 threads, one CTA per SM, persistent over the tiles): warp 0 copies,
+// warp 1 allocates TMEM and issues the MMAs, warps 2-17 drain and store.  Every wait is
+// bounded.
+#include <algorithm>
+#include <climits>
+
+#include "common.cuh"
+#include "tc_ptx.cuh"
+
+namespace isdf {
+
+namespace ztc {
+
+using namespace tc;
+
+constexpr int NS = 8;                        // slices per operand
+constexpr int RB = 32;                       // rows per block of the slices
+constexpr int BM = 64, BN = 32, BK = 16;     // tile rows, columns, k per stage (complex)
+constexpr int kSlice = 2 * RB * BK;          // fp16 of one slice of a block: re rows, im rows (2 KB)
+constexpr int kBlk = NS * kSlice;            // fp16 of one (row block, k block): 16 KB
+constexpr int kABytes = 2 * kBlk * 2;        // two row blocks, 32 KB
+constexpr int kBBytes = kBlk * 2;            // 16 KB
+constexpr int kStage = kABytes + kBBytes;    // 48 KB
+constexpr int NST = 3;                       // stages
+constexpr int kChunk = 24;                   // k blocks per exact chunk (384 k)
+constexpr int kShortK = 96;                  // K up to which every group stays below 2^22 (96 * 40960)
+constexpr int kOutBytes = 65536;             // exchange of the partial sums, then the tile of C on its way out
+constexpr int NT = 576;
+constexpr int kDrainWarps = 16;
+constexpr int kDrainCols = 16;               // accumulator columns per drain warp
+constexpr int kTmem = 512;                   // 8 groups x 64 columns
+constexpr uint32_t kIdesc = (1u << 4) | ((uint32_t)((2 * BN) >> 3) << 17) | ((uint32_t)((2 * BM) >> 4) << 24);
+constexpr int kBadExp = INT_MIN;            // row or column with a non-finite entry
+
+// K-major descriptor of 8 x 16-byte core matrices: the two core matrices of a 16-k row
+// are 128 bytes apart, 8-row groups 256 bytes.
+__device__ __forceinline__ uint64_t sdesc_core(uint32_t a) {
+  return (uint64_t)((a & 0x3FFFF) >> 4) | ((uint64_t)(128 >> 4) << 16) | ((uint64_t)(256 >> 4) << 32) |
+         ((uint64_t)1 << 46);
+}
+__device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
+  asm volatile(
+      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(smem_u32(dst)),
+      "l"(src), "r"(bytes), "r"(smem_u32(bar))
+      : "memory");
+}
+
+struct Args {
+  const __half *SA, *SB;    // slices
+  const int *eA, *eB;       // exponents [batch][rows]
+  double2* C;
+  int64_t ldc, sC;
+  double alpha;
+  int scale;                // alpha != 1 (the FP64 pipe is kept out of the loop)
+  int m, n, nkb;            // nkb: 16-k blocks
+  int mt, nt, mb, nb;       // tiles of 64 rows and 32 columns; 32-row blocks per batch entry of A and B
+  int64_t ntiles;
+  int lower;                // op(A) lower triangular: k < m0 + 64 only
+  int neg_ri, neg_ir, neg_ii;  // signs of re x im, im x re, im x im
+  int* err;
+};
+
+__device__ __noinline__ double scale_slow(unsigned long long T, int e) { return ldexp((double)T, e); }
+
+// +-(hi 2^-21 + lo 2^-49) (exact integers), times 2^e, rounded to FP64 in integer arithmetic.
+__device__ __forceinline__ double fixed_to_double(long long hi, long long lo, bool flip, int e) {
+  long long H = hi + (lo >> 28);
+  uint32_t l = (uint32_t)lo & 0x0FFFFFFFu;  // value = (H 2^28 + l) 2^-49
+  const bool neg = H < 0;
+  if (neg) {
+    H = (l == 0) ? -H : -H - 1;
+    l = (0x10000000u - l) & 0x0FFFFFFFu;
+  }
+  unsigned long long T;
+  int top;  // exponent of T's leading bit
+  if (H != 0) {
+    const int z = __clzll(H);
+    // the leading bits of H:l in 64 bits (z >= 1 as H > 0)
+    T = ((unsigned long long)H << z) | (((unsigned long long)l << 36) >> (64 - z));
+    top = 63 - z + 28 - 49 + e;
+  } else if (l != 0) {
+    const int z = __clzll((long long)l);
+    T = (unsigned long long)l << z;
+    top = 63 - z - 49 + e;
+  } else {
+    return 0.0;
+  }
+  const unsigned long long r = (T >> 11) + ((T >> 10) & 1);  // 53 bits, rounded; bit 52 adds to the exponent
+  const int be = 1022 + top;
+  unsigned long long v = r + ((unsigned long long)(unsigned)be << 52);
+  if ((unsigned)be >= 2045u) v = (unsigned long long)__double_as_longlong(scale_slow(T, top - 63));  // subnormal, overflow
+  if (neg != flip) v |= 1ULL << 63;
+  return __longlong_as_double((long long)v);
+}
+
+template <bool kShort>
+__global__ void __launch_bounds__(NT, 1) zgemm_tc_kernel(Args args) {
+  extern __shared__ __align__(1024) uint8_t smem[];
+  uint8_t* outS = smem + NST * kStage;
+  uint64_t* bars = reinterpret_cast<uint64_t*>(outS + kOutBytes);
+  uint64_t* full = bars;             // [NST] stage landed
+  uint64_t* empty = bars + NST;      // [NST] stage read by the MMAs
+  uint64_t* accf = bars + 2 * NST;   // chunk accumulated
+  uint64_t* drained = accf + 1;      // chunk drained
+  uint32_t* s_tmem = reinterpret_cast<uint32_t*>(drained + 1);
+  volatile int* s_err = reinterpret_cast<volatile int*>(s_tmem + 1);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < NST; ++s) {
+      mbar_init(&full[s], 1);
+      mbar_init(&empty[s], 1);
+    }
+    mbar_init(accf, 1);
+    mbar_init(drained, kDrainWarps);
+    *s_err = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(s_tmem)),
+                 "r"(kTmem)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = *s_tmem;
+  const int64_t per_batch = (int64_t)args.mt * args.nt;
+  // the column tiles of one row block are adjacent, so the CTAs of a wave share it through L2
+  auto tile_of = [&](int64_t t, int& b, int& ti, int& tj) {
+    b = (int)(t / per_batch);
+    const int rem = (int)(t % per_batch);
+    ti = rem / args.nt;
+    tj = rem % args.nt;
+  };
+  auto kblocks = [&](int ti) { return args.lower ? min(args.nkb, (ti + 1) * (BM / BK)) : args.nkb; };
+
+  if (warp == 0) {
+    if (lane == 0) {
+      int64_t it = 0;  // stages filled so far
+      bool ok = true;
+      for (int64_t t = blockIdx.x; t < args.ntiles && ok; t += gridDim.x) {
+        int b, ti, tj;
+        tile_of(t, b, ti, tj);
+        const int nk = kblocks(ti);
+        const __half* a0 = args.SA + ((int64_t)b * args.mb + 2 * ti) * args.nkb * kBlk;
+        // the second row block of the last tile may not exist: its rows are not stored
+        const __half* a1 = (2 * ti + 1 < args.mb) ? a0 + (int64_t)args.nkb * kBlk : a0;
+        const __half* bb = args.SB + ((int64_t)b * args.nb + tj) * args.nkb * kBlk;
+        for (int kb = 0; kb < nk; ++kb, ++it) {
+          const int s = (int)(it % NST);
+          if (!mbar_wait(&empty[s], (uint32_t)((it / NST) & 1) ^ 1, s_err, args.err, 41)) {
+            ok = false;
+            break;
+          }
+          uint8_t* st = smem + s * kStage;
+          mbar_expect_tx(&full[s], kStage);
+          bulk_load(st + kABytes, bb + (int64_t)kb * kBlk, kBBytes, &full[s]);
+          // per slice the two row blocks of A side by side
+#pragma unroll
+          for (int i = 0; i < NS; ++i) {
+            bulk_load(st + (2 * i) * kSlice * 2, a0 + (int64_t)kb * kBlk + i * kSlice, kSlice * 2, &full[s]);
+            bulk_load(st + (2 * i + 1) * kSlice * 2, a1 + (int64_t)kb * kBlk + i * kSlice, kSlice * 2, &full[s]);
+          }
+        }
+      }
+    }
+  } else if (warp == 1) {
+    if (lane == 0) {
+      int64_t it = 0, ch = 0;  // stages and chunks so far
+      bool ok = true;
+      for (int64_t t = blockIdx.x; t < args.ntiles && ok; t += gridDim.x) {
+        int b, ti, tj;
+        tile_of(t, b, ti, tj);
+        const int nk = kblocks(ti);
+        for (int kb = 0; kb < nk; ++kb, ++it) {
+          const bool first = (kb % kChunk) == 0;
+          if (first && ch > 0) {
+            if (!mbar_wait(drained, (uint32_t)((ch - 1) & 1), s_err, args.err, 42)) {
+              ok = false;
+              break;
+            }
+            tc_fence_after();
+          }
+          const int s = (int)(it % NST);
+          if (!mbar_wait(&full[s], (uint32_t)((it / NST) & 1), s_err, args.err, 43)) {
+            ok = false;
+            break;
+          }
+          tc_fence_after();
+          const uint32_t st = smem_u32(smem + s * kStage);
+          const uint64_t dA = sdesc_core(st), dB = sdesc_core(st + kABytes);
+          constexpr uint64_t oA = (2 * kSlice * 2) >> 4, oB = (kSlice * 2) >> 4;  // slice strides of the descriptors
+#pragma unroll
+          for (int i = 0; i < NS; ++i)
+#pragma unroll
+            for (int c = 0; c < NS - i; ++c)
+              umma_f16(tmem + (uint32_t)((i + c) * 2 * BN), dA + i * oA, dB + c * oB, kIdesc, (first && i == 0) ? 0u : 1u);
+          umma_commit(&empty[s]);
+          if ((kb % kChunk) == kChunk - 1 || kb == nk - 1) {
+            umma_commit(accf);
+            ++ch;
+          }
+        }
+      }
+    }
+  } else {
+    // drain: TMEM lane quarter q = warp % 4 (a hardware rule): row block q / 2, Re a (q even) or
+    // Im a (q odd); 16 columns: half 0 (Re b) or 1 (Im b) of the 64, sub-block 0 or 1 of the half
+    constexpr int kKeep = kDrainCols / 2;
+    const int q = warp & 3, cblk = (warp - 2) >> 2, half = cblk >> 1, sub = cblk & 1, odd = q & 1;
+    const uint32_t tbase = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(cblk * kDrainCols);
+    const int part = odd ^ half;  // what this warp's products go to: Re c or Im c
+    // signs of this warp's products and of its partner's
+    const bool neg = odd ? (half ? args.neg_ii : args.neg_ir) : (half ? args.neg_ri : 0);
+    const bool pneg = odd ? (half ? 0 : args.neg_ri) : (half ? args.neg_ir : args.neg_ii);
+    const long long pm = (neg != pneg) ? -1LL : 0LL;
+    // the two warps of a part exchange half of their columns: even q keeps the first eight, odd q
+    // the others.  Registers 0-7 hold the kept ones.
+    const uint32_t keep = (uint32_t)(odd * kKeep);
+    ulonglong2* xmine = reinterpret_cast<ulonglong2*>(outS) + (size_t)(q + 4 * cblk) * kKeep * 32 + lane;
+    const ulonglong2* xother =
+        reinterpret_cast<const ulonglong2*>(outS) + (size_t)((q ^ 1) + 4 * (cblk ^ 2)) * kKeep * 32 + lane;
+    const int row = (q >> 1) * 32 + lane, col0 = sub * kDrainCols + odd * kKeep;
+    double* out = reinterpret_cast<double*>(outS);
+    int64_t ch = 0;
+    bool ok = true;
+    for (int64_t t = blockIdx.x; t < args.ntiles; t += gridDim.x) {
+      int b, ti, tj;
+      tile_of(t, b, ti, tj);
+      const int nch = (kblocks(ti) + kChunk - 1) / kChunk;
+      long long hi[kDrainCols], lo[kDrainCols];
+#pragma unroll
+      for (int j = 0; j < kDrainCols; ++j) hi[j] = lo[j] = 0;
+      for (int c = 0; c < nch && ok; ++c, ++ch) {
+        ok = __all_sync(0xffffffffu, mbar_wait(accf, (uint32_t)(ch & 1), s_err, args.err, 44));
+        if (!ok) break;
+        tc_fence_after();
+#pragma unroll
+        for (int cb = 0; cb < kDrainCols / 4; ++cb) {
+          uint32_t v[NS][4];
+#pragma unroll
+          for (int g = 0; g < NS; ++g) tmem_ld4(tbase + (uint32_t)(g * 2 * BN) + ((uint32_t)(cb * 4) ^ keep), v[g]);
+          tmem_wait_ld();
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            int w[NS];
+#pragma unroll
+            for (int g = 0; g < NS; ++g) {
+              // exact integers; below 2^22 the addition of 1.5 2^23 puts them into the low bits
+              const float f = __uint_as_float(v[g][j]);
+              w[g] = kShort ? __float_as_int(f + 12582912.f) - 0x4B400000 : __float2int_rn(f);
+            }
+            // |w_g| < 2^24, and below 2^24 - 2^20 for g < 7: 128 w_g + w_(g+1) fits 32 bits
+            const int a0 = w[0] * 128 + w[1], a1 = w[2] * 128 + w[3];
+            const int a2 = w[4] * 128 + w[5], a3 = w[6] * 128 + w[7];
+            hi[cb * 4 + j] += (long long)a0 * 16384 + a1;
+            lo[cb * 4 + j] += (long long)a2 * 16384 + a3;
+          }
+        }
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(drained);
+      }
+      // a warp whose wait expired keeps the barriers below company, without storing
+      const int r = ti * BM + row, n0 = tj * BN;
+      const int ea = r < args.m ? args.eA[(int64_t)b * args.m + r] : 0;
+      const int* eb = args.eB + (int64_t)b * args.n;
+#pragma unroll
+      for (int j = 0; j < kKeep; ++j) {
+        xmine[j * 32] = make_ulonglong2((unsigned long long)hi[kKeep + j], (unsigned long long)lo[kKeep + j]);
+      }
+      asm volatile("bar.sync 1, 512;" ::: "memory");
+      double x[kKeep];
+#pragma unroll
+      for (int j = 0; j < kKeep; ++j) {
+        const ulonglong2 o = xother[j * 32];
+        const int n = n0 + col0 + j;
+        const int eb1 = n < args.n ? __ldg(eb + n) : 0;
+        // own +- the partner's, negated as a whole if the own sign is
+        x[j] = fixed_to_double(hi[j] + (((long long)o.x ^ pm) - pm), lo[j] + (((long long)o.y ^ pm) - pm), neg, -(ea + eb1));
+        if (ea == kBadExp || eb1 == kBadExp) x[j] = __longlong_as_double(0x7FF8000000000000LL);
+        if (args.scale) x[j] *= args.alpha;
+      }
+      asm volatile("bar.sync 1, 512;" ::: "memory");
+      // staged with the columns rotated by the row, so that lanes (rows) hit different banks
+#pragma unroll
+      for (int j = 0; j < kKeep; ++j) out[(row * BN + ((col0 + j) ^ lane)) * 2 + part] = x[j];
+      asm volatile("bar.sync 1, 512;" ::: "memory");
+      if (ok) {
+        double2* C = args.C + (int64_t)b * args.sC;
+        const int wv = warp - 2, n = n0 + lane;
+        const double2* o2 = reinterpret_cast<const double2*>(outS);
+#pragma unroll 4
+        for (int i = 0; i < BM / kDrainWarps; ++i) {
+          const int rr = wv * (BM / kDrainWarps) + i, gr = ti * BM + rr;
+          if (gr < args.m && n < args.n) C[(int64_t)gr * args.ldc + n] = o2[rr * BN + (lane ^ (rr & 31))];
+        }
+      }
+      asm volatile("bar.sync 1, 512;" ::: "memory");
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 1) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmem) : "memory");
+  }
+}
+
+// ---------------------------------------------------------------- slicing
+// Exponent ex with max 2^ex in [64, 128) from the bits of the largest magnitude.
+__device__ __forceinline__ int exp_of(unsigned long long mx) {
+  if (mx == 0) return 0;
+  const int f = (int)(mx >> 52);
+  if (f == 0x7FF) return kBadExp;
+  return f ? 6 - (f - 1023) : 6 - (63 - __clzll((long long)mx) - 1074);
+}
+
+// The 56-bit integer rint(x 2^(ex + 49)) plus 64 at each of the lower seven digits, so that
+// digit i is bits [7 (7 - i), +7) minus 64 (i >= 1) and s_0 the bits from 49 on.
+__device__ __forceinline__ long long digits_of(double x, int ex) {
+  const unsigned long long u = (unsigned long long)__double_as_longlong(x);
+  const int f = (int)((u >> 52) & 0x7FF);
+  unsigned long long m = u & 0xFFFFFFFFFFFFFULL;
+  if (f) m |= 1ULL << 52;
+  const int s = (f ? f : 1) - 1026 + ex;  // <= 3 for normal rows
+  unsigned long long F;
+  if (s >= 0)
+    F = m << s;
+  else
+    F = s > -55 ? (m + (1ULL << (-s - 1))) >> -s : 0ULL;
+  long long v = (long long)u < 0 ? -(long long)F : (long long)F;
+  constexpr long long kBias = 64LL * (1LL + (1LL << 7) + (1LL << 14) + (1LL << 21) + (1LL << 28) + (1LL << 35) + (1LL << 42));
+  return v + kBias;
+}
+
+// Slices of eight consecutive k of one row, part re or im of the chunk at dst (16 bytes per slice).
+// Digits as fp16 pairs: 1024 + u has the bits 0x6400 | u (u < 1024), minus 1024 + 64.
+__device__ __forceinline__ void store_planes(const long long (&F)[8], int part, __half* dst) {
+#pragma unroll
+  for (int s = 0; s < NS; ++s) {
+    uint32_t w[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      if (s == 0) {
+        const __half2 h = __floats2half2_rn((float)(int)(F[2 * i] >> 49), (float)(int)(F[2 * i + 1] >> 49));
+        w[i] = *reinterpret_cast<const uint32_t*>(&h);
+      } else {
+        const uint32_t u0 = (uint32_t)(F[2 * i] >> (7 * (NS - 1 - s))) & 127u;
+        const uint32_t u1 = (uint32_t)(F[2 * i + 1] >> (7 * (NS - 1 - s))) & 127u;
+        const uint32_t p = 0x64006400u | u0 | (u1 << 16);
+        const __half2 h = __hsub2(*reinterpret_cast<const __half2*>(&p), __floats2half2_rn(1088.f, 1088.f));
+        w[i] = *reinterpret_cast<const uint32_t*>(&h);
+      }
+    }
+    *reinterpret_cast<uint4*>(dst + s * kSlice + part * (RB * BK)) = make_uint4(w[0], w[1], w[2], w[3]);
+  }
+}
+
+__device__ __forceinline__ void emit_chunk(const double2 (&x)[8], int ex, __half* dst) {
+  long long F[8];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) F[i] = digits_of(x[i].x, ex);
+  store_planes(F, 0, dst);
+#pragma unroll
+  for (int i = 0; i < 8; ++i) F[i] = digits_of(x[i].y, ex);
+  store_planes(F, 1, dst);
+}
+
+__device__ __forceinline__ unsigned long long amax_bits(double2 v) {
+  constexpr long long kAbs = 0x7FFFFFFFFFFFFFFFLL;
+  const unsigned long long a = (unsigned long long)(__double_as_longlong(v.x) & kAbs);
+  const unsigned long long b = (unsigned long long)(__double_as_longlong(v.y) & kAbs);
+  return a > b ? a : b;
+}
+
+// Where chunk kc (eight k) of row r goes.
+__device__ __forceinline__ int64_t slot_of(int r, int kc, int nkb) {
+  return ((int64_t)(r / RB) * nkb + (kc >> 1)) * kBlk + ((r % RB) >> 3) * (2 * 64) + (kc & 1) * 64 + (r & 7) * 8;
+}
+
+// Rows stored contiguously along k: a block takes eight rows, one warp per row for the
+// largest entry, then eight lanes per 128-byte line of the slices.
+__global__ void __launch_bounds__(256) zslice_rows_kernel(const double2* __restrict__ X, int64_t ld, int64_t sX, int rows,
+                                                          int K, int nkb, int nblk, __half* __restrict__ S,
+                                                          int* __restrict__ ex) {
+  const int b = blockIdx.y, r0 = blockIdx.x * 8, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  X += (int64_t)b * sX;
+  S += (int64_t)b * nblk * nkb * kBlk;
+  __shared__ int se[8];
+  {
+    const int r = r0 + warp;
+    unsigned long long m = 0;
+    if (r < rows)
+      for (int k = lane; k < K; k += 32) m = max(m, amax_bits(X[(int64_t)r * ld + k]));
+    for (int o = 16; o; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if (lane == 0) {
+      const int e = exp_of(m);
+      se[warp] = e;
+      if (r < rows) ex[(int64_t)b * rows + r] = e;
+    }
+  }
+  __syncthreads();
+  const int r = r0 + (threadIdx.x & 7);
+  if (r >= rows) return;
+  const int e = se[threadIdx.x & 7];
+  const double2* row = X + (int64_t)r * ld;
+  for (int kc = threadIdx.x >> 3; kc < nkb * 2; kc += 32) {
+    double2 x[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) x[i] = (kc * 8 + i < K && e != kBadExp) ? row[kc * 8 + i] : make_double2(0.0, 0.0);
+    emit_chunk(x, e, S + slot_of(r, kc, nkb));
+  }
+}
+
+// Rows stored with stride ld along k (columns of the array), optionally gathered
+// (k -> idx[k], none where negative): a block takes 32 rows, lanes along them.
+__global__ void __launch_bounds__(256) zslice_cols_kernel(const double2* __restrict__ X, int64_t ld, int64_t sX, int rows,
+                                                          int K, int nkb, int nblk, const int32_t* __restrict__ idx,
+                                                          int64_t sIdx, __half* __restrict__ S, int* __restrict__ ex) {
+  const int b = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31, r = blockIdx.x * 32 + lane;
+  X += (int64_t)b * sX + r;
+  S += (int64_t)b * nblk * nkb * kBlk;
+  if (idx) idx += (int64_t)b * sIdx;
+  const bool in = r < rows;
+  auto at = [&](int k) {
+    const int kk = idx ? __ldg(idx + k) : k;
+    return (in && kk >= 0) ? X[(int64_t)kk * ld] : make_double2(0.0, 0.0);
+  };
+  __shared__ unsigned long long sm[8][32];
+  unsigned long long m = 0;
+#pragma unroll 4
+  for (int k = warp; k < K; k += 8) m = max(m, amax_bits(at(k)));
+  sm[warp][lane] = m;
+  __syncthreads();
+#pragma unroll
+  for (int w = 0; w < 8; ++w) m = max(m, sm[w][lane]);
+  const int e = exp_of(m);
+  if (!in) return;
+  if (warp == 0) ex[(int64_t)b * rows + r] = e;
+  for (int kc = warp; kc < nkb * 2; kc += 8) {
+    double2 x[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) x[i] = (kc * 8 + i < K && e != kBadExp) ? at(kc * 8 + i) : make_double2(0.0, 0.0);
+    emit_chunk(x, e, S + slot_of(r, kc, nkb));
+  }
+}
+
+inline int64_t cdiv(int64_t a, int64_t b) { return (a + b - 1) / b; }
+inline size_t slice_bytes(int rows, int k, int nb) { return (size_t)nb * cdiv(rows, RB) * cdiv(k, BK) * kBBytes; }
+
+// Slices of op(X) by rows (side A) or of op(X)^T (side B): `cols` when the wanted rows run
+// along the fast index of the array.
+cudaError_t slice(cudaStream_t st, bool cols, const double2* X, int64_t ld, int64_t sX, int rows, int K, int batch,
+                  const int32_t* idx, int64_t sIdx, __half* S, int* ex) {
+  const int nkb = (int)cdiv(K, BK), nblk = (int)cdiv(rows, RB);
+  if (cols)
+    zslice_cols_kernel<<<dim3((unsigned)cdiv(rows, 32), batch), 256, 0, st>>>(X, ld, sX, rows, K, nkb, nblk, idx, sIdx, S,
+                                                                             ex);
+  else
+    zslice_rows_kernel<<<dim3((unsigned)cdiv(rows, 8), batch), 256, 0, st>>>(X, ld, sX, rows, K, nkb, nblk, S, ex);
+  count_launch();
+  return cudaGetLastError();
+}
+
+}  // namespace ztc
+
+size_t zgemm_tc_work_bytes(int m, int n, int k, int nb, bool same) {
+  return ztc::slice_bytes(m, k, nb) + (same ? 0 : ztc::slice_bytes(n, k, nb)) + sizeof(int) * (size_t)nb * (m + n) + 256;
+}
+
+cudaError_t zgemm_tc(cudaStream_t st, char opA, char opB, int m, int n, int k, double alpha, const double2* A,
+                     int64_t lda, int64_t sA, const double2* B, int64_t ldb, int64_t sB, double2* C, int64_t ldc,
+                     int64_t sC, int batch, int lowerA, const int32_t* brow, int64_t sIdx, void* work,
+                     size_t work_bytes, int* err) {
+  using namespace ztc;
+  if (m <= 0 || n <= 0 || k <= 0 || batch <= 0) return cudaSuccess;
+  if (brow && opB != 'N') return cudaErrorInvalidValue;
+  const bool aT = opA == 'T' || opA == 'C', aC = opA == 'C' || opA == 'R';
+  const bool bT = opB == 'T' || opB == 'C', bC = opB == 'C' || opB == 'R';
+  const bool same = !brow && zgemm_tc_same(opA, opB, m, n, A, lda, sA, B, ldb, sB);
+  const size_t per = slice_bytes(m, k, 1) + (same ? 0 : slice_bytes(n, k, 1)) + sizeof(int) * (size_t)(m + n);
+  if (work_bytes < per + 256) return cudaErrorInvalidValue;
+  const int nbc = (int)std::min<size_t>((size_t)std::min(batch, 65535), (work_bytes - 256) / per);
+  int dev = 0, sms = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e != cudaSuccess) return e;
+  constexpr size_t smem = (size_t)NST * kStage + kOutBytes + 128;
+  const bool ks = k <= kShortK;
+  e = cudaFuncSetAttribute(ks ? zgemm_tc_kernel<true> : zgemm_tc_kernel<false>,
+                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  for (int b0 = 0; b0 < batch; b0 += nbc) {
+    const int nb = std::min(nbc, batch - b0);
+    __half* SA = reinterpret_cast<__half*>(work);
+    __half* SB = same ? SA : SA + slice_bytes(m, k, nb) / 2;
+    int* eA = reinterpret_cast<int*>(SB + slice_bytes(n, k, nb) / 2);  // n = m where SB is SA
+    int* eB = same ? eA : eA + (size_t)nb * m;
+    e = slice(st, aT, A + b0 * sA, lda, sA, m, k, nb, nullptr, 0, SA, eA);
+    if (e == cudaSuccess && !same)
+      e = slice(st, !bT, B + b0 * sB, ldb, sB, n, k, nb, brow ? brow + b0 * sIdx : nullptr, sIdx, SB, eB);
+    if (e != cudaSuccess) return e;
+    Args a{};
+    a.SA = SA;
+    a.SB = SB;
+    a.eA = eA;
+    a.eB = eB;
+    a.C = C + b0 * sC;
+    a.ldc = ldc;
+    a.sC = sC;
+    a.alpha = alpha;
+    a.scale = alpha != 1.0;
+    a.m = m;
+    a.n = n;
+    a.nkb = (int)cdiv(k, BK);
+    a.mt = (int)cdiv(m, BM);
+    a.nt = (int)cdiv(n, BN);
+    a.mb = (int)cdiv(m, RB);
+    a.nb = (int)cdiv(n, RB);
+    a.ntiles = (int64_t)nb * a.mt * a.nt;
+    a.lower = lowerA;
+    // a = ar + i ca ai, b = br + i cb bi:  Re = ar br - ca cb ai bi,  Im = cb ar bi + ca ai br
+    a.neg_ri = bC;
+    a.neg_ir = aC;
+    a.neg_ii = (aC == bC);
+    a.err = err;
+    const unsigned grid = (unsigned)std::min<int64_t>(a.ntiles, sms);
+    if (ks)
+      zgemm_tc_kernel<true><<<grid, NT, smem, st>>>(a);
+    else
+      zgemm_tc_kernel<false><<<grid, NT, smem, st>>>(a);
+    count_launch();
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
+}  // namespace isdf
