@@ -865,12 +865,14 @@ int isdf_coulomb_metric(isdf_handle* h, void* V_out) {
   const int64_t pp = (int64_t)np * np, xg = (int64_t)rx * ng;
   CK(cudaMemsetAsync(Vxi, 0, sizeof(double2) * (size_t)nk * pp, h->st));
   // FP64 and FP64_TC: FP64 arithmetic (an error in V_xi reaches E unamplified, as
-  // P dV_xi P^H with P = M W^T well scaled, so FP64_TC needs more than four slices here)
+  // P dV_xi P^H with P = M W^T well scaled, so FP64_TC needs more than four slices here).
+  // FP64_TC keeps the FMA chains: another order of rounding in V_xi moves single integrals
+  // of its fragments by up to 5e-8 of the larger ones (see isdf_fit_zeta)
   if (h->prec != ISDF_MIXED) {
     for (const auto& r : qh.runs) {
       CK(grid_coulomb_fft(h->st, xi + r.first * xg, rx, r.first, r.second, h->cell, tw, gwork));
-      ZM("grid_work_z", 'R', 'T', rx, rx, ng, h->volume, xi + r.first * xg, ng, xg,
-               xi + r.first * xg, ng, xg, Vxi + r.first * pp, np, pp, r.second);
+      ZM(h->prec == ISDF_FP64 ? "grid_work_z" : nullptr, 'R', 'T', rx, rx, ng, h->volume, xi + r.first * xg, ng, xg,
+         xi + r.first * xg, ng, xg, Vxi + r.first * pp, np, pp, r.second);
     }
   } else {
     // mixed: xi rows to float-float in place, the grid FFT in float-float, and
