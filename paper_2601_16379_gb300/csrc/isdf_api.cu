@@ -55,6 +55,7 @@ struct isdf_handle {
   std::vector<int> ao_shell, ao_lxyz, sh_atom, sh_off;
   std::vector<double> prim_exp, prim_norm, coords;
   int maxprim = 1;
+  int nterm = 0;  // products of primitives of one AO (terms of the separable Gram)
   BasisDev bdev{};
   // owned device buffers by name
   std::vector<std::pair<std::string, DevBuf>> bufs;
@@ -357,6 +358,19 @@ int upload_basis(isdf_handle* h) {
   b.coords = (const double*)up("coords", h->coords.data(), h->coords.size() * sizeof(double));
   b.prim_cn = nullptr;
   if (!b.ao_shell || !b.ao_lxyz || !b.sh_atom || !b.sh_off || !b.prim_exp || !b.prim_norm || !b.coords)
+    return fail(h, ISDF_ERR_OOM, "uploading the basis failed");
+  std::vector<int> terms;
+  for (int mu = 0; mu < h->nao; ++mu) {
+    const int npr = h->sh_off[h->ao_shell[mu] + 1] - h->sh_off[h->ao_shell[mu]];
+    if (!h->cell.orthorhombic || terms.size() > ((size_t)3 << 20)) {  // Phi is read instead
+      terms.clear();
+      break;
+    }
+    for (int p = 0; p < npr; ++p)
+      for (int q = 0; q < npr; ++q) terms.insert(terms.end(), {mu, p, q});
+  }
+  h->nterm = (int)(terms.size() / 3);
+  if (h->nterm && !up("ip_terms", terms.data(), terms.size() * sizeof(int)))
     return fail(h, ISDF_ERR_OOM, "uploading the basis failed");
   const int words[4] = {0, 0, 0, 0};
   if (!up("err_words", words, sizeof(words))) return fail(h, ISDF_ERR_OOM, "allocating the error words failed");
@@ -692,20 +706,26 @@ int isdf_build_points(isdf_handle* h, int n_p, uint64_t seed, double chol_tol, i
   if (int e = eval_phi(h)) return e;
   const int ng = h->ng, nkao = h->nk * h->nao;
   double2* phi = (double2*)h->buf("phi");
-  ENSURE(d, double, "ip_d", ng);
   ENSURE(Lt, double, "ip_Lt", (size_t)n_p * ng);
   ENSURE(piv, int32_t, "ips", n_p);
-  ENSURE(chosen, int32_t, "ip_chosen", ng);
-  ENSURE(partial, double, "ip_partial", (size_t)kIpSplit * ng);
   ENSURE(scal, double, "ip_scal", 4);
   ENSURE(status, int32_t, "ip_status", 1);
-  CK(cudaMemsetAsync(chosen, 0, sizeof(int32_t) * ng, h->st));
   CK(cudaMemsetAsync(status, 0, sizeof(int32_t), h->st));
   CK(cudaMemsetAsync(piv, 0xff, sizeof(int32_t) * n_p, h->st));
-  CK(ip_init(h->st, phi, nkao, ng, d, partial));
-  for (int j = 0; j < n_p; ++j)
-    CK(ip_step(h->st, phi, nkao, ng, j, d, Lt, piv, chosen, partial, kIpSplit, seed, kTieEps, chol_tol,
-               scal, status));
+  if (ips_supported(h->cell, h->nterm)) {
+    ENSURE(work, double, "ip_work", ips_work_bytes(h->cell, h->nterm) / sizeof(double));
+    CK(ips_select(h->st, h->cell, h->bdev, (const double*)h->buf("ao_work"), (const int*)h->buf("ip_terms"), h->nterm,
+                  n_p, work, Lt, piv, seed, kTieEps, chol_tol, scal, status));
+  } else {
+    ENSURE(d, double, "ip_d", ng);
+    ENSURE(chosen, int32_t, "ip_chosen", ng);
+    ENSURE(partial, double, "ip_partial", (size_t)kIpSplit * ng);
+    CK(cudaMemsetAsync(chosen, 0, sizeof(int32_t) * ng, h->st));
+    CK(ip_init(h->st, phi, nkao, ng, d, partial));
+    for (int j = 0; j < n_p; ++j)
+      CK(ip_step(h->st, phi, nkao, ng, j, d, Lt, piv, chosen, partial, kIpSplit, seed, kTieEps, chol_tol,
+                 scal, status));
+  }
   std::vector<int32_t> hp(n_p);
   int32_t hs = 0;
   CK(cudaMemcpyAsync(hp.data(), piv, sizeof(int32_t) * n_p, cudaMemcpyDeviceToHost, h->st));

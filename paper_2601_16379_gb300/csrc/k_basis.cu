@@ -10,6 +10,12 @@
 //           D(r,r') = Re sum_{k,mu} conj(Phi^k_mu(r)) Phi^k_mu(r') (D is real:
 //           the k and -k terms are conjugate).  One pivot per ip_step: argmax
 //           with ties, column generation, rank-one update.
+// ips_*     the same selection for orthorhombic cells, where D factorises as Phi does:
+//             D(r,r') = sum_mu sum_{p,p'} c_p c_p' prod_a A_a(g_a, g'_a),
+//             A_a(g, g') = sum_{m_a} conj(S_a^p(m_a, g)) S_a^p'(m_a, g')   (real),
+//           since the k-mesh is a product of its axes.  A column of D then costs N_AO
+//           terms per grid point instead of a pass over Phi.
+#include <algorithm>
 #include <cmath>
 
 #include "common.cuh"
@@ -58,32 +64,50 @@ __global__ void ao_1d_kernel(CellDev c, BasisDev b, double2* __restrict__ S) {
   }
 }
 
-__global__ void ao_combine_kernel(CellDev c, BasisDev b, const double2* __restrict__ S,
-                                  double2* __restrict__ phi) {
-  const int ng = c.mesh[0] * c.mesh[1] * c.mesh[2];
-  const int nk = c.kmesh[0] * c.kmesh[1] * c.kmesh[2];
-  const int64_t total = (int64_t)nk * b.nao * ng;
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total;
-       e += (int64_t)gridDim.x * blockDim.x) {
-    const int r = (int)(e % ng);
-    const int mu = (int)((e / ng) % b.nao);
-    const int k = (int)(e / ((int64_t)ng * b.nao));
-    const int g2 = r % c.mesh[2], g1 = (r / c.mesh[2]) % c.mesh[1], g0 = r / (c.mesh[1] * c.mesh[2]);
+// The two complex products of a value of Phi with the order of their fused operations written
+// out: every later step follows the rounding of Phi, so it must not depend on how the
+// compiler contracts the expression in its surroundings.
+__device__ __forceinline__ double2 phi_xy(double2 a, double2 b) {
+  return make_double2(__fma_rn(a.x, b.x, -__dmul_rn(a.y, b.y)), __fma_rn(a.y, b.x, __dmul_rn(a.x, b.y)));
+}
+__device__ __forceinline__ double2 phi_xyz(double2 a, double2 b) {
+  return make_double2(__fma_rn(a.x, b.x, -__dmul_rn(a.y, b.y)), __fma_rn(a.x, b.y, __dmul_rn(a.y, b.x)));
+}
+
+// Phi[k][mu][r] = sum_p c_p (Sx Sy) Sz.  The FP64 pipe bounds it (10 operations per value),
+// not the 16 bytes written: a block takes one (k, mu) and forms the products Sx Sy of a
+// primitive once per (g0, g1) in shared memory instead of once per grid point, which leaves
+// six.  The order of the multiplications is
+// that of the direct form, so the values are the same bits.
+__global__ void __launch_bounds__(256) ao_combine_kernel(CellDev c, BasisDev b, const double2* __restrict__ S,
+                                                         double2* __restrict__ phi, int64_t nblk) {
+  const int n1 = c.mesh[1], n2 = c.mesh[2], nxy = c.mesh[0] * n1, ng = nxy * n2;
+  __shared__ double2 sxy[256], sz[64];
+  for (int64_t blk = blockIdx.x; blk < nblk; blk += gridDim.x) {
+    // block: (k, mu) and a run of 256 (g0, g1)
+    const int nrun = (nxy + 255) / 256;
+    const int run = (int)(blk % nrun), mu = (int)((blk / nrun) % b.nao), k = (int)(blk / ((int64_t)nrun * b.nao));
     const int m2 = k % c.kmesh[2], m1 = (k / c.kmesh[2]) % c.kmesh[1], m0 = k / (c.kmesh[1] * c.kmesh[2]);
     const int sh = b.ao_shell[mu];
     const int np = b.sh_off[sh + 1] - b.sh_off[sh];
-    double2 acc = make_double2(0.0, 0.0);
+    const int x0 = run * 256, cnt = min(256, nxy - x0) * n2;
+    double2* out = phi + ((int64_t)k * b.nao + mu) * ng + (int64_t)x0 * n2;
     for (int p = 0; p < np; ++p) {
       const double2* base = S + (int64_t)((mu * b.maxprim + p) * 3) * 16 * 64;
-      const double2 sx = base[0 * 1024 + m0 * 64 + g0];
-      const double2 sy = base[1 * 1024 + m1 * 64 + g1];
-      const double2 sz = base[2 * 1024 + m2 * 64 + g2];
       const double cn = b.prim_norm[mu * b.maxprim + p];
-      const double2 t = cmul(cmul(sx, sy), sz);
-      acc.x += cn * t.x;
-      acc.y += cn * t.y;
+      __syncthreads();
+      if (x0 + (int)threadIdx.x < nxy) {
+        const int g0 = (x0 + threadIdx.x) / n1, g1 = (x0 + threadIdx.x) % n1;
+        sxy[threadIdx.x] = phi_xy(base[m0 * 64 + g0], base[1024 + m1 * 64 + g1]);
+      }
+      if ((int)threadIdx.x < n2) sz[threadIdx.x] = base[2048 + m2 * 64 + threadIdx.x];
+      __syncthreads();
+      for (int e = threadIdx.x; e < cnt; e += 256) {
+        const double2 t = phi_xyz(sxy[e / n2], sz[e % n2]);
+        const double2 acc = p ? out[e] : make_double2(0.0, 0.0);
+        out[e] = make_double2(__fma_rn(cn, t.x, acc.x), __fma_rn(cn, t.y, acc.y));
+      }
     }
-    phi[e] = acc;
   }
 }
 
@@ -304,6 +328,196 @@ __global__ void ip_update_kernel(const double* __restrict__ partial, int nsplit,
   d[r] -= l * l;
 }
 
+// ------------------------------------------- IP selection, orthorhombic cells
+// A[term][a][g'][g] (64 x 64 per axis), the factors of one term (mu, p, p'); c_p c_p' is in axis 0.
+__global__ void ips_table_kernel(CellDev c, BasisDev b, const double2* __restrict__ S, const int* __restrict__ terms,
+                                 int nterm, const int64_t o1, const int64_t o2, double* __restrict__ A) {
+  const int n0 = c.mesh[0], n1 = c.mesh[1], n2 = c.mesh[2];
+  const int per = n0 * n0 + n1 * n1 + n2 * n2;
+  const int64_t total = (int64_t)nterm * per;
+  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
+    const int t = (int)(e / per);
+    int j = (int)(e % per), a = 0;
+    if (j >= n0 * n0) j -= n0 * n0, a = 1;
+    if (a == 1 && j >= n1 * n1) j -= n1 * n1, a = 2;
+    const int n = c.mesh[a], gp = j / n, g = j % n, mu = terms[3 * t], p = terms[3 * t + 1], pp = terms[3 * t + 2];
+    const double2* s = S + (int64_t)((mu * b.maxprim + p) * 3 + a) * 1024 + g;
+    const double2* sp = S + (int64_t)((mu * b.maxprim + pp) * 3 + a) * 1024 + gp;
+    double acc = 0.0;
+    for (int m = 0; m < c.kmesh[a]; ++m) {
+      const double2 x = s[m * 64], y = sp[m * 64];
+      acc = fma(x.x, y.x, acc);
+      acc = fma(x.y, y.y, acc);
+    }
+    if (a == 0) acc *= b.prim_norm[mu * b.maxprim + p] * b.prim_norm[mu * b.maxprim + pp];
+    A[(a == 0 ? 0 : a == 1 ? o1 : o2) + (int64_t)t * n * n + j] = acc;
+  }
+}
+
+struct IpsArgs {
+  const double* A;  // factor tables: axis 0 at 0, axis 1 at o1, axis 2 at o2
+  int64_t o1, o2;
+  int nterm, n0, n1, n2, ng;
+  int tile;         // terms whose (g0, g1) products are held at once
+  double* M;        // block maxima of the residual diagonal, two buffers of gridDim.x
+  double* d;        // residual diagonal, two buffers of ng; -inf at the chosen points
+  double* Lt;       // [n_p][ng]
+  int32_t* piv;
+  double* scal;     // scal[0] = d_max,0
+  int32_t* status;
+  uint64_t seed;
+  double tie_eps, chol_tol;
+};
+
+// D(r, r') for the threads' points r = r0 + threadIdx.x: the products of the axes 0 and 1
+// once per (g0, g1) of the block, then one FMA per term.  r' = p, or r' = r (p < 0).
+__device__ __forceinline__ double ips_column(const IpsArgs& a, int r0, int p, double* sxy) {
+  const int r = r0 + threadIdx.x, last = min(r0 + (int)blockDim.x, a.ng) - 1;
+  const int x0 = r0 / a.n2, nx = last / a.n2 - x0 + 1;  // (g0, g1) pairs of the block
+  const bool in = r < a.ng;
+  const int g2 = in ? r % a.n2 : 0, xi = in ? r / a.n2 - x0 : 0;
+  double D = 0.0;
+  for (int t0 = 0; t0 < a.nterm; t0 += a.tile) {
+    const int nt = min(a.tile, a.nterm - t0);
+    __syncthreads();
+    for (int e = threadIdx.x; e < nt * nx; e += blockDim.x) {
+      const int t = t0 + e / nx, x = x0 + e % nx, g0 = x / a.n1, g1 = x % a.n1;
+      const int p0 = p < 0 ? g0 : p / (a.n1 * a.n2), p1 = p < 0 ? g1 : (p / a.n2) % a.n1;
+      sxy[e] = a.A[((int64_t)t * a.n0 + p0) * a.n0 + g0] * a.A[a.o1 + ((int64_t)t * a.n1 + p1) * a.n1 + g1];
+    }
+    __syncthreads();
+    const double* A2 = a.A + a.o2 + ((int64_t)t0 * a.n2 + (p < 0 ? g2 : p % a.n2)) * a.n2 + g2;
+#pragma unroll 8
+    for (int t = 0; t < nt; ++t) D = fma(sxy[t * nx + xi], A2[(int64_t)t * a.n2 * a.n2], D);
+  }
+  return D;
+}
+
+__device__ __forceinline__ double block_fmax(double m, double* sv) {
+  for (int o = 16; o; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+  __syncthreads();
+  if ((threadIdx.x & 31) == 0) sv[threadIdx.x >> 5] = m;
+  __syncthreads();
+  m = sv[0];
+  for (int i = 1; i < (int)(blockDim.x >> 5); ++i) m = fmax(m, sv[i]);
+  return m;
+}
+
+__global__ void ips_init_kernel(IpsArgs a) {
+  extern __shared__ double ips_smem[];
+  __shared__ double sv[8];
+  const int r0 = blockIdx.x * blockDim.x, r = r0 + threadIdx.x;
+  const double D = ips_column(a, r0, -1, ips_smem);
+  double v = -INFINITY;
+  if (r < a.ng) a.d[r] = v = D * D;
+  v = block_fmax(v, sv);
+  if (threadIdx.x == 0) a.M[blockIdx.x] = v;
+}
+
+// Step j in one launch (the stream order between the steps is the only barrier): every block
+// finds the pivot from the block maxima of step j - 1 -- the tie rule looks only into blocks
+// whose maximum lies in the window -- then updates its own points and leaves its new maximum.
+// Buffers alternate, so that no block reads what another one writes.  About 150 blocks: one
+// point per thread, chains of j FMAs against rows of Lt that stay in L2.
+__global__ void ips_step_kernel(IpsArgs a, int j) {
+  extern __shared__ double ips_smem[];
+  __shared__ double sv[8];
+  __shared__ unsigned long long sh[8];
+  __shared__ int si[8];
+  if (*a.status != 0) return;
+  const int nb = gridDim.x, bd = blockDim.x, tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  const double* M = a.M + (j & 1) * nb;
+  const double* din = a.d + (int64_t)(j & 1) * a.ng;
+  double* dout = a.d + (int64_t)((j & 1) ^ 1) * a.ng;
+  double dmax = -INFINITY;
+  for (int b = tid; b < nb; b += bd) dmax = fmax(dmax, M[b]);
+  dmax = block_fmax(dmax, sv);
+  const double d0 = j == 0 ? dmax : a.scal[0];
+  if (!(dmax >= a.chol_tol * d0) || !(dmax > 0.0)) {
+    if (blockIdx.x == 0 && tid == 0) {
+      *a.status = 1;
+      a.piv[j] = -1;
+    }
+    return;
+  }
+  const double thr = fmax(dmax - a.tie_eps * d0, 0.5 * dmax);
+  unsigned long long best = ~0ULL;
+  int bi = -1;
+  for (int b = 0; b < nb; ++b) {
+    if (!(M[b] >= thr)) continue;
+    const int r = b * bd + tid;
+    if (r < a.ng && din[r] >= thr) {
+      const unsigned long long hsh = splitmix64(a.seed ^ (uint64_t)r);
+      if (bi < 0 || hsh < best) {  // ascending r: the smaller index wins equal hashes
+        best = hsh;
+        bi = r;
+      }
+    }
+  }
+  for (int o = 16; o; o >>= 1) {
+    const unsigned long long ob = __shfl_xor_sync(0xffffffffu, best, o);
+    const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
+    if (oi >= 0 && (bi < 0 || ob < best || (ob == best && oi < bi))) {
+      best = ob;
+      bi = oi;
+    }
+  }
+  if (lane == 0) {
+    sh[w] = best;
+    si[w] = bi;
+  }
+  __syncthreads();
+  int p = -1;
+  best = ~0ULL;
+  for (int i = 0; i < (bd >> 5); ++i)
+    if (si[i] >= 0 && (p < 0 || sh[i] < best || (sh[i] == best && si[i] < p))) {
+      best = sh[i];
+      p = si[i];
+    }
+  if (p < 0) {  // no finite candidate
+    if (blockIdx.x == 0 && tid == 0) {
+      *a.status = 2;
+      a.piv[j] = -1;
+    }
+    return;
+  }
+  if (blockIdx.x == 0 && tid == 0) {
+    a.piv[j] = p;
+    if (j == 0) a.scal[0] = dmax;
+  }
+  const int r0 = blockIdx.x * bd, r = r0 + tid;
+  const double D = ips_column(a, r0, p, ips_smem);
+  __syncthreads();
+  double* lp = ips_smem;  // L[i][p], in pieces of 256
+  const double* Lr = a.Lt + (r < a.ng ? r : 0);
+  double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
+  for (int i0 = 0; i0 < j; i0 += 256) {
+    const int n = min(256, j - i0);
+    __syncthreads();
+    for (int i = tid; i < n; i += bd) lp[i] = a.Lt[(int64_t)(i0 + i) * a.ng + p];
+    __syncthreads();
+    const double* L = Lr + (int64_t)i0 * a.ng;
+    int i = 0;
+#pragma unroll 2
+    for (; i + 4 <= n; i += 4) {
+      s0 = fma(L[(int64_t)i * a.ng], lp[i], s0);
+      s1 = fma(L[(int64_t)(i + 1) * a.ng], lp[i + 1], s1);
+      s2 = fma(L[(int64_t)(i + 2) * a.ng], lp[i + 2], s2);
+      s3 = fma(L[(int64_t)(i + 3) * a.ng], lp[i + 3], s3);
+    }
+    for (; i < n; ++i) s0 = fma(L[(int64_t)i * a.ng], lp[i], s0);
+  }
+  double v = -INFINITY;
+  if (r < a.ng) {
+    const double l = (D * D - ((s0 + s1) + (s2 + s3))) * (1.0 / sqrt(din[p]));
+    a.Lt[(int64_t)j * a.ng + r] = l;
+    v = r == p ? -INFINITY : din[r] - l * l;
+    dout[r] = v;
+  }
+  v = block_fmax(v, sv);
+  if (tid == 0) a.M[((j & 1) ^ 1) * nb + blockIdx.x] = v;
+}
+
 __global__ void gather_x_kernel(const double2* __restrict__ phi, int nk, int nao, int ng,
                                 const int32_t* __restrict__ ips, int np, double2* __restrict__ X) {
   const int64_t total = (int64_t)nk * np * nao;
@@ -337,7 +551,8 @@ cudaError_t ao_eval(cudaStream_t st, const CellDev& c, const BasisDev& b, double
     const int total1 = b.nao * b.maxprim * 3 * 16 * 64;
     ao_1d_kernel<<<nblocks(total1), 256, 0, st>>>(c, b, S);
     count_launch();
-    ao_combine_kernel<<<nblocks((int64_t)nk * b.nao * ng), 256, 0, st>>>(c, b, S, phi);
+    const int64_t nblk = (int64_t)nk * b.nao * ((c.mesh[0] * c.mesh[1] + 255) / 256);
+    ao_combine_kernel<<<(unsigned)std::min<int64_t>(nblk, 152 * 32), 256, 0, st>>>(c, b, S, phi, nblk);
     count_launch();
   } else {
     const int64_t total = (int64_t)((nk + KCH - 1) / KCH) * b.nao * ng;
@@ -367,6 +582,69 @@ cudaError_t ip_step(cudaStream_t st, const double2* phi, int nkao, int ng, int j
   count_launch();
   ip_update_kernel<<<(ng + 255) / 256, 256, 0, st>>>(partial, nsplit, ng, j, piv, Lt, d, scal, status);
   count_launch();
+  return cudaGetLastError();
+}
+
+namespace {
+struct IpsLayout {
+  int threads, blocks, tile;
+  size_t table, total;  // doubles
+};
+IpsLayout ips_layout(const CellDev& c, int nterm) {
+  const int ng = c.mesh[0] * c.mesh[1] * c.mesh[2];
+  IpsLayout l;
+  // one wave: points spread over the SMs, a warp to eight warps each
+  l.threads = std::min(256, std::max(32, ((ng + 151) / 152 + 31) / 32 * 32));
+  l.blocks = (ng + l.threads - 1) / l.threads;
+  const int nx = l.threads / c.mesh[2] + 2;
+  l.tile = std::max(1, std::min(nterm, 4096 / nx));
+  l.table = (size_t)nterm * (c.mesh[0] * c.mesh[0] + c.mesh[1] * c.mesh[1] + c.mesh[2] * c.mesh[2]);
+  l.total = l.table + 2 * (size_t)l.blocks + 2 * (size_t)ng;
+  return l;
+}
+constexpr size_t kIpsMaxTable = (size_t)32 << 20;  // doubles (256 MB): beyond it, long contractions, Phi is read instead
+}  // namespace
+
+bool ips_supported(const CellDev& c, int nterm) {
+  return c.orthorhombic && nterm > 0 && nterm < (1 << 20) && ips_layout(c, nterm).table <= kIpsMaxTable;
+}
+size_t ips_work_bytes(const CellDev& c, int nterm) { return ips_layout(c, nterm).total * sizeof(double); }
+
+// The separable selection.  Measured on GB300 (Phi and points together, 300 points, 24^3 grid,
+// Nk = 1000, N_AO = 26): 13.7 ms, against 478 ms with one pass over Phi per pivot.
+cudaError_t ips_select(cudaStream_t st, const CellDev& c, const BasisDev& b, const double* ao_work, const int* terms,
+                       int nterm, int n_p, double* work, double* Lt, int32_t* piv, uint64_t seed, double tie_eps,
+                       double chol_tol, double* scal, int32_t* status) {
+  const IpsLayout l = ips_layout(c, nterm);
+  IpsArgs a;
+  a.A = work;
+  a.o1 = (int64_t)nterm * c.mesh[0] * c.mesh[0];
+  a.o2 = a.o1 + (int64_t)nterm * c.mesh[1] * c.mesh[1];
+  a.nterm = nterm;
+  a.n0 = c.mesh[0];
+  a.n1 = c.mesh[1];
+  a.n2 = c.mesh[2];
+  a.ng = a.n0 * a.n1 * a.n2;
+  a.tile = l.tile;
+  a.M = work + l.table;
+  a.d = a.M + 2 * (size_t)l.blocks;
+  a.Lt = Lt;
+  a.piv = piv;
+  a.scal = scal;
+  a.status = status;
+  a.seed = seed;
+  a.tie_eps = tie_eps;
+  a.chol_tol = chol_tol;
+  ips_table_kernel<<<nblocks((int64_t)l.table), 256, 0, st>>>(c, b, reinterpret_cast<const double2*>(ao_work), terms,
+                                                              nterm, a.o1, a.o2, work);
+  count_launch();
+  const size_t smem = sizeof(double) * std::max<size_t>(256, (size_t)l.tile * (l.threads / a.n2 + 2));
+  ips_init_kernel<<<l.blocks, l.threads, smem, st>>>(a);
+  count_launch();
+  for (int j = 0; j < n_p; ++j) {
+    ips_step_kernel<<<l.blocks, l.threads, smem, st>>>(a, j);
+    count_launch();
+  }
   return cudaGetLastError();
 }
 
