@@ -123,12 +123,15 @@ cudaError_t ips_select(cudaStream_t st, const CellDev& c, const BasisDev& b, con
 cudaError_t gather_x(cudaStream_t st, const double2* phi, int nk, int nao, int ng,
                      const int32_t* ips, int np, double2* X);
 
-// Pivoted Cholesky (batched) of Hermitian PSD A[b][n][n].  Lt[b][j][i] = L[i][j].
-cudaError_t pchol_batched(cudaStream_t st, const double2* A, int n, int batch, double tol,
-                          double2* Lt, int32_t* perm, int32_t* rank, double* dwork);
-// Wfull[b] (n x n): Wfull[i][perm[c]] = (L_S^{-1})[i][c], zero elsewhere.
-cudaError_t trinv_batched(cudaStream_t st, const double2* Lt, const int32_t* perm,
-                          const int32_t* rank, int n, int batch, double2* W, double2* work);
+// Pivoted Cholesky of the Hermitian PSD A[q][n][n], q in qlist (device, nq entries), whose rows
+// and columns from neff on are zero.  Lt[q][j][i] = L[i][j]; with `live`, rows that have been
+// pivots are left out of the later columns (the solve does not read them).
+cudaError_t pchol_batched(cudaStream_t st, const double2* A, int n, int neff, bool live, const int* qlist, int nq,
+                          double tol, double2* Lt, int32_t* perm, int32_t* rank);
+// Wfull[q] (n x n): Wfull[i][perm[c]] = (L_S^{-1})[i][c], zero elsewhere, for q in qlist; W and work
+// (L_S^{-1} in pivot order) are zeroed for all nk matrices; tmp: nk n n of scratch.
+cudaError_t trinv_batched(cudaStream_t st, const double2* Lt, const int32_t* perm, const int32_t* rank, int n, int nk,
+                          const int* qlist, int nq, double2* W, double2* work, double2* tmp);
 // Lpad[b][i][j] = L[i][j] (row-major, columns beyond the rank zero).
 cudaError_t lt_to_rowmajor(cudaStream_t st, const double2* Lt, const int32_t* rank, int n,
                            int batch, double2* L);

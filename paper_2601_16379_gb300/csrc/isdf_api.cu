@@ -301,6 +301,7 @@ void q_point_set(const KMesh& km, bool pair, std::vector<int>& qs, std::vector<d
 // of those of q.  Without pairing every q is its own representative.
 struct QHalf {
   std::vector<std::pair<int, int>> runs;  // (first q, count)
+  std::vector<int> list;                  // the computed q-points
   std::vector<int2> mirror;               // (q, -q) for q not computed
   int count = 0;                          // computed q-points
 };
@@ -315,6 +316,7 @@ QHalf fit_q_set(const KMesh& km, bool pair) {
       continue;
     }
     ++h.count;
+    h.list.push_back(q);
     if (!h.runs.empty() && h.runs.back().first + h.runs.back().second == q)
       ++h.runs.back().second;
     else
@@ -541,17 +543,27 @@ TileSchedule tuned_schedule(isdf_handle* h, int64_t ntiles, const std::function<
   return {t.cfg, t.band};
 }
 
-// Shared tail of both Coulomb routes: factor V_xi = L_xi L_xi^H, L^q = W^T L_xi
+// Shared tail of both Coulomb routes (V_xi zero beyond its first neff rows and columns; q and
+// its mirror list as uploaded by the caller): factor V_xi = L_xi L_xi^H, L^q = W^T L_xi
 // (so V^q = L^q L^q^H), optional output of V^q, precision copies for the fragments.
-int coulomb_tail(isdf_handle* h, double2* Vxi, void* V_out) {
+int coulomb_tail(isdf_handle* h, const QHalf& qh, int neff, double2* Vxi, void* V_out) {
   const int nk = h->nk, np = h->np;
   double2* W = (double2*)h->buf("W");
   // V_xi = L_xi L_xi^H ; L^q = W^T L_xi
   ENSURE(LtV, double2, "LtV", (size_t)nk * np * np);
   ENSURE(permV, int32_t, "permV", (size_t)nk * np);
   ENSURE(rankV, int32_t, "rankV", nk);
-  ENSURE(dwork, double, "chol_dwork", (size_t)nk * 2 * np);
-  CK(pchol_batched(h->st, Vxi, np, nk, 1e-15, LtV, permV, rankV, dwork));
+  ENSURE(qlist, int, "q_list", nk);
+  CK(cudaMemcpyAsync(qlist, qh.list.data(), sizeof(int) * qh.list.size(), cudaMemcpyHostToDevice, h->st));
+  // the factor of the conjugate matrix is the conjugate factor, bit for bit
+  CK(pchol_batched(h->st, Vxi, np, neff, false, qlist, qh.count, 1e-15, LtV, permV, rankV));
+  if (!qh.mirror.empty()) {
+    const int2* mir = (const int2*)h->buf("q_mirror");
+    const int nm = (int)qh.mirror.size();
+    CK(mirror_conj(h->st, LtV, (int64_t)np * np, mir, nm));
+    CK(mirror_copy(h->st, permV, np, mir, nm));
+    CK(mirror_copy(h->st, rankV, 1, mir, nm));
+  }
   h->ranks_v.assign(nk, 0);
   CK(cudaMemcpyAsync(h->ranks_v.data(), rankV, sizeof(int32_t) * nk, cudaMemcpyDeviceToHost, h->st));
   ENSURE(Lxi, double2, "W_work", (size_t)nk * np * np);
@@ -816,14 +828,13 @@ int isdf_fit_zeta(isdf_handle* h, double solve_tol, int32_t* rank_out) {
   ENSURE(LtPi, double2, "LtPi", (size_t)nk * np * np);
   ENSURE(permPi, int32_t, "permPi", (size_t)nk * np);
   ENSURE(rankPi, int32_t, "rankPi", nk);
-  ENSURE(dwork, double, "chol_dwork", (size_t)nk * 2 * np);
   ENSURE(W, double2, "W", (size_t)nk * np * np);
   ENSURE(wwork, double2, "W_work", (size_t)nk * np * np);
-  ENSURE(xi, double2, "xi", (size_t)nk * np * ng);
+  ENSURE(tri, double2, "Vxi", (size_t)nk * np * np);  // scratch of the triangular inverse
+  ENSURE(qlist, int, "q_list", nk);
   const int64_t pp = (int64_t)np * np;
-  for (const auto& r : qh.runs)
-    CK(pchol_batched(h->st, Pi + r.first * pp, np, r.second, solve_tol, LtPi + r.first * pp,
-                     permPi + (int64_t)r.first * np, rankPi + r.first, dwork + (int64_t)r.first * 2 * np));
+  CK(cudaMemcpyAsync(qlist, qh.list.data(), sizeof(int) * qh.list.size(), cudaMemcpyHostToDevice, h->st));
+  CK(pchol_batched(h->st, Pi, np, np, true, qlist, qh.count, solve_tol, LtPi, permPi, rankPi));
   if (!qh.mirror.empty()) {
     ENSURE(mir, int2, "q_mirror", qh.mirror.size());
     CK(cudaMemcpyAsync(mir, qh.mirror.data(), sizeof(int2) * qh.mirror.size(), cudaMemcpyHostToDevice, h->st));
@@ -840,10 +851,10 @@ int isdf_fit_zeta(isdf_handle* h, double solve_tol, int32_t* rank_out) {
   // xi^q = W eta^q has nonzero rows only below r_q: keep r_max rows per q
   const int rx = *std::max_element(h->ranks.begin(), h->ranks.end());
   const int64_t pg = (int64_t)np * ng, xg = (int64_t)rx * ng;
+  ENSURE(xi, double2, "xi", (size_t)nk * rx * ng);
+  CK(trinv_batched(h->st, LtPi, permPi, rankPi, np, nk, qlist, qh.count, W, wwork, tri));
   for (const auto& r : qh.runs) {
     const int q0 = r.first, nq = r.second;
-    CK(trinv_batched(h->st, LtPi + q0 * pp, permPi + (int64_t)q0 * np, rankPi + q0, np, nq, W + q0 * pp,
-                     wwork + q0 * pp));
     // xi^q = W eta^q = L_S^{-1} (eta^q rows in pivot order): triangular, gathered
     ZM(zw, 'N', 'N', rx, ng, rx, 1.0, wwork + q0 * pp, np, pp, eta + q0 * pg, ng, pg, xi + q0 * xg, ng, xg,
        nq, 1, permPi + (int64_t)q0 * np, np);
@@ -854,10 +865,10 @@ int isdf_fit_zeta(isdf_handle* h, double solve_tol, int32_t* rank_out) {
     CK(mirror_conj(h->st, xi, xg, mir, (int)qh.mirror.size()));
   }
   h->xi_rows = rx;
-  double tri = 0.0;  // triangular xi = W eta over the computed q: r_q^2 / 2 complex MACs per grid point
+  double tri_flops = 0.0;  // triangular xi = W eta over the computed q: r_q^2 / 2 complex MACs per grid point
   for (const auto& r : qh.runs)
-    for (int q = r.first; q < r.first + r.second; ++q) tri += (double)h->ranks[q] * h->ranks[q];
-  stt.flops = 8.0 * nk * (double)np * ng * nao + 4.0 * tri * ng;
+    for (int q = r.first; q < r.first + r.second; ++q) tri_flops += (double)h->ranks[q] * h->ranks[q];
+  stt.flops = 8.0 * nk * (double)np * ng * nao + 4.0 * tri_flops * ng;
   h->has_fit = true;
   h->has_xi = true;
   h->has_eta = true;
@@ -913,7 +924,7 @@ int isdf_coulomb_metric(isdf_handle* h, void* V_out) {
     CK(mirror_conj(h->st, Vxi, pp, mir, (int)qh.mirror.size()));
   }
   h->has_xi = false;  // xi was transformed in place (FP64) / is no longer needed
-  return coulomb_tail(h, Vxi, V_out);
+  return coulomb_tail(h, qh, rx, Vxi, V_out);
 }
 
 // Coulomb kernel without forming zeta (Eqs. 7-8): V_eta = Omega c'^* c'^T from
@@ -930,7 +941,7 @@ int isdf_coulomb_metric_eta(isdf_handle* h, void* V_out) {
   const int nk = h->nk, np = h->np, ng = h->ng;
   double2* eta = (double2*)h->buf("eta");
   double2* W = (double2*)h->buf("W");
-  double2* work = (double2*)h->buf("xi");  // the copy of eta is transformed in place
+  ENSURE(work, double2, "xi", (size_t)nk * np * ng);  // the copy of eta is transformed in place
   const double2* tw = (const double2*)h->buf("grid_tw");
   const KMesh km{{h->cell.kmesh[0], h->cell.kmesh[1], h->cell.kmesh[2]}};
   const QHalf qh = fit_q_set(km, h->q_sym);
@@ -959,7 +970,7 @@ int isdf_coulomb_metric_eta(isdf_handle* h, void* V_out) {
            (int64_t)np * np, nk);
   ZM("grid_work_z", 'R', 'N', np, np, np, 1.0, W, np, (int64_t)np * np, tmp, np, (int64_t)np * np, Vxi, np,
            (int64_t)np * np, nk);
-  return coulomb_tail(h, Vxi, V_out);
+  return coulomb_tail(h, qh, np, Vxi, V_out);
 }
 
 int isdf_fragment_eri(isdf_handle* h, int n_frag, const int32_t* n_orb, const void* const* C,

@@ -1,14 +1,21 @@
 // Batched FP64 factorisations for the least-squares solve (Eq. 3).
 //
-// pchol_batched  pivoted Cholesky of Hermitian PSD matrices, one block per
-//                matrix: pivot = largest remaining diagonal, where diagonals
-//                within 1e-11 * (largest initial diagonal) of it are ties
-//                resolved to the smallest index; stop when it is <= tol *
-//                largest initial diagonal.  Column j of L is stored as Lt[j][:].
+// pchol_batched  pivoted Cholesky of Hermitian PSD matrices: pivot = largest
+//                remaining diagonal, where diagonals within 1e-11 * (largest
+//                initial diagonal) of it are ties resolved to the smallest
+//                index; stop when it is <= tol * largest initial diagonal.
+//                Column j of L is stored as Lt[j][:].
 // trinv_batched  W = L_S^{-1} for the kept rows S = perm[:rank] (L_S is lower
 //                triangular in pivot order), scattered to Wfull[i][perm[c]] so
 //                that xi = Wfull * eta and zeta = Wfull^H * xi give the basic
 //                least-squares solution (zeta = 0 on dropped points).
+//
+// Both take a list of the matrices (q-points) to work on, so that one launch covers the
+// scattered representatives of the time-reversal pairs.
+#include <cooperative_groups.h>
+
+#include <algorithm>
+
 #include "common.cuh"
 
 namespace isdf {
@@ -17,137 +24,185 @@ namespace {
 
 constexpr double kTieEps = 1e-11;  // pivot tie window, relative to the largest initial diagonal
 
-__global__ void __launch_bounds__(512) pchol_kernel(const double2* __restrict__ A, int n, double tol,
-                                                    double2* __restrict__ Lt, int32_t* __restrict__ perm,
-                                                    int32_t* __restrict__ rank, double* __restrict__ dwork) {
-  const int b = blockIdx.x;
-  A += (int64_t)b * n * n;
-  Lt += (int64_t)b * n * n;
-  perm += (int64_t)b * n;
-  double* d = dwork + (int64_t)b * 2 * n;
-  double* used = d + n;
-  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5, nw = blockDim.x >> 5;
-  __shared__ double sv[32];
-  __shared__ int si[32];
-  __shared__ int s_p;
-  __shared__ double s_dp;
-  __shared__ double s_d0;
-  for (int i = tid; i < n; i += blockDim.x) {
-    d[i] = A[(int64_t)i * n + i].x;
-    used[i] = 0.0;
+// A cluster of C blocks per matrix, one row of L per thread.  What bounds it is the FP64 pipe
+// (six operations per complex product, 2 per clock and SM): n r^2 / 2 products are 28 ms on
+// one SM at n = 500, r = 270, so the rows are spread over C SMs; the residual diagonals live
+// in shared memory, double-buffered, and are read across the cluster.  Rows are written once
+// per column and read by their own thread; only the pivot's row of L is gathered per column.
+// live != 0: rows that were pivots are skipped from then on (nothing reads their later
+// columns); rows from neff on are zero.
+constexpr int kBp = 512;  // entries of the pivot's row of L staged at once
+__global__ void __launch_bounds__(256) pchol_kernel(const double2* __restrict__ A, int n, int neff, int live,
+                                                    const int* __restrict__ qlist, double tol, double2* Lt,
+                                                    int32_t* __restrict__ perm, int32_t* __restrict__ rank) {
+  namespace cg = cooperative_groups;
+  cg::cluster_group cl = cg::this_cluster();
+  const int C = (int)cl.num_blocks(), cr = (int)cl.block_rank();
+  const int64_t q = qlist[blockIdx.x / C];
+  A += q * n * n;
+  Lt += q * n * n;
+  perm += q * n;
+  const int bd = blockDim.x, tid = threadIdx.x, lane = tid & 31, w = tid >> 5, nw = bd >> 5;
+  const int per = (neff + C - 1) / C, i0 = cr * per, i1 = min(neff, i0 + per);  // rows of this block
+  extern __shared__ __align__(16) unsigned char chol_smem[];
+  double2* bp = reinterpret_cast<double2*>(chol_smem);           // [kBp] of the pivot's row of L
+  double* sd = reinterpret_cast<double*>(bp + kBp);              // [2][per] residual diagonals
+  unsigned char* used = reinterpret_cast<unsigned char*>(sd + 2 * per);  // [per]
+  __shared__ double sv[8], s_max[2], s_inv;
+  __shared__ int si[8], s_idx[2];
+  for (int i = i0 + tid; i < i1; i += bd) {
+    sd[i - i0] = A[(int64_t)i * n + i].x;
+    used[i - i0] = 0;
   }
   __syncthreads();
+  double d0 = 0.0;
   int r = 0;
-  for (int j = 0; j < n; ++j) {
+  for (int j = 0; j < neff; ++j) {
+    const int cur = j & 1;
+    double* d = sd + cur * per;
+    double* dn = sd + (cur ^ 1) * per;
     // largest remaining diagonal over unused rows
     double bv = -INFINITY;
-    for (int i = tid; i < n; i += blockDim.x)
-      if (used[i] == 0.0) bv = fmax(bv, d[i]);
+    for (int i = i0 + tid; i < i1; i += bd)
+      if (!used[i - i0]) bv = fmax(bv, d[i - i0]);
     for (int o = 16; o; o >>= 1) bv = fmax(bv, __shfl_xor_sync(0xffffffffu, bv, o));
     if (lane == 0) sv[w] = bv;
     __syncthreads();
     if (tid == 0) {
       double v = sv[0];
       for (int t = 1; t < nw; ++t) v = fmax(v, sv[t]);
-      if (j == 0) s_d0 = v;
-      s_dp = v;
+      s_max[cur] = v;
     }
-    __syncthreads();
-    const double dmax = s_dp;
-    if (!(dmax > tol * s_d0) || !(dmax > 0.0)) break;
+    cl.sync();
+    double dmax = -INFINITY;
+    for (int c = 0; c < C; ++c) dmax = fmax(dmax, *cl.map_shared_rank(&s_max[cur], c));
+    if (j == 0) d0 = dmax;
+    if (!(dmax > tol * d0) || !(dmax > 0.0)) break;
     // ties: every unused row within tie_eps * d_max,0 (and >= dmax/2) -> smallest index
-    const double thr = fmax(dmax - kTieEps * s_d0, 0.5 * dmax);
+    const double thr = fmax(dmax - kTieEps * d0, 0.5 * dmax);
     int bi = n;
-    for (int i = tid; i < n; i += blockDim.x)
-      if (used[i] == 0.0 && d[i] >= thr && i < bi) bi = i;
+    for (int i = i0 + tid; i < i1; i += bd)
+      if (!used[i - i0] && d[i - i0] >= thr && i < bi) bi = i;
     for (int o = 16; o; o >>= 1) bi = min(bi, __shfl_xor_sync(0xffffffffu, bi, o));
     if (lane == 0) si[w] = bi;
     __syncthreads();
     if (tid == 0) {
       int ii = si[0];
       for (int t = 1; t < nw; ++t) ii = min(ii, si[t]);
-      s_p = ii;
-      s_dp = ii < n ? d[ii] : 0.0;
+      s_idx[cur] = ii;
     }
-    __syncthreads();
-    const int p = s_p;
+    cl.sync();
+    int p = n;
+    for (int c = 0; c < C; ++c) p = min(p, *cl.map_shared_rank(&s_idx[cur], c));
     if (p >= n) break;  // no finite candidate
-    const double dp = s_dp;
-    const double inv = 1.0 / sqrt(dp);
-    for (int i = tid; i < n; i += blockDim.x) {
-      double2 acc = A[(int64_t)i * n + p];
-      for (int l = 0; l < j; ++l) {
-        const double2 a = Lt[(int64_t)l * n + i];
-        const double2 bp = Lt[(int64_t)l * n + p];
-        // acc -= a * conj(bp)
-        acc.x -= a.x * bp.x + a.y * bp.y;
-        acc.y -= a.y * bp.x - a.x * bp.y;
-      }
-      const double2 col = make_double2(acc.x * inv, acc.y * inv);
-      // write after all threads have read Lt[l][p] for l < j (row j is new)
-      Lt[(int64_t)j * n + i] = col;
-      d[i] -= col.x * col.x + col.y * col.y;
-    }
     if (tid == 0) {
-      used[p] = 1.0;
-      perm[j] = p;
+      const double dp = *cl.map_shared_rank(d + p % per, p / per);
+      s_inv = 1.0 / sqrt(dp);
     }
+    for (int ib = i0; ib < i1; ib += bd) {
+      const int i = ib + tid;
+      const bool on = i < i1 && !(live && used[i - i0]);
+      double2 acc = on ? A[(int64_t)i * n + p] : make_double2(0.0, 0.0);
+      for (int l0 = 0; l0 < j; l0 += kBp) {
+        const int nl = min(kBp, j - l0);
+        __syncthreads();
+        for (int l = tid; l < nl; l += bd) bp[l] = Lt[(int64_t)(l0 + l) * n + p];
+        __syncthreads();
+        if (!on) continue;
+        const double2* Li = Lt + (int64_t)l0 * n + i;
+#pragma unroll 8
+        for (int l = 0; l < nl; ++l) {
+          const double2 a = Li[(int64_t)l * n];
+          const double2 b = bp[l];
+          // acc -= a * conj(b)
+          acc.x -= a.x * b.x + a.y * b.y;
+          acc.y -= a.y * b.x - a.x * b.y;
+        }
+      }
+      if (j == 0) __syncthreads();  // s_inv
+      if (!on) continue;
+      const double inv = s_inv;
+      const double2 col = make_double2(acc.x * inv, acc.y * inv);
+      Lt[(int64_t)j * n + i] = col;
+      dn[i - i0] = d[i - i0] - (col.x * col.x + col.y * col.y);
+      if (i == p) used[i - i0] = 1;
+    }
+    if (cr == 0 && tid == 0) perm[j] = p;
     r = j + 1;
     __syncthreads();
   }
-  if (tid == 0) rank[b] = r;
-  // zero the unused columns so that consumers can read a full n x n array
-  for (int64_t e = (int64_t)r * n + tid; e < (int64_t)n * n; e += blockDim.x) Lt[e] = make_double2(0.0, 0.0);
-  for (int i = r + tid; i < n; i += blockDim.x) perm[i] = -1;
+  cl.sync();  // no block leaves while its shared memory may be read
+  if (cr == 0 && tid == 0) rank[q] = r;
+  // zero what was not computed so that consumers can read a full n x n array
+  const int64_t t0 = (int64_t)cr * bd + tid, step = (int64_t)C * bd;
+  for (int64_t e = (int64_t)r * n + t0; e < (int64_t)n * n; e += step) Lt[e] = make_double2(0.0, 0.0);
+  const int64_t pad = n - neff;
+  for (int64_t e = t0; e < (int64_t)r * pad; e += step) Lt[(e / pad) * n + neff + e % pad] = make_double2(0.0, 0.0);
+  for (int64_t i = r + t0; i < n; i += step) perm[i] = -1;
 }
 
-// work[b][i][c] = (L_S^{-1})[i][c]; thread per column c, forward substitution over i.
-__global__ void __launch_bounds__(256) trinv_kernel(const double2* __restrict__ Lt,
-                                                    const int32_t* __restrict__ perm,
-                                                    const int32_t* __restrict__ rank, int n,
-                                                    double2* __restrict__ work) {
-  const int b = blockIdx.y;
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  Lt += (int64_t)b * n * n;
-  perm += (int64_t)b * n;
-  work += (int64_t)b * n * n;
-  const int r = rank[b];
+// work[q][l][i] = L_S[i][l] = Lt[l][perm[i]] for l <= i < r: the rows of the triangular solve,
+// contiguous in i.
+__global__ void tri_gather_kernel(const double2* __restrict__ Lt, const int32_t* __restrict__ perm,
+                                  const int32_t* __restrict__ rank, const int* __restrict__ qlist, int n,
+                                  double2* __restrict__ out) {
+  const int64_t q = qlist[blockIdx.y];
+  const int r = rank[q];
+  for (int l = blockIdx.x; l < r; l += gridDim.x)
+    for (int i = l + threadIdx.x; i < r; i += blockDim.x)
+      out[q * n * n + (int64_t)l * n + i] = Lt[q * n * n + (int64_t)l * n + perm[q * n + i]];
+}
+
+// work[q][i][c] = (L_S^{-1})[i][c]: a warp per column c, its entries in shared memory (or, for
+// n beyond it, in row c of the scratch array).  Right-looking: entry l is final after l
+// updates and is taken from all later ones, which keeps every entry's order of summation
+// and leaves one division, not a sum, on the serial chain.
+__global__ void __launch_bounds__(256) trinv_kernel(const double2* __restrict__ Lc, const int32_t* __restrict__ rank,
+                                                    const int* __restrict__ qlist, int n, int in_smem,
+                                                    double2* __restrict__ scratch, double2* __restrict__ work) {
+  extern __shared__ __align__(16) unsigned char chol_smem[];
+  const int64_t q = qlist[blockIdx.y];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarp = blockDim.x >> 5;
+  const int c = blockIdx.x * nwarp + warp;
+  const int r = rank[q];
   if (c >= r) return;
-  // L_S[i][l] = Lt[l][perm[i]]
-  for (int i = 0; i < r; ++i) {
-    if (i < c) {
-      work[(int64_t)i * n + c] = make_double2(0.0, 0.0);
-      continue;
-    }
-    const int pi = perm[i];
-    double2 acc = make_double2(i == c ? 1.0 : 0.0, 0.0);
-    for (int l = c; l < i; ++l) {
-      const double2 Lil = Lt[(int64_t)l * n + pi];
-      const double2 wl = work[(int64_t)l * n + c];
-      acc.x -= Lil.x * wl.x - Lil.y * wl.y;
-      acc.y -= Lil.x * wl.y + Lil.y * wl.x;
-    }
-    const double2 Lii = Lt[(int64_t)i * n + pi];
+  Lc += q * n * n;
+  work += q * n * n;
+  double2* x = in_smem ? reinterpret_cast<double2*>(chol_smem) + (int64_t)warp * n : scratch + q * n * n + (int64_t)c * n;
+  for (int i = c + lane; i < r; i += 32) x[i] = make_double2(i == c ? 1.0 : 0.0, 0.0);
+  __syncwarp();
+  for (int l = c; l < r; ++l) {
+    const double2 acc = x[l], Lii = Lc[(int64_t)l * n + l];
     // acc / Lii
-    const double den = Lii.x * Lii.x + Lii.y * Lii.y;
-    work[(int64_t)i * n + c] =
-        make_double2((acc.x * Lii.x + acc.y * Lii.y) / den, (acc.y * Lii.x - acc.x * Lii.y) / den);
+    const double den = __fma_rn(Lii.x, Lii.x, __dmul_rn(Lii.y, Lii.y));
+    const double2 wl = make_double2(__ddiv_rn(__fma_rn(acc.x, Lii.x, __dmul_rn(acc.y, Lii.y)), den),
+                                    __ddiv_rn(__fma_rn(acc.y, Lii.x, -__dmul_rn(acc.x, Lii.y)), den));
+    if (lane == 0) work[(int64_t)l * n + c] = wl;
+    for (int i = l + 1 + lane; i < r; i += 32) {
+      const double2 Lil = Lc[(int64_t)l * n + i];
+      double2 a = x[i];
+      // the order of the fused operations is written out: the solve amplifies their rounding
+      a.x = __dsub_rn(a.x, __fma_rn(Lil.x, wl.x, -__dmul_rn(Lil.y, wl.y)));
+      a.y = __dsub_rn(a.y, __fma_rn(Lil.y, wl.x, __dmul_rn(Lil.x, wl.y)));
+      x[i] = a;
+    }
+    __syncwarp();
   }
 }
 
 __global__ void scatter_w_kernel(const double2* __restrict__ work, const int32_t* __restrict__ perm,
-                                 const int32_t* __restrict__ rank, int n, int batch,
+                                 const int32_t* __restrict__ rank, const int* __restrict__ qlist, int n, int nq,
                                  double2* __restrict__ W) {
-  const int64_t total = (int64_t)batch * n * n;
+  const int64_t total = (int64_t)nq * n * n;
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total;
        e += (int64_t)gridDim.x * blockDim.x) {
-    const int b = (int)(e / ((int64_t)n * n));
+    const int64_t b = qlist[e / ((int64_t)n * n)];
     const int i = (int)((e / n) % n);
     const int c = (int)(e % n);
     const int r = rank[b];
     if (i < r && c < r) {
-      const int col = perm[(int64_t)b * n + c];
-      W[(int64_t)b * n * n + (int64_t)i * n + col] = work[e];
+      const int col = perm[b * n + c];
+      W[b * n * n + (int64_t)i * n + col] = work[b * n * n + (int64_t)i * n + c];
     }
   }
 }
@@ -172,27 +227,63 @@ inline int nblocks(int64_t total) {
 
 }  // namespace
 
-cudaError_t pchol_batched(cudaStream_t st, const double2* A, int n, int batch, double tol, double2* Lt,
-                          int32_t* perm, int32_t* rank, double* dwork) {
-  if (n <= 0 || batch <= 0) return cudaSuccess;
-  pchol_kernel<<<batch, 512, 0, st>>>(A, n, tol, Lt, perm, rank, dwork);
+cudaError_t pchol_batched(cudaStream_t st, const double2* A, int n, int neff, bool live, const int* qlist, int nq,
+                          double tol, double2* Lt, int32_t* perm, int32_t* rank) {
+  if (n <= 0 || nq <= 0) return cudaSuccess;
+  // blocks per matrix: up to eight (the portable cluster) while they do not fill the SMs
+  // four times over and keep a warp of rows each
+  int C = 1;
+  while (C < 8 && nq * C < 152 * 4 && neff > 32 * C) C *= 2;
+  int threads = std::min(256, std::max(32, ((neff + C - 1) / C + 31) / 32 * 32));
+  auto smem_of = [&](int c) {
+    const size_t per = (size_t)(neff + c - 1) / c;
+    return kBp * sizeof(double2) + per * (2 * sizeof(double) + 1);
+  };
+  size_t smem = smem_of(C);
+  if (smem > 220 * 1024) return cudaErrorInvalidValue;
+  if (smem > 40 * 1024) {
+    cudaError_t e = cudaFuncSetAttribute(pchol_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+  }
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)(nq * C));
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = (unsigned)C;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  cudaError_t e = cudaLaunchKernelEx(&cfg, pchol_kernel, A, n, neff, live ? 1 : 0, qlist, tol, Lt, perm, rank);
   count_launch();
-  return cudaGetLastError();
+  return e != cudaSuccess ? e : cudaGetLastError();
 }
 
-cudaError_t trinv_batched(cudaStream_t st, const double2* Lt, const int32_t* perm, const int32_t* rank,
-                          int n, int batch, double2* W, double2* work) {
-  if (n <= 0 || batch <= 0) return cudaSuccess;
-  dim3 g((n + 255) / 256, batch);
-  // work holds L_S^{-1} in pivot order (lower triangular); entries outside the
-  // rank stay zero
-  cudaError_t e = cudaMemsetAsync(work, 0, sizeof(double2) * (size_t)batch * n * n, st);
+// work holds L_S^{-1} in pivot order (lower triangular, zero outside the rank); tmp: nk n n of scratch.
+cudaError_t trinv_batched(cudaStream_t st, const double2* Lt, const int32_t* perm, const int32_t* rank, int n, int nk,
+                          const int* qlist, int nq, double2* W, double2* work, double2* tmp) {
+  if (n <= 0 || nq <= 0) return cudaSuccess;
+  const size_t bytes = sizeof(double2) * (size_t)nk * n * n;
+  cudaError_t e = cudaMemsetAsync(work, 0, bytes, st);
   if (e != cudaSuccess) return e;
-  trinv_kernel<<<g, 256, 0, st>>>(Lt, perm, rank, n, work);
+  tri_gather_kernel<<<dim3((unsigned)std::min(n, 64), nq), 128, 0, st>>>(Lt, perm, rank, qlist, n, tmp);
   count_launch();
-  e = cudaMemsetAsync(W, 0, sizeof(double2) * (size_t)batch * n * n, st);
+  int warps = 8;
+  while (warps > 1 && (size_t)warps * n * sizeof(double2) > 64 * 1024) warps /= 2;
+  const size_t smem = (size_t)warps * n * sizeof(double2);
+  const bool in_smem = smem <= 200 * 1024;
+  if (in_smem && smem > 40 * 1024) {
+    e = cudaFuncSetAttribute(trinv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+  }
+  trinv_kernel<<<dim3((n + warps - 1) / warps, nq), warps * 32, in_smem ? smem : 0, st>>>(tmp, rank, qlist, n, in_smem, W,
+                                                                                         work);
+  count_launch();
+  e = cudaMemsetAsync(W, 0, bytes, st);
   if (e != cudaSuccess) return e;
-  scatter_w_kernel<<<nblocks((int64_t)batch * n * n), 256, 0, st>>>(work, perm, rank, n, batch, W);
+  scatter_w_kernel<<<nblocks((int64_t)nq * n * n), 256, 0, st>>>(work, perm, rank, qlist, n, nq, W);
   count_launch();
   return cudaGetLastError();
 }
