@@ -54,16 +54,21 @@ inline void count_launch() {
 }
 
 // ------------------------------------------------------------------- kernels
-// Batched complex GEMM, row-major: C_b = alpha * op(A_b) op(B_b) + beta * C_b.
+// Batched complex GEMM, row-major: C_b = alpha * op(A_b) op(B_b).
 // op: 'N' as is, 'T' transpose, 'C' conjugate transpose, 'R' conjugate only.
-cudaError_t zgemm(cudaStream_t st, char opA, char opB, int m, int n, int k, double2 alpha,
-                  const double2* A, int64_t lda, int64_t sA, const double2* B, int64_t ldb,
-                  int64_t sB, double2 beta, double2* C, int64_t ldc, int64_t sC, int batch);
-// C_b = A_b * gather_rows(B_b, brow_b) with A_b (m x m) lower triangular: the
-// k > row blocks are skipped.  Rows with brow < 0 contribute zero.
-cudaError_t ztrmm_gather(cudaStream_t st, int m, int n, const double2* A, int64_t lda, int64_t sA,
-                         const int32_t* brow, int64_t sIdx, const double2* B, int64_t ldb, int64_t sB, double2* C,
-                         int64_t ldc, int64_t sC, int batch);
+// What the caller knows of the operands:
+struct ZOpt {
+  int lowerA = 0;                   // op(A_b) is lower triangular
+  const int32_t* brow = nullptr;    // op(B_b) = rows brow[b sIdx + k] of B_b ('N'; zero where negative)
+  int64_t sIdx = 0;
+  const int* qmap = nullptr;        // batch entry i works on matrix qmap[i] of each array
+  const int32_t* krank = nullptr;   // by matrix: op(A_b) is zero from row and column krank on
+};
+// FP64 FMA chains in the order of k.
+cudaError_t zgemm(cudaStream_t st, char opA, char opB, int m, int n, int k, double alpha, const double2* A, int64_t lda,
+                  int64_t sA, const double2* B, int64_t ldb, int64_t sB, double2* C, int64_t ldc, int64_t sC, int batch,
+                  const ZOpt& o = ZOpt());
+// Complex64, with beta * C_b added.
 cudaError_t cgemm(cudaStream_t st, char opA, char opB, int m, int n, int k, float2 alpha,
                   const float2* A, int64_t lda, int64_t sA, const float2* B, int64_t ldb,
                   int64_t sB, float2 beta, float2* C, int64_t ldc, int64_t sC, int batch);
@@ -132,9 +137,9 @@ cudaError_t pchol_batched(cudaStream_t st, const double2* A, int n, int neff, bo
 // (L_S^{-1} in pivot order) are zeroed for all nk matrices; tmp: nk n n of scratch.
 cudaError_t trinv_batched(cudaStream_t st, const double2* Lt, const int32_t* perm, const int32_t* rank, int n, int nk,
                           const int* qlist, int nq, double2* W, double2* work, double2* tmp);
-// Lpad[b][i][j] = L[i][j] (row-major, columns beyond the rank zero).
-cudaError_t lt_to_rowmajor(cudaStream_t st, const double2* Lt, const int32_t* rank, int n,
-                           int batch, double2* L);
+// Lpad[q][i][j] = L[i][j] (row-major, columns beyond the rank zero) for q in qlist.
+cudaError_t lt_to_rowmajor(cudaStream_t st, const double2* Lt, const int32_t* rank, const int* qlist, int nq, int n,
+                           double2* L);
 
 // Grid FFT of rows x[q][I][r] (complex128), in place:
 //   x <- sqrt(w(q+G)) * (1/N_g) FFT(e^{-i q.r} x)   with w = 4 pi/|q+G|^2, 0 at q+G = 0.
@@ -297,7 +302,7 @@ cudaError_t hadamard_t(cudaStream_t st, const double2* a, const double2* c, int 
 
 // FP64-accurate complex GEMM on the tensor cores (k_ztc.cu): C_b = alpha op(A_b) op(B_b),
 // any K, eight exact slices per operand (36 fp16 products), no less accurate than an FP64
-// FMA chain.  lowerA and brow as in ztrmm_gather.  work: zgemm_tc_work_bytes for the batch
+// FMA chain.  work: zgemm_tc_work_bytes for the batch
 // entries of one chunk (one at least); err: device word set on a bounded-wait timeout.
 // zgemm_tc_same: op(A) op(A)^T or ^H of one array, whose slices serve both sides.
 inline bool zgemm_tc_same(char opA, char opB, int m, int n, const double2* A, int64_t lda, int64_t sA,
@@ -308,8 +313,7 @@ inline bool zgemm_tc_same(char opA, char opB, int m, int n, const double2* A, in
 size_t zgemm_tc_work_bytes(int m, int n, int k, int nb, bool same);
 cudaError_t zgemm_tc(cudaStream_t st, char opA, char opB, int m, int n, int k, double alpha, const double2* A,
                      int64_t lda, int64_t sA, const double2* B, int64_t ldb, int64_t sB, double2* C, int64_t ldc,
-                     int64_t sC, int batch, int lowerA, const int32_t* brow, int64_t sIdx, void* work,
-                     size_t work_bytes, int* err);
+                     int64_t sC, int batch, const ZOpt& o, void* work, size_t work_bytes, int* err);
 
 // FP64-accurate complex GEMM on the tensor cores for 2K <= 128 (k_emu.cu):
 // C_b = op(A_b) B_b, op 'N' or 'R' (conjugate), seven exact 7-bit slices per

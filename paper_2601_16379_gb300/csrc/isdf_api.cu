@@ -385,7 +385,7 @@ int upload_basis(isdf_handle* h) {
 // C_b = alpha op(A_b) op(B_b) in complex128 (FP64-accurate): on the tensor cores with its slices
 // in the buffer `wname` (batch entries in chunks of kSliceBytes), on the FP64 pipe where the
 // inner dimension is too short to pay for the slicing or the workspace cannot be had.
-// lowerA / brow as in ztrmm_gather.  A bounded wait that expires sets the handle's error
+// A bounded wait that expires sets the handle's error
 // word, read by tc_status at the next synchronisation point.
 // wname NULL keeps the FP64 pipe.
 //
@@ -397,29 +397,33 @@ constexpr size_t kSliceBytes = (size_t)512 << 20;
 constexpr int kMinTcK = 6;
 int zmul(isdf_handle* h, const char* wname, char opA, char opB, int m, int n, int k, double alpha, const double2* A,
          int64_t lda, int64_t sA, const double2* B, int64_t ldb, int64_t sB, double2* C, int64_t ldc, int64_t sC,
-         int batch, int lowerA = 0, const int32_t* brow = nullptr, int64_t sIdx = 0) {
+         int batch, const ZOpt& o = ZOpt()) {
   void* w = nullptr;
   size_t bytes = 0;
   if (wname && k >= kMinTcK) {
-    const bool same = !brow && zgemm_tc_same(opA, opB, m, n, A, lda, sA, B, ldb, sB);
+    const bool same = !o.brow && zgemm_tc_same(opA, opB, m, n, A, lda, sA, B, ldb, sB);
     bytes = std::min(zgemm_tc_work_bytes(m, n, k, batch, same),
                      std::max(zgemm_tc_work_bytes(m, n, k, 1, same), kSliceBytes));
     w = h->ensure_evict(wname, bytes);
   }
   if (w)
-    CK(zgemm_tc(h->st, opA, opB, m, n, k, alpha, A, lda, sA, B, ldb, sB, C, ldc, sC, batch, lowerA, brow, sIdx, w,
-                bytes, (int*)h->buf("err_words")));
-  else if (lowerA || brow)
-    CK(ztrmm_gather(h->st, m, n, A, lda, sA, brow, sIdx, B, ldb, sB, C, ldc, sC, batch));
+    CK(zgemm_tc(h->st, opA, opB, m, n, k, alpha, A, lda, sA, B, ldb, sB, C, ldc, sC, batch, o, w, bytes,
+                (int*)h->buf("err_words")));
   else
-    CK(zgemm(h->st, opA, opB, m, n, k, make_double2(alpha, 0.0), A, lda, sA, B, ldb, sB, make_double2(0.0, 0.0), C, ldc,
-             sC, batch));
+    CK(zgemm(h->st, opA, opB, m, n, k, alpha, A, lda, sA, B, ldb, sB, C, ldc, sC, batch, o));
   return ISDF_OK;
 }
 #define ZM(...)                          \
   do {                                   \
     if (int e_ = zmul(h, __VA_ARGS__)) return e_; \
   } while (0)
+
+// Columns of L^q that are not zero: the largest rank of V_xi.
+int l_cols(const isdf_handle* h) {
+  int nv = 1;
+  for (int32_t r : h->ranks_v) nv = std::max(nv, (int)r);
+  return nv;
+}
 
 // Synchronise the stream and report a bounded wait that expired on the way.
 int tc_status(isdf_handle* h, const char* what) {
@@ -555,30 +559,31 @@ int coulomb_tail(isdf_handle* h, const QHalf& qh, int neff, double2* Vxi, void* 
   ENSURE(rankV, int32_t, "rankV", nk);
   ENSURE(qlist, int, "q_list", nk);
   CK(cudaMemcpyAsync(qlist, qh.list.data(), sizeof(int) * qh.list.size(), cudaMemcpyHostToDevice, h->st));
-  // the factor of the conjugate matrix is the conjugate factor, bit for bit
+  // the representatives only: L^-q is the conjugate of L^q, bit for bit
   CK(pchol_batched(h->st, Vxi, np, neff, false, qlist, qh.count, 1e-15, LtV, permV, rankV));
-  if (!qh.mirror.empty()) {
-    const int2* mir = (const int2*)h->buf("q_mirror");
-    const int nm = (int)qh.mirror.size();
-    CK(mirror_conj(h->st, LtV, (int64_t)np * np, mir, nm));
-    CK(mirror_copy(h->st, permV, np, mir, nm));
-    CK(mirror_copy(h->st, rankV, 1, mir, nm));
-  }
+  const int2* mir = (const int2*)h->buf("q_mirror");
+  const int nm = (int)qh.mirror.size();
+  CK(mirror_copy(h->st, rankV, 1, mir, nm));
   h->ranks_v.assign(nk, 0);
   CK(cudaMemcpyAsync(h->ranks_v.data(), rankV, sizeof(int32_t) * nk, cudaMemcpyDeviceToHost, h->st));
   ENSURE(Lxi, double2, "W_work", (size_t)nk * np * np);
-  CK(lt_to_rowmajor(h->st, LtV, rankV, np, nk, Lxi));
+  CK(lt_to_rowmajor(h->st, LtV, rankV, qlist, qh.count, np, Lxi));
   ENSURE(Lq, double2, "Lq", (size_t)nk * np * np);
-  // L^q in another rounding moves the FP64_TC integrals by 6e-10 of themselves: FP64 FMA there
-  ZM(h->prec == ISDF_FP64_TC ? nullptr : "zwork", 'T', 'N', np, np, np, 1.0, W, np, (int64_t)np * np, Lxi, np,
-     (int64_t)np * np, Lq, np, (int64_t)np * np, nk);
+  // W has neff rows and L_xi neff rows and columns that are not zero.  L^q in another rounding
+  // moves the FP64_TC integrals by 6e-10 of themselves: FP64 FMA there
+  const int64_t pp = (int64_t)np * np;
+  ZOpt reps;
+  reps.qmap = qlist;
+  CK(cudaMemsetAsync(Lq, 0, sizeof(double2) * (size_t)nk * pp, h->st));
+  ZM(h->prec == ISDF_FP64_TC ? nullptr : "zwork", 'T', 'N', np, neff, neff, 1.0, W, np, pp, Lxi, np, pp, Lq, np, pp,
+     qh.count, reps);
+  CK(mirror_conj(h->st, Lq, pp, mir, nm));
   if (V_out) {
     // V^q = W^T V_xi conj(W)
     double2* tmp = Lxi;  // reuse
-    ZM("zwork", 'N', 'R', np, np, np, 1.0, Vxi, np, (int64_t)np * np, W, np, (int64_t)np * np, tmp, np,
-             (int64_t)np * np, nk);
-    ZM("zwork", 'T', 'N', np, np, np, 1.0, W, np, (int64_t)np * np, tmp, np, (int64_t)np * np,
-             (double2*)V_out, np, (int64_t)np * np, nk);
+    ZM("zwork", 'N', 'R', neff, np, neff, 1.0, Vxi, np, pp, W, np, pp, tmp, np, pp, qh.count, reps);
+    ZM("zwork", 'T', 'N', np, np, neff, 1.0, W, np, pp, tmp, np, pp, (double2*)V_out, np, pp, qh.count, reps);
+    CK(mirror_conj(h->st, (double2*)V_out, pp, mir, nm));
   }
   if (h->prec == ISDF_MIXED) {
     ENSURE(Xf, float2, "X_f", (size_t)nk * np * h->nao);
@@ -853,12 +858,14 @@ int isdf_fit_zeta(isdf_handle* h, double solve_tol, int32_t* rank_out) {
   const int64_t pg = (int64_t)np * ng, xg = (int64_t)rx * ng;
   ENSURE(xi, double2, "xi", (size_t)nk * rx * ng);
   CK(trinv_batched(h->st, LtPi, permPi, rankPi, np, nk, qlist, qh.count, W, wwork, tri));
-  for (const auto& r : qh.runs) {
-    const int q0 = r.first, nq = r.second;
-    // xi^q = W eta^q = L_S^{-1} (eta^q rows in pivot order): triangular, gathered
-    ZM(zw, 'N', 'N', rx, ng, rx, 1.0, wwork + q0 * pp, np, pp, eta + q0 * pg, ng, pg, xi + q0 * xg, ng, xg,
-       nq, 1, permPi + (int64_t)q0 * np, np);
-  }
+  // xi^q = W eta^q = L_S^{-1} (eta^q rows in pivot order): triangular, gathered, up to the rank
+  ZOpt tri_opt;
+  tri_opt.lowerA = 1;
+  tri_opt.brow = permPi;
+  tri_opt.sIdx = np;
+  tri_opt.qmap = qlist;
+  tri_opt.krank = rankPi;
+  ZM(zw, 'N', 'N', rx, ng, rx, 1.0, wwork, np, pp, eta, ng, pg, xi, ng, xg, qh.count, tri_opt);
   if (!qh.mirror.empty()) {
     const int2* mir = (const int2*)h->buf("q_mirror");
     CK(mirror_conj(h->st, W, pp, mir, (int)qh.mirror.size()));
@@ -900,11 +907,14 @@ int isdf_coulomb_metric(isdf_handle* h, void* V_out) {
   // FP64_TC keeps the FMA chains: another order of rounding in V_xi moves single integrals
   // of its fragments by up to 5e-8 of the larger ones (see isdf_fit_zeta)
   if (h->prec != ISDF_MIXED) {
-    for (const auto& r : qh.runs) {
+    for (const auto& r : qh.runs)
       CK(grid_coulomb_fft(h->st, xi + r.first * xg, rx, r.first, r.second, h->cell, tw, gwork));
-      ZM(h->prec == ISDF_FP64 ? "grid_work_z" : nullptr, 'R', 'T', rx, rx, ng, h->volume, xi + r.first * xg, ng, xg,
-         xi + r.first * xg, ng, xg, Vxi + r.first * pp, np, pp, r.second);
-    }
+    ENSURE(qlist, int, "q_list", nk);
+    CK(cudaMemcpyAsync(qlist, qh.list.data(), sizeof(int) * qh.list.size(), cudaMemcpyHostToDevice, h->st));
+    ZOpt reps;
+    reps.qmap = qlist;
+    ZM(h->prec == ISDF_FP64 ? "grid_work_z" : nullptr, 'R', 'T', rx, rx, ng, h->volume, xi, ng, xg, xi, ng, xg, Vxi, np, pp,
+       qh.count, reps);
   } else {
     // mixed: xi rows to float-float in place, the grid FFT in float-float, and
     // V_xi = Omega conj(c')c'^T on the tensor cores with four exact slices (~2^-28 relative;
@@ -921,7 +931,6 @@ int isdf_coulomb_metric(isdf_handle* h, void* V_out) {
   if (!qh.mirror.empty()) {
     ENSURE(mir, int2, "q_mirror", qh.mirror.size());
     CK(cudaMemcpyAsync(mir, qh.mirror.data(), sizeof(int2) * qh.mirror.size(), cudaMemcpyHostToDevice, h->st));
-    CK(mirror_conj(h->st, Vxi, pp, mir, (int)qh.mirror.size()));
   }
   h->has_xi = false;  // xi was transformed in place (FP64) / is no longer needed
   return coulomb_tail(h, qh, rx, Vxi, V_out);
@@ -1376,15 +1385,16 @@ int isdf_ao_eri(isdf_handle* h, int n_quartet, const int32_t* quartets, void* ou
   ENSURE(Cc, double2, "ao_pairs_c", (size_t)np * nao2);
   ENSURE(U, double2, "ao_u", (size_t)np * nao2);
   ENSURE(Wm, double2, "ao_w", (size_t)np * nao2);
+  const int nv = l_cols(h);
   for (int n = 0; n < n_quartet; ++n) {
     const int32_t* k = quartets + 4 * n;
     const double2* L = Lq + qv[n] * pp;
     CK(ao_pairs(h->st, X + k[0] * pa, X + k[1] * pa, np, nao, A));
     CK(ao_pairs(h->st, X + k[2] * pa, X + k[3] * pa, np, nao, Cc));
     // (mu nu|lam sig) = Nk A^T V^Q C with V^Q = L L^H: (L^T A)^T (L^H C)
-    ZM("zwork", 'T', 'N', np, (int)nao2, np, 1.0, L, np, 0, A, nao2, 0, U, nao2, 0, 1);
-    ZM("zwork", 'C', 'N', np, (int)nao2, np, 1.0, L, np, 0, Cc, nao2, 0, Wm, nao2, 0, 1);
-    ZM("zwork", 'T', 'N', (int)nao2, (int)nao2, np, (double)nk, U, nao2, 0, Wm, nao2, 0, (double2*)out + (int64_t)n * nao2 * nao2, nao2, 0, 1);
+    ZM("zwork", 'T', 'N', nv, (int)nao2, np, 1.0, L, np, 0, A, nao2, 0, U, nao2, 0, 1);
+    ZM("zwork", 'C', 'N', nv, (int)nao2, np, 1.0, L, np, 0, Cc, nao2, 0, Wm, nao2, 0, 1);
+    ZM("zwork", 'T', 'N', (int)nao2, (int)nao2, nv, (double)nk, U, nao2, 0, Wm, nao2, 0, (double2*)out + (int64_t)n * nao2 * nao2, nao2, 0, 1);
   }
   return tc_status(h, "isdf_ao_eri");
 }
@@ -1432,7 +1442,7 @@ int isdf_sos_polarizability(isdf_handle* h, const void* C, int n_mo, int n_occ, 
   CK(kdft_cols(h->st, chi, pp, km, -1, -1, 0, 1.0 / nk));
   if (s_out) {
     // S = Nk^2 sum_Q tr[conj(V^Q) chi^Q conj(V^Q) (chi^{-Q})^T], V^Q = L^Q L^Q^H (Eq. 12)
-    ZM("zwork", 'N', 'C', np, np, np, 1.0, Lq, np, pp, Lq, np, pp, Vq, np, pp, nk);
+    ZM("zwork", 'N', 'C', np, np, l_cols(h), 1.0, Lq, np, pp, Lq, np, pp, Vq, np, pp, nk);
     ZM("zwork", 'R', 'N', np, np, np, 1.0, Vq, np, pp, chi, np, pp, T1, np, pp, nk);
     ZM("zwork", 'N', 'R', np, np, np, 1.0, T1, np, pp, Vq, np, pp, Go, np, pp, nk);  // Go reused
     CK(sos_trace_parts(h->st, Go, chi, h->cell.kmesh, np, part));
@@ -1464,8 +1474,8 @@ int isdf_exchange(isdf_handle* h, const void* P, void* K_out) {
   ZM("zwork", 'N', 'C', np, np, nao, 1.0, t1, nao, (int64_t)np * nao, X, nao, (int64_t)np * nao, rho, np,
            (int64_t)np * np, nk);
   // V^q = L^q L^q^H
-  ZM("zwork", 'N', 'C', np, np, np, 1.0, Lq, np, (int64_t)np * np, Lq, np, (int64_t)np * np, Vd, np,
-           (int64_t)np * np, nk);
+  ZM("zwork", 'N', 'C', np, np, l_cols(h), 1.0, Lq, np, (int64_t)np * np, Lq, np, (int64_t)np * np, Vd, np,
+     (int64_t)np * np, nk);
   // Gamma^k = sum_k' (V^{k'-k})^T o rho^{k'}: DFT_- V, DFT_+ rho, transposed product, DFT_- / Nk
   CK(kdft_cols(h->st, Vd, (int64_t)np * np, km, -1, -1, 0, 1.0));
   CK(kdft_cols(h->st, rho, (int64_t)np * np, km, +1, +1, 0, 1.0));

@@ -208,14 +208,21 @@ __global__ void scatter_w_kernel(const double2* __restrict__ work, const int32_t
 }
 
 __global__ void lt_to_row_kernel(const double2* __restrict__ Lt, const int32_t* __restrict__ rank,
-                                 int n, int batch, double2* __restrict__ L) {
-  const int64_t total = (int64_t)batch * n * n;
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total;
-       e += (int64_t)gridDim.x * blockDim.x) {
-    const int b = (int)(e / ((int64_t)n * n));
-    const int i = (int)((e / n) % n);
-    const int j = (int)(e % n);
-    L[e] = (j < rank[b]) ? Lt[(int64_t)b * n * n + (int64_t)j * n + i] : make_double2(0.0, 0.0);
+                                 const int* __restrict__ qlist, int n, double2* __restrict__ L) {
+  // 32 x 32 tiles transposed through shared memory
+  __shared__ double2 t[32][33];
+  const int64_t q = qlist[blockIdx.z];
+  const int i0 = blockIdx.x * 32, j0 = blockIdx.y * 32, r = rank[q];
+  Lt += q * n * n;
+  L += q * n * n;
+  for (int y = threadIdx.y; y < 32; y += 8) {
+    const int j = j0 + y, i = i0 + threadIdx.x;
+    t[y][threadIdx.x] = (i < n && j < r) ? Lt[(int64_t)j * n + i] : make_double2(0.0, 0.0);
+  }
+  __syncthreads();
+  for (int y = threadIdx.y; y < 32; y += 8) {
+    const int i = i0 + y, j = j0 + threadIdx.x;
+    if (i < n && j < n) L[(int64_t)i * n + j] = t[threadIdx.x][y];
   }
 }
 
@@ -288,9 +295,11 @@ cudaError_t trinv_batched(cudaStream_t st, const double2* Lt, const int32_t* per
   return cudaGetLastError();
 }
 
-cudaError_t lt_to_rowmajor(cudaStream_t st, const double2* Lt, const int32_t* rank, int n, int batch,
+cudaError_t lt_to_rowmajor(cudaStream_t st, const double2* Lt, const int32_t* rank, const int* qlist, int nq, int n,
                            double2* L) {
-  lt_to_row_kernel<<<nblocks((int64_t)batch * n * n), 256, 0, st>>>(Lt, rank, n, batch, L);
+  if (n <= 0 || nq <= 0) return cudaSuccess;
+  const unsigned nt = (unsigned)((n + 31) / 32);
+  lt_to_row_kernel<<<dim3(nt, nt, nq), dim3(32, 8), 0, st>>>(Lt, rank, qlist, n, L);
   count_launch();
   return cudaGetLastError();
 }

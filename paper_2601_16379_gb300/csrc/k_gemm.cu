@@ -69,26 +69,30 @@ __device__ __forceinline__ float2 finish(float2 acc, float2 lo) {
 
 // Optional structure: lowerA skips the k > row part of a lower-triangular
 // op(A); brow (with batch stride sIdx) gathers the rows of B ('N' only):
-// op(B)[kk][n] = B[brow[kk]][n], 0 where brow[kk] < 0.
+// op(B)[kk][n] = B[brow[kk]][n], 0 where brow[kk] < 0.  qmap: batch entry z works on matrix
+// qmap[z] of each array; krank (by matrix): op(A) is zero from row and column krank on.
+// What is known to be zero is not multiplied; the order of the other terms stays.
 template <typename T, int BK>
 __global__ void __launch_bounds__(256, 2) gemm_kernel(char opA, char opB, int m, int n, int k, T alpha,
                                                    const T* __restrict__ A, int64_t lda, int64_t sA,
                                                    const T* __restrict__ B, int64_t ldb, int64_t sB,
                                                    T beta, T* __restrict__ C, int64_t ldc,
                                                    int64_t sC, int lowerA, const int32_t* __restrict__ brow,
-                                                   int64_t sIdx) {
+                                                   int64_t sIdx, const int* __restrict__ qmap,
+                                                   const int32_t* __restrict__ krank) {
   constexpr int BM = 64, BN = 64;
   __shared__ T As[BK][BM + 1];
   __shared__ T Bs[BK][BN + 1];
   const int tid = threadIdx.x;
   const int tx = tid % 16, ty = tid / 16;
   const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
-  const int64_t b = blockIdx.z;
+  const int64_t b = qmap ? qmap[blockIdx.z] : (int)blockIdx.z;
   A += b * sA;
   B += b * sB;
   C += b * sC;
   if (brow) brow += b * sIdx;
-  const int kend = lowerA ? min(k, m0 + BM) : k;
+  int kend = lowerA ? min(k, m0 + BM) : k;
+  if (krank) kend = krank[b] > m0 ? min(kend, krank[b]) : 0;
   const bool aT = (opA == 'T' || opA == 'C');
   const bool aC = (opA == 'C' || opA == 'R');
   const bool bT = (opB == 'T' || opB == 'C');
@@ -195,17 +199,20 @@ __global__ void __launch_bounds__(256, 2) gemm_kernel(char opA, char opB, int m,
 #pragma unroll
         for (int j = 0; j < 4; ++j) fold(acc[i][j], lo[i][j], part[i][j]);
     } else {
+      // rows m0 + 16 i .. + 15 of a lower-triangular op(A) end at k = m0 + 16 i + 15
+      const int lo_i = lowerA && k0 > m0 ? (k0 - m0) / 16 : 0;
 #pragma unroll
       for (int kk = 0; kk < BK; ++kk) {
-        T a[4], bb[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) a[i] = As[kk][ty + 16 * i];
+        T bb[4];
 #pragma unroll
         for (int j = 0; j < 4; ++j) bb[j] = Bs[kk][tx + 16 * j];
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
+        for (int i = 0; i < 4; ++i) {
+          if (i < lo_i) continue;
+          const T a = As[kk][ty + 16 * i];
 #pragma unroll
-          for (int j = 0; j < 4; ++j) cfma_t(acc[i][j], a[i], bb[j]);
+          for (int j = 0; j < 4; ++j) cfma_t(acc[i][j], a, bb[j]);
+        }
       }
     }
     __syncthreads();
@@ -236,15 +243,18 @@ template <typename T, int BK>
 static cudaError_t gemm_launch(cudaStream_t st, char opA, char opB, int m, int n, int k, T alpha,
                                const T* A, int64_t lda, int64_t sA, const T* B, int64_t ldb,
                                int64_t sB, T beta, T* C, int64_t ldc, int64_t sC, int batch,
-                               int lowerA = 0, const int32_t* brow = nullptr, int64_t sIdx = 0) {
+                               int lowerA = 0, const int32_t* brow = nullptr, int64_t sIdx = 0,
+                               const int* qmap = nullptr, const int32_t* krank = nullptr) {
   if (m <= 0 || n <= 0 || batch <= 0) return cudaSuccess;
   if (batch > 65535) {
     // split very large batches
     for (int b0 = 0; b0 < batch; b0 += 65535) {
       int nb = batch - b0 < 65535 ? batch - b0 : 65535;
-      cudaError_t e = gemm_launch<T, BK>(st, opA, opB, m, n, k, alpha, A + b0 * sA, lda, sA,
-                                         B + b0 * sB, ldb, sB, beta, C + b0 * sC, ldc, sC, nb, lowerA,
-                                         brow ? brow + b0 * sIdx : nullptr, sIdx);
+      const int64_t o = qmap ? 0 : b0;
+      cudaError_t e = gemm_launch<T, BK>(st, opA, opB, m, n, k, alpha, A + o * sA, lda, sA,
+                                         B + o * sB, ldb, sB, beta, C + o * sC, ldc, sC, nb, lowerA,
+                                         brow ? brow + o * sIdx : nullptr, sIdx, qmap ? qmap + b0 : nullptr,
+                                         krank ? krank + o : nullptr);
       if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
@@ -253,23 +263,16 @@ static cudaError_t gemm_launch(cudaStream_t st, char opA, char opB, int m, int n
   if (grid.y > 65535) return cudaErrorInvalidValue;
   if (brow && opB != 'N') return cudaErrorInvalidValue;
   gemm_kernel<T, BK><<<grid, 256, 0, st>>>(opA, opB, m, n, k, alpha, A, lda, sA, B, ldb, sB, beta,
-                                           C, ldc, sC, lowerA, brow, sIdx);
+                                           C, ldc, sC, lowerA, brow, sIdx, qmap, krank);
   count_launch();
   return cudaGetLastError();
 }
 
-cudaError_t zgemm(cudaStream_t st, char opA, char opB, int m, int n, int k, double2 alpha,
-                  const double2* A, int64_t lda, int64_t sA, const double2* B, int64_t ldb,
-                  int64_t sB, double2 beta, double2* C, int64_t ldc, int64_t sC, int batch) {
-  return gemm_launch<double2, 8>(st, opA, opB, m, n, k, alpha, A, lda, sA, B, ldb, sB, beta, C,
-                                 ldc, sC, batch);
-}
-
-cudaError_t ztrmm_gather(cudaStream_t st, int m, int n, const double2* A, int64_t lda, int64_t sA,
-                         const int32_t* brow, int64_t sIdx, const double2* B, int64_t ldb, int64_t sB, double2* C,
-                         int64_t ldc, int64_t sC, int batch) {
-  return gemm_launch<double2, 8>(st, 'N', 'N', m, n, m, make_double2(1.0, 0.0), A, lda, sA, B, ldb, sB,
-                                 make_double2(0.0, 0.0), C, ldc, sC, batch, 1, brow, sIdx);
+cudaError_t zgemm(cudaStream_t st, char opA, char opB, int m, int n, int k, double alpha, const double2* A, int64_t lda,
+                  int64_t sA, const double2* B, int64_t ldb, int64_t sB, double2* C, int64_t ldc, int64_t sC, int batch,
+                  const ZOpt& o) {
+  return gemm_launch<double2, 8>(st, opA, opB, m, n, k, make_double2(alpha, 0.0), A, lda, sA, B, ldb, sB,
+                                 make_double2(0.0, 0.0), C, ldc, sC, batch, o.lowerA, o.brow, o.sIdx, o.qmap, o.krank);
 }
 
 cudaError_t cgemm(cudaStream_t st, char opA, char opB, int m, int n, int k, float2 alpha,

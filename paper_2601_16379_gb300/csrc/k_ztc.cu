@@ -97,6 +97,8 @@ struct Args {
   int mt, nt, mb, nb;       // tiles of 64 rows and 32 columns; 32-row blocks per batch entry of A and B
   int64_t ntiles;
   int lower;                // op(A) lower triangular: k < m0 + 64 only
+  const int* qmap;          // batch entry -> matrix (or NULL)
+  const int32_t* krank;     // by matrix: op(A) is zero from row and column krank on (or NULL)
   int neg_ri, neg_ir, neg_ii;  // signs of re x im, im x re, im x im
   int* err;
 };
@@ -175,7 +177,14 @@ __global__ void __launch_bounds__(NT, 1) zgemm_tc_kernel(Args args) {
     ti = rem / args.nt;
     tj = rem % args.nt;
   };
-  auto kblocks = [&](int ti) { return args.lower ? min(args.nkb, (ti + 1) * (BM / BK)) : args.nkb; };
+  auto kblocks = [&](int b, int ti) {
+    int nk = args.lower ? min(args.nkb, (ti + 1) * (BM / BK)) : args.nkb;
+    if (args.krank) {
+      const int r = args.krank[args.qmap ? args.qmap[b] : b];
+      nk = r > ti * BM ? min(nk, (r + BK - 1) / BK) : 0;
+    }
+    return nk;
+  };
 
   if (warp == 0) {
     if (lane == 0) {
@@ -184,7 +193,7 @@ __global__ void __launch_bounds__(NT, 1) zgemm_tc_kernel(Args args) {
       for (int64_t t = blockIdx.x; t < args.ntiles && ok; t += gridDim.x) {
         int b, ti, tj;
         tile_of(t, b, ti, tj);
-        const int nk = kblocks(ti);
+        const int nk = kblocks(b, ti);
         const __half* a0 = args.SA + ((int64_t)b * args.mb + 2 * ti) * args.nkb * kBlk;
         // the second row block of the last tile may not exist: its rows are not stored
         const __half* a1 = (2 * ti + 1 < args.mb) ? a0 + (int64_t)args.nkb * kBlk : a0;
@@ -214,7 +223,7 @@ __global__ void __launch_bounds__(NT, 1) zgemm_tc_kernel(Args args) {
       for (int64_t t = blockIdx.x; t < args.ntiles && ok; t += gridDim.x) {
         int b, ti, tj;
         tile_of(t, b, ti, tj);
-        const int nk = kblocks(ti);
+        const int nk = kblocks(b, ti);
         for (int kb = 0; kb < nk; ++kb, ++it) {
           const bool first = (kb % kChunk) == 0;
           if (first && ch > 0) {
@@ -270,7 +279,7 @@ __global__ void __launch_bounds__(NT, 1) zgemm_tc_kernel(Args args) {
     for (int64_t t = blockIdx.x; t < args.ntiles; t += gridDim.x) {
       int b, ti, tj;
       tile_of(t, b, ti, tj);
-      const int nch = (kblocks(ti) + kChunk - 1) / kChunk;
+      const int nch = (kblocks(b, ti) + kChunk - 1) / kChunk;
       long long hi[kDrainCols], lo[kDrainCols];
 #pragma unroll
       for (int j = 0; j < kDrainCols; ++j) hi[j] = lo[j] = 0;
@@ -330,7 +339,7 @@ __global__ void __launch_bounds__(NT, 1) zgemm_tc_kernel(Args args) {
       for (int j = 0; j < kKeep; ++j) out[(row * BN + ((col0 + j) ^ lane)) * 2 + part] = x[j];
       asm volatile("bar.sync 1, 512;" ::: "memory");
       if (ok) {
-        double2* C = args.C + (int64_t)b * args.sC;
+        double2* C = args.C + (int64_t)(args.qmap ? args.qmap[b] : b) * args.sC;
         const int wv = warp - 2, n = n0 + lane;
         const double2* o2 = reinterpret_cast<const double2*>(outS);
 #pragma unroll 4
@@ -425,10 +434,10 @@ __device__ __forceinline__ int64_t slot_of(int r, int kc, int nkb) {
 // Rows stored contiguously along k: a block takes eight rows, one warp per row for the
 // largest entry, then eight lanes per 128-byte line of the slices.
 __global__ void __launch_bounds__(256) zslice_rows_kernel(const double2* __restrict__ X, int64_t ld, int64_t sX, int rows,
-                                                          int K, int nkb, int nblk, __half* __restrict__ S,
-                                                          int* __restrict__ ex) {
+                                                          int K, int nkb, int nblk, const int* __restrict__ qmap,
+                                                          __half* __restrict__ S, int* __restrict__ ex) {
   const int b = blockIdx.y, r0 = blockIdx.x * 8, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  X += (int64_t)b * sX;
+  X += (int64_t)(qmap ? qmap[b] : b) * sX;
   S += (int64_t)b * nblk * nkb * kBlk;
   __shared__ int se[8];
   {
@@ -460,11 +469,13 @@ __global__ void __launch_bounds__(256) zslice_rows_kernel(const double2* __restr
 // (k -> idx[k], none where negative): a block takes 32 rows, lanes along them.
 __global__ void __launch_bounds__(256) zslice_cols_kernel(const double2* __restrict__ X, int64_t ld, int64_t sX, int rows,
                                                           int K, int nkb, int nblk, const int32_t* __restrict__ idx,
-                                                          int64_t sIdx, __half* __restrict__ S, int* __restrict__ ex) {
+                                                          int64_t sIdx, const int* __restrict__ qmap,
+                                                          __half* __restrict__ S, int* __restrict__ ex) {
   const int b = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31, r = blockIdx.x * 32 + lane;
-  X += (int64_t)b * sX + r;
+  const int qb = qmap ? qmap[b] : b;
+  X += (int64_t)qb * sX + r;
   S += (int64_t)b * nblk * nkb * kBlk;
-  if (idx) idx += (int64_t)b * sIdx;
+  if (idx) idx += (int64_t)qb * sIdx;
   const bool in = r < rows;
   auto at = [&](int k) {
     const int kk = idx ? __ldg(idx + k) : k;
@@ -495,13 +506,13 @@ inline size_t slice_bytes(int rows, int k, int nb) { return (size_t)nb * cdiv(ro
 // Slices of op(X) by rows (side A) or of op(X)^T (side B): `cols` when the wanted rows run
 // along the fast index of the array.
 cudaError_t slice(cudaStream_t st, bool cols, const double2* X, int64_t ld, int64_t sX, int rows, int K, int batch,
-                  const int32_t* idx, int64_t sIdx, __half* S, int* ex) {
+                  const int32_t* idx, int64_t sIdx, const int* qmap, __half* S, int* ex) {
   const int nkb = (int)cdiv(K, BK), nblk = (int)cdiv(rows, RB);
   if (cols)
-    zslice_cols_kernel<<<dim3((unsigned)cdiv(rows, 32), batch), 256, 0, st>>>(X, ld, sX, rows, K, nkb, nblk, idx, sIdx, S,
-                                                                             ex);
+    zslice_cols_kernel<<<dim3((unsigned)cdiv(rows, 32), batch), 256, 0, st>>>(X, ld, sX, rows, K, nkb, nblk, idx, sIdx,
+                                                                             qmap, S, ex);
   else
-    zslice_rows_kernel<<<dim3((unsigned)cdiv(rows, 8), batch), 256, 0, st>>>(X, ld, sX, rows, K, nkb, nblk, S, ex);
+    zslice_rows_kernel<<<dim3((unsigned)cdiv(rows, 8), batch), 256, 0, st>>>(X, ld, sX, rows, K, nkb, nblk, qmap, S, ex);
   count_launch();
   return cudaGetLastError();
 }
@@ -514,14 +525,13 @@ size_t zgemm_tc_work_bytes(int m, int n, int k, int nb, bool same) {
 
 cudaError_t zgemm_tc(cudaStream_t st, char opA, char opB, int m, int n, int k, double alpha, const double2* A,
                      int64_t lda, int64_t sA, const double2* B, int64_t ldb, int64_t sB, double2* C, int64_t ldc,
-                     int64_t sC, int batch, int lowerA, const int32_t* brow, int64_t sIdx, void* work,
-                     size_t work_bytes, int* err) {
+                     int64_t sC, int batch, const ZOpt& o, void* work, size_t work_bytes, int* err) {
   using namespace ztc;
   if (m <= 0 || n <= 0 || k <= 0 || batch <= 0) return cudaSuccess;
-  if (brow && opB != 'N') return cudaErrorInvalidValue;
+  if (o.brow && opB != 'N') return cudaErrorInvalidValue;
   const bool aT = opA == 'T' || opA == 'C', aC = opA == 'C' || opA == 'R';
   const bool bT = opB == 'T' || opB == 'C', bC = opB == 'C' || opB == 'R';
-  const bool same = !brow && zgemm_tc_same(opA, opB, m, n, A, lda, sA, B, ldb, sB);
+  const bool same = !o.brow && zgemm_tc_same(opA, opB, m, n, A, lda, sA, B, ldb, sB);
   const size_t per = slice_bytes(m, k, 1) + (same ? 0 : slice_bytes(n, k, 1)) + sizeof(int) * (size_t)(m + n);
   if (work_bytes < per + 256) return cudaErrorInvalidValue;
   const int nbc = (int)std::min<size_t>((size_t)std::min(batch, 65535), (work_bytes - 256) / per);
@@ -540,16 +550,19 @@ cudaError_t zgemm_tc(cudaStream_t st, char opA, char opB, int m, int n, int k, d
     __half* SB = same ? SA : SA + slice_bytes(m, k, nb) / 2;
     int* eA = reinterpret_cast<int*>(SB + slice_bytes(n, k, nb) / 2);  // n = m where SB is SA
     int* eB = same ? eA : eA + (size_t)nb * m;
-    e = slice(st, aT, A + b0 * sA, lda, sA, m, k, nb, nullptr, 0, SA, eA);
+    // with a map the arrays stay where they are and the map moves on
+    const int* qm = o.qmap ? o.qmap + b0 : nullptr;
+    const int64_t s0 = qm ? 0 : b0;
+    e = slice(st, aT, A + s0 * sA, lda, sA, m, k, nb, nullptr, 0, qm, SA, eA);
     if (e == cudaSuccess && !same)
-      e = slice(st, !bT, B + b0 * sB, ldb, sB, n, k, nb, brow ? brow + b0 * sIdx : nullptr, sIdx, SB, eB);
+      e = slice(st, !bT, B + s0 * sB, ldb, sB, n, k, nb, o.brow ? o.brow + s0 * o.sIdx : nullptr, o.sIdx, qm, SB, eB);
     if (e != cudaSuccess) return e;
     Args a{};
     a.SA = SA;
     a.SB = SB;
     a.eA = eA;
     a.eB = eB;
-    a.C = C + b0 * sC;
+    a.C = C + s0 * sC;
     a.ldc = ldc;
     a.sC = sC;
     a.alpha = alpha;
@@ -562,7 +575,9 @@ cudaError_t zgemm_tc(cudaStream_t st, char opA, char opB, int m, int n, int k, d
     a.mb = (int)cdiv(m, RB);
     a.nb = (int)cdiv(n, RB);
     a.ntiles = (int64_t)nb * a.mt * a.nt;
-    a.lower = lowerA;
+    a.lower = o.lowerA;
+    a.qmap = qm;
+    a.krank = o.krank ? o.krank + s0 : nullptr;
     // a = ar + i ca ai, b = br + i cb bi:  Re = ar br - ca cb ai bi,  Im = cb ar bi + ca ai br
     a.neg_ri = bC;
     a.neg_ir = aC;
