@@ -63,6 +63,7 @@ struct ZOpt {
   int64_t sIdx = 0;
   const int* qmap = nullptr;        // batch entry i works on matrix qmap[i] of each array
   const int32_t* krank = nullptr;   // by matrix: op(A_b) is zero from row and column krank on
+  int slices = 8;                   // zgemm_tc: 8, or 7 for k <= kZgemm7MaxK
 };
 // FP64 FMA chains in the order of k.
 cudaError_t zgemm(cudaStream_t st, char opA, char opB, int m, int n, int k, double alpha, const double2* A, int64_t lda,
@@ -302,28 +303,20 @@ cudaError_t hadamard_t(cudaStream_t st, const double2* a, const double2* c, int 
 
 // FP64-accurate complex GEMM on the tensor cores (k_ztc.cu): C_b = alpha op(A_b) op(B_b),
 // any K, eight exact slices per operand (36 fp16 products), no less accurate than an FP64
-// FMA chain.  work: zgemm_tc_work_bytes for the batch
+// FMA chain; or seven (28 products, ~2^-48), the fixed arithmetic of g and T in the mixed and
+// FP64_TC paths.  work: zgemm_tc_work_bytes for the batch
 // entries of one chunk (one at least); err: device word set on a bounded-wait timeout.
 // zgemm_tc_same: op(A) op(A)^T or ^H of one array, whose slices serve both sides.
+constexpr int kZgemm7MaxK = 64;
 inline bool zgemm_tc_same(char opA, char opB, int m, int n, const double2* A, int64_t lda, int64_t sA,
                           const double2* B, int64_t ldb, int64_t sB) {
   const bool aT = opA == 'T' || opA == 'C', bT = opB == 'T' || opB == 'C';
   return A == B && lda == ldb && sA == sB && m == n && aT != bT;
 }
-size_t zgemm_tc_work_bytes(int m, int n, int k, int nb, bool same);
+size_t zgemm_tc_work_bytes(int slices, int m, int n, int k, int nb, bool same);
 cudaError_t zgemm_tc(cudaStream_t st, char opA, char opB, int m, int n, int k, double alpha, const double2* A,
                      int64_t lda, int64_t sA, const double2* B, int64_t ldb, int64_t sB, double2* C, int64_t ldc,
                      int64_t sC, int batch, const ZOpt& o, void* work, size_t work_bytes, int* err);
-
-// FP64-accurate complex GEMM on the tensor cores for 2K <= 128 (k_emu.cu):
-// C_b = op(A_b) B_b, op 'N' or 'R' (conjugate), seven exact 7-bit slices per
-// operand.  work: zgemm_emu_work_bytes(M, N, K, batch) bytes; err: device word
-// set on a bounded-wait timeout.
-bool zgemm_emu_supported(int K);
-size_t zgemm_emu_work_bytes(int M, int N, int K, int batch);
-cudaError_t zgemm_emu(cudaStream_t st, char opA, int M, int N, int K, const double2* A, int64_t lda, int64_t sA,
-                      const double2* B, int64_t ldb, int64_t sB, double2* C, int64_t ldc, int64_t sC, int batch,
-                      void* work, int* err);
 
 // Precision conversions.
 cudaError_t z2c(cudaStream_t st, const double2* in, float2* out, int64_t n);

@@ -400,10 +400,10 @@ int zmul(isdf_handle* h, const char* wname, char opA, char opB, int m, int n, in
          int batch, const ZOpt& o = ZOpt()) {
   void* w = nullptr;
   size_t bytes = 0;
-  if (wname && k >= kMinTcK) {
+  if (wname && (k >= kMinTcK || o.slices == 7)) {
     const bool same = !o.brow && zgemm_tc_same(opA, opB, m, n, A, lda, sA, B, ldb, sB);
-    bytes = std::min(zgemm_tc_work_bytes(m, n, k, batch, same),
-                     std::max(zgemm_tc_work_bytes(m, n, k, 1, same), kSliceBytes));
+    bytes = std::min(zgemm_tc_work_bytes(o.slices, m, n, k, batch, same),
+                     std::max(zgemm_tc_work_bytes(o.slices, m, n, k, 1, same), kSliceBytes));
     w = h->ensure_evict(wname, bytes);
   }
   if (w)
@@ -809,20 +809,10 @@ int isdf_fit_zeta(isdf_handle* h, double solve_tol, int32_t* rank_out) {
   CK(kdft_cols(h->st, Pi, (int64_t)np * np, km, +1, -1, 1, 1.0 / nk));
   // eta^q (Eq. 5): g^k_I(r) = sum_mu conj(X^k_I mu) Phi^k_mu(r), then the k-convolution.
   ENSURE(eta, double2, "eta", (size_t)nk * np * ng);
-  if (!fp64 && zgemm_emu_supported(nao)) {
-    const size_t per_k = zgemm_emu_work_bytes(np, ng, nao, 1);
-    const int nkc = (int)std::max<size_t>(1, std::min<size_t>((size_t)nk, ((size_t)4 << 30) / per_k));
-    ENSURE(gw, uint8_t, "grid_work_z", zgemm_emu_work_bytes(np, ng, nao, nkc));
-    for (int k0 = 0; k0 < nk; k0 += nkc) {
-      const int nb = std::min(nkc, nk - k0);
-      CK(zgemm_emu(h->st, 'R', np, ng, nao, X + (int64_t)k0 * np * nao, nao, (int64_t)np * nao,
-                   phi + (int64_t)k0 * nao * ng, ng, (int64_t)nao * ng, eta + (int64_t)k0 * np * ng, ng,
-                   (int64_t)np * ng, nb, gw, (int*)h->buf("err_words")));
-    }
-  } else {
-    ZM(zw, 'R', 'N', np, ng, nao, 1.0, X, nao, (int64_t)np * nao, phi, ng, (int64_t)nao * ng, eta, ng,
-       (int64_t)np * ng, nk);
-  }
+  ZOpt g_opt;
+  if (!fp64 && nao <= kZgemm7MaxK) g_opt.slices = 7;
+  ZM(fp64 || g_opt.slices == 7 ? "grid_work_z" : nullptr, 'R', 'N', np, ng, nao, 1.0, X, nao, (int64_t)np * nao, phi, ng,
+     (int64_t)nao * ng, eta, ng, (int64_t)np * ng, nk, g_opt);
   // the k-convolution of Algorithm 1 over the grid columns: FP64 in the FP64 path,
   // float-float (~2^-44 relative, FP32 arithmetic) in the others
   if (h->prec == ISDF_FP64)
@@ -1219,14 +1209,10 @@ int isdf_fragment_eri(isdf_handle* h, int n_frag, const int32_t* n_orb, const vo
             // T = X C FP64-class (seven exact slices; see isdf_fit_zeta on the fixed arithmetic; FP64
             // beyond N_AO = 64), then float-float in place for the DFT and the pair rows
             double2* Tz = reinterpret_cast<double2*>(T);
-            if (zgemm_emu_supported(nao)) {
-              ENSURE(tew, uint8_t, "frag_T_emu", zgemm_emu_work_bytes(np, nfmax, nao, nk));
-              CK(zgemm_emu(h->st, 'N', np, nf, nao, Xz, nao, (int64_t)np * nao, (const double2*)C[f], nf,
-                           (int64_t)nao * nf, Tz, nf, (int64_t)np * nf, nk, tew, errw));
-            } else {
-              ZM(nullptr, 'N', 'N', np, nf, nao, 1.0, Xz, nao, (int64_t)np * nao, (const double2*)C[f], nf,
-                 (int64_t)nao * nf, Tz, nf, (int64_t)np * nf, nk);
-            }
+            ZOpt t_opt;
+            if (nao <= kZgemm7MaxK) t_opt.slices = 7;
+            ZM(t_opt.slices == 7 ? "tc_zwork" : nullptr, 'N', 'N', np, nf, nao, 1.0, Xz, nao, (int64_t)np * nao,
+               (const double2*)C[f], nf, (int64_t)nao * nf, Tz, nf, (int64_t)np * nf, nk, t_opt);
             ffcomplex* Tff = reinterpret_cast<ffcomplex*>(Tz);
             CK(z2ff(h->st, Tz, Tff, (int64_t)nk * np * nf));
             CK(kdft_cols_ff(h->st, Tff, (int64_t)np * nf, km, +1, +1, 0, 1.0));

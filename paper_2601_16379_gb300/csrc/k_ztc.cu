@@ -29,6 +29,10 @@
 // N = 128 would need the accumulators of two passes, whose 64-bit sums (16 bytes per entry)
 // would fill the register file.
 //
+// Seven slices (K <= 64): the form in which the mixed and FP64_TC paths have their g and T, with
+// ~2^-48 of the rows' largest entries; digits and sums are those of that form bit for bit, on
+// the same kernel.
+//
 // A row (column) with an infinity or NaN gives NaN in its whole row (column) of C.
 //
 // Layout of the slices.  The slicing kernels write them in the exact order in which the
@@ -54,14 +58,17 @@ namespace ztc {
 
 using namespace tc;
 
-constexpr int NS = 8;                        // slices per operand
 constexpr int RB = 32;                       // rows per block of the slices
 constexpr int BM = 64, BN = 32, BK = 16;     // tile rows, columns, k per stage (complex)
 constexpr int kSlice = 2 * RB * BK;          // fp16 of one slice of a block: re rows, im rows (2 KB)
-constexpr int kBlk = NS * kSlice;            // fp16 of one (row block, k block): 16 KB
-constexpr int kABytes = 2 * kBlk * 2;        // two row blocks, 32 KB
-constexpr int kBBytes = kBlk * 2;            // 16 KB
-constexpr int kStage = kABytes + kBBytes;    // 48 KB
+// of one (row block, k block) for NS slices: 16 KB at eight
+template <int NS>
+struct Blk {
+  static constexpr int kElems = NS * kSlice;
+  static constexpr int kBytesA = 2 * kElems * 2;      // two row blocks
+  static constexpr int kBytesB = kElems * 2;
+  static constexpr int kStage = kBytesA + kBytesB;    // 48 KB at eight slices
+};
 constexpr int NST = 3;                       // stages
 constexpr int kChunk = 24;                   // k blocks per exact chunk (384 k)
 constexpr int kShortK = 96;                  // K up to which every group stays below 2^22 (96 * 40960)
@@ -136,8 +143,50 @@ __device__ __forceinline__ double fixed_to_double(long long hi, long long lo, bo
   return __longlong_as_double((long long)v);
 }
 
-template <bool kShort>
+// T rounded to `keep` leading bits, half to even (its low bits zero).
+__device__ __forceinline__ unsigned long long round_even(unsigned long long T, int drop) {
+  if (drop <= 0) return T;
+  const unsigned long long r = T >> drop, rem = T & ((1ULL << drop) - 1), half = 1ULL << (drop - 1);
+  return (r + (rem > half || (rem == half && (r & 1)))) << drop;
+}
+
+__device__ __noinline__ double seven_slow(long long T1, int v0, int e) {
+  // the magnitudes at which a sum of 64-bit integers could wrap, or an exponent range end
+  return ldexp(fma((double)v0, 4398046511104.0, (double)T1), e - 42);
+}
+
+// The seven-slice form: groups g = 0..6 of weight 2^{-7 g} summed in FP64 from the smallest to the
+// largest, acc = fma(v_g, 2^{-7 g}, acc).  The sum is exact up to group 2, so that it is
+// T1 = sum_{g>=1} v_g 2^{7 (6 - g)} rounded to 53 bits, plus v0 2^42, rounded to 53 bits; times
+// 2^(e - 42).
+__device__ __forceinline__ double seven_to_double(long long T1, int v0, bool flip, int e) {
+  unsigned long long m = (unsigned long long)(T1 < 0 ? -T1 : T1);
+  if (m >> 53) {
+    m = round_even(m, 64 - __clzll((long long)m) - 53);
+    T1 = T1 < 0 ? -(long long)m : (long long)m;
+  }
+  unsigned long long v;
+  const bool wide = v0 >= (1 << 20) || v0 <= -(1 << 20);
+  const long long X = T1 + (long long)((unsigned long long)(long long)v0 << 42);
+  m = (unsigned long long)(X < 0 ? -X : X);
+  if (m == 0 && !wide) return 0.0;
+  const int z = __clzll((long long)m);
+  const unsigned long long T = m << z;
+  unsigned long long r = T >> 11;
+  const unsigned rem = (unsigned)T & 0x7FFu;
+  r += (rem + 0x3FFu + ((unsigned)r & 1u)) >> 11;
+  const int be = 1022 + 63 - z + e - 42;
+  v = r + ((unsigned long long)(unsigned)be << 52);
+  if (X < 0) v |= 1ULL << 63;
+  if (wide || (unsigned)be >= 2045u) v = (unsigned long long)__double_as_longlong(seven_slow(T1, v0, e));
+  if (flip) v ^= 1ULL << 63;
+  return __longlong_as_double((long long)v);
+}
+
+// NS = 8: the exact sum of the groups, rounded once.  NS = 7: see seven_to_double.
+template <int NS, bool kShort>
 __global__ void __launch_bounds__(NT, 1) zgemm_tc_kernel(Args args) {
+  constexpr int kBlk = Blk<NS>::kElems, kABytes = Blk<NS>::kBytesA, kStage = Blk<NS>::kStage;
   extern __shared__ __align__(1024) uint8_t smem[];
   uint8_t* outS = smem + NST * kStage;
   uint64_t* bars = reinterpret_cast<uint64_t*>(outS + kOutBytes);
@@ -206,7 +255,7 @@ __global__ void __launch_bounds__(NT, 1) zgemm_tc_kernel(Args args) {
           }
           uint8_t* st = smem + s * kStage;
           mbar_expect_tx(&full[s], kStage);
-          bulk_load(st + kABytes, bb + (int64_t)kb * kBlk, kBBytes, &full[s]);
+          bulk_load(st + kABytes, bb + (int64_t)kb * kBlk, Blk<NS>::kBytesB, &full[s]);
           // per slice the two row blocks of A side by side
 #pragma unroll
           for (int i = 0; i < NS; ++i) {
@@ -302,9 +351,16 @@ __global__ void __launch_bounds__(NT, 1) zgemm_tc_kernel(Args args) {
               const float f = __uint_as_float(v[g][j]);
               w[g] = kShort ? __float_as_int(f + 12582912.f) - 0x4B400000 : __float2int_rn(f);
             }
+            if constexpr (NS == 7) {
+              // groups 1-6 below 2^22 (64 * 36864): weights 2^35 .. 1; group 0 apart
+              const int a0 = w[1] * 128 + w[2], a1 = w[3] * 128 + w[4], a2 = w[5] * 128 + w[6];
+              hi[cb * 4 + j] += (long long)a0 * (1 << 28) + (long long)a1 * (1 << 14) + a2;
+              lo[cb * 4 + j] += w[0];
+              continue;
+            }
             // |w_g| < 2^24, and below 2^24 - 2^20 for g < 7: 128 w_g + w_(g+1) fits 32 bits
             const int a0 = w[0] * 128 + w[1], a1 = w[2] * 128 + w[3];
-            const int a2 = w[4] * 128 + w[5], a3 = w[6] * 128 + w[7];
+            const int a2 = w[4] * 128 + w[5], a3 = w[6] * 128 + w[NS - 1];
             hi[cb * 4 + j] += (long long)a0 * 16384 + a1;
             lo[cb * 4 + j] += (long long)a2 * 16384 + a3;
           }
@@ -329,7 +385,8 @@ __global__ void __launch_bounds__(NT, 1) zgemm_tc_kernel(Args args) {
         const int n = n0 + col0 + j;
         const int eb1 = n < args.n ? __ldg(eb + n) : 0;
         // own +- the partner's, negated as a whole if the own sign is
-        x[j] = fixed_to_double(hi[j] + (((long long)o.x ^ pm) - pm), lo[j] + (((long long)o.y ^ pm) - pm), neg, -(ea + eb1));
+        const long long h = hi[j] + (((long long)o.x ^ pm) - pm), l = lo[j] + (((long long)o.y ^ pm) - pm);
+        x[j] = NS == 7 ? seven_to_double(h, (int)l, neg, -(ea + eb1)) : fixed_to_double(h, l, neg, -(ea + eb1));
         if (ea == kBadExp || eb1 == kBadExp) x[j] = __longlong_as_double(0x7FF8000000000000LL);
         if (args.scale) x[j] *= args.alpha;
       }
@@ -389,6 +446,7 @@ __device__ __forceinline__ long long digits_of(double x, int ex) {
 // Slices of eight consecutive k of one row, part re or im of the chunk at dst (16 bytes per slice).
 // Digits as fp16 pairs: 1024 + u has the bits 0x6400 | u (u < 1024), minus 1024 + 64.
 __device__ __forceinline__ void store_planes(const long long (&F)[8], int part, __half* dst) {
+  constexpr int NS = 8;
 #pragma unroll
   for (int s = 0; s < NS; ++s) {
     uint32_t w[4];
@@ -409,14 +467,67 @@ __device__ __forceinline__ void store_planes(const long long (&F)[8], int part, 
   }
 }
 
+// The seven-slice form takes the digits one after the other, each the nearest integer (half to
+// even) of what is left: |s_i| <= 64.  x 2^ex as a 62-bit integer (v 2^55), a last bit that
+// stands for anything below it.
+__device__ __forceinline__ long long digits7_of(double x, int ex) {
+  const unsigned long long u = (unsigned long long)__double_as_longlong(x);
+  const int f = (int)((u >> 52) & 0x7FF);
+  unsigned long long m = u & 0xFFFFFFFFFFFFFULL;
+  if (f) m |= 1ULL << 52;
+  const int s = (f ? f : 1) - 1020 + ex;  // <= 9 for normal rows
+  unsigned long long F;
+  if (s >= 0)
+    F = m << s;
+  else if (s > -63)
+    F = (m >> -s) | ((m & ((1ULL << -s) - 1)) != 0);
+  else
+    F = m != 0;
+  return (long long)u < 0 ? -(long long)F : (long long)F;
+}
+
+__device__ __forceinline__ void store_planes7(long long (&F)[8], int part, __half* dst) {
+#pragma unroll
+  for (int s = 0; s < 7; ++s) {
+    const int pos = 55 - 7 * s;
+    const long long half = 1LL << (pos - 1);
+    uint32_t w[4];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const long long t = F[i] + half;
+      long long q = t >> pos;
+      if ((t & ((1LL << pos) - 1)) == 0) q &= ~1LL;  // a tie: to even
+      F[i] -= q << pos;
+      const uint32_t h = 0x6400u | ((uint32_t)((int)q + 128) & 1023u);
+      if (i & 1)
+        w[i >> 1] |= h << 16;
+      else
+        w[i >> 1] = h;
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const __half2 h = __hsub2(*reinterpret_cast<const __half2*>(&w[i]), __floats2half2_rn(1152.f, 1152.f));
+      w[i] = *reinterpret_cast<const uint32_t*>(&h);
+    }
+    *reinterpret_cast<uint4*>(dst + s * kSlice + part * (RB * BK)) = make_uint4(w[0], w[1], w[2], w[3]);
+  }
+}
+
+template <int NS>
 __device__ __forceinline__ void emit_chunk(const double2 (&x)[8], int ex, __half* dst) {
   long long F[8];
 #pragma unroll
-  for (int i = 0; i < 8; ++i) F[i] = digits_of(x[i].x, ex);
-  store_planes(F, 0, dst);
+  for (int p = 0; p < 2; ++p) {
 #pragma unroll
-  for (int i = 0; i < 8; ++i) F[i] = digits_of(x[i].y, ex);
-  store_planes(F, 1, dst);
+    for (int i = 0; i < 8; ++i) {
+      const double v = p ? x[i].y : x[i].x;
+      F[i] = NS == 7 ? digits7_of(v, ex) : digits_of(v, ex);
+    }
+    if constexpr (NS == 7)
+      store_planes7(F, p, dst);
+    else
+      store_planes(F, p, dst);
+  }
 }
 
 __device__ __forceinline__ unsigned long long amax_bits(double2 v) {
@@ -427,18 +538,20 @@ __device__ __forceinline__ unsigned long long amax_bits(double2 v) {
 }
 
 // Where chunk kc (eight k) of row r goes.
+template <int NS>
 __device__ __forceinline__ int64_t slot_of(int r, int kc, int nkb) {
-  return ((int64_t)(r / RB) * nkb + (kc >> 1)) * kBlk + ((r % RB) >> 3) * (2 * 64) + (kc & 1) * 64 + (r & 7) * 8;
+  return ((int64_t)(r / RB) * nkb + (kc >> 1)) * Blk<NS>::kElems + ((r % RB) >> 3) * (2 * 64) + (kc & 1) * 64 + (r & 7) * 8;
 }
 
 // Rows stored contiguously along k: a block takes eight rows, one warp per row for the
 // largest entry, then eight lanes per 128-byte line of the slices.
+template <int NS>
 __global__ void __launch_bounds__(256) zslice_rows_kernel(const double2* __restrict__ X, int64_t ld, int64_t sX, int rows,
                                                           int K, int nkb, int nblk, const int* __restrict__ qmap,
                                                           __half* __restrict__ S, int* __restrict__ ex) {
   const int b = blockIdx.y, r0 = blockIdx.x * 8, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   X += (int64_t)(qmap ? qmap[b] : b) * sX;
-  S += (int64_t)b * nblk * nkb * kBlk;
+  S += (int64_t)b * nblk * nkb * Blk<NS>::kElems;
   __shared__ int se[8];
   {
     const int r = r0 + warp;
@@ -461,12 +574,13 @@ __global__ void __launch_bounds__(256) zslice_rows_kernel(const double2* __restr
     double2 x[8];
 #pragma unroll
     for (int i = 0; i < 8; ++i) x[i] = (kc * 8 + i < K && e != kBadExp) ? row[kc * 8 + i] : make_double2(0.0, 0.0);
-    emit_chunk(x, e, S + slot_of(r, kc, nkb));
+    emit_chunk<NS>(x, e, S + slot_of<NS>(r, kc, nkb));
   }
 }
 
 // Rows stored with stride ld along k (columns of the array), optionally gathered
 // (k -> idx[k], none where negative): a block takes 32 rows, lanes along them.
+template <int NS>
 __global__ void __launch_bounds__(256) zslice_cols_kernel(const double2* __restrict__ X, int64_t ld, int64_t sX, int rows,
                                                           int K, int nkb, int nblk, const int32_t* __restrict__ idx,
                                                           int64_t sIdx, const int* __restrict__ qmap,
@@ -474,7 +588,7 @@ __global__ void __launch_bounds__(256) zslice_cols_kernel(const double2* __restr
   const int b = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31, r = blockIdx.x * 32 + lane;
   const int qb = qmap ? qmap[b] : b;
   X += (int64_t)qb * sX + r;
-  S += (int64_t)b * nblk * nkb * kBlk;
+  S += (int64_t)b * nblk * nkb * Blk<NS>::kElems;
   if (idx) idx += (int64_t)qb * sIdx;
   const bool in = r < rows;
   auto at = [&](int k) {
@@ -496,34 +610,39 @@ __global__ void __launch_bounds__(256) zslice_cols_kernel(const double2* __restr
     double2 x[8];
 #pragma unroll
     for (int i = 0; i < 8; ++i) x[i] = (kc * 8 + i < K && e != kBadExp) ? at(kc * 8 + i) : make_double2(0.0, 0.0);
-    emit_chunk(x, e, S + slot_of(r, kc, nkb));
+    emit_chunk<NS>(x, e, S + slot_of<NS>(r, kc, nkb));
   }
 }
 
 inline int64_t cdiv(int64_t a, int64_t b) { return (a + b - 1) / b; }
-inline size_t slice_bytes(int rows, int k, int nb) { return (size_t)nb * cdiv(rows, RB) * cdiv(k, BK) * kBBytes; }
+inline size_t slice_bytes(int slices, int rows, int k, int nb) {
+  return (size_t)nb * cdiv(rows, RB) * cdiv(k, BK) * slices * kSlice * 2;
+}
 
 // Slices of op(X) by rows (side A) or of op(X)^T (side B): `cols` when the wanted rows run
 // along the fast index of the array.
+template <int NS>
 cudaError_t slice(cudaStream_t st, bool cols, const double2* X, int64_t ld, int64_t sX, int rows, int K, int batch,
                   const int32_t* idx, int64_t sIdx, const int* qmap, __half* S, int* ex) {
   const int nkb = (int)cdiv(K, BK), nblk = (int)cdiv(rows, RB);
   if (cols)
-    zslice_cols_kernel<<<dim3((unsigned)cdiv(rows, 32), batch), 256, 0, st>>>(X, ld, sX, rows, K, nkb, nblk, idx, sIdx,
+    zslice_cols_kernel<NS><<<dim3((unsigned)cdiv(rows, 32), batch), 256, 0, st>>>(X, ld, sX, rows, K, nkb, nblk, idx, sIdx,
                                                                              qmap, S, ex);
   else
-    zslice_rows_kernel<<<dim3((unsigned)cdiv(rows, 8), batch), 256, 0, st>>>(X, ld, sX, rows, K, nkb, nblk, qmap, S, ex);
+    zslice_rows_kernel<NS><<<dim3((unsigned)cdiv(rows, 8), batch), 256, 0, st>>>(X, ld, sX, rows, K, nkb, nblk, qmap, S, ex);
   count_launch();
   return cudaGetLastError();
 }
 
 }  // namespace ztc
 
-size_t zgemm_tc_work_bytes(int m, int n, int k, int nb, bool same) {
-  return ztc::slice_bytes(m, k, nb) + (same ? 0 : ztc::slice_bytes(n, k, nb)) + sizeof(int) * (size_t)nb * (m + n) + 256;
+size_t zgemm_tc_work_bytes(int slices, int m, int n, int k, int nb, bool same) {
+  return ztc::slice_bytes(slices, m, k, nb) + (same ? 0 : ztc::slice_bytes(slices, n, k, nb)) +
+         sizeof(int) * (size_t)nb * (m + n) + 256;
 }
 
-cudaError_t zgemm_tc(cudaStream_t st, char opA, char opB, int m, int n, int k, double alpha, const double2* A,
+template <int NS>
+static cudaError_t zgemm_tc_impl(cudaStream_t st, char opA, char opB, int m, int n, int k, double alpha, const double2* A,
                      int64_t lda, int64_t sA, const double2* B, int64_t ldb, int64_t sB, double2* C, int64_t ldc,
                      int64_t sC, int batch, const ZOpt& o, void* work, size_t work_bytes, int* err) {
   using namespace ztc;
@@ -532,30 +651,30 @@ cudaError_t zgemm_tc(cudaStream_t st, char opA, char opB, int m, int n, int k, d
   const bool aT = opA == 'T' || opA == 'C', aC = opA == 'C' || opA == 'R';
   const bool bT = opB == 'T' || opB == 'C', bC = opB == 'C' || opB == 'R';
   const bool same = !o.brow && zgemm_tc_same(opA, opB, m, n, A, lda, sA, B, ldb, sB);
-  const size_t per = slice_bytes(m, k, 1) + (same ? 0 : slice_bytes(n, k, 1)) + sizeof(int) * (size_t)(m + n);
+  const size_t per = slice_bytes(NS, m, k, 1) + (same ? 0 : slice_bytes(NS, n, k, 1)) + sizeof(int) * (size_t)(m + n);
   if (work_bytes < per + 256) return cudaErrorInvalidValue;
   const int nbc = (int)std::min<size_t>((size_t)std::min(batch, 65535), (work_bytes - 256) / per);
   int dev = 0, sms = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return e;
-  constexpr size_t smem = (size_t)NST * kStage + kOutBytes + 128;
-  const bool ks = k <= kShortK;
-  e = cudaFuncSetAttribute(ks ? zgemm_tc_kernel<true> : zgemm_tc_kernel<false>,
+  constexpr size_t smem = (size_t)NST * Blk<NS>::kStage + kOutBytes + 128;
+  const bool ks = NS == 7 || k <= kShortK;
+  e = cudaFuncSetAttribute(ks ? zgemm_tc_kernel<NS, true> : zgemm_tc_kernel<NS, NS == 7>,
                            cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   for (int b0 = 0; b0 < batch; b0 += nbc) {
     const int nb = std::min(nbc, batch - b0);
     __half* SA = reinterpret_cast<__half*>(work);
-    __half* SB = same ? SA : SA + slice_bytes(m, k, nb) / 2;
-    int* eA = reinterpret_cast<int*>(SB + slice_bytes(n, k, nb) / 2);  // n = m where SB is SA
+    __half* SB = same ? SA : SA + slice_bytes(NS, m, k, nb) / 2;
+    int* eA = reinterpret_cast<int*>(SB + slice_bytes(NS, n, k, nb) / 2);  // n = m where SB is SA
     int* eB = same ? eA : eA + (size_t)nb * m;
     // with a map the arrays stay where they are and the map moves on
     const int* qm = o.qmap ? o.qmap + b0 : nullptr;
     const int64_t s0 = qm ? 0 : b0;
-    e = slice(st, aT, A + s0 * sA, lda, sA, m, k, nb, nullptr, 0, qm, SA, eA);
+    e = slice<NS>(st, aT, A + s0 * sA, lda, sA, m, k, nb, nullptr, 0, qm, SA, eA);
     if (e == cudaSuccess && !same)
-      e = slice(st, !bT, B + s0 * sB, ldb, sB, n, k, nb, o.brow ? o.brow + s0 * o.sIdx : nullptr, o.sIdx, qm, SB, eB);
+      e = slice<NS>(st, !bT, B + s0 * sB, ldb, sB, n, k, nb, o.brow ? o.brow + s0 * o.sIdx : nullptr, o.sIdx, qm, SB, eB);
     if (e != cudaSuccess) return e;
     Args a{};
     a.SA = SA;
@@ -585,14 +704,26 @@ cudaError_t zgemm_tc(cudaStream_t st, char opA, char opB, int m, int n, int k, d
     a.err = err;
     const unsigned grid = (unsigned)std::min<int64_t>(a.ntiles, sms);
     if (ks)
-      zgemm_tc_kernel<true><<<grid, NT, smem, st>>>(a);
+      zgemm_tc_kernel<NS, true><<<grid, NT, smem, st>>>(a);
     else
-      zgemm_tc_kernel<false><<<grid, NT, smem, st>>>(a);
+      zgemm_tc_kernel<NS, NS == 7><<<grid, NT, smem, st>>>(a);
     count_launch();
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
+}
+
+cudaError_t zgemm_tc(cudaStream_t st, char opA, char opB, int m, int n, int k, double alpha, const double2* A,
+                     int64_t lda, int64_t sA, const double2* B, int64_t ldb, int64_t sB, double2* C, int64_t ldc,
+                     int64_t sC, int batch, const ZOpt& o, void* work, size_t work_bytes, int* err) {
+  if (o.slices == 7) {
+    if (k > kZgemm7MaxK) return cudaErrorInvalidValue;
+    return zgemm_tc_impl<7>(st, opA, opB, m, n, k, alpha, A, lda, sA, B, ldb, sB, C, ldc, sC, batch, o, work, work_bytes,
+                            err);
+  }
+  return zgemm_tc_impl<8>(st, opA, opB, m, n, k, alpha, A, lda, sA, B, ldb, sB, C, ldc, sC, batch, o, work, work_bytes,
+                          err);
 }
 
 }  // namespace isdf
