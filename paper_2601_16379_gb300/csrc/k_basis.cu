@@ -16,6 +16,7 @@
 //           since the k-mesh is a product of its axes.  A column of D then costs N_AO
 //           terms per grid point instead of a pass over Phi.
 #include <algorithm>
+#include <climits>
 #include <cmath>
 
 #include "common.cuh"
@@ -354,12 +355,15 @@ __global__ void ips_table_kernel(CellDev c, BasisDev b, const double2* __restric
   }
 }
 
+constexpr int kLp = 512;  // entries of the pivot's row staged at once
+
 struct IpsArgs {
   const double* A;  // factor tables: axis 0 at 0, axis 1 at o1, axis 2 at o2
   int64_t o1, o2;
   int nterm, n0, n1, n2, ng;
+  int R;            // points per block
   int tile;         // terms whose (g0, g1) products are held at once
-  double* M;        // block maxima of the residual diagonal, two buffers of gridDim.x
+  long long* M;     // block maxima of the residual diagonal (order_key), two buffers of gridDim.x
   double* d;        // residual diagonal, two buffers of ng; -inf at the chosen points
   double* Lt;       // [n_p][ng]
   int32_t* piv;
@@ -369,88 +373,139 @@ struct IpsArgs {
   double tie_eps, chol_tol;
 };
 
-// D(r, r') for the threads' points r = r0 + threadIdx.x: the products of the axes 0 and 1
-// once per (g0, g1) of the block, then one FMA per term.  r' = p, or r' = r (p < 0).
-__device__ __forceinline__ double ips_column(const IpsArgs& a, int r0, int p, double* sxy) {
-  const int r = r0 + threadIdx.x, last = min(r0 + (int)blockDim.x, a.ng) - 1;
+// A block has R = a.R points and G groups of R threads; the terms of D and the rows of Lt are
+// dealt out to the groups, whose partial sums meet in shared memory: a chain of j loads and
+// FP64 FMAs per point would leave the chip waiting (one warp's worth of points per scheduler).
+
+// The FP64 pipe (2 operations per clock and SM) also does comparisons, so maxima are taken on
+// order-preserving integers, and what one thread can compute, one thread does.
+
+// Sum over the groups of one value per thread, in the first group.
+__device__ __forceinline__ double group_sum(double v, int R, int G, double* red) {
+  __syncthreads();
+  red[threadIdx.x] = v;
+  __syncthreads();
+  double s = v;
+  if ((int)threadIdx.x < R)
+    for (int g = 1; g < G; ++g) s += red[g * R + threadIdx.x];
+  return s;
+}
+
+// Integer with the order of the double; NaN below everything (as fmax ignores it).
+__device__ __forceinline__ long long order_key(double x) {
+  const long long b = __double_as_longlong(x);
+  if ((b & 0x7FFFFFFFFFFFFFFFLL) > 0x7FF0000000000000LL) return LLONG_MIN;
+  return b ^ ((b >> 63) & 0x7FFFFFFFFFFFFFFFLL);
+}
+__device__ __forceinline__ double order_value(long long k) {
+  return __longlong_as_double(k ^ ((k >> 63) & 0x7FFFFFFFFFFFFFFFLL));
+}
+
+// D(r, r') for the points r = r0 + threadIdx.x % R: the products of the axes 0 and 1 once per
+// (g0, g1) of the block, then one FMA per term.  r' = p, or r' = r (p < 0).
+__device__ __forceinline__ double ips_column(const IpsArgs& a, int r0, int p, double* sxy, double* red) {
+  const int R = a.R, G = blockDim.x / R, lr = threadIdx.x % R, grp = threadIdx.x / R;
+  const int r = r0 + lr, last = min(r0 + R, a.ng) - 1;
   const int x0 = r0 / a.n2, nx = last / a.n2 - x0 + 1;  // (g0, g1) pairs of the block
   const bool in = r < a.ng;
   const int g2 = in ? r % a.n2 : 0, xi = in ? r / a.n2 - x0 : 0;
+  const int p0f = p < 0 ? 0 : p / (a.n1 * a.n2), p1f = p < 0 ? 0 : (p / a.n2) % a.n1, p2 = p < 0 ? g2 : p % a.n2;
   double D = 0.0;
   for (int t0 = 0; t0 < a.nterm; t0 += a.tile) {
     const int nt = min(a.tile, a.nterm - t0);
     __syncthreads();
     for (int e = threadIdx.x; e < nt * nx; e += blockDim.x) {
       const int t = t0 + e / nx, x = x0 + e % nx, g0 = x / a.n1, g1 = x % a.n1;
-      const int p0 = p < 0 ? g0 : p / (a.n1 * a.n2), p1 = p < 0 ? g1 : (p / a.n2) % a.n1;
+      const int p0 = p < 0 ? g0 : p0f, p1 = p < 0 ? g1 : p1f;
       sxy[e] = a.A[((int64_t)t * a.n0 + p0) * a.n0 + g0] * a.A[a.o1 + ((int64_t)t * a.n1 + p1) * a.n1 + g1];
     }
     __syncthreads();
-    const double* A2 = a.A + a.o2 + ((int64_t)t0 * a.n2 + (p < 0 ? g2 : p % a.n2)) * a.n2 + g2;
-#pragma unroll 8
-    for (int t = 0; t < nt; ++t) D = fma(sxy[t * nx + xi], A2[(int64_t)t * a.n2 * a.n2], D);
+    const double* A2 = a.A + a.o2 + ((int64_t)t0 * a.n2 + p2) * a.n2 + g2;
+#pragma unroll 4
+    for (int t = grp; t < nt; t += G) D = fma(sxy[t * nx + xi], A2[(int64_t)t * a.n2 * a.n2], D);
   }
-  return D;
+  return group_sum(D, R, G, red);
 }
 
-__device__ __forceinline__ double block_fmax(double m, double* sv) {
-  for (int o = 16; o; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+__device__ __forceinline__ long long block_kmax(long long m, long long* sv) {
+  for (int o = 16; o; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
   __syncthreads();
   if ((threadIdx.x & 31) == 0) sv[threadIdx.x >> 5] = m;
   __syncthreads();
   m = sv[0];
-  for (int i = 1; i < (int)(blockDim.x >> 5); ++i) m = fmax(m, sv[i]);
+  for (int i = 1; i < (int)(blockDim.x >> 5); ++i) m = max(m, sv[i]);
   return m;
 }
 
-__global__ void ips_init_kernel(IpsArgs a) {
+__global__ void __launch_bounds__(1024) ips_init_kernel(IpsArgs a) {
   extern __shared__ double ips_smem[];
-  __shared__ double sv[8];
-  const int r0 = blockIdx.x * blockDim.x, r = r0 + threadIdx.x;
-  const double D = ips_column(a, r0, -1, ips_smem);
-  double v = -INFINITY;
-  if (r < a.ng) a.d[r] = v = D * D;
-  v = block_fmax(v, sv);
+  __shared__ long long sv[32];
+  const int r0 = blockIdx.x * a.R, r = r0 + threadIdx.x;
+  const double D = ips_column(a, r0, -1, ips_smem + blockDim.x, ips_smem);
+  long long v = LLONG_MIN;
+  if ((int)threadIdx.x < a.R && r < a.ng) {
+    a.d[r] = D * D;
+    v = order_key(D * D);
+  }
+  v = block_kmax(v, sv);
   if (threadIdx.x == 0) a.M[blockIdx.x] = v;
 }
 
 // Step j in one launch (the stream order between the steps is the only barrier): every block
 // finds the pivot from the block maxima of step j - 1 -- the tie rule looks only into blocks
 // whose maximum lies in the window -- then updates its own points and leaves its new maximum.
-// Buffers alternate, so that no block reads what another one writes.  About 150 blocks: one
-// point per thread, chains of j FMAs against rows of Lt that stay in L2.
-__global__ void ips_step_kernel(IpsArgs a, int j) {
+// Buffers alternate, so that no block reads what another one writes.  About 150 blocks.
+__global__ void __launch_bounds__(1024) ips_step_kernel(IpsArgs a, int j) {
   extern __shared__ double ips_smem[];
-  __shared__ double sv[8];
-  __shared__ unsigned long long sh[8];
-  __shared__ int si[8];
+  __shared__ long long sv[32], s_thr;
+  __shared__ unsigned long long sh[32];
+  __shared__ int si[32], s_list[32], s_n, s_stop;
+  __shared__ double s_inv;
   if (*a.status != 0) return;
-  const int nb = gridDim.x, bd = blockDim.x, tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-  const double* M = a.M + (j & 1) * nb;
+  const int nb = gridDim.x, bd = blockDim.x, tid = threadIdx.x, lane = tid & 31, w = tid >> 5, R = a.R, G = bd / R;
+  const long long* M = a.M + (j & 1) * nb;
   const double* din = a.d + (int64_t)(j & 1) * a.ng;
   double* dout = a.d + (int64_t)((j & 1) ^ 1) * a.ng;
-  double dmax = -INFINITY;
-  for (int b = tid; b < nb; b += bd) dmax = fmax(dmax, M[b]);
-  dmax = block_fmax(dmax, sv);
-  const double d0 = j == 0 ? dmax : a.scal[0];
-  if (!(dmax >= a.chol_tol * d0) || !(dmax > 0.0)) {
+  if (tid == 0) s_n = 0;
+  const double d0r = a.scal[0];
+  long long kmax = LLONG_MIN;
+  for (int b = tid; b < nb; b += bd) kmax = max(kmax, M[b]);
+  kmax = block_kmax(kmax, sv);
+  const double dmax = order_value(kmax);
+  if (tid == 0) {
+    const double d0 = j == 0 ? dmax : d0r;
+    s_stop = kmax == LLONG_MIN || !(dmax >= a.chol_tol * d0) || !(dmax > 0.0);
+    s_thr = order_key(fmax(dmax - a.tie_eps * d0, 0.5 * dmax));
+  }
+  __syncthreads();
+  if (s_stop) {
     if (blockIdx.x == 0 && tid == 0) {
       *a.status = 1;
       a.piv[j] = -1;
     }
     return;
   }
-  const double thr = fmax(dmax - a.tie_eps * d0, 0.5 * dmax);
+  const long long thr = s_thr;
+  // blocks with candidates (a list of up to 32; beyond it every block is looked at)
+  for (int b = tid; b < nb; b += bd)
+    if (M[b] >= thr) {
+      const int i = atomicAdd(&s_n, 1);
+      if (i < 32) s_list[i] = b;
+    }
+  __syncthreads();
+  const int nl = s_n;
   unsigned long long best = ~0ULL;
   int bi = -1;
-  for (int b = 0; b < nb; ++b) {
-    if (!(M[b] >= thr)) continue;
-    const int r = b * bd + tid;
-    if (r < a.ng && din[r] >= thr) {
-      const unsigned long long hsh = splitmix64(a.seed ^ (uint64_t)r);
-      if (bi < 0 || hsh < best) {  // ascending r: the smaller index wins equal hashes
-        best = hsh;
-        bi = r;
+  for (int i = 0; i < (nl <= 32 ? nl : nb); ++i) {
+    const int b = nl <= 32 ? s_list[i] : i;
+    for (int x = tid; x < R; x += bd) {
+      const int r = b * R + x;
+      if (r < a.ng && order_key(din[r]) >= thr) {
+        const unsigned long long hsh = splitmix64(a.seed ^ (uint64_t)r);
+        if (bi < 0 || hsh < best || (hsh == best && r < bi)) {
+          best = hsh;
+          bi = r;
+        }
       }
     }
   }
@@ -485,36 +540,39 @@ __global__ void ips_step_kernel(IpsArgs a, int j) {
     a.piv[j] = p;
     if (j == 0) a.scal[0] = dmax;
   }
-  const int r0 = blockIdx.x * bd, r = r0 + tid;
-  const double D = ips_column(a, r0, p, ips_smem);
-  __syncthreads();
-  double* lp = ips_smem;  // L[i][p], in pieces of 256
-  const double* Lr = a.Lt + (r < a.ng ? r : 0);
-  double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
-  for (int i0 = 0; i0 < j; i0 += 256) {
-    const int n = min(256, j - i0);
+  double* red = ips_smem;                // [bd]
+  double* sxy = ips_smem + bd;           // term products, then L[i][p] in pieces of kLp
+  const int r0 = blockIdx.x * R, lr = tid % R, grp = tid / R, r = r0 + lr;
+  const bool in = r < a.ng;
+  const double dr = in ? din[r] : 0.0;
+  if (tid == bd - 1) s_inv = 1.0 / sqrt(din[p]);
+  const double D = ips_column(a, r0, p, sxy, red);
+  const double* Lr = a.Lt + (in ? r : 0);
+  double s0 = 0.0, s1 = 0.0;
+  for (int i0 = 0; i0 < j; i0 += kLp) {
+    const int n = min(kLp, j - i0);
     __syncthreads();
-    for (int i = tid; i < n; i += bd) lp[i] = a.Lt[(int64_t)(i0 + i) * a.ng + p];
+    for (int i = tid; i < n; i += bd) sxy[i] = a.Lt[(int64_t)(i0 + i) * a.ng + p];
     __syncthreads();
     const double* L = Lr + (int64_t)i0 * a.ng;
-    int i = 0;
-#pragma unroll 2
-    for (; i + 4 <= n; i += 4) {
-      s0 = fma(L[(int64_t)i * a.ng], lp[i], s0);
-      s1 = fma(L[(int64_t)(i + 1) * a.ng], lp[i + 1], s1);
-      s2 = fma(L[(int64_t)(i + 2) * a.ng], lp[i + 2], s2);
-      s3 = fma(L[(int64_t)(i + 3) * a.ng], lp[i + 3], s3);
+    int i = grp;
+#pragma unroll 4
+    for (; i + G < n; i += 2 * G) {
+      s0 = fma(L[(int64_t)i * a.ng], sxy[i], s0);
+      s1 = fma(L[(int64_t)(i + G) * a.ng], sxy[i + G], s1);
     }
-    for (; i < n; ++i) s0 = fma(L[(int64_t)i * a.ng], lp[i], s0);
+    if (i < n) s0 = fma(L[(int64_t)i * a.ng], sxy[i], s0);
   }
-  double v = -INFINITY;
-  if (r < a.ng) {
-    const double l = (D * D - ((s0 + s1) + (s2 + s3))) * (1.0 / sqrt(din[p]));
+  const double sum = group_sum(s0 + s1, R, G, red);
+  long long v = LLONG_MIN;
+  if (grp == 0 && in) {
+    const double l = (D * D - sum) * s_inv;  // set before the barriers of the sums
     a.Lt[(int64_t)j * a.ng + r] = l;
-    v = r == p ? -INFINITY : din[r] - l * l;
-    dout[r] = v;
+    const double dn = r == p ? -INFINITY : dr - l * l;
+    dout[r] = dn;
+    v = order_key(dn);
   }
-  v = block_fmax(v, sv);
+  v = block_kmax(v, sv);
   if (tid == 0) a.M[((j & 1) ^ 1) * nb + blockIdx.x] = v;
 }
 
@@ -587,16 +645,18 @@ cudaError_t ip_step(cudaStream_t st, const double2* phi, int nkao, int ng, int j
 
 namespace {
 struct IpsLayout {
-  int threads, blocks, tile;
+  int R, G, blocks, tile;  // points per block, thread groups
   size_t table, total;  // doubles
 };
 IpsLayout ips_layout(const CellDev& c, int nterm) {
   const int ng = c.mesh[0] * c.mesh[1] * c.mesh[2];
   IpsLayout l;
-  // one wave: points spread over the SMs, a warp to eight warps each
-  l.threads = std::min(256, std::max(32, ((ng + 151) / 152 + 31) / 32 * 32));
-  l.blocks = (ng + l.threads - 1) / l.threads;
-  const int nx = l.threads / c.mesh[2] + 2;
+  // one wave: the points spread over the SMs, a warp to eight warps of them each, and up to
+  // eight groups of threads on the same points (c5: 9.3 ms, 13.7 with one group)
+  l.R = std::min(256, std::max(32, ((ng + 151) / 152 + 31) / 32 * 32));
+  l.G = std::max(1, std::min(8, 1024 / l.R));
+  l.blocks = (ng + l.R - 1) / l.R;
+  const int nx = l.R / c.mesh[2] + 2;
   l.tile = std::max(1, std::min(nterm, 4096 / nx));
   l.table = (size_t)nterm * (c.mesh[0] * c.mesh[0] + c.mesh[1] * c.mesh[1] + c.mesh[2] * c.mesh[2]);
   l.total = l.table + 2 * (size_t)l.blocks + 2 * (size_t)ng;
@@ -611,7 +671,7 @@ bool ips_supported(const CellDev& c, int nterm) {
 size_t ips_work_bytes(const CellDev& c, int nterm) { return ips_layout(c, nterm).total * sizeof(double); }
 
 // The separable selection.  Measured on GB300 (Phi and points together, 300 points, 24^3 grid,
-// Nk = 1000, N_AO = 26): 13.7 ms, against 478 ms with one pass over Phi per pivot.
+// Nk = 1000, N_AO = 26): 9.3 ms, against 478 ms with one pass over Phi per pivot.
 cudaError_t ips_select(cudaStream_t st, const CellDev& c, const BasisDev& b, const double* ao_work, const int* terms,
                        int nterm, int n_p, double* work, double* Lt, int32_t* piv, uint64_t seed, double tie_eps,
                        double chol_tol, double* scal, int32_t* status) {
@@ -625,9 +685,10 @@ cudaError_t ips_select(cudaStream_t st, const CellDev& c, const BasisDev& b, con
   a.n1 = c.mesh[1];
   a.n2 = c.mesh[2];
   a.ng = a.n0 * a.n1 * a.n2;
+  a.R = l.R;
   a.tile = l.tile;
-  a.M = work + l.table;
-  a.d = a.M + 2 * (size_t)l.blocks;
+  a.M = reinterpret_cast<long long*>(work + l.table);
+  a.d = work + l.table + 2 * (size_t)l.blocks;
   a.Lt = Lt;
   a.piv = piv;
   a.scal = scal;
@@ -638,11 +699,12 @@ cudaError_t ips_select(cudaStream_t st, const CellDev& c, const BasisDev& b, con
   ips_table_kernel<<<nblocks((int64_t)l.table), 256, 0, st>>>(c, b, reinterpret_cast<const double2*>(ao_work), terms,
                                                               nterm, a.o1, a.o2, work);
   count_launch();
-  const size_t smem = sizeof(double) * std::max<size_t>(256, (size_t)l.tile * (l.threads / a.n2 + 2));
-  ips_init_kernel<<<l.blocks, l.threads, smem, st>>>(a);
+  const int threads = l.R * l.G;
+  const size_t smem = sizeof(double) * (threads + std::max<size_t>(kLp, (size_t)l.tile * (l.R / a.n2 + 2)));
+  ips_init_kernel<<<l.blocks, threads, smem, st>>>(a);
   count_launch();
   for (int j = 0; j < n_p; ++j) {
-    ips_step_kernel<<<l.blocks, l.threads, smem, st>>>(a, j);
+    ips_step_kernel<<<l.blocks, threads, smem, st>>>(a, j);
     count_launch();
   }
   return cudaGetLastError();
