@@ -158,8 +158,16 @@ void grid_twiddles(const int mesh[3], double2* host192);
 
 // Real k-mesh DFT out of place, keeping the q with qslot[q] >= 0 (complex64 output):
 //   out[qslot[q]][col] = scale sum_k e^{s 2 pi i m_q.m_k/n} in[k][col].
+// With `keep` the columns col = a np + I are the rows a of M and only the entries inv[j][I] = c >= 0 of
+// the position j = qslot[q] are written, at out[(j rows + a) pitch + c] (rows = ncol / np); rowmax[a]
+// (bits, zeroed by the caller) receives the largest |component| among them.
+struct KeepCols {
+  const int16_t* inv = nullptr;
+  int np = 0, pitch = 0;
+  unsigned* rowmax = nullptr;
+};
 cudaError_t kdft_real_f(cudaStream_t st, const float* in, float2* out, int64_t ncol, KMesh km, int s, float scale,
-                        const int* qslot);
+                        const int* qslot, const KeepCols& keep = KeepCols());
 // Real pair rows of the time-reversal basis: for pairs o = (p < q) in lexicographic
 // order Zr[R][2o][I] = 2 Re(conj(t_p) t_q), Zr[R][2o+1][I] = 2 Im(conj(t_p) t_q), and
 // Zr[R][2P + p][I] = |t_p|^2 (P = n_f (n_f - 1)/2), t = t[R][I][p] complex64.
@@ -259,26 +267,23 @@ int vxi_tc_chunk(int rx, int ng, size_t budget);
 size_t vxi_tc_work_bytes(int rx, int ng, int qc);
 cudaError_t vxi_tc(cudaStream_t st, const ffcomplex* c, int64_t qs, int rx, int ng, int nq, double omega,
                    double2* V, int64_t ldv, int64_t vs, void* work, int qc, int* err);
-// B^q = M^q L^q (w_q^{1/2} folded into L) on the tensor cores with three slices
-// per operand (an integer and two fp16 remainders), over the structural nonzeros
-// of L^q only: the rp = max_q r_q
-// pivot columns perm_q[c] (c < rank_q) of M^q and the nj output columns.  M^q is
-// stored by position j in the sum (q = qmap[j]) with q stride sq; B^q is written
-// in place over it with row pitch nj.  prepare: slices of L for all q (once per
-// L); rowscale: exponents of the gathered M rows over the sum; chunk: the
-// positions j0..j0+nq-1 of the sum.
+// Exponents e with max 2^e in [64, 128) from the bits of the rows' largest entries.
+cudaError_t row_exponents(cudaStream_t st, const unsigned* mx, int64_t rows, int* row_exp);
+// B^q = M^q L^q (w_q^{1/2} folded into L) on the tensor cores with three slices per operand (an
+// integer and two fp16 remainders), over the structural nonzeros of L^q only: M holds the
+// gathered pivot columns perm_q[c], c < r_q <= rp, of the nS positions of the sum (q = qmap[j]) with row
+// pitch pm (even), B the nj output columns with row pitch nj; both are [position][row].
+// prepare: slices of L by position (once per L) and the column map of KeepCols; bmax[a]
+// (zeroed by the caller) receives the bits of the largest |component| of row a of B.
 int mlgemm_tc_kp(int rp);
 int mlgemm_tc_nj_pad(int nj);
 bool mlgemm_tc_supported(int rp);
-size_t mlgemm_tc_lslice_bytes(int nk, int rp, int nj);
-size_t mlgemm_tc_split_bytes(int64_t n2, int rp, int nq);
-cudaError_t mlgemm_tc_prepare(cudaStream_t st, const double2* L, const double* sw, int nk, int np, const int* perm,
-                              const int* rank, int rp, int nj, void* lsl, int* col_exp);
-cudaError_t mlgemm_tc_rowscale(cudaStream_t st, const float2* M, int64_t sq, int np, const int* qmap, int nS,
-                               const int* perm, const int* rank, int rp, int64_t n2, int* row_exp);
-cudaError_t mlgemm_tc_chunk(cudaStream_t st, float2* M, int64_t sq, const int* qmap, int64_t n2, int np,
-                            const int* perm, const int* rank, int rp, int nj, int j0, int nq, const int* row_exp,
-                            void* split, const void* lsl, const int* col_exp, int nk, int* err);
+size_t mlgemm_tc_lslice_bytes(int nS, int rp, int nj);
+cudaError_t mlgemm_tc_prepare(cudaStream_t st, const double2* L, const double* sw, int np, const int* qmap, int nS,
+                              const int* perm, const int* rank, int rp, int nj, void* lsl, float* col_scale, int16_t* inv);
+cudaError_t mlgemm_tc(cudaStream_t st, const float2* M, int pm, float2* B, const int* qmap, int nS, int64_t rows,
+                      const int* rank, int rp, int nj, const int* row_exp, const void* lsl, const float* col_scale,
+                      unsigned* bmax, int* err);
 // eri[p][q][r][s] (complex64) = E[(p q)][(s r)] (complex128) * scale
 cudaError_t eri_permute_zc(cudaStream_t st, const double2* E, int nf, double scale, float2* eri);
 

@@ -1086,19 +1086,23 @@ int isdf_fragment_eri(isdf_handle* h, int n_frag, const int32_t* n_orb, const vo
     // B = M L on the tensor cores (three remainder slices; five exact ones in FP64_TC) when the
     // 2 r_q gathered columns fit their exact accumulation, else on the
     // compensated SIMT GEMM
-    const bool tc_ml = tc64 || mlgemm_tc_supported(rp);
+    const bool tc_ml = tc64 || (mlgemm_tc_supported(rp) && np <= 32767);
     float2* Lwf = nullptr;
     void* lsl = nullptr;
-    int* lexp = nullptr;
+    int* lexp = nullptr;  // column exponents of L (FP64_TC) or inverse scales (mixed)
+    int16_t* inv = nullptr;  // kept columns of M (mixed): position in the pivot order
     if (tc_ml) {
-      lsl = h->ensure_evict("frag_Lsl", tc64 ? mlgemm5_tc_lslice_bytes(nk, rp, nj) : mlgemm_tc_lslice_bytes(nk, rp, nj));
+      lsl = h->ensure_evict("frag_Lsl", tc64 ? mlgemm5_tc_lslice_bytes(nk, rp, nj) : mlgemm_tc_lslice_bytes(nS, rp, nj));
       lexp = (int*)h->ensure_evict("frag_Lexp",
                                    sizeof(int) * (size_t)nk * (tc64 ? mlgemm5_tc_nj_pad(nj) : mlgemm_tc_nj_pad(nj)));
       if (!lsl || !lexp) return fail(h, ISDF_ERR_OOM, "device allocation of the slices of L failed");
-      if (tc64)
+      if (tc64) {
         CK(mlgemm5_tc_prepare(h->st, Lq, swd, nk, np, permPi, rankPi, rp, nj, lsl, lexp));
-      else
-        CK(mlgemm_tc_prepare(h->st, Lq, swd, nk, np, permPi, rankPi, rp, nj, lsl, lexp));
+      } else {
+        inv = (int16_t*)h->ensure_evict("frag_inv", sizeof(int16_t) * (size_t)nS * np);
+        if (!inv) return fail(h, ISDF_ERR_OOM, "device allocation of the column map failed");
+        CK(mlgemm_tc_prepare(h->st, Lq, swd, np, qmap, nS, permPi, rankPi, rp, nj, lsl, reinterpret_cast<float*>(lexp), inv));
+      }
     } else {
       Lwf = (float2*)h->ensure_evict("frag_Lwf", sizeof(float2) * (size_t)nk * pp);
       if (!Lwf) return fail(h, ISDF_ERR_OOM, "device allocation of frag_Lwf failed");
@@ -1122,7 +1126,11 @@ int isdf_fragment_eri(isdf_handle* h, int n_frag, const int32_t* n_orb, const vo
         row0[i] = rows;
         rows += (i + 1 < grp.size()) ? (n2f + 127) / 128 * 128 : n2f;
       }
-      const int64_t sq = rows * np;  // q stride of M
+      // mixed: M holds the gathered columns only (pitch pm) and B has its own array; else B
+      // overwrites M
+      const int pm = inv ? (rp + 3) / 4 * 4 : np;
+      const int64_t sqZ = rows * np, sq = rows * pm;  // position strides of Z and M
+      const int64_t sqB = inv ? rows * nj : sq;
       int nfmax = 0;
       double flops3 = 0.0, flops4 = 0.0, flops5 = 0.0;
       for (int f : grp) {
@@ -1138,12 +1146,13 @@ int isdf_fragment_eri(isdf_handle* h, int n_frag, const int32_t* n_orb, const vo
       ENSURE(T, float2, "frag_T", (size_t)nk * np * nfmax * (tc64 ? 2 : 1));
       // real pair rows Z(R) of the time-reversal basis, and M^q (then B^q) of the
       // q of the sum, stored by their position in it
-      ENSURE(Zr, uint8_t, "frag_Zr", zsz * (size_t)nk * sq);
-      ENSURE(M, uint8_t, "frag_Mf", msz * (size_t)nS * sq);
+      ENSURE(Zr, uint8_t, "frag_Zr", zsz * (size_t)nk * sqZ);
+      ENSURE(M, uint8_t, "frag_Mf", msz * (size_t)nS * (inv ? sq + sqB : sq));
       float* Zr_f = reinterpret_cast<float*>(Zr);
       ffloat* Zr_ff = reinterpret_cast<ffloat*>(Zr);
       float2* M_f = reinterpret_cast<float2*>(M);
       ffcomplex* M_ff = reinterpret_cast<ffcomplex*>(M);
+      float2* B_f = inv ? M_f + (int64_t)nS * sq : M_f;
       ENSURE(trpart, double2, "frag_traces_part", std::max<size_t>(2 * (size_t)n2max, syrk_tc_eri_part_count()));
       // tiles of every fragment's diagonal block, in the autotuned band order
       std::vector<int2>& tl = h->tiles_host;
@@ -1180,10 +1189,7 @@ int isdf_fragment_eri(isdf_handle* h, int n_frag, const int32_t* n_orb, const vo
       auto syrk_split_bytes = [&](int64_t kc) {
         return tc64 ? syrk4_tc_split_bytes(rows, kc) : syrk_tc_split_bytes(rows, kc);
       };
-      auto ml_split_bytes = [&](int nq) -> size_t {
-        if (!tc_ml) return 0;
-        return tc64 ? mlgemm5_tc_split_bytes(rows, rp, nq) : mlgemm_tc_split_bytes(rows, rp, nq);
-      };
+      auto ml_split_bytes = [&](int nq) -> size_t { return tc64 ? mlgemm5_tc_split_bytes(rows, rp, nq) : 0; };
       const size_t per_q = std::max(syrk_split_bytes(nj), ml_split_bytes(1));
       const int qc = (int)std::max<int64_t>(1, std::min<int64_t>(nS, (int64_t)(h->split_budget / per_q)));
       ENSURE(split, uint8_t, "tc_split", std::max(syrk_split_bytes((int64_t)qc * nj), ml_split_bytes(qc)));
@@ -1193,6 +1199,7 @@ int isdf_fragment_eri(isdf_handle* h, int n_frag, const int32_t* n_orb, const vo
         if (!Bc) return fail(h, ISDF_ERR_OOM, "device allocation of frag_Bc failed");
       }
       ENSURE(rexp, int, "tc_rowexp", rows);
+      ENSURE(rmax, unsigned, "tc_rowmax", 2 * rows);  // bits of the rows' largest entries: M, then B
       ENSURE(tiles_d, int2, "tc_tiles", tl.size());
       ENSURE(tile_of_d, int, "tc_tile_of", tof.size());
       ENSURE(orb_d, int2, "tc_orbits", orb.size());
@@ -1227,14 +1234,18 @@ int isdf_fragment_eri(isdf_handle* h, int n_frag, const int32_t* n_orb, const vo
           }
           const int64_t pad = (i + 1 < grp.size()) ? row0[i + 1] - row0[i] - n2f : 0;
           if (pad > 0)
-            CK(cudaMemset2DAsync(Zr + zsz * (size_t)((row0[i] + n2f) * np), zsz * (size_t)sq, 0,
+            CK(cudaMemset2DAsync(Zr + zsz * (size_t)((row0[i] + n2f) * np), zsz * (size_t)sqZ, 0,
                                  zsz * (size_t)(pad * np), nk, h->st));
         }
         // the R -> q DFT keeps only the q of the sum (M^{-q} = conj(M^q))
         if (tc64)
-          CK(kdft_real_ff(h->st, Zr_ff, M_ff, sq, km, +1, 1.0 / nk, qslot_d));
-        else
-          CK(kdft_real_f(h->st, Zr_f, M_f, sq, km, +1, 1.f / nk, qslot_d));
+          CK(kdft_real_ff(h->st, Zr_ff, M_ff, sqZ, km, +1, 1.0 / nk, qslot_d));
+        else if (inv) {
+          // and of these only the pivot columns, leaving the largest entry of each row
+          CK(cudaMemsetAsync(rmax, 0, sizeof(unsigned) * 2 * (size_t)rows, h->st));
+          CK(kdft_real_f(h->st, Zr_f, M_f, sqZ, km, +1, 1.f / nk, qslot_d, KeepCols{inv, np, pm, rmax}));
+        } else
+          CK(kdft_real_f(h->st, Zr_f, M_f, sqZ, km, +1, 1.f / nk, qslot_d));
       }
       {
         StageTimer stt(h, 4, flops4);
@@ -1245,12 +1256,9 @@ int isdf_fragment_eri(isdf_handle* h, int n_frag, const int32_t* n_orb, const vo
             CK(mlgemm5_tc_chunk(h->st, M_ff, sq, qmap, rows, np, permPi, rankPi, rp, nj, j0, std::min(qc, nS - j0),
                                 rexp, split, lsl, lexp, nk, errw));
         } else if (tc_ml) {
-          // row exponents of the gathered M over the q of the sum, then B^q = M^q L^q
-          // over M^q, q-chunk by q-chunk
-          CK(mlgemm_tc_rowscale(h->st, M_f, sq, np, qmap, nS, permPi, rankPi, rp, rows, rexp));
-          for (int j0 = 0; j0 < nS; j0 += qc)
-            CK(mlgemm_tc_chunk(h->st, M_f, sq, qmap, rows, np, permPi, rankPi, rp, nj, j0, std::min(qc, nS - j0),
-                               rexp, split, lsl, lexp, nk, errw));
+          CK(row_exponents(h->st, rmax, rows, rexp));
+          CK(mlgemm_tc(h->st, M_f, pm, B_f, qmap, nS, rows, rankPi, rp, nj, rexp, lsl,
+                       reinterpret_cast<const float*>(lexp), rmax + rows, errw));
         } else {
           // consecutive q of a run sit at consecutive positions
           for (const auto& r : runs)
@@ -1271,6 +1279,8 @@ int isdf_fragment_eri(isdf_handle* h, int n_frag, const int32_t* n_orb, const vo
         StageTimer stt(h, 5, flops5);
         if (tc64)
           CK(syrk4_tc_rowscale(h->st, M_ff, sq, ldB, nj, nS, rows, rexp));
+        else if (inv)
+          CK(row_exponents(h->st, rmax + rows, rows, rexp));
         else
           CK(syrk_tc_rowscale(h->st, M_f, sq, ldB, nj, nullptr, nS, rows, rexp));
         // per-row sums of the left-out diagonal products, accumulated chunk by chunk
@@ -1283,7 +1293,7 @@ int isdf_fragment_eri(isdf_handle* h, int n_frag, const int32_t* n_orb, const vo
           if (cudaMemcpyAsync(tiles_d, tl.data(), tl.size() * sizeof(int2), cudaMemcpyHostToDevice, h->st) !=
               cudaSuccess)
             return -1;
-          return syrk_tc_chunk(h->st, M_f, sq, ldB, nj, nullptr, rows, 0, nq0, rexp, split, tiles_d,
+          return syrk_tc_chunk(h->st, B_f, sqB, ldB, nj, nullptr, rows, 0, nq0, rexp, split, tiles_d,
                                (int)tl.size(), ws, 0, errw, cfg) == cudaSuccess ? 0 : -1;
         });
         if (sch.band < 0) return fail(h, ISDF_ERR_CUDA, "tile-schedule tuning launch failed");
@@ -1299,7 +1309,7 @@ int isdf_fragment_eri(isdf_handle* h, int n_frag, const int32_t* n_orb, const vo
             StageTimer stk(h, 6, flops5 * nv_chunk / std::max(sum_nv, 1.0));
             CK(syrk4_tc_mma(h->st, split, rows, nq, nj, tiles_d, (int)tl.size(), ws, j0 > 0, errw));
           } else {
-            CK(syrk_tc_split(h->st, M_f, sq, ldB, nj, nullptr, rows, j0, nq, rexp, split, dcorr));
+            CK(syrk_tc_split(h->st, B_f, sqB, ldB, nj, nullptr, rows, j0, nq, rexp, split, dcorr));
             StageTimer stk(h, 6, flops5 * nv_chunk / std::max(sum_nv, 1.0));
             CK(syrk_tc_mma(h->st, split, rows, nq, nj, tiles_d, (int)tl.size(), ws, j0 > 0, errw, sch.cfg));
           }

@@ -350,7 +350,7 @@ template <typename T, int L>
 __global__ void __launch_bounds__(256) kdft_real_cubic_kernel(const typename CT<T>::R* __restrict__ in,
                                                               T* __restrict__ out, int64_t ncol, int lct, int padk,
                                                               const int* __restrict__ qslot, Twiddles16 tw,
-                                                              double scale, int vec) {
+                                                              double scale, int vec, KeepCols keep) {
   using R = typename CT<T>::R;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* s = reinterpret_cast<T*>(smem_raw);
@@ -396,6 +396,19 @@ __global__ void __launch_bounds__(256) kdft_real_cubic_kernel(const typename CT<
   __syncthreads();
   kmesh_dft_cubic<T, L>(s, lct, padk, twc, tws);
   const R h = (R)(0.5 * scale);
+  // blockDim.x is a multiple of ct: a thread's working column is fixed
+  const int cth = threadIdx.x & (ct - 1);
+  const int64_t colt = c0 + 2 * (int64_t)cth;
+  int64_t row0 = 0, row1 = 0;
+  int I0 = 0, I1 = 0;
+  if (keep.inv) {
+    row0 = colt / keep.np;
+    I0 = (int)(colt % keep.np);
+    row1 = (colt + 1) / keep.np;
+    I1 = (int)((colt + 1) % keep.np);
+  }
+  const int64_t per_pos = keep.inv ? ncol / keep.np * keep.pitch : ncol;
+  float mx0 = 0.f, mx1 = 0.f;
   for (int e = threadIdx.x; e < nk * ct; e += blockDim.x) {
     const int k = e >> lct, c = e & (ct - 1);
     const int64_t col = c0 + 2 * (int64_t)c;
@@ -404,9 +417,37 @@ __global__ void __launch_bounds__(256) kdft_real_cubic_kernel(const typename CT<
       const int m0 = k / (L * L), m1 = (k / L) % L, m2 = k % L;
       const int km = (((L - m0) % L) * L + (L - m1) % L) * L + (L - m2) % L;
       const T zq = s[cidx<T, L>(k, c, lct, padk)], zm = s[cidx<T, L>(km, c, lct, padk)];
-      T* o = out + (int64_t)j * ncol + col;
-      o[0] = CT<T>::mk(h * (zq.x + zm.x), h * (zq.y - zm.y));
-      if (col + 1 < ncol) o[1] = CT<T>::mk(h * (zq.y + zm.y), h * (zm.x - zq.x));
+      const T x = CT<T>::mk(h * (zq.x + zm.x), h * (zq.y - zm.y)), y = CT<T>::mk(h * (zq.y + zm.y), h * (zm.x - zq.x));
+      if (!keep.inv) {
+        T* o = out + (int64_t)j * ncol + col;
+        o[0] = x;
+        if (col + 1 < ncol) o[1] = y;
+      } else {
+        const int16_t* iv = keep.inv + (int64_t)j * keep.np;
+        T* o = out + (int64_t)j * per_pos;
+        const int i0 = iv[I0], i1 = col + 1 < ncol ? iv[I1] : -1;
+        if (i0 >= 0) {
+          o[row0 * keep.pitch + i0] = x;
+          if constexpr (sizeof(T) == 8) mx0 = fmaxf(mx0, fmaxf(fabsf((float)x.x), fabsf((float)x.y)));
+        }
+        if (i1 >= 0) {
+          o[row1 * keep.pitch + i1] = y;
+          if constexpr (sizeof(T) == 8) mx1 = fmaxf(mx1, fmaxf(fabsf((float)y.x), fabsf((float)y.y)));
+        }
+      }
+    }
+  }
+  if constexpr (sizeof(T) == 8) {
+    if (keep.rowmax) {
+      for (int o = 16; o >= ct; o >>= 1) {
+        mx0 = fmaxf(mx0, __shfl_xor_sync(0xffffffffu, mx0, o));
+        mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, o));
+      }
+      if ((int)(threadIdx.x & 31) < ct && colt < ncol) {
+        if (__float_as_uint(mx0) > keep.rowmax[row0]) atomicMax(keep.rowmax + row0, __float_as_uint(mx0));
+        if (colt + 1 < ncol && __float_as_uint(mx1) > keep.rowmax[row1])
+          atomicMax(keep.rowmax + row1, __float_as_uint(mx1));
+      }
     }
   }
 }
@@ -415,7 +456,7 @@ template <typename T>
 __global__ void __launch_bounds__(256) kdft_real_cols_kernel(const typename CT<T>::R* __restrict__ in,
                                                              T* __restrict__ out, int64_t ncol, KMesh km, int ct,
                                                              const int* __restrict__ qslot, Twiddles16 tw,
-                                                             double scale) {
+                                                             double scale, KeepCols keep) {
   using R = typename CT<T>::R;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* s = reinterpret_cast<T*>(smem_raw);
@@ -440,7 +481,19 @@ __global__ void __launch_bounds__(256) kdft_real_cols_kernel(const typename CT<T
     const int j = qslot[k];
     if (col < ncol && j >= 0) {
       const T v = s[e];
-      out[(int64_t)j * ncol + col] = CT<T>::mk(v.x * (R)scale, v.y * (R)scale);
+      const T x = CT<T>::mk(v.x * (R)scale, v.y * (R)scale);
+      if (!keep.inv) {
+        out[(int64_t)j * ncol + col] = x;
+      } else {
+        const int64_t row = col / keep.np;
+        const int i = keep.inv[(int64_t)j * keep.np + col % keep.np];
+        if (i < 0) continue;
+        out[((int64_t)j * (ncol / keep.np) + row) * keep.pitch + i] = x;
+        if constexpr (sizeof(T) == 8) {
+          const unsigned b = __float_as_uint(fmaxf(0.f, fmaxf(fabsf((float)x.x), fabsf((float)x.y))));
+          if (keep.rowmax && b > keep.rowmax[row]) atomicMax(keep.rowmax + row, b);
+        }
+      }
     }
   }
 }
@@ -466,7 +519,7 @@ cudaError_t kdft_cubic_launch(cudaStream_t st, TS* data, int64_t ncol, int mode,
   while (lct < 5 && ((int64_t)nk * sizeof(T) << (lct + 1)) <= 65536) ++lct;
   const int padk = kdft_cubic_pad(L, 1 << lct, (int)sizeof(T));
   const size_t smem = ((size_t)nk << lct) * sizeof(T) + (size_t)(nk / L) * padk * sizeof(T);
-  if (smem > 48 * 1024) {
+  if (smem > 40 * 1024) {
     cudaError_t e = cudaFuncSetAttribute(kdft_cubic_kernel<T, L, TS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)smem);
     if (e != cudaSuccess) return e;
@@ -480,13 +533,13 @@ cudaError_t kdft_cubic_launch(cudaStream_t st, TS* data, int64_t ncol, int mode,
 
 template <typename T, int L>
 cudaError_t kdft_real_cubic_launch(cudaStream_t st, const typename CT<T>::R* in, T* out, int64_t ncol,
-                                   const Twiddles16& tw, double scale, const int* qslot) {
+                                   const Twiddles16& tw, double scale, const int* qslot, const KeepCols& keep) {
   constexpr int nk = L * L * L;
   int lct = 0;
   while (lct < 5 && ((int64_t)nk * sizeof(T) << (lct + 1)) <= 65536) ++lct;
   const int padk = kdft_cubic_pad(L, 1 << lct, (int)sizeof(T));
   const size_t smem = ((size_t)nk << lct) * sizeof(T) + (size_t)(nk / L) * padk * sizeof(T);
-  if (smem > 48 * 1024) {
+  if (smem > 40 * 1024) {
     cudaError_t e = cudaFuncSetAttribute(kdft_real_cubic_kernel<T, L>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)smem);
     if (e != cudaSuccess) return e;
@@ -498,7 +551,7 @@ cudaError_t kdft_real_cubic_launch(cudaStream_t st, const typename CT<T>::R* in,
   constexpr int kEpv = 16 / (int)sizeof(T);
   const int vec = ((reinterpret_cast<uintptr_t>(in) & 15) == 0 && (ncol % (2 * kEpv)) == 0 &&
                    (1 << lct) % kEpv == 0) ? 1 : 0;
-  kdft_real_cubic_kernel<T, L><<<(unsigned)nblk, 256, smem, st>>>(in, out, ncol, lct, padk, qslot, tw, scale, vec);
+  kdft_real_cubic_kernel<T, L><<<(unsigned)nblk, 256, smem, st>>>(in, out, ncol, lct, padk, qslot, tw, scale, vec, keep);
   count_launch();
   return cudaGetLastError();
 }
@@ -569,7 +622,7 @@ cudaError_t kdft_launch(cudaStream_t st, TS* data, int64_t ncol, KMesh km, int s
   if (ct < 1) ct = 1;
   if (ct > 32) ct = 32;
   size_t smem = (size_t)nk * ct * sizeof(T);
-  if (smem > 48 * 1024) {
+  if (smem > 40 * 1024) {
     cudaError_t e = cudaFuncSetAttribute(kdft_cols_kernel<T, TS>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
@@ -584,7 +637,7 @@ cudaError_t kdft_launch(cudaStream_t st, TS* data, int64_t ncol, KMesh km, int s
 
 template <typename T>
 cudaError_t kdft_real_launch(cudaStream_t st, const typename CT<T>::R* in, T* out, int64_t ncol, KMesh km, int s,
-                             double scale, const int* qslot) {
+                             double scale, const int* qslot, const KeepCols& keep = KeepCols()) {
   const int nk = km.n[0] * km.n[1] * km.n[2];
   for (int a = 0; a < 3; ++a)
     if (km.n[a] < 1 || km.n[a] > 16) return cudaErrorInvalidValue;
@@ -592,12 +645,12 @@ cudaError_t kdft_real_launch(cudaStream_t st, const typename CT<T>::R* in, T* ou
   const Twiddles16 tw = make_tw(km.n, s);
   if (km.n[0] == km.n[1] && km.n[1] == km.n[2]) {
     switch (km.n[0]) {
-      case 2: return kdft_real_cubic_launch<T, 2>(st, in, out, ncol, tw, scale, qslot);
-      case 3: return kdft_real_cubic_launch<T, 3>(st, in, out, ncol, tw, scale, qslot);
-      case 4: return kdft_real_cubic_launch<T, 4>(st, in, out, ncol, tw, scale, qslot);
-      case 6: return kdft_real_cubic_launch<T, 6>(st, in, out, ncol, tw, scale, qslot);
-      case 8: return kdft_real_cubic_launch<T, 8>(st, in, out, ncol, tw, scale, qslot);
-      case 10: return kdft_real_cubic_launch<T, 10>(st, in, out, ncol, tw, scale, qslot);
+      case 2: return kdft_real_cubic_launch<T, 2>(st, in, out, ncol, tw, scale, qslot, keep);
+      case 3: return kdft_real_cubic_launch<T, 3>(st, in, out, ncol, tw, scale, qslot, keep);
+      case 4: return kdft_real_cubic_launch<T, 4>(st, in, out, ncol, tw, scale, qslot, keep);
+      case 6: return kdft_real_cubic_launch<T, 6>(st, in, out, ncol, tw, scale, qslot, keep);
+      case 8: return kdft_real_cubic_launch<T, 8>(st, in, out, ncol, tw, scale, qslot, keep);
+      case 10: return kdft_real_cubic_launch<T, 10>(st, in, out, ncol, tw, scale, qslot, keep);
       default: break;
     }
   }
@@ -605,14 +658,14 @@ cudaError_t kdft_real_launch(cudaStream_t st, const typename CT<T>::R* in, T* ou
   if (ct < 1) ct = 1;
   if (ct > 32) ct = 32;
   const size_t smem = (size_t)nk * ct * sizeof(T);
-  if (smem > 48 * 1024) {
+  if (smem > 40 * 1024) {
     cudaError_t e = cudaFuncSetAttribute(kdft_real_cols_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)smem);
     if (e != cudaSuccess) return e;
   }
   const int64_t nblk = (ncol + ct - 1) / ct;
   if (nblk > 2147483647LL) return cudaErrorInvalidValue;
-  kdft_real_cols_kernel<T><<<(unsigned)nblk, 256, smem, st>>>(in, out, ncol, km, ct, qslot, tw, scale);
+  kdft_real_cols_kernel<T><<<(unsigned)nblk, 256, smem, st>>>(in, out, ncol, km, ct, qslot, tw, scale, keep);
   count_launch();
   return cudaGetLastError();
 }
@@ -915,7 +968,7 @@ cudaError_t pair_launch(cudaStream_t st, const T* t, int nk, int np, int nf, T* 
   if (nk > 65535) return cudaErrorInvalidValue;
   const size_t smem = (size_t)np * (kPairQ + 1) * sizeof(T);
   if (smem > 200 * 1024) return cudaErrorInvalidValue;
-  if (smem > 48 * 1024) {
+  if (smem > 40 * 1024) {
     cudaError_t e = cudaFuncSetAttribute(pair_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
   }
@@ -931,7 +984,7 @@ cudaError_t pair_real_launch(cudaStream_t st, const T* t, int nk, int np, int nf
   if (nk > 65535) return cudaErrorInvalidValue;
   const size_t smem = (size_t)np * (kPairQ + 1) * sizeof(T);
   if (smem > 200 * 1024) return cudaErrorInvalidValue;
-  if (smem > 48 * 1024) {
+  if (smem > 40 * 1024) {
     cudaError_t e = cudaFuncSetAttribute(pair_real_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
   }
@@ -943,8 +996,8 @@ cudaError_t pair_real_launch(cudaStream_t st, const T* t, int nk, int np, int nf
 }  // namespace
 
 cudaError_t kdft_real_f(cudaStream_t st, const float* in, float2* out, int64_t ncol, KMesh km, int s, float scale,
-                        const int* qslot) {
-  return kdft_real_launch<float2>(st, in, out, ncol, km, s, scale, qslot);
+                        const int* qslot, const KeepCols& keep) {
+  return kdft_real_launch<float2>(st, in, out, ncol, km, s, scale, qslot, keep);
 }
 cudaError_t pair_products_real_f(cudaStream_t st, const float2* t, int nk, int np, int nf, float* Zr, int64_t row0,
                                  int64_t rows) {

@@ -1,7 +1,7 @@
 // Tensor-core (tcgen05) kernels of the fragment ERIs, Eq. 19:
 //     E = sum_q B^q B^q^H   with  B^q = M^q L^q   (V^q = L^q L^q^H).
 // syrk_tc_kernel forms E (below); mlgemm_tc_kernel forms B (further down, with
-// four slices instead of three).
+// three slices).
 //
 // Structural zeros of L^q.  Pi^q is factorised with truncation to rank r_q
 // (pivots perm_q[0..r_q)), W = L_S^{-1} is nonzero only in the columns
@@ -66,10 +66,8 @@ namespace tc {
 constexpr int BM = 128;        // A' rows per tile (64 complex rows of E)
 constexpr int BN = 128;        // B' rows per tile (complex columns of E)
 constexpr int BK = 64;         // fp16 per row per stage (one 128-byte swizzle row)
-constexpr int STAGES = 2;                   // B = M L pipeline depth
 constexpr int NSLICE = 2;                   // fp16 slices per value in E': s1 (integer), s2 (remainder)
 constexpr int TMEM_COLS = 512;              // g0 and g1, each two 128-column FP32 buffers
-constexpr int NTHREADS = 192;
 // E' kernel: warp 0 TMA, warp 1 MMA, 16 drain warps (TMEM lane quarter warp % 4, 32 of
 // the 128 columns each), whose registers hold the tile's float-float running sums
 constexpr int kSyrkThreads = 576, kDrainWarps = 16, kDrainCols = 32;
@@ -291,43 +289,49 @@ __global__ void rrow_scale_kernel(BView B, int64_t K, int* __restrict__ row_exp)
   for (int64_t k = threadIdx.x; k < K; k += blockDim.x) m = fmaxf(m, amax2(B.at(a, k)));
   __shared__ float sm[32];
   m = block_max(m, sm);
-  if (threadIdx.x == 0) row_exp[a] = slice_exp(m);
+  if (threadIdx.x == 0) row_exp[a] = min(slice_exp(m), 127);
 }
 
-// Two slices of x = v 2^ex (|x| < 128): the integer s1 = rint(x) and the fp16
-// remainder s2 = fp16(x - s1); dd = x - s1 - s2 exactly (FP32).
-__device__ __forceinline__ void slice2(float v, int ex, float& s1, __half& s2, float& dd) {
-  const float x = ldexpf(v, ex);
-  s1 = rintf(x);
-  const float r = x - s1;
-  s2 = __float2half_rn(r);
-  dd = r - __half2float(s2);
+// rint(x) for |x| < 2^22 by two additions (the conversion pipe runs at an eighth of their rate).
+__device__ __forceinline__ float rint_small(float x) { return __fadd_rn(__fadd_rn(x, 12582912.f), -12582912.f); }
+__device__ __forceinline__ uint32_t half2_bits(float a, float b) {
+  const __half2 h = __floats2half2_rn(a, b);
+  return *reinterpret_cast<const uint32_t*>(&h);
 }
 
-// Slices of the R rows for the sum positions j0 .. j0 + nq - 1, one block per
+// Two slices of x = v 2^e (|x| < 128), the integer s1 = rint(x) and the fp16 remainder s2 = fp16(x - s1), with
+// dd = x - s1 - s2 exactly (FP32), of the R rows for the sum positions j0 .. j0 + nq - 1, one block per
 // row a: columns 2 (jl nJ + J) and + 1 hold the (re, im) of B at (position
 // j0 + jl, J); columns beyond 2 nq nJ (up to the padded width K2) are zero.
 // With corr, the block also adds to corr[a] the part of E'_aa (in slice units)
 // that the slices do not represent, sum of x^2 - (s1 + s2)^2 = dd (2 x - dd), so
 // that the finish makes the diagonal exact; off the diagonal the representation
 // error is of either sign and averages out.
+// A row's values of one position are contiguous: a warp takes a position at a time.
 __global__ void __launch_bounds__(256) rsplit_kernel(BView B, int64_t j0, int nq, int64_t K2,
                                                      const int* __restrict__ row_exp, __half* __restrict__ S1,
                                                      __half* __restrict__ S2, double* __restrict__ corr) {
-  const int64_t a = blockIdx.x, half = K2 / 2, ncol = (int64_t)nq * B.nJ;
-  const int ex = row_exp[a];
+  const int64_t a = blockIdx.x;
+  const int ex = row_exp[a], nJ = (int)B.nJ, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const float sc = ldexpf(1.f, ex);
   float d = 0.f;
-  for (int64_t c2 = threadIdx.x; c2 < half; c2 += blockDim.x) {
-    const float2 x = (c2 < ncol) ? B.at(a, j0 * B.nJ + c2) : make_float2(0.f, 0.f);
-    float r1, i1, rd, id;
-    __half r2, i2;
-    slice2(x.x, ex, r1, r2, rd);
-    slice2(x.y, ex, i1, i2, id);
-    const int64_t at = a * K2 + 2 * c2;
-    *reinterpret_cast<__half2*>(S1 + at) = __floats2half2_rn(r1, i1);
-    *reinterpret_cast<__half2*>(S2 + at) = __halves2half2(r2, i2);
-    d += rd * (2.f * ldexpf(x.x, ex) - rd) + id * (2.f * ldexpf(x.y, ex) - id);
+  auto put = [&](float2 v, int64_t at) {
+    const float x = v.x * sc, y = v.y * sc, r1 = rint_small(x), i1 = rint_small(y), rx = x - r1, ry = y - i1;
+    const __half2 h2 = __floats2half2_rn(rx, ry);
+    const float2 f2 = __half22float2(h2);
+    const float rd = rx - f2.x, id = ry - f2.y;
+    *reinterpret_cast<uint32_t*>(S1 + at) = half2_bits(r1, i1);
+    *reinterpret_cast<__half2*>(S2 + at) = h2;
+    d += rd * (2.f * x - rd) + id * (2.f * y - id);
+  };
+  for (int jl = warp; jl < nq; jl += 8) {
+    const int64_t slot = B.qmap ? (int64_t)__ldg(B.qmap + j0 + jl) : j0 + jl;
+    const float2* p = B.p + slot * B.sQ + a * B.sA;
+    const int64_t at = a * K2 + 2 * (int64_t)jl * nJ;
+#pragma unroll 4
+    for (int J = lane; J < nJ; J += 32) put(p[J], at + 2 * J);
   }
+  for (int64_t c = 2 * (int64_t)nq * nJ + threadIdx.x; c < K2; c += 256) S1[a * K2 + c] = S2[a * K2 + c] = __half(0.f);
   if (!corr) return;
   __shared__ double sd[8];
   double v = d;
@@ -538,174 +542,51 @@ __global__ void __launch_bounds__(256) eri_traces_final_kernel(const double2* __
 // 2^-18 of it and accumulate in FP32 over at most kMlMaxK terms.  The epilogue
 // forms g0 + (g1 + g2) once and rescales.  Simulated on the c2 data against the
 // exact products: E_J within ~1e-9 Ha (four 7-bit slices with ten products: ~2e-8).
-// Tiles of 128 x 64 with K rows of 32 fp16 in two stages: 72 KB of shared memory and
-// 256 TMEM columns per CTA, so that two CTAs share an SM and one's set-up and
-// epilogue overlap the other's MMAs (each tile runs only 2 r_q / 32 k-blocks).
+//
+// One kernel slices M and multiplies.  What bounds the product is the tensor pipe (six
+// products) as long as M is read once and B written once; slices of M in memory would cost
+// 12 + 12 bytes per value on top of the 8 + 8 (measured: the separate slicing pass and the
+// GEMM on 128 x 64 tiles took 27 ms at Nk = 1000, 16,000 rows, r = 128).  So a persistent
+// CTA takes 128 rows of one q: producer warps load the gathered columns of M, cut them and
+// write the slices in the MMA's shared-memory layout, the slices of L come by TMA (a q's
+// stay in L2 while its row blocks pass), and passes of up to 64 complex columns (N = 128: an
+// MMA of 128 x N x 16 takes N/2 clocks only from N = 128 on) accumulate in three 128-column
+// TMEM groups.  The next pass's MMAs wait only for the TMEM reads of the one before.
+// The epilogue also leaves the rows' largest entries for the slicing of B.
+//
+// Kernel roles (704 threads): warp 0 TMA, warp 1 TMEM and MMAs, warps 2-13 producers (three groups
+// that take the k-blocks in turn, each with its next one in flight), warps 14-21 epilogue.
 constexpr int MSL = 3;                                     // slices per operand
-constexpr int MBN = 64;                                    // B' rows per tile (N of the MMA)
-constexpr int MBJ = MBN / 2;                               // complex columns of B per tile
+constexpr int MBJ = 32;                                    // columns of L are padded to a multiple of it
 constexpr int MBK = 32;                                    // fp16 of K per stage row (64-byte swizzle)
+constexpr int MPN = 128;                                   // B' rows per pass (64 complex columns)
 constexpr int MA_BYTES = BM * MBK * 2;                     // 8 KB per slice
-constexpr int MB_BYTES = MBN * MBK * 2;                    // 4 KB per slice
-constexpr int MSTAGE_BYTES = MSL * (MA_BYTES + MB_BYTES);  // 36 KB
-constexpr int kMlTmem = 256;                               // three 64-column groups
+constexpr int MB_BYTES = MPN * MBK * 2;                    // 8 KB per slice
+constexpr int MBOX = 64 * MBK * 2;                         // bytes of one TMA box (64 rows)
+constexpr int MSTAGE_BYTES = MSL * (MA_BYTES + MB_BYTES);  // 48 KB
+constexpr int MSTAGES = 3;
+constexpr int MGROUPS = 3;                                 // producer groups of four warps
+constexpr int MTHREADS = 64 + 128 * MGROUPS + 256;
+constexpr int MEPI = 8;                                    // epilogue warps
+constexpr int kMlPitch = MPN + 2;                          // floats per staged row (bank-conflict padding)
+constexpr int kMlOut = BM * kMlPitch * 4;
+constexpr int kMlTmem = 512;                               // three 128-column groups
 constexpr int kMlMaxK = 640;                               // K' bound for exact accumulation
-constexpr uint32_t kIdescMl = (1u << 4) | ((uint32_t)(MBN >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
+constexpr uint32_t kIdescMl = (1u << 4) | ((uint32_t)(BM >> 4) << 24);  // N >> 3 at bit 17 is added per pass
 
 struct MlArgs {
-  float2* out;          // B: element (a, J) of sum position j = j0 + ql at out[j sq + a nj + J]
+  const float2* M;      // gathered: element (a, c) of sum position j at M[j sqM + a pm + c], c < r_q
+  float2* B;            // element (a, J) of position j at B[j sqB + a nj + J]
+  const int* row_exp;   // e_a, [rows]
+  const float* col_scale;  // 2^-f_qJ, [position][nj_pad], zero for J >= nj
   const int* qmap;      // q of each sum position
-  const int* row_exp;   // e_a, [n2]
-  const int* col_exp;   // f_qJ, [Nk][nj_pad] indexed by q (nj_pad: complex columns, multiple of MBJ)
-  int64_t sq;           // q stride of out
-  int n2, nj, nj_pad, j0, nkb;
+  const int* rank;      // r_q by q
+  unsigned* bmax;       // [rows]: bits of the largest |component| of the rows of B
+  int64_t sqM, sqB;
+  int pm, rows, nj, nj_pad, mt, nkb, npass;
+  int64_t units;        // mt x positions
   int* err;
 };
-
-__global__ void __launch_bounds__(NTHREADS, 2)
-    mlgemm_tc_kernel(const __grid_constant__ CUtensorMap mA1, const __grid_constant__ CUtensorMap mA2,
-                     const __grid_constant__ CUtensorMap mA3, const __grid_constant__ CUtensorMap mB1,
-                     const __grid_constant__ CUtensorMap mB2, const __grid_constant__ CUtensorMap mB3, MlArgs args) {
-  extern __shared__ __align__(1024) uint8_t smem_raw[];
-  uint8_t* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
-  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + STAGES * MSTAGE_BYTES);
-  uint64_t* full = bars;               // [STAGES]
-  uint64_t* empty = bars + STAGES;     // [STAGES]
-  uint64_t* accf = bars + 2 * STAGES;  // accumulation finished
-  uint32_t* s_tmem = reinterpret_cast<uint32_t*>(bars + 2 * STAGES + 1);
-  volatile int* s_err = reinterpret_cast<volatile int*>(s_tmem + 1);
-
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  // the output-column tiles of one row block are adjacent in launch order, so
-  // they run together and share the row block's slices through L2
-  const int ntj = args.nj_pad / MBJ;
-  const int ti = blockIdx.x / ntj, tj = blockIdx.x % ntj, ql = blockIdx.y;
-  const int pos = args.j0 + ql;                      // position in the sum (storage of B)
-  const int slot = args.qmap ? args.qmap[pos] : pos;  // its q (slices and exponents of L)
-  const int nkb = args.nkb;
-
-  if (threadIdx.x == 0) {
-    for (int s = 0; s < STAGES; ++s) {
-      mbar_init(&full[s], 1);
-      mbar_init(&empty[s], 1);
-    }
-    mbar_init(accf, 1);
-    *s_err = 0;
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  }
-  if (warp == 1) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(s_tmem)),
-                 "r"(kMlTmem)
-                 : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-  }
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  const uint32_t tmem_base = *s_tmem;
-
-  if (warp == 0) {
-    if (lane == 0) {
-      const CUtensorMap* ma[MSL] = {&mA1, &mA2, &mA3};
-      const CUtensorMap* mb[MSL] = {&mB1, &mB2, &mB3};
-      const int arow = ql * args.n2 + ti * BM, brow = slot * 2 * args.nj_pad + tj * MBN;
-      for (int kb = 0; kb < nkb; ++kb) {
-        const int s = kb % STAGES, r = kb / STAGES;
-        if (!mbar_wait(&empty[s], (r & 1) ^ 1, s_err, args.err, 11)) break;
-        uint8_t* st = smem + s * MSTAGE_BYTES;
-        mbar_expect_tx(&full[s], MSTAGE_BYTES);
-        const int x = kb * MBK;
-#pragma unroll
-        for (int i = 0; i < MSL; ++i) {
-          tma_load_2d(st + i * MA_BYTES, ma[i], &full[s], x, arow);
-          tma_load_2d(st + MSL * MA_BYTES + i * MB_BYTES, mb[i], &full[s], x, brow);
-        }
-      }
-    }
-  } else if (warp == 1) {
-    if (lane == 0) {
-      const uint32_t g0 = tmem_base, g1 = tmem_base + MBN, g2 = tmem_base + 2 * MBN;
-      bool ok = true;
-      for (int kb = 0; kb < nkb && ok; ++kb) {
-        const int s = kb % STAGES, r = kb / STAGES;
-        if (!mbar_wait(&full[s], r & 1, s_err, args.err, 12)) {
-          ok = false;
-          break;
-        }
-        tc_fence_after();
-        const uint8_t* st = smem + s * MSTAGE_BYTES;
-        uint64_t dA[MSL], dB[MSL];
-#pragma unroll
-        for (int i = 0; i < MSL; ++i) {
-          dA[i] = sdesc_k<MBK>(st + i * MA_BYTES);
-          dB[i] = sdesc_k<MBK>(st + MSL * MA_BYTES + i * MB_BYTES);
-        }
-#pragma unroll
-        for (int kk = 0; kk < MBK / 16; ++kk) {
-          const uint64_t off = (uint64_t)(kk * 32) >> 4;
-          const uint32_t acc = (kb == 0 && kk == 0) ? 0u : 1u;
-          umma_f16(g0, dA[0] + off, dB[0] + off, kIdescMl, acc);
-          umma_f16(g1, dA[0] + off, dB[1] + off, kIdescMl, acc);
-          umma_f16(g1, dA[1] + off, dB[0] + off, kIdescMl, 1u);
-          umma_f16(g2, dA[0] + off, dB[2] + off, kIdescMl, acc);
-          umma_f16(g2, dA[1] + off, dB[1] + off, kIdescMl, 1u);
-          umma_f16(g2, dA[2] + off, dB[0] + off, kIdescMl, 1u);
-        }
-        umma_commit(&empty[s]);
-      }
-      if (ok) umma_commit(accf);
-    }
-  } else {
-    // epilogue: warps 2..5 -> TMEM lane quarter (warp % 4); lane r is row a of M, TMEM
-    // column n is B' row n of the tile: complex column Jl = n / 2, part n % 2 (Re, Im)
-    const int q = warp & 3;
-    const int r = q * 32 + lane;             // row of the tile
-    const int64_t a = (int64_t)ti * BM + r;  // row of M (of the q-point's block)
-    // warp-uniform, so that the .sync.aligned TMEM loads are taken by whole warps
-    const bool okw = __all_sync(0xffffffffu, mbar_wait(accf, 0, s_err, args.err, 13));
-    tc_fence_after();
-    // the operand stages are idle now: stage the 128 x MBJ complex tile for coalesced stores
-    constexpr int kPitch = MBN + 2;     // floats per staged row (bank-conflict padding)
-    float* tileS = reinterpret_cast<float*>(smem);
-    const int ea = (okw && a < args.n2) ? args.row_exp[a] : 0;
-    const int* fcol = args.col_exp + (int64_t)slot * args.nj_pad + tj * MBJ;
-#pragma unroll 1
-    for (int cb = 0; cb < MBN / 32; ++cb) {
-      uint32_t v0[32] = {}, v1[32] = {}, v2[32] = {};
-      if (okw) {
-        const uint32_t lo = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(cb * 32);
-        tmem_ld32(lo, v0);
-        tmem_ld32(lo + MBN, v1);
-        tmem_ld32(lo + 2 * MBN, v2);
-      }
-#pragma unroll
-      for (int j = 0; j < 32; ++j) {
-        const float v = __uint_as_float(v0[j]) + (__uint_as_float(v1[j]) + __uint_as_float(v2[j]));
-        const int n = cb * 32 + j;
-        tileS[r * kPitch + n] = ldexpf(v, -(ea + fcol[n >> 1]));
-      }
-    }
-    asm volatile("bar.sync 1, 128;" ::: "memory");
-    if (okw) {
-      const int t = threadIdx.x - 64;
-      float2* outq = args.out + (int64_t)pos * args.sq;
-      for (int idx = t; idx < BM * MBJ; idx += 128) {
-        const int ar = idx / MBJ, Jl = idx % MBJ;
-        const int64_t aa = (int64_t)ti * BM + ar;
-        const int J = tj * MBJ + Jl;
-        if (aa < args.n2 && J < args.nj)
-          outq[aa * args.nj + J] = *reinterpret_cast<const float2*>(tileS + ar * kPitch + 2 * Jl);
-      }
-    }
-  }
-  tc_fence_before();
-  __syncthreads();
-  if (warp == 1) {
-    tc_fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(kMlTmem)
-                 : "memory");
-  }
-}
 
 __device__ __forceinline__ float round_int(float x) { return rintf(x); }
 __device__ __forceinline__ double round_int(double x) { return rint(x); }
@@ -722,88 +603,355 @@ __device__ __forceinline__ void slice3r(R v, __half& h1, __half& h2, __half& h3)
   h3 = __float2half_rn((float)r2);
 }
 
-// Row exponents of M over the gathered columns of the q-points of the sum:
-// max over positions Q < nS and c < r_q of |M^{q}_{a, perm_q[c]}|, q = qmap[Q],
-// with M^q stored at position Q.
-__global__ void mrow_scale_kernel(const float2* __restrict__ M, int64_t sq, int np, const int* __restrict__ qmap,
-                                  int nS, const int* __restrict__ perm, const int* __restrict__ rank, int rp,
-                                  int* __restrict__ row_exp) {
-  const int64_t a = blockIdx.x;
-  float m = 0.f;
-  for (int64_t k = threadIdx.x; k < (int64_t)nS * rp; k += blockDim.x) {
-    const int Q = (int)(k / rp), c = (int)(k % rp);
-    const int q = qmap[Q];
-    if (c < rank[q]) m = fmaxf(m, amax2(M[(int64_t)Q * sq + a * np + perm[(int64_t)q * np + c]]));
-  }
-  __shared__ float sm[32];
-  m = block_max(m, sm);
-  if (threadIdx.x == 0) row_exp[a] = slice_exp(m);
+// slice3r of two values, packed by slice.
+__device__ __forceinline__ void slice3_pair(float x, float y, uint32_t (&out)[3]) {
+  const float sx = rint_small(x), sy = rint_small(y), rx = x - sx, ry = y - sy;
+  const __half2 h2 = __floats2half2_rn(rx, ry);
+  const float2 f2 = __half22float2(h2);
+  out[0] = half2_bits(sx, sy);
+  out[1] = *reinterpret_cast<const uint32_t*>(&h2);
+  out[2] = half2_bits(rx - f2.x, ry - f2.y);
 }
 
-// A' slices of M for the sum positions j0..j0+nq-1 (M^q stored by position,
-// q = qmap[j]): block ql holds row a = P_a over Kp columns: the gathered columns
-// perm_q[c], c < r_q, as (re, im) pairs, zero beyond.
-__global__ void msplit_kernel(const float2* __restrict__ M, int64_t sq, int np, const int* __restrict__ qmap,
-                              const int* __restrict__ perm, const int* __restrict__ rank, int64_t n2, int j0, int nq,
-                              int Kp, const int* __restrict__ row_exp, __half* __restrict__ S1,
-                              __half* __restrict__ S2, __half* __restrict__ S3) {
-  const int64_t half = Kp / 2, total = (int64_t)nq * n2 * half;
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t ql = e / (n2 * half), rem = e % (n2 * half);
-    const int64_t a = rem / half, c = rem % half;
-    const int q = qmap[j0 + ql];
-    float2 v = make_float2(0.f, 0.f);
-    if (c < rank[q]) v = M[(int64_t)(j0 + ql) * sq + a * np + perm[(int64_t)q * np + c]];
-    const int ex = row_exp[a];
-    __half r1, r2, r3, i1, i2, i3;
-    slice3r<float>(ldexpf(v.x, ex), r1, r2, r3);
-    slice3r<float>(ldexpf(v.y, ex), i1, i2, i3);
-    const int64_t at = (ql * n2 + a) * Kp + 2 * c;
-    *reinterpret_cast<__half2*>(S1 + at) = __halves2half2(r1, i1);
-    *reinterpret_cast<__half2*>(S2 + at) = __halves2half2(r2, i2);
-    *reinterpret_cast<__half2*>(S3 + at) = __halves2half2(r3, i3);
+__device__ __forceinline__ uint32_t pack2(__half a, __half b) {
+  const __half2 h = __halves2half2(a, b);
+  return *reinterpret_cast<const uint32_t*>(&h);
+}
+
+__global__ void __launch_bounds__(MTHREADS, 1)
+    mlgemm_tc_kernel(const __grid_constant__ CUtensorMap mB1, const __grid_constant__ CUtensorMap mB2,
+                     const __grid_constant__ CUtensorMap mB3, MlArgs args) {
+  extern __shared__ __align__(1024) uint8_t smem_raw[];
+  uint8_t* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
+  float* tileS = reinterpret_cast<float*>(smem + MSTAGES * MSTAGE_BYTES);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + MSTAGES * MSTAGE_BYTES + kMlOut);
+  uint64_t* full = bars;                 // [MSTAGES] slices of L landed, four producer warps done
+  uint64_t* empty = bars + MSTAGES;      // [MSTAGES] read by the MMAs
+  uint64_t* accf = bars + 2 * MSTAGES;   // pass accumulated
+  uint64_t* drained = accf + 1;          // pass read out of TMEM
+  uint32_t* s_tmem = reinterpret_cast<uint32_t*>(drained + 1);
+  volatile int* s_err = reinterpret_cast<volatile int*>(s_tmem + 1);
+
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int nkb = args.nkb, npass = args.npass;
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < MSTAGES; ++s) {
+      mbar_init(&full[s], 1 + 4);
+      mbar_init(&empty[s], 1);
+    }
+    mbar_init(accf, 1);
+    mbar_init(drained, MEPI);
+    *s_err = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(s_tmem)),
+                 "r"(kMlTmem)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem_base = *s_tmem;
+  // B' rows of pass p: 128, or 64 where at most 32 complex columns are left
+  auto pass_n = [&](int p) { return args.nj_pad - p * (MPN / 2) > MPN / 4 ? MPN : MPN / 2; };
+
+  if (warp == 0) {
+    if (lane == 0) {
+      const CUtensorMap* mb[MSL] = {&mB1, &mB2, &mB3};
+      int64_t it = 0;
+      bool ok = true;
+      for (int64_t u = blockIdx.x; u < args.units && ok; u += gridDim.x) {
+        const int pos = (int)(u / args.mt);
+        for (int p = 0; p < npass && ok; ++p) {
+          const int boxes = pass_n(p) / 64, brow = pos * 2 * args.nj_pad + p * MPN;
+          for (int kb = 0; kb < nkb; ++kb, ++it) {
+            const int s = (int)(it % MSTAGES);
+            if (!mbar_wait(&empty[s], (uint32_t)((it / MSTAGES) & 1) ^ 1, s_err, args.err, 11)) {
+              ok = false;
+              break;
+            }
+            uint8_t* st = smem + s * MSTAGE_BYTES + MSL * MA_BYTES;
+            mbar_expect_tx(&full[s], MSL * boxes * MBOX);
+            for (int i = 0; i < MSL; ++i)
+              for (int b = 0; b < boxes; ++b)
+                tma_load_2d(st + i * MB_BYTES + b * MBOX, mb[i], &full[s], kb * MBK, brow + b * 64);
+          }
+        }
+      }
+    }
+  } else if (warp == 1) {
+    if (lane == 0) {
+      int64_t it = 0, ps = 0;
+      bool ok = true;
+      for (int64_t u = blockIdx.x; u < args.units && ok; u += gridDim.x)
+        for (int p = 0; p < npass && ok; ++p, ++ps) {
+          const uint32_t idesc = kIdescMl | ((uint32_t)(pass_n(p) >> 3) << 17);
+          const uint32_t g0 = tmem_base, g1 = tmem_base + MPN, g2 = tmem_base + 2 * MPN;
+          if (ps > 0 && !mbar_wait(drained, (uint32_t)((ps - 1) & 1), s_err, args.err, 14)) {
+            ok = false;
+            break;
+          }
+          tc_fence_after();
+          for (int kb = 0; kb < nkb; ++kb, ++it) {
+            const int s = (int)(it % MSTAGES);
+            if (!mbar_wait(&full[s], (uint32_t)((it / MSTAGES) & 1), s_err, args.err, 12)) {
+              ok = false;
+              break;
+            }
+            tc_fence_after();
+            const uint8_t* st = smem + s * MSTAGE_BYTES;
+            uint64_t dA[MSL], dB[MSL];
+#pragma unroll
+            for (int i = 0; i < MSL; ++i) {
+              dA[i] = sdesc_k<MBK>(st + i * MA_BYTES);
+              dB[i] = sdesc_k<MBK>(st + MSL * MA_BYTES + i * MB_BYTES);
+            }
+#pragma unroll
+            for (int kk = 0; kk < MBK / 16; ++kk) {
+              const uint64_t off = (uint64_t)(kk * 32) >> 4;
+              const uint32_t acc = (kb == 0 && kk == 0) ? 0u : 1u;
+              umma_f16(g0, dA[0] + off, dB[0] + off, idesc, acc);
+              umma_f16(g1, dA[0] + off, dB[1] + off, idesc, acc);
+              umma_f16(g1, dA[1] + off, dB[0] + off, idesc, 1u);
+              umma_f16(g2, dA[0] + off, dB[2] + off, idesc, acc);
+              umma_f16(g2, dA[1] + off, dB[1] + off, idesc, 1u);
+              umma_f16(g2, dA[2] + off, dB[0] + off, idesc, 1u);
+            }
+            umma_commit(&empty[s]);
+          }
+          if (ok) umma_commit(accf);
+        }
+    }
+  } else if (warp < 2 + 4 * MGROUPS) {
+    // producers: group g takes the stages it = g, g + MGROUPS, ...; lanes 8 per row, two complex values
+    // each, so that a warp's load covers four 128-byte runs of M and its store whole rows of the
+    // swizzled layout.  A group's next block is in flight while the others' are cut.
+    const int grp = (warp - 2) >> 2, t = ((warp - 2) & 3) * 32 + lane, l8 = t & 7, rr = t >> 3;
+    const int per_unit = npass * nkb;
+    // the unit the loads are in: its row of this thread, its rank, rows left
+    int64_t lu = blockIdx.x;
+    const float2* lm = nullptr;
+    int lr = 0, lrows = 0, lrem = grp, lkb = 0;
+    auto enter = [&]() {
+      if (lu >= args.units) return;
+      const int pos = (int)(lu / args.mt), ti = (int)(lu % args.mt);
+      lr = __ldg(args.rank + __ldg(args.qmap + pos));
+      lrows = args.rows - ti * BM;
+      lm = args.M + (int64_t)pos * args.sqM + ((int64_t)ti * BM + rr) * args.pm + l8 * 2;
+    };
+    auto forward = [&]() {  // brings lrem below per_unit
+      if (lrem >= per_unit) {
+        do {
+          lrem -= per_unit;
+          lu += gridDim.x;
+        } while (lrem >= per_unit);
+        enter();
+      }
+      lkb = lrem % nkb;
+    };
+    float4 x[8];
+    auto load = [&]() {
+      const int col = lkb * (MBK / 2) + l8 * 2, rows = col < lr ? lrows : 0;
+      const float2* m = lm + lkb * (MBK / 2);
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        x[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (i * 16 + rr < rows) {
+          x[i] = __ldg(reinterpret_cast<const float4*>(m + (int64_t)i * 16 * args.pm));
+          if (col + 1 >= lr) x[i].z = x[i].w = 0.f;  // beyond the rank: not written
+        }
+      }
+    };
+    float sc[8];
+    int64_t it = grp, su = -1;
+    enter();
+    forward();
+    if (lu < args.units) load();
+    while (lu < args.units) {
+      if (su != lu) {
+        su = lu;
+        const int a0 = (int)(lu % args.mt) * BM + rr;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          const int ex = a0 + i * 16 < args.rows ? __ldg(args.row_exp + a0 + i * 16) : 0;  // -121 .. 127
+          sc[i] = __int_as_float((ex + 127) << 23);
+        }
+      }
+      const int s = (int)(it % MSTAGES);
+      if (!__all_sync(0xffffffffu, mbar_wait(&empty[s], (uint32_t)((it / MSTAGES) & 1) ^ 1, s_err, args.err, 15))) break;
+      uint8_t* st = smem + s * MSTAGE_BYTES;
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const int row = i * 16 + rr;
+        uint32_t h[3], g[3];
+        slice3_pair(x[i].x * sc[i], x[i].y * sc[i], h);
+        slice3_pair(x[i].z * sc[i], x[i].w * sc[i], g);
+        uint8_t* d = st + row * (MBK * 2) + (((l8 >> 1) ^ ((row >> 1) & 3)) << 4) + (l8 & 1) * 8;
+#pragma unroll
+        for (int k = 0; k < MSL; ++k) *reinterpret_cast<uint2*>(d + k * MA_BYTES) = make_uint2(h[k], g[k]);
+      }
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&full[s]);
+      it += MGROUPS;
+      lrem += MGROUPS;
+      forward();
+      if (lu < args.units) load();
+    }
+  } else {
+    // epilogue: TMEM lane quarter warp % 4; the two warps of a quarter take half of the pass's columns
+    // each.  Lane r is row a of M, TMEM column n is B' row n: complex column n / 2, part n % 2.
+    const int q = warp & 3, half = (warp - 2 - 4 * MGROUPS) >> 2, r = q * 32 + lane;
+    int64_t ps = 0;
+    bool ok = true;
+    for (int64_t u = blockIdx.x; u < args.units; u += gridDim.x) {
+      const int pos = (int)(u / args.mt), ti = (int)(u % args.mt), a = ti * BM + r;
+      const float rs = a < args.rows ? ldexpf(1.f, -args.row_exp[a]) : 0.f;
+      float m = 0.f;
+      for (int p = 0; p < npass; ++p, ++ps) {
+        const int N = pass_n(p), n0 = half * (N / 2);
+        if (ok) ok = __all_sync(0xffffffffu, mbar_wait(accf, (uint32_t)(ps & 1), s_err, args.err, 13));
+        if (ok) {
+          tc_fence_after();
+          // 2^-f_qJ, zero for J >= nj
+          const float* fcol = args.col_scale + (int64_t)pos * args.nj_pad + p * (MPN / 2);
+#pragma unroll 1
+          for (int cb = n0; cb < n0 + N / 2; cb += 8) {
+            uint32_t v0[8], v1[8], v2[8];
+            const uint32_t lo = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)cb;
+            tmem_ld8(lo, v0);
+            tmem_ld8(lo + MPN, v1);
+            tmem_ld8(lo + 2 * MPN, v2);
+            const float4 f = __ldg(reinterpret_cast<const float4*>(fcol + (cb >> 1)));
+            const float fs[4] = {f.x, f.y, f.z, f.w};
+            tmem_wait_ld();
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              const float x = __uint_as_float(v0[2 * j]) + (__uint_as_float(v1[2 * j]) + __uint_as_float(v2[2 * j]));
+              const float y =
+                  __uint_as_float(v0[2 * j + 1]) + (__uint_as_float(v1[2 * j + 1]) + __uint_as_float(v2[2 * j + 1]));
+              const float2 z = make_float2(x * rs * fs[j], y * rs * fs[j]);
+              m = fmaxf(m, fmaxf(fabsf(z.x), fabsf(z.y)));
+              *reinterpret_cast<float2*>(tileS + r * kMlPitch + cb + 2 * j) = z;
+            }
+          }
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(drained);
+        }
+        // a warp whose wait expired keeps the barriers below company, without storing
+        asm volatile("bar.sync 1, 256;" ::: "memory");
+        if (ok) {
+          const int lg = N == MPN ? 6 : 5, t = threadIdx.x - (MTHREADS - 256), Jl = t & ((1 << lg) - 1), rstep = 256 >> lg;
+          if (p * (MPN / 2) + Jl < args.nj) {
+            const float* src = tileS + (t >> lg) * kMlPitch + 2 * Jl;
+            float2* out = args.B + (int64_t)pos * args.sqB + (int64_t)(ti * BM + (t >> lg)) * args.nj + p * (MPN / 2) + Jl;
+            const int last = min(BM, args.rows - ti * BM);
+#pragma unroll 8
+            for (int ar = t >> lg; ar < last; ar += rstep) {
+              *out = *reinterpret_cast<const float2*>(src);
+              out += (int64_t)rstep * args.nj;
+              src += rstep * kMlPitch;
+            }
+          }
+        }
+        asm volatile("bar.sync 1, 256;" ::: "memory");
+      }
+      if (ok && a < args.rows) {
+        const unsigned bits = __float_as_uint(m);
+        if (bits > args.bmax[a]) atomicMax(args.bmax + a, bits);
+      }
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 1) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(kMlTmem)
+                 : "memory");
   }
 }
 
-// B' slices of w_q^{1/2} L^q: block (row, q), row = 2 J + part, is R_J = (Re L, -Im L)
-// (part 0) or I_J = (Im L, Re L) (part 1) over the gathered rows perm_q(c) of column J,
+// Row exponents from the bits of the rows' largest entries.
+__global__ void row_exp_kernel(const unsigned* __restrict__ mx, int64_t rows, int* __restrict__ row_exp) {
+  const int64_t a = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  // at most 2^127, a float (rows below 2^-121 keep fewer digits of what is subnormal anyway)
+  if (a < rows) row_exp[a] = min(slice_exp(__uint_as_float(mx[a])), 127);
+}
+
+// inv[j][I] = c where perm_q[c] = I, c < r_q (q = qmap[j]), else -1.
+__global__ void inv_perm_kernel(const int* __restrict__ qmap, const int* __restrict__ perm, const int* __restrict__ rank,
+                                int np, int16_t* __restrict__ inv) {
+  const int j = blockIdx.x, q = qmap[j], r = rank[q];
+  for (int I = threadIdx.x; I < np; I += blockDim.x) inv[(int64_t)j * np + I] = -1;
+  __syncthreads();
+  for (int c = threadIdx.x; c < r; c += blockDim.x) inv[(int64_t)j * np + perm[(int64_t)q * np + c]] = (int16_t)c;
+}
+
+// B' slices of w_q^{1/2} L^q for the positions of the sum: block (32 columns J, position), row = 2 J + part, is
+// R_J = (Re L, -Im L) (part 0) or I_J = (Im L, Re L) (part 1) over the gathered rows perm_q(c) of column J,
 // scaled by 2^f_qJ (largest component of the column in [64, 128)); columns J >= nj,
-// c >= r_q and beyond 2 r_q are zero.  Layout [q][2 nj_pad][Kp] per slice;
-// exponents [q][nj_pad].
-__global__ void lslice_kernel(const double2* __restrict__ L, const double* __restrict__ sw, int np,
-                              const int* __restrict__ perm, const int* __restrict__ rank, int nj, int nj_pad, int Kp,
-                              __half* __restrict__ S1, __half* __restrict__ S2, __half* __restrict__ S3,
-                              int* __restrict__ col_exp) {
-  const int q = blockIdx.y, J = blockIdx.x >> 1, part = blockIdx.x & 1;
+// c >= r_q and beyond 2 r_q are zero.  Layout [position][2 nj_pad][Kp] per slice; the inverse scales
+// [position][nj_pad].  Rows of L are read along J and the slices written along c, through shared memory.
+__global__ void __launch_bounds__(256) lslice_kernel(const double2* __restrict__ L, const double* __restrict__ sw, int np,
+                                                     const int* __restrict__ qmap, const int* __restrict__ perm,
+                                                     const int* __restrict__ rank, int nj, int nj_pad, int Kp,
+                                                     __half* __restrict__ S1, __half* __restrict__ S2,
+                                                     __half* __restrict__ S3, float* __restrict__ col_scale) {
+  const int j = blockIdx.y, q = qmap[j], J0 = blockIdx.x * 32, tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
   const double w = sw[q];
-  const int r = rank[q];
+  const int r = rank[q], J = J0 + tx;
   const double2* Lq = L + (int64_t)q * np * np;
   const int* pq = perm + (int64_t)q * np;
+  __shared__ double sm[8][32];
+  __shared__ uint32_t sd[3][32][33];
   double m = 0.0;
   if (J < nj)
-    for (int c = threadIdx.x; c < r; c += blockDim.x) {
+    for (int c = ty; c < r; c += 8) {
       const double2 v = Lq[(int64_t)pq[c] * np + J];
       m = fmax(m, fmax(fabs(v.x * w), fabs(v.y * w)));
     }
-  __shared__ double sm[32];
-  m = block_max(m, sm);
-  const int ex = (m > 0.0 && isfinite(m)) ? 6 - ilogb(m) : 0;
-  if (threadIdx.x == 0 && part == 0) col_exp[(int64_t)q * nj_pad + J] = ex;
-  const int64_t row = ((int64_t)q * 2 * nj_pad + blockIdx.x) * Kp;
-  for (int c = threadIdx.x; c < Kp / 2; c += blockDim.x) {
-    double re = 0.0, im = 0.0;
-    if (J < nj && c < r) {
-      const double2 v = Lq[(int64_t)pq[c] * np + J];
-      const double lr = ldexp(v.x * w, ex), li = ldexp(v.y * w, ex);
-      re = part ? li : lr;
-      im = part ? lr : -li;
+  sm[ty][tx] = m;
+  __syncthreads();
+  for (int i = 0; i < 8; ++i) m = fmax(m, sm[i][tx]);
+  // within what a float's power of two holds
+  const int ex = (m > 0.0 && isfinite(m)) ? max(-126, min(126, 6 - ilogb(m))) : 0;
+  if (ty == 0) col_scale[(int64_t)j * nj_pad + J] = J < nj ? ldexpf(1.f, -ex) : 0.f;
+  __half* const S[3] = {S1, S2, S3};
+  for (int c0 = 0; c0 < Kp / 2; c0 += 32) {
+    __syncthreads();
+    for (int cc = ty; cc < 32; cc += 8) {
+      const int c = c0 + cc;
+      double lr = 0.0, li = 0.0;
+      if (J < nj && c < r) {
+        const double2 v = Lq[(int64_t)pq[c] * np + J];
+        lr = ldexp(v.x * w, ex);
+        li = ldexp(v.y * w, ex);
+      }
+      __half a1, a2, a3, b1, b2, b3;
+      slice3r<double>(lr, a1, a2, a3);
+      slice3r<double>(li, b1, b2, b3);
+      sd[0][tx][cc] = pack2(a1, b1);
+      sd[1][tx][cc] = pack2(a2, b2);
+      sd[2][tx][cc] = pack2(a3, b3);
     }
-    __half a1, a2, a3, b1, b2, b3;
-    slice3r<double>(re, a1, a2, a3);
-    slice3r<double>(im, b1, b2, b3);
-    *reinterpret_cast<__half2*>(S1 + row + 2 * c) = __halves2half2(a1, b1);
-    *reinterpret_cast<__half2*>(S2 + row + 2 * c) = __halves2half2(a2, b2);
-    *reinterpret_cast<__half2*>(S3 + row + 2 * c) = __halves2half2(a3, b3);
+    __syncthreads();
+    // row 2 Jl + part of the block, lanes along c
+    for (int e = ty; e < 64; e += 8) {
+      const int Jl = e >> 1, part = e & 1, c = c0 + tx;
+      if (c >= Kp / 2) continue;
+      const int64_t at = ((int64_t)j * 2 * nj_pad + 2 * (J0 + Jl) + part) * Kp + 2 * c;
+#pragma unroll
+      for (int i = 0; i < 3; ++i) {
+        const uint32_t x = sd[i][Jl][tx];
+        // (re, -im) or (im, re); the slices of -x are those of x negated
+        const uint32_t y = part ? (x >> 16) | (x << 16) : x ^ 0x80000000u;
+        *reinterpret_cast<uint32_t*>(S[i] + at) = y;
+      }
+    }
   }
 }
 
@@ -945,60 +1093,75 @@ cudaError_t syrk_tc_finish_eri_z(cudaStream_t st, const void* ws, int ntiles, co
   return finish_eri_impl<double2>(st, ws, ntiles, tile_of_d, orb, nf, row_exp, corr, scale, eri, gamma, part, out4);
 }
 
+cudaError_t row_exponents(cudaStream_t st, const unsigned* mx, int64_t rows, int* row_exp) {
+  if (rows <= 0) return cudaSuccess;
+  tc::row_exp_kernel<<<(unsigned)((rows + 255) / 256), 256, 0, st>>>(mx, rows, row_exp);
+  count_launch();
+  return cudaGetLastError();
+}
+
 // ---- B = M L on the tensor cores, three slices (host side)
 int mlgemm_tc_kp(int rp) { return (int)tc::round_up(2 * (int64_t)rp, tc::BK); }
 int mlgemm_tc_nj_pad(int nj) { return (int)tc::round_up(nj, tc::MBJ); }
 bool mlgemm_tc_supported(int rp) { return rp > 0 && mlgemm_tc_kp(rp) <= tc::kMlMaxK; }
-size_t mlgemm_tc_lslice_bytes(int nk, int rp, int nj) {
-  return (size_t)tc::MSL * nk * (2 * mlgemm_tc_nj_pad(nj)) * mlgemm_tc_kp(rp) * sizeof(__half) + 256;
-}
-size_t mlgemm_tc_split_bytes(int64_t n2, int rp, int nq) {
-  return (size_t)tc::MSL * nq * n2 * mlgemm_tc_kp(rp) * sizeof(__half) + 256;
+size_t mlgemm_tc_lslice_bytes(int nS, int rp, int nj) {
+  return (size_t)tc::MSL * nS * (2 * mlgemm_tc_nj_pad(nj)) * mlgemm_tc_kp(rp) * sizeof(__half) + 256;
 }
 
-cudaError_t mlgemm_tc_prepare(cudaStream_t st, const double2* L, const double* sw, int nk, int np, const int* perm,
-                              const int* rank, int rp, int nj, void* lsl, int* col_exp) {
+cudaError_t mlgemm_tc_prepare(cudaStream_t st, const double2* L, const double* sw, int np, const int* qmap, int nS,
+                              const int* perm, const int* rank, int rp, int nj, void* lsl, float* col_scale, int16_t* inv) {
   using namespace tc;
+  if (np > 32767) return cudaErrorInvalidValue;
   const int Kp = mlgemm_tc_kp(rp), njp = mlgemm_tc_nj_pad(nj);
-  const size_t per = (size_t)nk * 2 * njp * Kp;
+  const size_t per = (size_t)nS * 2 * njp * Kp;
   __half* S1 = reinterpret_cast<__half*>(lsl);
-  lslice_kernel<<<dim3(2 * njp, nk), 128, 0, st>>>(L, sw, np, perm, rank, nj, njp, Kp, S1, S1 + per, S1 + 2 * per,
-                                                    col_exp);
+  lslice_kernel<<<dim3(njp / 32, nS), 256, 0, st>>>(L, sw, np, qmap, perm, rank, nj, njp, Kp, S1, S1 + per, S1 + 2 * per,
+                                                    col_scale);
+  count_launch();
+  inv_perm_kernel<<<nS, 128, 0, st>>>(qmap, perm, rank, np, inv);
   count_launch();
   return cudaGetLastError();
 }
 
-cudaError_t mlgemm_tc_rowscale(cudaStream_t st, const float2* M, int64_t sq, int np, const int* qmap, int nS,
-                               const int* perm, const int* rank, int rp, int64_t n2, int* row_exp) {
-  tc::mrow_scale_kernel<<<(unsigned)n2, 256, 0, st>>>(M, sq, np, qmap, nS, perm, rank, rp, row_exp);
-  count_launch();
-  return cudaGetLastError();
-}
-
-cudaError_t mlgemm_tc_chunk(cudaStream_t st, float2* M, int64_t sq, const int* qmap, int64_t n2, int np,
-                            const int* perm, const int* rank, int rp, int nj, int j0, int nq, const int* row_exp,
-                            void* split, const void* lsl, const int* col_exp, int nk, int* err) {
+cudaError_t mlgemm_tc(cudaStream_t st, const float2* M, int pm, float2* B, const int* qmap, int nS, int64_t rows,
+                      const int* rank, int rp, int nj, const int* row_exp, const void* lsl, const float* col_scale,
+                      unsigned* bmax, int* err) {
   using namespace tc;
-  if (n2 <= 0 || nq <= 0) return cudaSuccess;
-  if (!mlgemm_tc_supported(rp)) return cudaErrorInvalidValue;
+  if (rows <= 0 || nS <= 0) return cudaSuccess;
+  if (!mlgemm_tc_supported(rp) || pm < rp || pm % 2 != 0 || rows > 2147483647LL - BM) return cudaErrorInvalidValue;
   const int Kp = mlgemm_tc_kp(rp), njp = mlgemm_tc_nj_pad(nj);
-  const size_t pa = (size_t)nq * n2 * Kp, pb = (size_t)nk * 2 * njp * Kp;
-  __half* S1 = reinterpret_cast<__half*>(split);
-  msplit_kernel<<<nblk((int64_t)nq * n2 * (Kp / 2)), 256, 0, st>>>(M, sq, np, qmap, perm, rank, n2, j0, nq, Kp,
-                                                                   row_exp, S1, S1 + pa, S1 + 2 * pa);
-  count_launch();
+  const size_t pb = (size_t)nS * 2 * njp * Kp;
   const __half* L1 = reinterpret_cast<const __half*>(lsl);
-  CUtensorMap mA[MSL], mB[MSL];
+  CUtensorMap mB[MSL];
   for (int i = 0; i < MSL; ++i)
-    if (!make_map(&mA[i], S1 + i * pa, Kp, (int64_t)nq * n2, Kp, BM, MBK) ||
-        !make_map(&mB[i], L1 + i * pb, Kp, (int64_t)nk * 2 * njp, Kp, MBN, MBK))
-      return cudaErrorInvalidValue;
-  const size_t smem = (size_t)STAGES * MSTAGE_BYTES + 1024 + 256;
+    if (!make_map(&mB[i], L1 + i * pb, Kp, (int64_t)nS * 2 * njp, Kp, 64, MBK)) return cudaErrorInvalidValue;
+  const size_t smem = (size_t)MSTAGES * MSTAGE_BYTES + kMlOut + 1024 + 256;
   cudaError_t e = cudaFuncSetAttribute(mlgemm_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  const int mt = (int)((n2 + BM - 1) / BM), ntj = njp / MBJ;
-  MlArgs args{M, qmap, row_exp, col_exp, sq, (int)n2, nj, njp, j0, Kp / MBK, err};
-  mlgemm_tc_kernel<<<dim3(mt * ntj, nq), NTHREADS, smem, st>>>(mA[0], mA[1], mA[2], mB[0], mB[1], mB[2], args);
+  int dev = 0, sms = 0;
+  e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e != cudaSuccess) return e;
+  MlArgs a{};
+  a.M = M;
+  a.B = B;
+  a.row_exp = row_exp;
+  a.col_scale = col_scale;
+  a.qmap = qmap;
+  a.rank = rank;
+  a.bmax = bmax;
+  a.sqM = rows * pm;
+  a.sqB = rows * nj;
+  a.pm = pm;
+  a.rows = (int)rows;
+  a.nj = nj;
+  a.nj_pad = njp;
+  a.mt = (int)((rows + BM - 1) / BM);
+  a.nkb = Kp / MBK;
+  a.npass = (njp + MPN / 2 - 1) / (MPN / 2);
+  a.units = (int64_t)a.mt * nS;
+  a.err = err;
+  mlgemm_tc_kernel<<<(unsigned)std::min<int64_t>(a.units, sms), MTHREADS, smem, st>>>(mB[0], mB[1], mB[2], a);
   count_launch();
   return cudaGetLastError();
 }
