@@ -81,8 +81,9 @@ cudaError_t cgemm(cudaStream_t st, char opA, char opB, int m, int n, int k, floa
 struct KMesh {
   int n[3];
 };
+// radix: mixed-radix axes on every mesh (else by the direct sum on meshes without a kernel of their own).
 cudaError_t kdft_cols(cudaStream_t st, double2* data, int64_t ncol, KMesh km, int s1, int s2,
-                      int mode, double scale);
+                      int mode, double scale, bool radix);
 cudaError_t kdft_cols_f(cudaStream_t st, float2* data, int64_t ncol, KMesh km, int s1, int s2,
                         int mode, float scale);
 
@@ -147,8 +148,9 @@ cudaError_t lt_to_rowmajor(cudaStream_t st, const double2* Lt, const int32_t* ra
 // dtw: device table of 3 x 64 forward twiddles exp(-2 pi i j/n_a) (grid_twiddles);
 // work: grid_coulomb_work_bytes(nq) bytes of device scratch (phase and weight tables).
 size_t grid_coulomb_work_bytes(int nq, const CellDev& c);
+// radix: two passes and mixed-radix axes, else the direct sums in their fixed order.
 cudaError_t grid_coulomb_fft(cudaStream_t st, double2* x, int rows_per_q, int q0, int nq,
-                             const CellDev& c, const double2* dtw, void* work);
+                             const CellDev& c, const double2* dtw, void* work, bool radix);
 cudaError_t grid_coulomb_fft_f(cudaStream_t st, float2* x, int rows_per_q, int q0, int nq,
                                const CellDev& c, const double2* dtw, void* work);
 // the same in float-float (FP32 arithmetic, ~2^-44), in place on float-float data

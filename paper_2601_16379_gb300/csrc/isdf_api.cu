@@ -806,7 +806,7 @@ int isdf_fit_zeta(isdf_handle* h, double solve_tol, int32_t* rank_out) {
   ENSURE(Pi, double2, "Pi", (size_t)nk * np * np);
   ZM(zw, 'R', 'T', np, np, nao, 1.0, X, nao, (int64_t)np * nao, X, nao, (int64_t)np * nao, Pi,
            np, (int64_t)np * np, nk);
-  CK(kdft_cols(h->st, Pi, (int64_t)np * np, km, +1, -1, 1, 1.0 / nk));
+  CK(kdft_cols(h->st, Pi, (int64_t)np * np, km, +1, -1, 1, 1.0 / nk, fp64));
   // eta^q (Eq. 5): g^k_I(r) = sum_mu conj(X^k_I mu) Phi^k_mu(r), then the k-convolution.
   ENSURE(eta, double2, "eta", (size_t)nk * np * ng);
   ZOpt g_opt;
@@ -816,7 +816,7 @@ int isdf_fit_zeta(isdf_handle* h, double solve_tol, int32_t* rank_out) {
   // the k-convolution of Algorithm 1 over the grid columns: FP64 in the FP64 path,
   // float-float (~2^-44 relative, FP32 arithmetic) in the others
   if (h->prec == ISDF_FP64)
-    CK(kdft_cols(h->st, eta, (int64_t)np * ng, km, +1, -1, 1, 1.0 / nk));
+    CK(kdft_cols(h->st, eta, (int64_t)np * ng, km, +1, -1, 1, 1.0 / nk, true));
   else
     CK(kdft_cols_zff(h->st, eta, (int64_t)np * ng, km, +1, -1, 1, 1.0 / nk));
   // Pi^q = L L^H (pivoted), W = L_S^{-1}
@@ -898,7 +898,8 @@ int isdf_coulomb_metric(isdf_handle* h, void* V_out) {
   // of its fragments by up to 5e-8 of the larger ones (see isdf_fit_zeta)
   if (h->prec != ISDF_MIXED) {
     for (const auto& r : qh.runs)
-      CK(grid_coulomb_fft(h->st, xi + r.first * xg, rx, r.first, r.second, h->cell, tw, gwork));
+      CK(grid_coulomb_fft(h->st, xi + r.first * xg, rx, r.first, r.second, h->cell, tw, gwork,
+                          h->prec == ISDF_FP64));
     ENSURE(qlist, int, "q_list", nk);
     CK(cudaMemcpyAsync(qlist, qh.list.data(), sizeof(int) * qh.list.size(), cudaMemcpyHostToDevice, h->st));
     ZOpt reps;
@@ -953,7 +954,8 @@ int isdf_coulomb_metric_eta(isdf_handle* h, void* V_out) {
   for (const auto& r : qh.runs) {
     CK(cudaMemcpyAsync(work + r.first * pg, eta + r.first * pg, sizeof(double2) * (size_t)(r.second * pg),
                        cudaMemcpyDeviceToDevice, h->st));
-    CK(grid_coulomb_fft(h->st, work + r.first * pg, np, r.first, r.second, h->cell, tw, gwork));
+    CK(grid_coulomb_fft(h->st, work + r.first * pg, np, r.first, r.second, h->cell, tw, gwork,
+                        h->prec == ISDF_FP64));
     ZM("grid_work_z", 'R', 'T', np, np, ng, h->volume, work + r.first * pg, ng, pg,
              work + r.first * pg, ng, pg, Veta + r.first * pp, np, pp, r.second);
   }
@@ -1057,9 +1059,9 @@ int isdf_fragment_eri(isdf_handle* h, int n_frag, const int32_t* n_orb, const vo
         StageTimer stt(h, 3, frag_m_flops(nk, np, nf, nao, km));
         ZM("tc_zwork", 'N', 'N', np, nf, nao, 1.0, X, nao, (int64_t)np * nao, Cf, nf, (int64_t)nao * nf, T,
                  nf, (int64_t)np * nf, nk);
-        CK(kdft_cols(h->st, T, (int64_t)np * nf, km, +1, +1, 0, 1.0));
+        CK(kdft_cols(h->st, T, (int64_t)np * nf, km, +1, +1, 0, 1.0, true));
         CK(pair_products(h->st, T, nk, np, nf, M));
-        CK(kdft_cols(h->st, M, n2 * np, km, +1, +1, 0, 1.0 / nk));
+        CK(kdft_cols(h->st, M, n2 * np, km, +1, +1, 0, 1.0 / nk, true));
       }
       {
         // B = [w_q^{1/2} M^q L^q]_{q in S}, compact: B[a][slot(q) nj + J], the nj
@@ -1432,10 +1434,10 @@ int isdf_sos_polarizability(isdf_handle* h, const void* C, int n_mo, int n_occ, 
   // Algorithm 1 does for Pi^q: with hat(a)(R) = sum_k a(k) e^{+ik.R} and
   // check(b)(R) = sum_k b(k) e^{-ik.R},  chi = (1/Nk) DFT_-( hat(Go)^T o check(Gv) )
   const KMesh km{{h->cell.kmesh[0], h->cell.kmesh[1], h->cell.kmesh[2]}};
-  CK(kdft_cols(h->st, Go, pp, km, +1, +1, 0, 1.0));
-  CK(kdft_cols(h->st, Gv, pp, km, -1, -1, 0, 1.0));
+  CK(kdft_cols(h->st, Go, pp, km, +1, +1, 0, 1.0, true));
+  CK(kdft_cols(h->st, Gv, pp, km, -1, -1, 0, 1.0, true));
   CK(hadamard_t(h->st, Go, Gv, np, nk, chi));
-  CK(kdft_cols(h->st, chi, pp, km, -1, -1, 0, 1.0 / nk));
+  CK(kdft_cols(h->st, chi, pp, km, -1, -1, 0, 1.0 / nk, true));
   if (s_out) {
     // S = Nk^2 sum_Q tr[conj(V^Q) chi^Q conj(V^Q) (chi^{-Q})^T], V^Q = L^Q L^Q^H (Eq. 12)
     ZM("zwork", 'N', 'C', np, np, l_cols(h), 1.0, Lq, np, pp, Lq, np, pp, Vq, np, pp, nk);
@@ -1473,10 +1475,10 @@ int isdf_exchange(isdf_handle* h, const void* P, void* K_out) {
   ZM("zwork", 'N', 'C', np, np, l_cols(h), 1.0, Lq, np, (int64_t)np * np, Lq, np, (int64_t)np * np, Vd, np,
      (int64_t)np * np, nk);
   // Gamma^k = sum_k' (V^{k'-k})^T o rho^{k'}: DFT_- V, DFT_+ rho, transposed product, DFT_- / Nk
-  CK(kdft_cols(h->st, Vd, (int64_t)np * np, km, -1, -1, 0, 1.0));
-  CK(kdft_cols(h->st, rho, (int64_t)np * np, km, +1, +1, 0, 1.0));
+  CK(kdft_cols(h->st, Vd, (int64_t)np * np, km, -1, -1, 0, 1.0, true));
+  CK(kdft_cols(h->st, rho, (int64_t)np * np, km, +1, +1, 0, 1.0, true));
   CK(hadamard_t(h->st, Vd, rho, np, nk, rho));
-  CK(kdft_cols(h->st, rho, (int64_t)np * np, km, -1, -1, 0, 1.0 / nk));
+  CK(kdft_cols(h->st, rho, (int64_t)np * np, km, -1, -1, 0, 1.0 / nk, true));
   // K^k = -(1/Nk) X^k^H Gamma^k X^k
   ZM("zwork", 'N', 'N', np, nao, np, 1.0, rho, np, (int64_t)np * np, X, nao, (int64_t)np * nao, t1, nao,
            (int64_t)np * nao, nk);

@@ -7,10 +7,11 @@
 //                (Eq. 6), producing sqrt(w) c(G) so that V = Omega c'^H c'.
 // pair_products  the outer product of Algorithm 2 in supercell space.
 //
-// All transforms are direct per-axis DFTs staged through shared memory (mesh
-// axes are at most 16 points for the k-mesh and 64 for the grid), with the
-// twiddles exp(+-2 pi i j/n) tabulated on the host.
+// All transforms are per-axis DFTs staged through shared memory (mesh axes are at most 16
+// points for the k-mesh and 64 for the grid), with the twiddles exp(+-2 pi i j/n) tabulated
+// on the host: mixed radix in registers, or direct sums where a path keeps their rounding.
 #include <cmath>
+#include <type_traits>
 #include <vector>
 
 #include "common.cuh"
@@ -249,6 +250,60 @@ struct Dft<R, 5, S, L, 5> {
     xi[3] = t2i - u2r;
   }
 };
+
+// The same passes with the mixed-radix transforms (a 5-point axis costs 8 FP64 operations per value
+// instead of 30): the FP64 path's meshes without a kernel of their own.  The direct form above
+// keeps the arithmetic of the other paths (see isdf_fit_zeta).
+template <typename T, int L>
+__device__ __forceinline__ void kmesh_line(T* s, int base, int step, const typename CT<T>::R* tc,
+                                           const typename CT<T>::R* ts) {
+  using R = typename CT<T>::R;
+  R vr[L], vi[L];
+#pragma unroll
+  for (int i = 0; i < L; ++i) {
+    const T v = s[base + i * step];
+    vr[i] = v.x;
+    vi[i] = v.y;
+  }
+  Dft<R, L, 1, L>::run(vr, vi, tc, ts);
+#pragma unroll
+  for (int i = 0; i < L; ++i) s[base + i * step] = CT<T>::mk(vr[i], vi[i]);
+}
+
+template <typename T>
+__device__ void kmesh_dft_radix(T* s, int ct, const int n[3], const typename CT<T>::R* tc,
+                                const typename CT<T>::R* ts) {
+  const int nk = n[0] * n[1] * n[2];
+  for (int a = 2; a >= 0; --a) {
+    const int L = n[a];
+    if (L == 1) continue;
+    const int stride = (a == 2) ? 1 : (a == 1 ? n[2] : n[1] * n[2]);
+    const int nlines = (nk / L) * ct;
+    for (int line = threadIdx.x; line < nlines; line += blockDim.x) {
+      const int c = line % ct, rest = line / ct, hi = rest / stride, lo = rest % stride;
+      const int base = (hi * stride * L + lo) * ct + c, step = stride * ct;
+      const typename CT<T>::R *tca = tc + a * 16, *tsa = ts + a * 16;
+      switch (L) {
+        case 2: kmesh_line<T, 2>(s, base, step, tca, tsa); break;
+        case 3: kmesh_line<T, 3>(s, base, step, tca, tsa); break;
+        case 4: kmesh_line<T, 4>(s, base, step, tca, tsa); break;
+        case 5: kmesh_line<T, 5>(s, base, step, tca, tsa); break;
+        case 6: kmesh_line<T, 6>(s, base, step, tca, tsa); break;
+        case 7: kmesh_line<T, 7>(s, base, step, tca, tsa); break;
+        case 8: kmesh_line<T, 8>(s, base, step, tca, tsa); break;
+        case 9: kmesh_line<T, 9>(s, base, step, tca, tsa); break;
+        case 10: kmesh_line<T, 10>(s, base, step, tca, tsa); break;
+        case 11: kmesh_line<T, 11>(s, base, step, tca, tsa); break;
+        case 12: kmesh_line<T, 12>(s, base, step, tca, tsa); break;
+        case 13: kmesh_line<T, 13>(s, base, step, tca, tsa); break;
+        case 14: kmesh_line<T, 14>(s, base, step, tca, tsa); break;
+        case 15: kmesh_line<T, 15>(s, base, step, tca, tsa); break;
+        default: kmesh_line<T, 16>(s, base, step, tca, tsa); break;
+      }
+    }
+    __syncthreads();
+  }
+}
 
 // Cubic mesh of compile-time side L: the three per-axis passes in place on
 // s[k][c] (Nk x ct, ct = 2^lct columns), line per thread, with the mixed-radix
@@ -556,7 +611,7 @@ cudaError_t kdft_real_cubic_launch(cudaStream_t st, const typename CT<T>::R* in,
   return cudaGetLastError();
 }
 
-template <typename T, typename TS = T>
+template <typename T, typename TS = T, bool kRadix = false>
 __global__ void __launch_bounds__(256) kdft_cols_kernel(TS* __restrict__ data, int64_t ncol, KMesh km,
                                                         int ct, int mode, Twiddles16 tw1,
                                                         Twiddles16 tw2, double scale) {
@@ -580,14 +635,20 @@ __global__ void __launch_bounds__(256) kdft_cols_kernel(TS* __restrict__ data, i
     s[e] = v;
   }
   __syncthreads();
-  kmesh_dft_smem<T>(s, ct, km.n, tw1c, tw1s);
+  auto dft = [&](const R* c, const R* sn) {
+    if constexpr (kRadix)
+      kmesh_dft_radix<T>(s, ct, km.n, c, sn);
+    else
+      kmesh_dft_smem<T>(s, ct, km.n, c, sn);
+  };
+  dft(tw1c, tw1s);
   if (mode == 1) {
     for (int e = threadIdx.x; e < nk * ct; e += blockDim.x) {
       T v = s[e];
       s[e] = CT<T>::mk(v.x * v.x + v.y * v.y, 0);
     }
     __syncthreads();
-    kmesh_dft_smem<T>(s, ct, km.n, tw2c, tw2s);
+    dft(tw2c, tw2s);
   }
   for (int e = threadIdx.x; e < nk * ct; e += blockDim.x) {
     const int k = e / ct, c = e % ct;
@@ -599,7 +660,7 @@ __global__ void __launch_bounds__(256) kdft_cols_kernel(TS* __restrict__ data, i
   }
 }
 
-template <typename T, typename TS = T>
+template <typename T, typename TS = T, bool kRadix = false>
 cudaError_t kdft_launch(cudaStream_t st, TS* data, int64_t ncol, KMesh km, int s1, int s2, int mode,
                         double scale) {
   const int nk = km.n[0] * km.n[1] * km.n[2];
@@ -623,13 +684,13 @@ cudaError_t kdft_launch(cudaStream_t st, TS* data, int64_t ncol, KMesh km, int s
   if (ct > 32) ct = 32;
   size_t smem = (size_t)nk * ct * sizeof(T);
   if (smem > 40 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(kdft_cols_kernel<T, TS>,
+    cudaError_t e = cudaFuncSetAttribute(kdft_cols_kernel<T, TS, kRadix>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
   }
   int64_t nblk = (ncol + ct - 1) / ct;
   if (nblk > 2147483647LL) return cudaErrorInvalidValue;
-  kdft_cols_kernel<T, TS><<<(unsigned)nblk, 256, smem, st>>>(data, ncol, km, ct, mode,
+  kdft_cols_kernel<T, TS, kRadix><<<(unsigned)nblk, 256, smem, st>>>(data, ncol, km, ct, mode,
                                                          make_tw(km.n, s1), make_tw(km.n, s2), scale);
   count_launch();
   return cudaGetLastError();
@@ -714,66 +775,218 @@ __global__ void phase_kernel(T* __restrict__ x, int64_t rows_per_q, int q0, int 
   }
 }
 
-// One axis of the forward grid DFT, lines of length L with element stride S.
-// Block: lpb lines x L outputs; smem holds the lines.
+// One axis of the forward grid DFT, lines of length L with element stride S, by the direct sum.
+// A block takes 4 (256 / L) lines; a thread one output j of four of them, so that a twiddle read
+// and its index serve four products and four independent chains run side by side, each in the
+// order of the sum.  The line pitch is odd: threads on consecutive lines hit distinct banks.
+// Bound by its FP32 (float-float) or FP64 operations: 24^3 grid, 64 k-points, 850 rows:
+// 106 -> 79 ms in float-float against one line per thread.
+constexpr int kAxisLines = 4;
 template <typename T>
-__global__ void __launch_bounds__(256) grid_axis_kernel(T* __restrict__ x, int64_t nrows, int ng,
-                                                        int L, int64_t S, int lpb,
+__global__ void __launch_bounds__(256) grid_axis_kernel(T* __restrict__ x, int64_t total_lines, int ng,
+                                                        int L, int S, int groups,
                                                         const double2* __restrict__ tw) {
   using R = typename CT<T>::R;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* tws = reinterpret_cast<T*>(smem_raw);  // 64 twiddles in the working precision
   T* s = reinterpret_cast<T*>(smem_raw + 64 * sizeof(double2));
-  const int64_t lines_per_row = ng / L;
-  const int64_t total_lines = nrows * lines_per_row;
-  const int64_t l0 = (int64_t)blockIdx.x * lpb;
+  const int lpr = ng / L, pitch = L | 1, lpb = kAxisLines * groups;
+  const int64_t l0 = (int64_t)blockIdx.x * lpb, row0 = l0 / lpr;
+  const int lr0 = (int)(l0 - row0 * lpr), nl = (int)min((int64_t)lpb, total_lines - l0);
   for (int t = threadIdx.x; t < L; t += blockDim.x) tws[t] = CT<T>::mk((R)tw[t].x, (R)tw[t].y);
-  // line id -> base element offset
-  auto base_of = [&](int64_t line) -> int64_t {
-    const int64_t row = line / lines_per_row;
-    const int64_t lr = line % lines_per_row;  // index over the other axes
-    const int64_t hi = lr / S, lo = lr % S;
-    return row * ng + hi * S * L + lo;
+  x += row0 * ng;
+  // line li of the block -> element offset of its first point
+  auto base_of = [&](int li) -> int64_t {
+    const int lr = lr0 + li, row = lr / lpr, r = lr - row * lpr;  // r over the other axes
+    return (int64_t)row * ng + (r / S) * S * L + r % S;
   };
   for (int e = threadIdx.x; e < lpb * L; e += blockDim.x) {
-    int li, i;
-    if (S == 1) {
-      li = e / L;
-      i = e % L;
-    } else {
-      li = e % lpb;
-      i = e / lpb;
-    }
-    const int64_t line = l0 + li;
+    const int li = S == 1 ? e / L : e % lpb, i = S == 1 ? e - li * L : e / lpb;
     T v = CT<T>::mk(0, 0);
-    if (line < total_lines) v = x[base_of(line) + (int64_t)i * S];
-    s[li * L + i] = v;
+    if (li < nl) v = x[base_of(li) + (int64_t)i * S];
+    s[li * pitch + i] = v;
   }
   __syncthreads();
-  for (int e = threadIdx.x; e < lpb * L; e += blockDim.x) {
-    int li, j;
-    if (S == 1) {
-      li = e / L;
-      j = e % L;
-    } else {
-      li = e % lpb;
-      j = e / lpb;
+  if (threadIdx.x >= groups * L) return;
+  const int g = S == 1 ? threadIdx.x / L : threadIdx.x % groups, j = S == 1 ? threadIdx.x - g * L : threadIdx.x / groups;
+  const T* sl = s + g * pitch;
+  R ax[kAxisLines], ay[kAxisLines];
+#pragma unroll
+  for (int c = 0; c < kAxisLines; ++c) ax[c] = ay[c] = 0;
+  int t = 0;
+  for (int i = 0; i < L; ++i) {
+    const T w = tws[t];
+#pragma unroll
+    for (int c = 0; c < kAxisLines; ++c) {
+      const T v = sl[c * groups * pitch + i];
+      ax[c] += v.x * w.x - v.y * w.y;
+      ay[c] += v.x * w.y + v.y * w.x;
     }
-    const int64_t line = l0 + li;
-    if (line >= total_lines) continue;
-    const T* sl = s + li * L;
-    R ax = 0, ay = 0;
+    t += j;
+    if (t >= L) t -= L;
+  }
+#pragma unroll
+  for (int c = 0; c < kAxisLines; ++c) {
+    const int li = g + c * groups;
+    if (li < nl) x[base_of(li) + (int64_t)j * S] = CT<T>::mk(ax[c], ay[c]);
+  }
+}
+
+// ---- the FP64 path's grid transform: two passes over memory and mixed radix.
+// The direct form takes six passes and 6 L FP64 operations per value and axis (2 per clock and
+// SM: 18 of 34 ms of the c2 fit and metric).  Here a block takes one (g1, g2) plane -- phase,
+// axis 2, axis 1 -- and a second kernel axis 0 and the weight.  An axis of length L = P Q goes in two
+// steps of in-register transforms of at most 8 points; other lengths (a prime above 8 in them) by
+// the direct sum over that factor, four FMAs per product.  Measured with the k-transforms: fit and
+// metric of 125 k-points on an 18^3 grid 33.9 -> 18.1 ms, ragged quartets 20.5 -> 13.0.
+// FP64_TC keeps the direct sums: see isdf_fit_zeta.
+constexpr int kRadMax = 8;
+__host__ __device__ inline int radix_p(int L) {  // P: both factors <= 8 if possible, else the largest factor <= 8
+  int best = 1;
+  for (int p = 2; p <= kRadMax; ++p)
+    if (L % p == 0) {
+      const int q = L / p, bq = L / best;
+      const bool ok = q <= kRadMax, bok = best > 1 && bq <= kRadMax;
+      // the more even split where both are small, else the larger P
+      if (ok ? (!bok || (q > p ? q : p) < (bq > best ? bq : best)) : !bok) best = p;
+    }
+  return best;
+}
+
+template <int N>
+__device__ __forceinline__ void grid_small(double2* s, int base, int step, const double2* tw, int tstep) {
+  double vr[N], vi[N], wc[N], ws[N];
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    const double2 v = s[base + i * step], w = tw[i * tstep];
+    vr[i] = v.x;
+    vi[i] = v.y;
+    wc[i] = w.x;
+    ws[i] = w.y;
+  }
+  Dft<double, N, 1, N>::run(vr, vi, wc, ws);
+#pragma unroll
+  for (int i = 0; i < N; ++i) s[base + i * step] = make_double2(vr[i], vi[i]);
+}
+__device__ __forceinline__ void grid_small_any(int n, double2* s, int base, int step, const double2* tw, int tstep) {
+  switch (n) {
+    case 2: grid_small<2>(s, base, step, tw, tstep); break;
+    case 3: grid_small<3>(s, base, step, tw, tstep); break;
+    case 4: grid_small<4>(s, base, step, tw, tstep); break;
+    case 5: grid_small<5>(s, base, step, tw, tstep); break;
+    case 6: grid_small<6>(s, base, step, tw, tstep); break;
+    case 7: grid_small<7>(s, base, step, tw, tstep); break;
+    case 8: grid_small<8>(s, base, step, tw, tstep); break;
+    default: break;
+  }
+}
+
+// Transform of all lines (fixed o, l) of s[(o L + i) inner + l], o < outer, l < inner, along i; tw: the L-th
+// roots.  The result for frequency k sits at i = (k mod P) (L / P) + k / P.  tmp: as large as s, used
+// (and returned as the result) where L / P > 8.
+__device__ double2* grid_lines(double2* s, double2* tmp, int outer, int inner, int L, int P, const double2* tw) {
+  const int Q = L / P;
+  if (P > 1) {
+    for (int e = threadIdx.x; e < outer * Q * inner; e += blockDim.x) {
+      const int l = e % inner, r = e / inner, n2 = r % Q, o = r / Q, base = (o * L + n2) * inner + l;
+      grid_small_any(P, s, base, Q * inner, tw, Q);
+      for (int k1 = 1; k1 < P; ++k1) {
+        double2* v = s + base + k1 * Q * inner;
+        if (n2) *v = cmul(*v, tw[(n2 * k1) % L]);
+      }
+    }
+    __syncthreads();
+  }
+  if (Q == 1) return s;
+  if (Q <= kRadMax) {
+    for (int e = threadIdx.x; e < outer * P * inner; e += blockDim.x) {
+      const int l = e % inner, r = e / inner, k1 = r % P, o = r / P;
+      grid_small_any(Q, s, (o * L + k1 * Q) * inner + l, inner, tw, P);
+    }
+    __syncthreads();
+    return s;
+  }
+  for (int e = threadIdx.x; e < outer * L * inner; e += blockDim.x) {
+    const int l = e % inner, r = e / inner, k2 = r % Q, base = (r / Q) * Q * inner + l;
+    double ax = 0.0, ay = 0.0;
     int t = 0;
-    for (int i = 0; i < L; ++i) {
-      const T w = tws[t];
-      const T v = sl[i];
-      ax += v.x * w.x - v.y * w.y;
-      ay += v.x * w.y + v.y * w.x;
-      t += j;
-      if (t >= L) t -= L;
-      if (t >= L) t %= L;
+    for (int n2 = 0; n2 < Q; ++n2) {
+      const double2 v = s[base + n2 * inner], w = tw[t * P];
+      ax = fma(v.x, w.x, ax);
+      ax = fma(-v.y, w.y, ax);
+      ay = fma(v.x, w.y, ay);
+      ay = fma(v.y, w.x, ay);
+      t += k2;
+      if (t >= Q) t -= Q;
     }
-    x[base_of(line) + (int64_t)j * S] = CT<T>::mk(ax, ay);
+    tmp[e] = make_double2(ax, ay);
+  }
+  __syncthreads();
+  return tmp;
+}
+
+// x[row][g0][.][.] -> transformed along axes 1 and 2 after the phase exp(-i q.r).
+__global__ void __launch_bounds__(256) grid_plane_kernel(double2* __restrict__ x, int64_t rows_per_q, int q0,
+                                                         GridFFTParams p, const double2* __restrict__ ph,
+                                                         const double2* __restrict__ dtw, int P1, int P2, int two) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int n1 = p.n[1], n2 = p.n[2], np = n1 * n2;
+  double2* s = reinterpret_cast<double2*>(smem_raw);
+  double2* tmp = two ? s + np : s;
+  double2 *t1 = s + (two ? 2 : 1) * np, *t2 = t1 + 64, *f1 = t2 + 64, *f2 = f1 + 64;
+  const int64_t blk = blockIdx.x;
+  const int g0 = (int)(blk % p.n[0]);
+  const int64_t row = blk / p.n[0];
+  const int q = q0 + (int)(row / rows_per_q);
+  const int m2 = q % p.kmesh[2], m1 = (q / p.kmesh[2]) % p.kmesh[1], m0 = q / (p.kmesh[1] * p.kmesh[2]);
+  double2* xp = x + blk * np;
+  for (int t = threadIdx.x; t < 64; t += blockDim.x) {
+    t1[t] = dtw[64 + t];
+    t2[t] = dtw[128 + t];
+    f1[t] = cmul(ph[m0 * 64 + g0], ph[1024 + m1 * 64 + t]);
+    f2[t] = ph[2048 + m2 * 64 + t];
+  }
+  __syncthreads();
+  for (int e = threadIdx.x; e < np; e += blockDim.x) s[e] = cmul(xp[e], cmul(f1[e / n2], f2[e % n2]));
+  __syncthreads();
+  double2* a = grid_lines(s, tmp, n1, 1, n2, P2, t2);
+  double2* b = a == s ? tmp : s;
+  a = grid_lines(a, b, 1, n2, n1, P1, t1);
+  const int Q1 = n1 / P1, Q2 = n2 / P2;
+  for (int e = threadIdx.x; e < np; e += blockDim.x) {
+    const int k1 = e / n2, k2 = e % n2;
+    xp[e] = a[((k1 % P1) * Q1 + k1 / P1) * n2 + (k2 % P2) * Q2 + k2 / P2];
+  }
+}
+
+// Axis 0 of 32 columns of a row, times the weight.
+__global__ void __launch_bounds__(256) grid_axis0_kernel(double2* __restrict__ x, int64_t rows_per_q, GridFFTParams p,
+                                                         const double* __restrict__ sw, const double2* __restrict__ dtw,
+                                                         int P0, int two) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  constexpr int C = 32;
+  const int n0 = p.n[0], np = p.n[1] * p.n[2];
+  double2* s = reinterpret_cast<double2*>(smem_raw);
+  double2* tmp = two ? s + n0 * C : s;
+  double2* t0 = s + (two ? 2 : 1) * n0 * C;
+  const int nch = (np + C - 1) / C, c0 = (int)(blockIdx.x % nch) * C, nc = min(C, np - c0);
+  const int64_t row = blockIdx.x / nch;
+  double2* xr = x + row * n0 * np + c0;
+  const double* w = sw + (row / rows_per_q) * n0 * np + c0;
+  for (int t = threadIdx.x; t < 64; t += blockDim.x) t0[t] = dtw[t];
+  for (int e = threadIdx.x; e < n0 * C; e += blockDim.x) {
+    const int g = e / C, c = e % C;
+    s[e] = c < nc ? xr[(int64_t)g * np + c] : make_double2(0.0, 0.0);
+  }
+  __syncthreads();
+  const double2* a = grid_lines(s, tmp, 1, C, n0, P0, t0);
+  const int Q0 = n0 / P0;
+  for (int e = threadIdx.x; e < n0 * C; e += blockDim.x) {
+    const int k = e / C, c = e % C;
+    if (c >= nc) continue;
+    const double2 v = a[((k % P0) * Q0 + k / P0) * C + c];
+    const double f = w[(int64_t)k * np + c];
+    xr[(int64_t)k * np + c] = make_double2(v.x * f, v.y * f);
   }
 }
 
@@ -822,7 +1035,7 @@ __global__ void coulomb_weight_kernel(T* __restrict__ x, int64_t rows_per_q, int
 
 template <typename T>
 cudaError_t grid_fft_launch(cudaStream_t st, T* x, int rows_per_q, int q0, int nq, const CellDev& c,
-                            const double2* dtw, void* work) {
+                            const double2* dtw, void* work, bool radix = false) {
   GridFFTParams p;
   for (int a = 0; a < 3; ++a) {
     p.n[a] = c.mesh[a];
@@ -840,24 +1053,43 @@ cudaError_t grid_fft_launch(cudaStream_t st, T* x, int rows_per_q, int q0, int n
   double* sw = reinterpret_cast<double*>(ph + 3 * 16 * 64);   // nq x ng weight table
   phase_table_kernel<<<12, 256, 0, st>>>(p, ph);
   count_launch();
-  phase_kernel<T><<<nb, 256, 0, st>>>(x, rows_per_q, q0, nq, p, ph);
-  count_launch();
+  if (!radix) {
+    phase_kernel<T><<<nb, 256, 0, st>>>(x, rows_per_q, q0, nq, p, ph);
+    count_launch();
+  }
   {
     int nbw = (int)(((int64_t)nq * ng + 255) / 256);
     if (nbw > 152 * 64) nbw = 152 * 64;
     weight_table_kernel<<<nbw, 256, 0, st>>>(q0, nq, p, sw);
     count_launch();
   }
+  if constexpr (std::is_same<T, double2>::value) {
+    if (radix) {
+      const int n0 = c.mesh[0], np = c.mesh[1] * c.mesh[2];
+      const int P0 = radix_p(n0), P1 = radix_p(c.mesh[1]), P2 = radix_p(c.mesh[2]);
+      const int two = c.mesh[1] / P1 > kRadMax || c.mesh[2] / P2 > kRadMax, two0 = n0 / P0 > kRadMax;
+      const size_t s1 = ((size_t)np * (1 + two) + 256) * sizeof(double2), s0 = ((size_t)n0 * 32 * (1 + two0) + 64) * sizeof(double2);
+      const int64_t planes = nrows * n0, chunks = nrows * ((np + 31) / 32);
+      if (planes > 2147483647LL || chunks > 2147483647LL) return cudaErrorInvalidValue;
+      cudaError_t e = cudaFuncSetAttribute(grid_plane_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s1);
+      if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(grid_axis0_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s0);
+      if (e != cudaSuccess) return e;
+      grid_plane_kernel<<<(unsigned)planes, 256, s1, st>>>(x, rows_per_q, q0, p, ph, dtw, P1, P2, two);
+      count_launch();
+      grid_axis0_kernel<<<(unsigned)chunks, 256, s0, st>>>(x, rows_per_q, p, sw, dtw, P0, two0);
+      count_launch();
+      return cudaGetLastError();
+    }
+  }
   for (int a = 2; a >= 0; --a) {
     const int L = c.mesh[a];
     if (L == 1) continue;
     const int64_t S = (a == 2) ? 1 : (a == 1 ? c.mesh[2] : (int64_t)c.mesh[1] * c.mesh[2]);
-    int lpb = 256 / L;
-    if (lpb < 1) lpb = 1;
-    const int64_t total_lines = nrows * (ng / L);
-    const int64_t nblk = (total_lines + lpb - 1) / lpb;
-    const size_t smem = (size_t)lpb * L * sizeof(T) + 64 * sizeof(double2);
-    grid_axis_kernel<T><<<(unsigned)nblk, 256, smem, st>>>(x, nrows, ng, L, S, lpb, dtw + a * 64);
+    const int groups = 256 / L, lpb = kAxisLines * groups;
+    const int64_t total_lines = nrows * (ng / L), nblk = (total_lines + lpb - 1) / lpb;
+    const size_t smem = (size_t)lpb * (L | 1) * sizeof(T) + 64 * sizeof(double2);
+    grid_axis_kernel<T><<<(unsigned)nblk, 256, smem, st>>>(x, total_lines, ng, L, (int)S, groups, dtw + a * 64);
     count_launch();
   }
   coulomb_weight_kernel<T><<<nb, 256, 0, st>>>(x, rows_per_q, nq, ng, sw);
@@ -1006,8 +1238,9 @@ cudaError_t pair_products_real_f(cudaStream_t st, const float2* t, int nk, int n
 }
 
 cudaError_t kdft_cols(cudaStream_t st, double2* data, int64_t ncol, KMesh km, int s1, int s2,
-                      int mode, double scale) {
-  return kdft_launch<double2>(st, data, ncol, km, s1, s2, mode, scale);
+                      int mode, double scale, bool radix) {
+  return radix ? kdft_launch<double2, double2, true>(st, data, ncol, km, s1, s2, mode, scale)
+               : kdft_launch<double2>(st, data, ncol, km, s1, s2, mode, scale);
 }
 cudaError_t kdft_cols_f(cudaStream_t st, float2* data, int64_t ncol, KMesh km, int s1, int s2,
                         int mode, float scale) {
@@ -1017,8 +1250,8 @@ size_t grid_coulomb_work_bytes(int nq, const CellDev& c) {
   return 3 * 16 * 64 * sizeof(double2) + (size_t)nq * c.mesh[0] * c.mesh[1] * c.mesh[2] * sizeof(double);
 }
 cudaError_t grid_coulomb_fft(cudaStream_t st, double2* x, int rows_per_q, int q0, int nq,
-                             const CellDev& c, const double2* dtw, void* work) {
-  return grid_fft_launch<double2>(st, x, rows_per_q, q0, nq, c, dtw, work);
+                             const CellDev& c, const double2* dtw, void* work, bool radix) {
+  return grid_fft_launch<double2>(st, x, rows_per_q, q0, nq, c, dtw, work, radix);
 }
 cudaError_t grid_coulomb_fft_f(cudaStream_t st, float2* x, int rows_per_q, int q0, int nq,
                                const CellDev& c, const double2* dtw, void* work) {
