@@ -14,6 +14,7 @@
 #include <cuda_runtime.h>
 
 #include <cmath>
+#include <cstdint>
 
 namespace isdf {
 
@@ -24,8 +25,33 @@ struct ffloat {
   __host__ __device__ __forceinline__ ffloat(int v) : hi((float)v), lo(0.f) {}
   __host__ __device__ __forceinline__ ffloat(float v) : hi(v), lo(0.f) {}
   // from double: the float nearest to v and the float nearest to the rest
-  __host__ __device__ __forceinline__ ffloat(double v) : hi((float)v), lo((float)(v - (double)(float)v)) {}
-  __host__ __device__ __forceinline__ double to_double() const { return (double)hi + (double)lo; }
+  // (on the device in integer arithmetic where v's exponent is inside the range that keeps both
+  // parts normal: conversions run on the FP64 pipe, at two a clock and SM)
+  __host__ __device__ __forceinline__ ffloat(double v) {
+#ifdef __CUDA_ARCH__
+    const uint32_t h = (uint32_t)__double2hiint(v), l = (uint32_t)__double2loint(v), e = (h >> 20) & 0x7ffu;
+    if (e - 953u < 190u) {  // 2^-70 <= |v| < 2^120
+      const uint32_t f = (((h & 0x7fffffffu) - (896u << 20)) << 3) | (l >> 29), rest = l & 0x1fffffffu;
+      const uint32_t up = rest + (f & 1u) > 0x10000000u;  // to nearest, ties to even
+      const int r = (int)rest - (int)(up << 29);
+      hi = __uint_as_float((f + up) | (h & 0x80000000u));
+      lo = __int2float_rn((h >> 31) ? -r : r) * __uint_as_float((e - 948u) << 23);  // r 2^(e - 1075)
+      return;
+    }
+#endif
+    hi = (float)v;
+    lo = (float)(v - (double)hi);
+  }
+  __host__ __device__ __forceinline__ double to_double() const { return widen(hi) + widen(lo); }
+  // (double)f, a normal f by its bits
+  __host__ __device__ static __forceinline__ double widen(float f) {
+#ifdef __CUDA_ARCH__
+    const uint32_t u = __float_as_uint(f);
+    if (((u >> 23) & 0xffu) - 1u < 254u)
+      return __hiloint2double((int)((((u & 0x7fffffffu) >> 3) + (896u << 20)) | (u & 0x80000000u)), (int)(u << 29));
+#endif
+    return (double)f;
+  }
 };
 
 // complex float-float (16 bytes, the size of a complex128)
