@@ -365,6 +365,7 @@ __global__ void __launch_bounds__(256) rsplit_kernel(BView B, int64_t j0, int nq
 // written as complex64 (mixed) or complex128 (FP64_TC); eri may be NULL, and
 // gamma NULL skips the traces.  Per-block partials go to part[blk] (J) and
 // part[gridDim.x + blk] (K); the fixed grid keeps the sums reproducible.
+// part[2 gridDim.x].x: whether gamma is Hermitian (gamma_herm_kernel).
 __device__ __forceinline__ ffloat ep_ff(const float* __restrict__ wh, const float* __restrict__ wl,
                                         const int* __restrict__ tile_of, int nt, int64_t i, int64_t j,
                                         const int* __restrict__ row_exp, ffloat sc) {
@@ -379,66 +380,138 @@ __device__ __forceinline__ ffloat ep_ff(const float* __restrict__ wh, const floa
   return ff_ldexp(v, -(row_exp[i] + row_exp[j])) * sc;
 }
 
-__device__ __forceinline__ void put_c(float2* e, double re, double im) { *e = make_float2((float)re, (float)im); }
-__device__ __forceinline__ void put_c(double2* e, double re, double im) { *e = make_double2(re, im); }
-
 struct BlockVals {
   double U, X, Y, Z;
 };
 
-// ERIs and trace terms of the block (row orbit (p, q), column orbit (x, y)); a
-// diagonal orbit has q == p (resp. y == x).
+// Trace terms of the block (row orbit (p, q), column orbit (x, y)); a diagonal orbit has q == p
+// (resp. y == x).  (r1, i1) = (pq|yx), (r2, i2) = (pq|xy) as in the table above.
+__device__ __forceinline__ void block_traces(const double2* __restrict__ g, int nf, int p, int q, int x, int y,
+                                             const BlockVals& b, double r1, double i1, double r2, double i2,
+                                             double& aj, double& ak) {
+  auto gm = [&](int i, int j) { return g[(int64_t)i * nf + j]; };
+  if (p != q && x != y) {
+    const double2 A = gm(p, q), B = gm(y, x);
+    aj += b.U * A.x * B.x - b.Z * A.y * B.y + b.X * A.x * B.y - b.Y * A.y * B.x;
+    const double2 w1 = cmul(gm(p, x), gm(y, q)), w2 = cmul(gm(p, y), gm(x, q));
+    ak += 2.0 * (w1.x * r1 - w1.y * i1 + w2.x * r2 - w2.y * i2);
+  } else if (p != q) {
+    const double2 A = gm(p, q), w = cmul(gm(p, x), gm(x, q));
+    aj += gm(x, x).x * (A.x * b.U - A.y * b.Y);
+    ak += 2.0 * (w.x * r1 - w.y * i1);
+  } else if (x != y) {
+    const double2 B = gm(y, x), w = cmul(gm(p, x), gm(y, p));
+    aj += gm(p, p).x * (B.x * b.U + B.y * b.X);
+    ak += 2.0 * (w.x * r1 - w.y * i1);
+  } else {
+    const double2 w = gm(p, x);
+    aj += gm(p, p).x * gm(x, x).x * b.U;
+    ak += (w.x * w.x + w.y * w.y) * b.U;
+  }
+}
+
+__device__ __forceinline__ void put_part(float& o, double v) { o = ffloat(v).hi; }
+__device__ __forceinline__ void put_part(double& o, double v) { o = v; }
+
+// ERIs and trace terms of the block (o1, o2) and, with mirror, of (o2, o1).  The FP64 pipe bounds
+// this (two operations a clock and SM): the mirrored block has the same four numbers up to
+// conjugation, so each is formed and narrowed once; and for a Hermitian gamma its trace terms
+// equal the block's (A' = conj B, B' = conj A; the exchange products conjugate along with
+// their integrals), so they count twice instead of being formed twice.
 template <typename TO>
 __device__ __forceinline__ void emit_block(TO* __restrict__ eri, const double2* __restrict__ g, int nf, int p,
-                                           int q, int x, int y, const BlockVals& b, double& aj, double& ak) {
+                                           int q, int x, int y, const BlockVals& b, bool mirror, bool herm,
+                                           double& aj, double& ak) {
   const bool pr = p != q, pc = x != y;
-  auto at = [&](int i0, int i1, int i2, int i3) { return eri + (((int64_t)i0 * nf + i1) * nf + i2) * nf + i3; };
-  auto gm = [&](int i, int j) { return g[(int64_t)i * nf + j]; };
+  double r1, i1, r2 = 0.0, i2 = 0.0;
   if (pr && pc) {
-    const double r1 = 0.25 * (b.U + b.Z), i1 = 0.25 * (b.Y - b.X), r2 = 0.25 * (b.U - b.Z), i2 = 0.25 * (b.X + b.Y);
-    if (eri) {
-      put_c(at(p, q, y, x), r1, i1);
-      put_c(at(p, q, x, y), r2, i2);
-      put_c(at(q, p, y, x), r2, -i2);
-      put_c(at(q, p, x, y), r1, -i1);
-    }
-    if (g) {
-      const double2 A = gm(p, q), B = gm(y, x);
-      aj += b.U * A.x * B.x - b.Z * A.y * B.y + b.X * A.x * B.y - b.Y * A.y * B.x;
-      const double2 w1 = cmul(gm(p, x), gm(y, q)), w2 = cmul(gm(p, y), gm(x, q));
-      ak += 2.0 * (w1.x * r1 - w1.y * i1 + w2.x * r2 - w2.y * i2);
-    }
-  } else if (pr) {
-    const double r = 0.5 * b.U, im = 0.5 * b.Y;
-    if (eri) {
-      put_c(at(p, q, x, x), r, im);
-      put_c(at(q, p, x, x), r, -im);
-    }
-    if (g) {
-      const double2 A = gm(p, q);
-      aj += gm(x, x).x * (A.x * b.U - A.y * b.Y);
-      const double2 w = cmul(gm(p, x), gm(x, q));
-      ak += 2.0 * (w.x * r - w.y * im);
-    }
-  } else if (pc) {
-    const double r = 0.5 * b.U, im = -0.5 * b.X;
-    if (eri) {
-      put_c(at(p, p, y, x), r, im);
-      put_c(at(p, p, x, y), r, -im);
-    }
-    if (g) {
-      const double2 B = gm(y, x);
-      aj += gm(p, p).x * (B.x * b.U + B.y * b.X);
-      const double2 w = cmul(gm(p, x), gm(y, p));
-      ak += 2.0 * (w.x * r - w.y * im);
-    }
+    r1 = 0.25 * (b.U + b.Z), i1 = 0.25 * (b.Y - b.X), r2 = 0.25 * (b.U - b.Z), i2 = 0.25 * (b.X + b.Y);
+  } else if (pr || pc) {
+    r1 = 0.5 * b.U, i1 = pr ? 0.5 * b.Y : -0.5 * b.X;
   } else {
-    if (eri) put_c(at(p, p, x, x), b.U, 0.0);
-    if (g) {
-      const double2 w = gm(p, x);
-      aj += gm(p, p).x * gm(x, x).x * b.U;
-      ak += (w.x * w.x + w.y * w.y) * b.U;
+    r1 = b.U, i1 = 0.0;
+  }
+  if (eri) {
+    auto at = [&](int i0, int i1, int i2, int i3) { return eri + (((int64_t)i0 * nf + i1) * nf + i2) * nf + i3; };
+    auto cj = [](TO v) {
+      v.y = -v.y;
+      return v;
+    };
+    TO z1, z2;
+    put_part(z1.x, r1);
+    put_part(z1.y, i1);
+    if (pr && pc) {
+      put_part(z2.x, r2);
+      put_part(z2.y, i2);
+      *at(p, q, y, x) = z1;
+      *at(p, q, x, y) = z2;
+      *at(q, p, y, x) = cj(z2);
+      *at(q, p, x, y) = cj(z1);
+      if (mirror) {  // (xy|qp) = conj (pq|yx)^(X <-> Y) and so on
+        *at(x, y, q, p) = cj(z1);
+        *at(x, y, p, q) = z2;
+        *at(y, x, q, p) = cj(z2);
+        *at(y, x, p, q) = z1;
+      }
+    } else if (pr) {
+      *at(p, q, x, x) = z1;
+      *at(q, p, x, x) = cj(z1);
+      if (mirror) {
+        *at(x, x, q, p) = cj(z1);
+        *at(x, x, p, q) = z1;
+      }
+    } else if (pc) {
+      *at(p, p, y, x) = z1;
+      *at(p, p, x, y) = cj(z1);
+      if (mirror) {
+        *at(x, y, p, p) = cj(z1);
+        *at(y, x, p, p) = z1;
+      }
+    } else {
+      *at(p, p, x, x) = z1;
+      if (mirror) *at(x, x, p, p) = z1;
     }
+  }
+  if (!g) return;
+  double tj = 0.0, tk = 0.0;
+  block_traces(g, nf, p, q, x, y, b, r1, i1, r2, i2, tj, tk);
+  if (mirror && herm) {
+    tj += tj;
+    tk += tk;
+  } else if (mirror) {
+    block_traces(g, nf, x, y, p, q, BlockVals{b.U, b.Y, b.X, b.Z}, r1, -i1, r2, i2, tj, tk);
+  }
+  aj += tj;
+  ak += tk;
+}
+
+// flag = gamma is Hermitian to 2^-44 of its mean modulus, the rounding of a C n C^H (one block)
+__global__ void __launch_bounds__(1024) gamma_herm_kernel(const double2* __restrict__ g, int nf,
+                                                          double2* __restrict__ flag) {
+  __shared__ double sm[32], sd[32];
+  double m = 0.0, d = 0.0;
+  for (int e = threadIdx.x; e < nf * nf; e += blockDim.x) {
+    const double2 u = g[e], v = g[(e % nf) * nf + e / nf];
+    m += fabs(u.x) + fabs(u.y);
+    d = fmax(d, fabs(u.x - v.x) + fabs(u.y + v.y));
+    if (!(fabs(u.x) + fabs(u.y) <= 1e300)) d = INFINITY;
+  }
+  m /= (double)nf * nf;
+  for (int o = 16; o; o >>= 1) {
+    m += __shfl_xor_sync(0xffffffffu, m, o);
+    d = fmax(d, __shfl_xor_sync(0xffffffffu, d, o));
+  }
+  if ((threadIdx.x & 31) == 0) {
+    sm[threadIdx.x >> 5] = m;
+    sd[threadIdx.x >> 5] = d;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < 32; ++w) {
+      sm[0] += sm[w];
+      sd[0] = fmax(sd[0], sd[w]);
+    }
+    *flag = make_double2(sd[0] <= sm[0] * 0x1p-44 ? 1.0 : 0.0, 0.0);
   }
 }
 
@@ -453,6 +526,7 @@ __global__ void __launch_bounds__(256) syrk_eri_kernel(const float* __restrict__
   const int nch = (no + 255) / 256;
   const int64_t ntask = (int64_t)no * nch;
   const ffloat sc(scale);
+  const bool herm = gam && part[2 * gridDim.x].x != 0.0;
   double aj = 0.0, ak = 0.0;
   for (int64_t task = blockIdx.x; task < ntask; task += gridDim.x) {
     const int o2 = (int)(task / nch), o1 = (int)(task % nch) * 256 + (int)threadIdx.x;
@@ -471,8 +545,7 @@ __global__ void __launch_bounds__(256) syrk_eri_kernel(const float* __restrict__
       b.U += ldexp(corr[u1], -2 * row_exp[u1]) * scale;
       if (pr) b.Z += ldexp(corr[u1 + 1], -2 * row_exp[u1 + 1]) * scale;
     }
-    emit_block<TO>(eri, gam, nf, r.x, r.y, c.x, c.y, b, aj, ak);
-    if (o1 != o2) emit_block<TO>(eri, gam, nf, c.x, c.y, r.x, r.y, BlockVals{b.U, b.Y, b.X, b.Z}, aj, ak);
+    emit_block<TO>(eri, gam, nf, r.x, r.y, c.x, c.y, b, o1 != o2, herm, aj, ak);
   }
   if (!gam) return;
   __shared__ double sj[256], sk[256];
@@ -1062,7 +1135,7 @@ cudaError_t syrk_tc_mma(cudaStream_t st, void* split, int64_t n2, int nq, int64_
 }
 
 constexpr int kEriBlocks = 152 * 16;  // fixed grid of the fused finish (reproducible traces)
-size_t syrk_tc_eri_part_count() { return 2 * (size_t)kEriBlocks; }
+size_t syrk_tc_eri_part_count() { return 2 * (size_t)kEriBlocks + 1; }  // partials, Hermitian flag
 
 template <typename TO>
 static cudaError_t finish_eri_impl(cudaStream_t st, const void* ws, int ntiles, const int* tile_of_d,
@@ -1073,6 +1146,10 @@ static cudaError_t finish_eri_impl(cudaStream_t st, const void* ws, int ntiles, 
   const float* wh = reinterpret_cast<const float*>(ws);
   const float* wl = wh + (size_t)ntiles * BN * BM;
   const int64_t n2 = (int64_t)nf * nf, nt = (n2 + BM - 1) / BM;
+  if (gamma) {
+    gamma_herm_kernel<<<1, 1024, 0, st>>>(gamma, nf, part + 2 * kEriBlocks);
+    count_launch();
+  }
   syrk_eri_kernel<TO><<<kEriBlocks, 256, 0, st>>>(wh, wl, tile_of_d, (int)nt, orb, nf, row_exp, corr, scale, eri,
                                                   gamma, part);
   count_launch();
