@@ -1,17 +1,25 @@
 // Batched complex GEMM on the SIMT pipes (FP64 and FP32).
 //
 // C_b = alpha * op(A_b) * op(B_b) + beta * C_b, row-major, op in {N, T, C, R}.
-// Used for the small-K contractions of the fit (G^k = X^k^* X^k^T, g^k = X^k^* Phi^k,
-// T^k = X^k C^k), the explicit-factor products of the solve, and the FP64 path's
-// Coulomb and fragment contractions (Eqs. 4-6, 19-20).
+// FP64: the products whose arithmetic the mixed and FP64_TC paths fix to FMA chains (Pi and
+// xi = W eta of the fit, V_xi and L of FP64_TC), and inner sizes too short for the tensor-core
+// product.  FP32: T^k = X^k C^k of the mixed path.
 //
 // Tiling: 64 x 64 output tile per 256-thread block, each thread owns a 4 x 4
 // sub-tile spread with stride 16 (conflict-free shared reads), K staged 8 (FP64)
 // or 16 (FP32) at a time through shared memory.
 //
+// The FP64 form is bound by the FP64 pipe (2 FMA per clock and SM: a full tile takes 4.2 us per
+// unit of K), so that a tile whose rows or columns end early, at the matrix or at its rank, forms
+// its 16-row and 16-column parts up to there only: a rank just above a multiple of 64 had paid
+// for a whole further tile (FP64_TC fit and metric at Nk = 216, 24^3 grid: 818 -> 675 ms where the
+// rank is above 128, 501 ms as before where it is 125).
+//
 // FP32 accumulation is compensated: each K tile is summed in FP32, then folded
 // into a float-float running sum with TwoSum (Knuth), so the rounding error is
 // that of a 16-term FP32 sum plus ~2^-48 of the total instead of growing with K.
+#include <type_traits>
+
 #include "common.cuh"
 
 namespace isdf {
@@ -93,6 +101,8 @@ __global__ void __launch_bounds__(256, 2) gemm_kernel(char opA, char opB, int m,
   if (brow) brow += b * sIdx;
   int kend = lowerA ? min(k, m0 + BM) : k;
   if (krank) kend = krank[b] > m0 ? min(kend, krank[b]) : 0;
+  // 16-row and 16-column parts of the tile that hold something
+  const int nrow = min(4, ((krank ? min(m, krank[b]) : m) - m0 + 15) / 16), ncol = min(4, (n - n0 + 15) / 16);
   const bool aT = (opA == 'T' || opA == 'C');
   const bool aC = (opA == 'C' || opA == 'R');
   const bool bT = (opB == 'T' || opB == 'C');
@@ -201,19 +211,26 @@ __global__ void __launch_bounds__(256, 2) gemm_kernel(char opA, char opB, int m,
     } else {
       // rows m0 + 16 i .. + 15 of a lower-triangular op(A) end at k = m0 + 16 i + 15
       const int lo_i = lowerA && k0 > m0 ? (k0 - m0) / 16 : 0;
+      auto step = [&](auto whole) {  // all four column parts, or the first ncol
 #pragma unroll
-      for (int kk = 0; kk < BK; ++kk) {
-        T bb[4];
+        for (int kk = 0; kk < BK; ++kk) {
+          T bb[4];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) bb[j] = Bs[kk][tx + 16 * j];
+          for (int j = 0; j < 4; ++j) bb[j] = Bs[kk][tx + 16 * j];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          if (i < lo_i) continue;
-          const T a = As[kk][ty + 16 * i];
+          for (int i = 0; i < 4; ++i) {
+            if (i < lo_i || i >= nrow) continue;
+            const T a = As[kk][ty + 16 * i];
 #pragma unroll
-          for (int j = 0; j < 4; ++j) cfma_t(acc[i][j], a, bb[j]);
+            for (int j = 0; j < 4; ++j)
+              if (whole.value || j < ncol) cfma_t(acc[i][j], a, bb[j]);
+          }
         }
-      }
+      };
+      if (ncol == 4)
+        step(std::true_type{});
+      else
+        step(std::false_type{});
     }
     __syncthreads();
   }

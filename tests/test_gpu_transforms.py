@@ -61,3 +61,9 @@ def test_metric_on_edge_meshes(cuda, lib_built, kmesh, mesh, prec):
 def test_factorisation_sizes(cuda, lib_built, n_p):
     """tau = 1e-6 keeps more pivots than one pass of the factorisation holds; the bound scales with it."""
     _check(cuda, _cell((2, 1, 3), (12, 10, 14)), n_p, 0, tau=1e-6, tol=1e-5)
+
+
+@pytest.mark.parametrize("n_p", [1, 16, 17, 63, 65, 79, 81, 130])
+def test_partial_tiles_of_the_fixed_chains(cuda, lib_built, n_p):
+    """xi, V_xi and L of FP64_TC on 64 x 64 tiles of which only some 16-row and 16-column parts are formed."""
+    _check(cuda, _cell((2, 1, 3), (12, 10, 14)), n_p, 2, tau=1e-6, tol=1e-5)
