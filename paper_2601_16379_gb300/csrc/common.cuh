@@ -151,9 +151,7 @@ size_t grid_coulomb_work_bytes(int nq, const CellDev& c);
 // radix: two passes and mixed-radix axes, else the direct sums in their fixed order.
 cudaError_t grid_coulomb_fft(cudaStream_t st, double2* x, int rows_per_q, int q0, int nq,
                              const CellDev& c, const double2* dtw, void* work, bool radix);
-cudaError_t grid_coulomb_fft_f(cudaStream_t st, float2* x, int rows_per_q, int q0, int nq,
-                               const CellDev& c, const double2* dtw, void* work);
-// the same in float-float (FP32 arithmetic, ~2^-44), in place on float-float data
+// the mixed-radix form in float-float (FP32 arithmetic, ~2^-44), in place on float-float data
 cudaError_t grid_coulomb_fft_ff(cudaStream_t st, ffcomplex* x, int rows_per_q, int q0, int nq,
                                 const CellDev& c, const double2* dtw, void* work);
 void grid_twiddles(const int mesh[3], double2* host192);

@@ -779,8 +779,7 @@ __global__ void phase_kernel(T* __restrict__ x, int64_t rows_per_q, int q0, int 
 // A block takes 4 (256 / L) lines; a thread one output j of four of them, so that a twiddle read
 // and its index serve four products and four independent chains run side by side, each in the
 // order of the sum.  The line pitch is odd: threads on consecutive lines hit distinct banks.
-// Bound by its FP32 (float-float) or FP64 operations: 24^3 grid, 64 k-points, 850 rows:
-// 106 -> 79 ms in float-float against one line per thread.
+// Bound by its FP64 operations (the FP64_TC path's form, which keeps the rounding of the direct sum).
 constexpr int kAxisLines = 4;
 template <typename T>
 __global__ void __launch_bounds__(256) grid_axis_kernel(T* __restrict__ x, int64_t total_lines, int ng,
@@ -832,13 +831,16 @@ __global__ void __launch_bounds__(256) grid_axis_kernel(T* __restrict__ x, int64
   }
 }
 
-// ---- the FP64 path's grid transform: two passes over memory and mixed radix.
+// ---- the grid transform of the FP64 path and, in float-float, of the mixed path: two passes over
+// memory and mixed radix.
 // The direct form takes six passes and 6 L FP64 operations per value and axis (2 per clock and
 // SM: 18 of 34 ms of the c2 fit and metric).  Here a block takes one (g1, g2) plane -- phase,
 // axis 2, axis 1 -- and a second kernel axis 0 and the weight.  An axis of length L = P Q goes in two
 // steps of in-register transforms of at most 8 points; other lengths (a prime above 8 in them) by
 // the direct sum over that factor, four FMAs per product.  Measured with the k-transforms: fit and
 // metric of 125 k-points on an 18^3 grid 33.9 -> 18.1 ms, ragged quartets 20.5 -> 13.0.
+// In float-float (as accurate as the direct sum of L terms, and FP32-bound there): fit and metric of 64
+// k-points on a 32^3 grid 527 -> 463 ms.
 // FP64_TC keeps the direct sums: see isdf_fit_zeta.
 constexpr int kRadMax = 8;
 __host__ __device__ inline int radix_p(int L) {  // P: both factors <= 8 if possible, else the largest factor <= 8
@@ -853,22 +855,27 @@ __host__ __device__ inline int radix_p(int L) {  // P: both factors <= 8 if poss
   return best;
 }
 
-template <int N>
-__device__ __forceinline__ void grid_small(double2* s, int base, int step, const double2* tw, int tstep) {
-  double vr[N], vi[N], wc[N], ws[N];
+__device__ __forceinline__ double mac(double a, double b, double c) { return fma(a, b, c); }
+__device__ __forceinline__ ffloat mac(ffloat a, ffloat b, ffloat c) { return c + a * b; }
+
+template <int N, typename T>
+__device__ __forceinline__ void grid_small(T* s, int base, int step, const T* tw, int tstep) {
+  using R = typename CT<T>::R;
+  R vr[N], vi[N], wc[N], ws[N];
 #pragma unroll
   for (int i = 0; i < N; ++i) {
-    const double2 v = s[base + i * step], w = tw[i * tstep];
+    const T v = s[base + i * step], w = tw[i * tstep];
     vr[i] = v.x;
     vi[i] = v.y;
     wc[i] = w.x;
     ws[i] = w.y;
   }
-  Dft<double, N, 1, N>::run(vr, vi, wc, ws);
+  Dft<R, N, 1, N>::run(vr, vi, wc, ws);
 #pragma unroll
-  for (int i = 0; i < N; ++i) s[base + i * step] = make_double2(vr[i], vi[i]);
+  for (int i = 0; i < N; ++i) s[base + i * step] = CT<T>::mk(vr[i], vi[i]);
 }
-__device__ __forceinline__ void grid_small_any(int n, double2* s, int base, int step, const double2* tw, int tstep) {
+template <typename T>
+__device__ __forceinline__ void grid_small_any(int n, T* s, int base, int step, const T* tw, int tstep) {
   switch (n) {
     case 2: grid_small<2>(s, base, step, tw, tstep); break;
     case 3: grid_small<3>(s, base, step, tw, tstep); break;
@@ -884,14 +891,16 @@ __device__ __forceinline__ void grid_small_any(int n, double2* s, int base, int 
 // Transform of all lines (fixed o, l) of s[(o L + i) inner + l], o < outer, l < inner, along i; tw: the L-th
 // roots.  The result for frequency k sits at i = (k mod P) (L / P) + k / P.  tmp: as large as s, used
 // (and returned as the result) where L / P > 8.
-__device__ double2* grid_lines(double2* s, double2* tmp, int outer, int inner, int L, int P, const double2* tw) {
+template <typename T>
+__device__ T* grid_lines(T* s, T* tmp, int outer, int inner, int L, int P, const T* tw) {
+  using R = typename CT<T>::R;
   const int Q = L / P;
   if (P > 1) {
     for (int e = threadIdx.x; e < outer * Q * inner; e += blockDim.x) {
       const int l = e % inner, r = e / inner, n2 = r % Q, o = r / Q, base = (o * L + n2) * inner + l;
       grid_small_any(P, s, base, Q * inner, tw, Q);
       for (int k1 = 1; k1 < P; ++k1) {
-        double2* v = s + base + k1 * Q * inner;
+        T* v = s + base + k1 * Q * inner;
         if (n2) *v = cmul(*v, tw[(n2 * k1) % L]);
       }
     }
@@ -908,49 +917,52 @@ __device__ double2* grid_lines(double2* s, double2* tmp, int outer, int inner, i
   }
   for (int e = threadIdx.x; e < outer * L * inner; e += blockDim.x) {
     const int l = e % inner, r = e / inner, k2 = r % Q, base = (r / Q) * Q * inner + l;
-    double ax = 0.0, ay = 0.0;
+    R ax = 0.0, ay = 0.0;
     int t = 0;
     for (int n2 = 0; n2 < Q; ++n2) {
-      const double2 v = s[base + n2 * inner], w = tw[t * P];
-      ax = fma(v.x, w.x, ax);
-      ax = fma(-v.y, w.y, ax);
-      ay = fma(v.x, w.y, ay);
-      ay = fma(v.y, w.x, ay);
+      const T v = s[base + n2 * inner], w = tw[t * P];
+      ax = mac(v.x, w.x, ax);
+      ax = mac(-v.y, w.y, ax);
+      ay = mac(v.x, w.y, ay);
+      ay = mac(v.y, w.x, ay);
       t += k2;
       if (t >= Q) t -= Q;
     }
-    tmp[e] = make_double2(ax, ay);
+    tmp[e] = CT<T>::mk(ax, ay);
   }
   __syncthreads();
   return tmp;
 }
 
 // x[row][g0][.][.] -> transformed along axes 1 and 2 after the phase exp(-i q.r).
-__global__ void __launch_bounds__(256) grid_plane_kernel(double2* __restrict__ x, int64_t rows_per_q, int q0,
+template <typename T>
+__global__ void __launch_bounds__(256) grid_plane_kernel(T* __restrict__ x, int64_t rows_per_q, int q0,
                                                          GridFFTParams p, const double2* __restrict__ ph,
                                                          const double2* __restrict__ dtw, int P1, int P2, int two) {
+  using R = typename CT<T>::R;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int n1 = p.n[1], n2 = p.n[2], np = n1 * n2;
-  double2* s = reinterpret_cast<double2*>(smem_raw);
-  double2* tmp = two ? s + np : s;
-  double2 *t1 = s + (two ? 2 : 1) * np, *t2 = t1 + 64, *f1 = t2 + 64, *f2 = f1 + 64;
+  T* s = reinterpret_cast<T*>(smem_raw);
+  T* tmp = two ? s + np : s;
+  T *t1 = s + (two ? 2 : 1) * np, *t2 = t1 + 64, *f1 = t2 + 64, *f2 = f1 + 64;
   const int64_t blk = blockIdx.x;
   const int g0 = (int)(blk % p.n[0]);
   const int64_t row = blk / p.n[0];
   const int q = q0 + (int)(row / rows_per_q);
   const int m2 = q % p.kmesh[2], m1 = (q / p.kmesh[2]) % p.kmesh[1], m0 = q / (p.kmesh[1] * p.kmesh[2]);
-  double2* xp = x + blk * np;
+  T* xp = x + blk * np;
   for (int t = threadIdx.x; t < 64; t += blockDim.x) {
-    t1[t] = dtw[64 + t];
-    t2[t] = dtw[128 + t];
-    f1[t] = cmul(ph[m0 * 64 + g0], ph[1024 + m1 * 64 + t]);
-    f2[t] = ph[2048 + m2 * 64 + t];
+    auto get = [](const double2& v) { return CT<T>::mk((R)v.x, (R)v.y); };
+    t1[t] = get(dtw[64 + t]);
+    t2[t] = get(dtw[128 + t]);
+    f1[t] = cmul(get(ph[m0 * 64 + g0]), get(ph[1024 + m1 * 64 + t]));
+    f2[t] = get(ph[2048 + m2 * 64 + t]);
   }
   __syncthreads();
   for (int e = threadIdx.x; e < np; e += blockDim.x) s[e] = cmul(xp[e], cmul(f1[e / n2], f2[e % n2]));
   __syncthreads();
-  double2* a = grid_lines(s, tmp, n1, 1, n2, P2, t2);
-  double2* b = a == s ? tmp : s;
+  T* a = grid_lines(s, tmp, n1, 1, n2, P2, t2);
+  T* b = a == s ? tmp : s;
   a = grid_lines(a, b, 1, n2, n1, P1, t1);
   const int Q1 = n1 / P1, Q2 = n2 / P2;
   for (int e = threadIdx.x; e < np; e += blockDim.x) {
@@ -960,33 +972,35 @@ __global__ void __launch_bounds__(256) grid_plane_kernel(double2* __restrict__ x
 }
 
 // Axis 0 of 32 columns of a row, times the weight.
-__global__ void __launch_bounds__(256) grid_axis0_kernel(double2* __restrict__ x, int64_t rows_per_q, GridFFTParams p,
+template <typename T>
+__global__ void __launch_bounds__(256) grid_axis0_kernel(T* __restrict__ x, int64_t rows_per_q, GridFFTParams p,
                                                          const double* __restrict__ sw, const double2* __restrict__ dtw,
                                                          int P0, int two) {
+  using R = typename CT<T>::R;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   constexpr int C = 32;
   const int n0 = p.n[0], np = p.n[1] * p.n[2];
-  double2* s = reinterpret_cast<double2*>(smem_raw);
-  double2* tmp = two ? s + n0 * C : s;
-  double2* t0 = s + (two ? 2 : 1) * n0 * C;
+  T* s = reinterpret_cast<T*>(smem_raw);
+  T* tmp = two ? s + n0 * C : s;
+  T* t0 = s + (two ? 2 : 1) * n0 * C;
   const int nch = (np + C - 1) / C, c0 = (int)(blockIdx.x % nch) * C, nc = min(C, np - c0);
   const int64_t row = blockIdx.x / nch;
-  double2* xr = x + row * n0 * np + c0;
+  T* xr = x + row * n0 * np + c0;
   const double* w = sw + (row / rows_per_q) * n0 * np + c0;
-  for (int t = threadIdx.x; t < 64; t += blockDim.x) t0[t] = dtw[t];
+  for (int t = threadIdx.x; t < 64; t += blockDim.x) t0[t] = CT<T>::mk((R)dtw[t].x, (R)dtw[t].y);
   for (int e = threadIdx.x; e < n0 * C; e += blockDim.x) {
     const int g = e / C, c = e % C;
-    s[e] = c < nc ? xr[(int64_t)g * np + c] : make_double2(0.0, 0.0);
+    s[e] = c < nc ? xr[(int64_t)g * np + c] : CT<T>::mk(0.0, 0.0);
   }
   __syncthreads();
-  const double2* a = grid_lines(s, tmp, 1, C, n0, P0, t0);
+  const T* a = grid_lines(s, tmp, 1, C, n0, P0, t0);
   const int Q0 = n0 / P0;
   for (int e = threadIdx.x; e < n0 * C; e += blockDim.x) {
     const int k = e / C, c = e % C;
     if (c >= nc) continue;
-    const double2 v = a[((k % P0) * Q0 + k / P0) * C + c];
-    const double f = w[(int64_t)k * np + c];
-    xr[(int64_t)k * np + c] = make_double2(v.x * f, v.y * f);
+    const T v = a[((k % P0) * Q0 + k / P0) * C + c];
+    const R f = (R)w[(int64_t)k * np + c];
+    xr[(int64_t)k * np + c] = CT<T>::mk(v.x * f, v.y * f);
   }
 }
 
@@ -1053,9 +1067,11 @@ cudaError_t grid_fft_launch(cudaStream_t st, T* x, int rows_per_q, int q0, int n
   double* sw = reinterpret_cast<double*>(ph + 3 * 16 * 64);   // nq x ng weight table
   phase_table_kernel<<<12, 256, 0, st>>>(p, ph);
   count_launch();
-  if (!radix) {
-    phase_kernel<T><<<nb, 256, 0, st>>>(x, rows_per_q, q0, nq, p, ph);
-    count_launch();
+  if constexpr (std::is_same<T, double2>::value) {
+    if (!radix) {
+      phase_kernel<T><<<nb, 256, 0, st>>>(x, rows_per_q, q0, nq, p, ph);
+      count_launch();
+    }
   }
   {
     int nbw = (int)(((int64_t)nq * ng + 255) / 256);
@@ -1063,38 +1079,39 @@ cudaError_t grid_fft_launch(cudaStream_t st, T* x, int rows_per_q, int q0, int n
     weight_table_kernel<<<nbw, 256, 0, st>>>(q0, nq, p, sw);
     count_launch();
   }
-  if constexpr (std::is_same<T, double2>::value) {
-    if (radix) {
-      const int n0 = c.mesh[0], np = c.mesh[1] * c.mesh[2];
-      const int P0 = radix_p(n0), P1 = radix_p(c.mesh[1]), P2 = radix_p(c.mesh[2]);
-      const int two = c.mesh[1] / P1 > kRadMax || c.mesh[2] / P2 > kRadMax, two0 = n0 / P0 > kRadMax;
-      const size_t s1 = ((size_t)np * (1 + two) + 256) * sizeof(double2), s0 = ((size_t)n0 * 32 * (1 + two0) + 64) * sizeof(double2);
-      const int64_t planes = nrows * n0, chunks = nrows * ((np + 31) / 32);
-      if (planes > 2147483647LL || chunks > 2147483647LL) return cudaErrorInvalidValue;
-      cudaError_t e = cudaFuncSetAttribute(grid_plane_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s1);
-      if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(grid_axis0_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s0);
-      if (e != cudaSuccess) return e;
-      grid_plane_kernel<<<(unsigned)planes, 256, s1, st>>>(x, rows_per_q, q0, p, ph, dtw, P1, P2, two);
-      count_launch();
-      grid_axis0_kernel<<<(unsigned)chunks, 256, s0, st>>>(x, rows_per_q, p, sw, dtw, P0, two0);
-      count_launch();
-      return cudaGetLastError();
-    }
-  }
-  for (int a = 2; a >= 0; --a) {
-    const int L = c.mesh[a];
-    if (L == 1) continue;
-    const int64_t S = (a == 2) ? 1 : (a == 1 ? c.mesh[2] : (int64_t)c.mesh[1] * c.mesh[2]);
-    const int groups = 256 / L, lpb = kAxisLines * groups;
-    const int64_t total_lines = nrows * (ng / L), nblk = (total_lines + lpb - 1) / lpb;
-    const size_t smem = (size_t)lpb * (L | 1) * sizeof(T) + 64 * sizeof(double2);
-    grid_axis_kernel<T><<<(unsigned)nblk, 256, smem, st>>>(x, total_lines, ng, L, (int)S, groups, dtw + a * 64);
+  if (radix) {
+    const int n0 = c.mesh[0], np = c.mesh[1] * c.mesh[2];
+    const int P0 = radix_p(n0), P1 = radix_p(c.mesh[1]), P2 = radix_p(c.mesh[2]);
+    const int two = c.mesh[1] / P1 > kRadMax || c.mesh[2] / P2 > kRadMax, two0 = n0 / P0 > kRadMax;
+    const size_t s1 = ((size_t)np * (1 + two) + 256) * sizeof(T), s0 = ((size_t)n0 * 32 * (1 + two0) + 64) * sizeof(T);
+    const int64_t planes = nrows * n0, chunks = nrows * ((np + 31) / 32);
+    if (planes > 2147483647LL || chunks > 2147483647LL) return cudaErrorInvalidValue;
+    cudaError_t e = cudaFuncSetAttribute(grid_plane_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s1);
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(grid_axis0_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s0);
+    if (e != cudaSuccess) return e;
+    grid_plane_kernel<T><<<(unsigned)planes, 256, s1, st>>>(x, rows_per_q, q0, p, ph, dtw, P1, P2, two);
     count_launch();
+    grid_axis0_kernel<T><<<(unsigned)chunks, 256, s0, st>>>(x, rows_per_q, p, sw, dtw, P0, two0);
+    count_launch();
+    return cudaGetLastError();
   }
-  coulomb_weight_kernel<T><<<nb, 256, 0, st>>>(x, rows_per_q, nq, ng, sw);
-  count_launch();
-  return cudaGetLastError();
+  if constexpr (std::is_same<T, double2>::value) {
+    for (int a = 2; a >= 0; --a) {
+      const int L = c.mesh[a];
+      if (L == 1) continue;
+      const int64_t S = (a == 2) ? 1 : (a == 1 ? c.mesh[2] : (int64_t)c.mesh[1] * c.mesh[2]);
+      const int groups = 256 / L, lpb = kAxisLines * groups;
+      const int64_t total_lines = nrows * (ng / L), nblk = (total_lines + lpb - 1) / lpb;
+      const size_t smem = (size_t)lpb * (L | 1) * sizeof(T) + 64 * sizeof(double2);
+      grid_axis_kernel<T><<<(unsigned)nblk, 256, smem, st>>>(x, total_lines, ng, L, (int)S, groups, dtw + a * 64);
+      count_launch();
+    }
+    coulomb_weight_kernel<T><<<nb, 256, 0, st>>>(x, rows_per_q, nq, ng, sw);
+    count_launch();
+    return cudaGetLastError();
+  }
+  return cudaErrorInvalidValue;
 }
 
 // Z[R][(p q)][I] = conj(t[R][I][p]) t[R][I][q].  Block (p-tile of kPairP, R):
@@ -1253,13 +1270,9 @@ cudaError_t grid_coulomb_fft(cudaStream_t st, double2* x, int rows_per_q, int q0
                              const CellDev& c, const double2* dtw, void* work, bool radix) {
   return grid_fft_launch<double2>(st, x, rows_per_q, q0, nq, c, dtw, work, radix);
 }
-cudaError_t grid_coulomb_fft_f(cudaStream_t st, float2* x, int rows_per_q, int q0, int nq,
-                               const CellDev& c, const double2* dtw, void* work) {
-  return grid_fft_launch<float2>(st, x, rows_per_q, q0, nq, c, dtw, work);
-}
 cudaError_t grid_coulomb_fft_ff(cudaStream_t st, ffcomplex* x, int rows_per_q, int q0, int nq,
                                 const CellDev& c, const double2* dtw, void* work) {
-  return grid_fft_launch<ffcomplex>(st, x, rows_per_q, q0, nq, c, dtw, work);
+  return grid_fft_launch<ffcomplex>(st, x, rows_per_q, q0, nq, c, dtw, work, true);
 }
 
 void grid_twiddles(const int mesh[3], double2* host192) {

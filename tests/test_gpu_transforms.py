@@ -63,6 +63,20 @@ def test_factorisation_sizes(cuda, lib_built, n_p):
     _check(cuda, _cell((2, 1, 3), (12, 10, 14)), n_p, 0, tau=1e-6, tol=1e-5)
 
 
+@pytest.mark.parametrize("kmesh,mesh", [
+    ((1, 1, 2), (64, 1, 9)),
+    ((1, 5, 7), (11, 13, 17)),
+    ((3, 1, 4), (8, 61, 4)),
+    ((2, 3, 1), (34, 38, 7)),
+    ((2, 2, 2), (24, 32, 21)),
+    ((3, 2, 1), (6, 5, 49)),
+])
+def test_metric_in_float_float(cuda, lib_built, kmesh, mesh):
+    """The mixed path's grid transform: V_xi is cut to four slices (2^-28 of its rows' largest entries),
+    which the solve multiplies by up to 1 / tau in sums of at most 14 x 14 terms: 7e-4 of the largest entry."""
+    _check(cuda, _cell(kmesh, mesh), min(14, int(np.prod(mesh)) // 3), 1, tol=1e-3)
+
+
 @pytest.mark.parametrize("n_p", [1, 16, 17, 63, 65, 79, 81, 130])
 def test_partial_tiles_of_the_fixed_chains(cuda, lib_built, n_p):
     """xi, V_xi and L of FP64_TC on 64 x 64 tiles of which only some 16-row and 16-column parts are formed."""
