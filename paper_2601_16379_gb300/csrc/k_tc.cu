@@ -521,12 +521,13 @@ __global__ void __launch_bounds__(256) syrk_eri_kernel(const float* __restrict__
                                                        const int2* __restrict__ orb, int nf,
                                                        const int* __restrict__ row_exp, const double* __restrict__ corr,
                                                        double scale, TO* __restrict__ eri,
-                                                       const double2* __restrict__ gam, double2* __restrict__ part) {
+                                                       const double2* __restrict__ gam, double2* __restrict__ part,
+                                                       int tested) {
   const int no = nf * (nf + 1) / 2, P = nf * (nf - 1) / 2;
   const int nch = (no + 255) / 256;
   const int64_t ntask = (int64_t)no * nch;
   const ffloat sc(scale);
-  const bool herm = gam && part[2 * gridDim.x].x != 0.0;
+  const bool herm = gam && tested && part[2 * gridDim.x].x != 0.0;
   double aj = 0.0, ak = 0.0;
   for (int64_t task = blockIdx.x; task < ntask; task += gridDim.x) {
     const int o2 = (int)(task / nch), o1 = (int)(task % nch) * 256 + (int)threadIdx.x;
@@ -969,6 +970,11 @@ __global__ void inv_perm_kernel(const int* __restrict__ qmap, const int* __restr
 // scaled by 2^f_qJ (largest component of the column in [64, 128)); columns J >= nj,
 // c >= r_q and beyond 2 r_q are zero.  Layout [position][2 nj_pad][Kp] per slice; the inverse scales
 // [position][nj_pad].  Rows of L are read along J and the slices written along c, through shared memory.
+// A block takes CW values of c at a time.  Bound by the FP64 pipe (~40 operations per value at two a
+// clock and SM, ~10 us per 32 x 32 values): where the blocks of 32 columns do not fill the SMs, the
+// values of c are split over blockIdx.z too, each block finding the scales anew in integers
+// (5 positions, rank ~70: 39 -> 13.5 us; 20 positions, rank ~100: 46 -> 32).
+template <int CW>
 __global__ void __launch_bounds__(256) lslice_kernel(const double2* __restrict__ L, const double* __restrict__ sw, int np,
                                                      const int* __restrict__ qmap, const int* __restrict__ perm,
                                                      const int* __restrict__ rank, int nj, int nj_pad, int Kp,
@@ -979,24 +985,29 @@ __global__ void __launch_bounds__(256) lslice_kernel(const double2* __restrict__
   const int r = rank[q], J = J0 + tx;
   const double2* Lq = L + (int64_t)q * np * np;
   const int* pq = perm + (int64_t)q * np;
-  __shared__ double sm[8][32];
-  __shared__ uint32_t sd[3][32][33];
-  double m = 0.0;
+  __shared__ unsigned long long sm[8][32];
+  __shared__ uint32_t sd[3][32][CW + 1];
+  constexpr unsigned long long kAbs = 0x7FFFFFFFFFFFFFFFULL, kInf = 0x7FF0000000000000ULL;
+  unsigned long long mb = 0;  // bits of the largest |component| of the column, NaN left out
   if (J < nj)
     for (int c = ty; c < r; c += 8) {
       const double2 v = Lq[(int64_t)pq[c] * np + J];
-      m = fmax(m, fmax(fabs(v.x * w), fabs(v.y * w)));
+      const unsigned long long a = (unsigned long long)__double_as_longlong(v.x) & kAbs;
+      const unsigned long long b = (unsigned long long)__double_as_longlong(v.y) & kAbs;
+      if (a <= kInf) mb = max(mb, a);
+      if (b <= kInf) mb = max(mb, b);
     }
-  sm[ty][tx] = m;
+  sm[ty][tx] = mb;
   __syncthreads();
-  for (int i = 0; i < 8; ++i) m = fmax(m, sm[i][tx]);
+  for (int i = 0; i < 8; ++i) mb = max(mb, sm[i][tx]);
+  const double m = __longlong_as_double((long long)mb) * w;  // w >= 0: the largest |component| w
   // within what a float's power of two holds
   const int ex = (m > 0.0 && isfinite(m)) ? max(-126, min(126, 6 - ilogb(m))) : 0;
-  if (ty == 0) col_scale[(int64_t)j * nj_pad + J] = J < nj ? ldexpf(1.f, -ex) : 0.f;
+  if (ty == 0 && blockIdx.z == 0) col_scale[(int64_t)j * nj_pad + J] = J < nj ? ldexpf(1.f, -ex) : 0.f;
   __half* const S[3] = {S1, S2, S3};
-  for (int c0 = 0; c0 < Kp / 2; c0 += 32) {
+  for (int c0 = blockIdx.z * CW; c0 < Kp / 2; c0 += gridDim.z * CW) {
     __syncthreads();
-    for (int cc = ty; cc < 32; cc += 8) {
+    for (int cc = ty; cc < CW; cc += 8) {
       const int c = c0 + cc;
       double lr = 0.0, li = 0.0;
       if (J < nj && c < r) {
@@ -1013,13 +1024,13 @@ __global__ void __launch_bounds__(256) lslice_kernel(const double2* __restrict__
     }
     __syncthreads();
     // row 2 Jl + part of the block, lanes along c
-    for (int e = ty; e < 64; e += 8) {
-      const int Jl = e >> 1, part = e & 1, c = c0 + tx;
+    for (int t = threadIdx.x; t < 64 * CW; t += 256) {
+      const int e = t / CW, Jl = e >> 1, part = e & 1, cc = t % CW, c = c0 + cc;
       if (c >= Kp / 2) continue;
       const int64_t at = ((int64_t)j * 2 * nj_pad + 2 * (J0 + Jl) + part) * Kp + 2 * c;
 #pragma unroll
       for (int i = 0; i < 3; ++i) {
-        const uint32_t x = sd[i][Jl][tx];
+        const uint32_t x = sd[i][Jl][cc];
         // (re, -im) or (im, re); the slices of -x are those of x negated
         const uint32_t y = part ? (x >> 16) | (x << 16) : x ^ 0x80000000u;
         *reinterpret_cast<uint32_t*>(S[i] + at) = y;
@@ -1134,6 +1145,9 @@ cudaError_t syrk_tc_mma(cudaStream_t st, void* split, int64_t n2, int nq, int64_
                   : syrk_launch<64, 3>(st, sl, n2, K2, tiles_d, ntiles, ws, accumulate, err);
 }
 
+// The test of gamma takes 13 us (one block) and saves an eighth of a finish of ~30 us at 33 orbitals,
+// ~750 us on average over 23 to 120.
+constexpr int kHermMin = 48;
 constexpr int kEriBlocks = 152 * 16;  // fixed grid of the fused finish (reproducible traces)
 size_t syrk_tc_eri_part_count() { return 2 * (size_t)kEriBlocks + 1; }  // partials, Hermitian flag
 
@@ -1146,12 +1160,13 @@ static cudaError_t finish_eri_impl(cudaStream_t st, const void* ws, int ntiles, 
   const float* wh = reinterpret_cast<const float*>(ws);
   const float* wl = wh + (size_t)ntiles * BN * BM;
   const int64_t n2 = (int64_t)nf * nf, nt = (n2 + BM - 1) / BM;
-  if (gamma) {
+  const int tested = gamma && nf >= kHermMin;
+  if (tested) {
     gamma_herm_kernel<<<1, 1024, 0, st>>>(gamma, nf, part + 2 * kEriBlocks);
     count_launch();
   }
   syrk_eri_kernel<TO><<<kEriBlocks, 256, 0, st>>>(wh, wl, tile_of_d, (int)nt, orb, nf, row_exp, corr, scale, eri,
-                                                  gamma, part);
+                                                  gamma, part, tested);
   count_launch();
   if (gamma) {
     eri_traces_final_kernel<<<1, 256, 0, st>>>(part, kEriBlocks, out4);
@@ -1192,8 +1207,17 @@ cudaError_t mlgemm_tc_prepare(cudaStream_t st, const double2* L, const double* s
   const int Kp = mlgemm_tc_kp(rp), njp = mlgemm_tc_nj_pad(nj);
   const size_t per = (size_t)nS * 2 * njp * Kp;
   __half* S1 = reinterpret_cast<__half*>(lsl);
-  lslice_kernel<<<dim3(njp / 32, nS), 256, 0, st>>>(L, sw, np, qmap, perm, rank, nj, njp, Kp, S1, S1 + per, S1 + 2 * per,
-                                                    col_scale);
+  // below two blocks per SM the values of c are split over blocks too
+  int dev = 0, sms = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e != cudaSuccess) return e;
+  if ((int64_t)(njp / 32) * nS < 2 * sms)
+    lslice_kernel<8><<<dim3(njp / 32, nS, (Kp / 2 + 7) / 8), 256, 0, st>>>(L, sw, np, qmap, perm, rank, nj, njp, Kp, S1,
+                                                                           S1 + per, S1 + 2 * per, col_scale);
+  else
+    lslice_kernel<32><<<dim3(njp / 32, nS), 256, 0, st>>>(L, sw, np, qmap, perm, rank, nj, njp, Kp, S1, S1 + per,
+                                                          S1 + 2 * per, col_scale);
   count_launch();
   inv_perm_kernel<<<nS, 128, 0, st>>>(qmap, perm, rank, np, inv);
   count_launch();
