@@ -454,14 +454,18 @@ __global__ void __launch_bounds__(1024) ips_init_kernel(IpsArgs a) {
 // Step j in one launch (the stream order between the steps is the only barrier): every block
 // finds the pivot from the block maxima of step j - 1 -- the tie rule looks only into blocks
 // whose maximum lies in the window -- then updates its own points and leaves its new maximum.
-// Buffers alternate, so that no block reads what another one writes.  About 150 blocks.
+// The maxima and the diagonal alternate between two buffers, and a step reads piv only below j, so
+// that no block reads what another one of its launch writes (scal[0], written at j = 0, is used
+// from j = 1 on).  About 150 blocks, more on grids above 152 x 256 points.
 __global__ void __launch_bounds__(1024) ips_step_kernel(IpsArgs a, int j) {
   extern __shared__ double ips_smem[];
   __shared__ long long sv[32], s_thr;
   __shared__ unsigned long long sh[32];
   __shared__ int si[32], s_list[32], s_n, s_stop;
   __shared__ double s_inv;
-  if (*a.status != 0) return;
+  // a selection that has stopped: piv[j - 1] is -1 from its last step on and fixed for this launch (the
+  // status is written by this very launch, so that warps of one block could see it differ)
+  if (j > 0 && a.piv[j - 1] < 0) return;
   const int nb = gridDim.x, bd = blockDim.x, tid = threadIdx.x, lane = tid & 31, w = tid >> 5, R = a.R, G = bd / R;
   const long long* M = a.M + (j & 1) * nb;
   const double* din = a.d + (int64_t)(j & 1) * a.ng;
