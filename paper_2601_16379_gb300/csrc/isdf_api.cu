@@ -134,9 +134,7 @@ struct isdf_handle {
     for (auto& b : bufs)
       if (b.first == name) {
         if (b.second.bytes >= bytes) return b.second.p;
-        cudaFree(b.second.p);
-        b.second.p = nullptr;
-        b.second.bytes = 0;
+        drop(b);
         if (cudaMalloc(&b.second.p, bytes) != cudaSuccess) {
           cudaGetLastError();
           return nullptr;
@@ -153,13 +151,13 @@ struct isdf_handle {
     bufs.emplace_back(name, d);
     return d.p;
   }
-  void release(const char* name) {
-    for (auto& b : bufs)
-      if (b.first == name && b.second.p) {
-        cudaFree(b.second.p);
-        b.second.p = nullptr;
-        b.second.bytes = 0;
-      }
+  // Free a buffer; what it held is gone, whether or not the caller can allocate it again.
+  void drop(std::pair<std::string, DevBuf>& b) {
+    cudaFree(b.second.p);
+    b.second.p = nullptr;
+    b.second.bytes = 0;
+    if (b.first == "eta") has_eta = false;
+    if (b.first == "xi") has_xi = false;
   }
   // Two groups of large buffers never live at once when HBM is short: the
   // grid-sized fit intermediates (eta, xi and their work) and the per-fragment
@@ -177,13 +175,10 @@ struct isdf_handle {
     for (auto& b : bufs) {
       const bool other = frag ? in_fit_group(b.first) : in_frag_group(b.first);
       if (other && b.second.p) {
-        cudaFree(b.second.p);
-        b.second.p = nullptr;
-        b.second.bytes = 0;
+        drop(b);
         freed = true;
       }
     }
-    if (freed && frag) has_xi = has_eta = false;
     return freed;
   }
   void* ensure_evict(const char* name, size_t bytes) {
@@ -448,10 +443,10 @@ int finish_points(isdf_handle* h) {
   const int np = h->np;
   double2* phi = (double2*)h->buf("phi");
   int32_t* ipsd = (int32_t*)h->buf("ips");
+  h->has_points = h->has_fit = h->has_xi = h->has_eta = h->has_coulomb = false;
   ENSURE(X, double2, "X", (size_t)h->nk * np * h->nao);
   CK(gather_x(h->st, phi, h->nk, h->nao, h->ng, ipsd, np, X));
   h->has_points = true;
-  h->has_fit = h->has_xi = h->has_eta = h->has_coulomb = false;
   return ISDF_OK;
 }
 
@@ -558,6 +553,9 @@ int coulomb_tail(isdf_handle* h, const QHalf& qh, int neff, double2* Vxi, void* 
   ENSURE(permV, int32_t, "permV", (size_t)nk * np);
   ENSURE(rankV, int32_t, "rankV", nk);
   ENSURE(qlist, int, "q_list", nk);
+  ENSURE(Lxi, double2, "W_work", (size_t)nk * np * np);
+  ENSURE(Lq, double2, "Lq", (size_t)nk * np * np);
+  h->has_coulomb = false;  // until the new factors stand
   CK(cudaMemcpyAsync(qlist, qh.list.data(), sizeof(int) * qh.list.size(), cudaMemcpyHostToDevice, h->st));
   // the representatives only: L^-q is the conjugate of L^q, bit for bit
   CK(pchol_batched(h->st, Vxi, np, neff, false, qlist, qh.count, 1e-15, LtV, permV, rankV));
@@ -566,9 +564,7 @@ int coulomb_tail(isdf_handle* h, const QHalf& qh, int neff, double2* Vxi, void* 
   CK(mirror_copy(h->st, rankV, 1, mir, nm));
   h->ranks_v.assign(nk, 0);
   CK(cudaMemcpyAsync(h->ranks_v.data(), rankV, sizeof(int32_t) * nk, cudaMemcpyDeviceToHost, h->st));
-  ENSURE(Lxi, double2, "W_work", (size_t)nk * np * np);
   CK(lt_to_rowmajor(h->st, LtV, rankV, qlist, qh.count, np, Lxi));
-  ENSURE(Lq, double2, "Lq", (size_t)nk * np * np);
   // W has neff rows and L_xi neff rows and columns that are not zero.  L^q in another rounding
   // moves the FP64_TC integrals by 6e-10 of themselves: FP64 FMA there
   const int64_t pp = (int64_t)np * np;
@@ -809,6 +805,7 @@ int isdf_fit_zeta(isdf_handle* h, double solve_tol, int32_t* rank_out) {
   CK(kdft_cols(h->st, Pi, (int64_t)np * np, km, +1, -1, 1, 1.0 / nk, fp64));
   // eta^q (Eq. 5): g^k_I(r) = sum_mu conj(X^k_I mu) Phi^k_mu(r), then the k-convolution.
   ENSURE(eta, double2, "eta", (size_t)nk * np * ng);
+  h->has_eta = false;  // until the new fit stands
   ZOpt g_opt;
   if (!fp64 && nao <= kZgemm7MaxK) g_opt.slices = 7;
   ZM(fp64 || g_opt.slices == 7 ? "grid_work_z" : nullptr, 'R', 'N', np, ng, nao, 1.0, X, nao, (int64_t)np * nao, phi, ng,
@@ -828,6 +825,8 @@ int isdf_fit_zeta(isdf_handle* h, double solve_tol, int32_t* rank_out) {
   ENSURE(tri, double2, "Vxi", (size_t)nk * np * np);  // scratch of the triangular inverse
   ENSURE(qlist, int, "q_list", nk);
   const int64_t pp = (int64_t)np * np;
+  // from here on the factors, ranks and xi of an earlier fit, and the metric on them, are overwritten
+  h->has_fit = h->has_xi = h->has_coulomb = false;
   CK(cudaMemcpyAsync(qlist, qh.list.data(), sizeof(int) * qh.list.size(), cudaMemcpyHostToDevice, h->st));
   CK(pchol_batched(h->st, Pi, np, np, true, qlist, qh.count, solve_tol, LtPi, permPi, rankPi));
   if (!qh.mirror.empty()) {
@@ -891,6 +890,13 @@ int isdf_coulomb_metric(isdf_handle* h, void* V_out) {
   ENSURE(Vxi, double2, "Vxi", (size_t)nk * np * np);
   ENSURE(gwork, uint8_t, "grid_work", grid_coulomb_work_bytes(nk, h->cell));
   const int64_t pp = (int64_t)np * np, xg = (int64_t)rx * ng;
+  const int qcv = vxi_tc_chunk(rx, ng, (size_t)4 << 30);
+  void* vwork = nullptr;
+  if (h->prec == ISDF_MIXED) {
+    ENSURE(vw, uint8_t, "grid_work_v", vxi_tc_work_bytes(rx, ng, qcv));
+    vwork = vw;
+  }
+  h->has_xi = false;  // xi is transformed in place
   CK(cudaMemsetAsync(Vxi, 0, sizeof(double2) * (size_t)nk * pp, h->st));
   // FP64 and FP64_TC: FP64 arithmetic (an error in V_xi reaches E unamplified, as
   // P dV_xi P^H with P = M W^T well scaled, so FP64_TC needs more than four slices here).
@@ -910,8 +916,6 @@ int isdf_coulomb_metric(isdf_handle* h, void* V_out) {
     // mixed: xi rows to float-float in place, the grid FFT in float-float, and
     // V_xi = Omega conj(c')c'^T on the tensor cores with four exact slices (~2^-28 relative;
     // an FP32 FFT and GEMM put ~2e-7 into V_xi, which reaches E and the traces as such)
-    const int qcv = vxi_tc_chunk(rx, ng, (size_t)4 << 30);
-    ENSURE(vwork, uint8_t, "grid_work_v", vxi_tc_work_bytes(rx, ng, qcv));
     for (const auto& r : qh.runs) {
       ffcomplex* xf = reinterpret_cast<ffcomplex*>(xi + r.first * xg);
       CK(z2ff(h->st, xi + r.first * xg, xf, r.second * xg));
@@ -923,7 +927,6 @@ int isdf_coulomb_metric(isdf_handle* h, void* V_out) {
     ENSURE(mir, int2, "q_mirror", qh.mirror.size());
     CK(cudaMemcpyAsync(mir, qh.mirror.data(), sizeof(int2) * qh.mirror.size(), cudaMemcpyHostToDevice, h->st));
   }
-  h->has_xi = false;  // xi was transformed in place (FP64) / is no longer needed
   return coulomb_tail(h, qh, rx, Vxi, V_out);
 }
 

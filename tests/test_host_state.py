@@ -1,0 +1,118 @@
+"""Host side of the library (isdf_api.cu) on the CPU, over fakes of the CUDA runtime and the kernels
+(host_fakes.cpp): what a handle still offers after an allocation has failed, after a bounded device
+wait has expired, and after a new fit.
+"""
+import ctypes as ct
+import subprocess
+from pathlib import Path
+
+import numpy as np
+import pytest
+
+from paper_2601_16379_gb300 import binding as B
+from paper_2601_16379_gb300 import workloads as W
+
+ROOT = Path(__file__).resolve().parents[1]
+CSRC = ROOT / "paper_2601_16379_gb300" / "csrc"
+CUDA_INCLUDE = "/usr/local/cuda/include"
+
+OOM, TIMEOUT, STATE = -2, -5, -6
+
+
+@pytest.fixture(scope="module")
+def fake_lib(tmp_path_factory):
+    out = tmp_path_factory.mktemp("host") / "libisdf_host.so"
+    inc = ["-I", str(ROOT / "include"), "-I", str(CSRC), "-I", CUDA_INCLUDE]
+    subprocess.run(["g++", "-x", "c++", "-std=c++17", "-O1", "-fPIC", "-shared", "-w", "-Wl,-Bsymbolic", *inc,
+                    str(CSRC / "isdf_api.cu"), str(ROOT / "tests" / "host_fakes.cpp"), "-o", str(out)], check=True)
+    lib = B.load(str(out))
+    for f in ("fake_used", "fake_peak", "fake_last_work"):
+        getattr(lib, f).restype = ct.c_size_t
+    lib.fake_capacity.argtypes = [ct.c_size_t]
+    return lib
+
+
+@pytest.fixture
+def fake(fake_lib, monkeypatch):
+    monkeypatch.setattr(B, "_lib", fake_lib)
+    fake_lib.fake_reset()
+    yield fake_lib
+    fake_lib.fake_reset()
+
+
+def _cell(kmesh=(2, 1, 2), mesh=(6, 5, 4)):
+    sh = [W.Shell(0, 0, (0.6,), (1.0,)), W.Shell(1, 1, (0.9,), (1.0,))]
+    return W.custom_cell(5.0, [[0.01, 0.02, 0.03], [0.37, 0.52, 0.21]], sh, kmesh, mesh)
+
+
+def _handle(prec=B.ISDF_FP64, n_p=12, **kw):
+    g = B.Isdf(_cell(**kw), prec)
+    g.set_points(np.arange(n_p))
+    return g
+
+
+def _code(call, *args):
+    with pytest.raises(B.IsdfError) as e:
+        call(*args)
+    return e.value.code
+
+
+OUT = ct.addressof((ct.c_double * (1 << 16))())  # stands for the caller's buffers, which the fakes do not touch
+
+
+def test_xi_is_gone_after_its_growth_failed_in_the_eta_route(fake):
+    g = _handle()
+    g.fit_zeta(1e-3)                     # xi holds 4 of 12 rows
+    fake.fake_capacity(fake.fake_used())
+    assert _code(g.coulomb_metric_eta) == OOM
+    assert _code(g.coulomb_metric) == STATE and _code(g.get, 3, OUT) == STATE
+    assert fake.fake_nulls() == 0
+    fake.fake_capacity(1 << 40)
+    g.coulomb_metric_eta()               # eta still stands
+    g.close()
+
+
+def test_a_fit_that_fails_leaves_no_fit(fake):
+    g = _handle()
+    g.fit_zeta(1e-3)
+    fake.fake_rank(9)                    # a smaller tolerance: more rows of xi
+    fake.fake_capacity(fake.fake_used())
+    assert _code(g.fit_zeta, 1e-9) == OOM
+    assert _code(g.coulomb_metric) == STATE and _code(g.coulomb_metric_eta) == STATE
+    assert _code(g.get, 3, OUT) == STATE and fake.fake_nulls() == 0
+    fake.fake_capacity(1 << 40)
+    g.fit_zeta(1e-9)
+    g.coulomb_metric()
+    assert fake.fake_nulls() == 0
+    g.close()
+
+
+def test_points_whose_vectors_do_not_fit_leave_no_points(fake):
+    g = _handle(n_p=12)
+    fake.fake_capacity(fake.fake_used() + 1024)  # the indices fit, X does not
+    assert _code(g.set_points, np.arange(40)) == OOM
+    assert _code(g.fit_zeta, 1e-3) == STATE and fake.fake_nulls() == 0
+    g.close()
+
+
+@pytest.mark.parametrize("prec", [B.ISDF_FP64, B.ISDF_MIXED, B.ISDF_FP64_TC])
+def test_a_fit_that_fails_ends_the_metric_only_once_it_touches_its_factors(fake, prec):
+    g = _handle(prec)
+    g.fit_zeta(1e-3)
+    g.coulomb_metric()
+    C = np.zeros((4, 4, 3), np.complex128)
+    frag = lambda: g.fragment_eri([_Ptr(C)], traces=False)  # noqa: E731
+    frag()
+    fake.fake_rank(9)
+    fake.fake_capacity(0)
+    assert _code(g.fit_zeta, 1e-9) == OOM          # at xi: new pivots beside the old L
+    assert _code(frag) == STATE and _code(g.exchange, OUT, OUT) == STATE
+    g.close()
+
+
+class _Ptr:
+    def __init__(self, a):
+        self.a, self.shape = a, a.shape
+
+    def data_ptr(self):
+        return self.a.ctypes.data
