@@ -65,6 +65,7 @@ struct isdf_handle {
   std::vector<int32_t> ranks_v;  // rank n_q of V_xi^q (columns of L^q), per q
   int xi_rows = 0;               // rows of xi kept per q: max_q r_q (rows beyond r_q are zero)
   std::string err;
+  bool err_unread = false;       // kernels that may set the device error word since it was last read
   int64_t launches = 0;
   std::vector<int2> tiles_host;
   std::vector<int> tile_of_host;
@@ -332,7 +333,19 @@ int check_device(isdf_handle* h) {
   if (e != cudaSuccess) return fail(h, ISDF_ERR_CUDA, "cudaGetDevice: %s", cudaGetErrorString(e));
   if (dev != h->device)
     return fail(h, ISDF_ERR_STATE, "current device %d differs from the handle's device %d", dev, h->device);
+  // a call that returned before it read the error word leaves nothing to this one
+  if (h->err_unread) {
+    e = cudaMemsetAsync(h->buf("err_words"), 0, sizeof(int), h->st);
+    if (e != cudaSuccess) return fail(h, ISDF_ERR_CUDA, "clearing the error word: %s", cudaGetErrorString(e));
+    h->err_unread = false;
+  }
   return ISDF_OK;
+}
+
+// The device word in which a kernel reports a bounded wait that expired, read by tc_status.
+int* err_word(isdf_handle* h) {
+  h->err_unread = true;
+  return (int*)h->buf("err_words");
 }
 
 int upload_basis(isdf_handle* h) {
@@ -403,7 +416,7 @@ int zmul(isdf_handle* h, const char* wname, char opA, char opB, int m, int n, in
   }
   if (w)
     CK(zgemm_tc(h->st, opA, opB, m, n, k, alpha, A, lda, sA, B, ldb, sB, C, ldc, sC, batch, o, w, bytes,
-                (int*)h->buf("err_words")));
+                err_word(h)));
   else
     CK(zgemm(h->st, opA, opB, m, n, k, alpha, A, lda, sA, B, ldb, sB, C, ldc, sC, batch, o));
   return ISDF_OK;
@@ -426,6 +439,7 @@ int tc_status(isdf_handle* h, const char* what) {
   int* w = (int*)h->buf("err_words");
   CK(cudaMemcpyAsync(&err, w, sizeof(int), cudaMemcpyDeviceToHost, h->st));
   CK(cudaStreamSynchronize(h->st));
+  h->err_unread = false;
   if (err == 0) return ISDF_OK;
   CK(cudaMemsetAsync(w, 0, sizeof(int), h->st));
   return fail(h, ISDF_ERR_TIMEOUT, "%s: bounded device wait expired (code %d)", what, err);
@@ -855,6 +869,9 @@ int isdf_fit_zeta(isdf_handle* h, double solve_tol, int32_t* rank_out) {
   tri_opt.qmap = qlist;
   tri_opt.krank = rankPi;
   ZM(zw, 'N', 'N', rx, ng, rx, 1.0, wwork, np, pp, eta, ng, pg, xi, ng, xg, qh.count, tri_opt);
+  // xi stands only if no wait of its product expired (FMA chains have none)
+  if (zw)
+    if (int e = tc_status(h, "xi of the fit")) return e;
   if (!qh.mirror.empty()) {
     const int2* mir = (const int2*)h->buf("q_mirror");
     CK(mirror_conj(h->st, W, pp, mir, (int)qh.mirror.size()));
@@ -920,7 +937,7 @@ int isdf_coulomb_metric(isdf_handle* h, void* V_out) {
       ffcomplex* xf = reinterpret_cast<ffcomplex*>(xi + r.first * xg);
       CK(z2ff(h->st, xi + r.first * xg, xf, r.second * xg));
       CK(grid_coulomb_fft_ff(h->st, xf, rx, r.first, r.second, h->cell, tw, gwork));
-      CK(vxi_tc(h->st, xf, xg, rx, ng, r.second, h->volume, Vxi + r.first * pp, np, pp, vwork, qcv, (int*)h->buf("err_words")));
+      CK(vxi_tc(h->st, xf, xg, rx, ng, r.second, h->volume, Vxi + r.first * pp, np, pp, vwork, qcv, err_word(h)));
     }
   }
   if (!qh.mirror.empty()) {
@@ -1034,7 +1051,7 @@ int isdf_fragment_eri(isdf_handle* h, int n_frag, const int32_t* n_orb, const vo
   const bool any_tr = (ej_out || ek_out) && gamma;
   ENSURE(trall, double, "frag_traces", 4 * (size_t)n_frag);
   CK(cudaMemsetAsync(trall, 0, sizeof(double) * 4 * (size_t)n_frag, h->st));
-  int* errw = (int*)h->buf("err_words");
+  int* errw = err_word(h);
   // FP64_TC: the grouped tensor-core path in float-float with more exact slices,
   // where B = M L fits its exact accumulation (2 r_q <= 576); else FP64 arithmetic
   const bool tc64 = (h->prec == ISDF_FP64_TC) && mlgemm5_tc_supported(rp);

@@ -110,6 +110,42 @@ def test_a_fit_that_fails_ends_the_metric_only_once_it_touches_its_factors(fake,
     g.close()
 
 
+def _wide():
+    """Eight orbitals: every product of the FP64 fit is long enough for the tensor cores."""
+    sh = [W.Shell(a, l, (x,), (1.0,)) for a in (0, 1) for l, x in ((0, 0.6), (1, 0.9))]
+    g = B.Isdf(W.custom_cell(5.0, [[0.01, 0.02, 0.03], [0.37, 0.52, 0.21]], sh, (2, 1, 2), (6, 5, 4)), B.ISDF_FP64)
+    g.set_points(np.arange(12))
+    return g
+
+
+@pytest.mark.parametrize("product", [0, 1, 2])  # G, g, xi
+def test_a_wait_that_expires_in_any_product_fails_the_fit(fake, product):
+    g = _wide()
+    fake.fake_rank(9)
+    fake.fake_arm(product)
+    assert _code(g.fit_zeta, 1e-3) == TIMEOUT
+    assert _code(g.coulomb_metric) == STATE and _code(g.get, 3, OUT) == STATE
+    g.fit_zeta(1e-3)
+    assert fake.fake_tc_calls() >= 5
+    g.coulomb_metric()
+    g.close()
+
+
+def test_a_call_does_not_report_the_wait_of_one_before(fake):
+    g = _wide()
+    fake.fake_rank(9)
+    g.fit_zeta(1e-3)
+    g.coulomb_metric()
+    small, large = (_Ptr(np.zeros((4, 8, n), np.complex128)) for n in (3, 64))
+    g.fragment_eri([small], traces=False)
+    fake.fake_capacity(fake.fake_used())
+    fake.fake_arm(0)                                  # in the first fragment; the second does not fit
+    assert _code(g.fragment_eri, [small, large]) == OOM
+    fake.fake_capacity(1 << 40)
+    g.exchange(OUT, OUT)
+    g.close()
+
+
 class _Ptr:
     def __init__(self, a):
         self.a, self.shape = a, a.shape
