@@ -237,6 +237,11 @@ int isdf_set_time_reversal(isdf_handle* h, int enable);
  * contracted in chunks of q-points that fit this limit, each chunk adding to
  * the same accumulator, so a smaller limit costs only more launches.  Default
  * 12 GiB; values below one q-point's slices give one q-point per chunk.
+ * Every mode: also the limit (with 512 MiB) for the integer slices of the
+ * complex128 tensor-core products, which go in chunks of batch entries (one at
+ * least; the same bits for any limit).  Where the device has no memory for the
+ * slices of one entry, products of the FP64 path run on the FP64 pipe instead;
+ * those whose arithmetic the other modes fix return ISDF_ERR_OOM.
  * Returns ISDF_ERR_ARG for 0. */
 int isdf_set_workspace_limit(isdf_handle* h, uint64_t bytes);
 

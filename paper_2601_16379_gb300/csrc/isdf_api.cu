@@ -167,7 +167,7 @@ struct isdf_handle {
   // them, or isdf_coulomb_metric_eta, then needs a new isdf_fit_zeta).
   static bool in_frag_group(const std::string& n) { return n.rfind("frag_", 0) == 0 || n.rfind("tc_", 0) == 0; }
   static bool in_fit_group(const std::string& n) {
-    return n == "eta" || n == "xi" || n == "grid_work" || n == "grid_work_z" || n == "grid_work_v";
+    return n == "eta" || n == "xi" || n == "grid_work" || n == "grid_work_v";
   }
   bool evict_other(const char* name) {
     const std::string n(name);
@@ -182,8 +182,19 @@ struct isdf_handle {
     }
     return freed;
   }
+  // The slices of a complex128 product (zmul) are dead as soon as it is enqueued: they give way
+  // to whatever else does not fit.
+  bool drop_slices() {
+    for (auto& b : bufs)
+      if (b.first == "zslices" && b.second.p) {
+        drop(b);
+        return true;
+      }
+    return false;
+  }
   void* ensure_evict(const char* name, size_t bytes) {
     void* p = ensure(name, bytes);
+    if (!p && drop_slices()) p = ensure(name, bytes);
     if (!p && evict_other(name)) p = ensure(name, bytes);
     return p;
   }
@@ -390,12 +401,15 @@ int upload_basis(isdf_handle* h) {
   return ISDF_OK;
 }
 
-// C_b = alpha op(A_b) op(B_b) in complex128 (FP64-accurate): on the tensor cores with its slices
-// in the buffer `wname` (batch entries in chunks of kSliceBytes), on the FP64 pipe where the
-// inner dimension is too short to pay for the slicing or the workspace cannot be had.
-// A bounded wait that expires sets the handle's error
-// word, read by tc_status at the next synchronisation point.
-// wname NULL keeps the FP64 pipe.
+// C_b = alpha op(A_b) op(B_b) in complex128 (FP64-accurate): with `who` on the tensor cores, its slices
+// in the buffer "zslices" (see isdf_handle::drop_slices) for as many batch entries at a time as fit
+// kSliceBytes, the workspace limit and the free memory, one at least; on the FP64 pipe
+// with `who` NULL and where the inner dimension is too short to pay for the slicing.
+// Where not even one entry's slices can be had: eight slices stand for FP64 FMA chains, which take their
+// place as the form without a workspace (nothing else is freed for them); seven slices are the fixed
+// arithmetic of their products (see isdf_fit_zeta), for which the group other than that of `who` is freed,
+// else the call fails.  A bounded wait that expires sets the handle's error word, read by tc_status at the next
+// synchronisation point.
 //
 // kMinTcK: a 64 x 64 tile of the SIMT kernel takes 4.3 us per unit of K however few tiles there
 // are, the tensor path ~23 us for the smallest product (three launches): measured 43 against
@@ -403,16 +417,20 @@ int upload_basis(isdf_handle* h) {
 // 1600 x 1600 x 1680, so that the line lies below K = 8.
 constexpr size_t kSliceBytes = (size_t)512 << 20;
 constexpr int kMinTcK = 6;
-int zmul(isdf_handle* h, const char* wname, char opA, char opB, int m, int n, int k, double alpha, const double2* A,
+int zmul(isdf_handle* h, const char* who, char opA, char opB, int m, int n, int k, double alpha, const double2* A,
          int64_t lda, int64_t sA, const double2* B, int64_t ldb, int64_t sB, double2* C, int64_t ldc, int64_t sC,
          int batch, const ZOpt& o = ZOpt()) {
   void* w = nullptr;
   size_t bytes = 0;
-  if (wname && (k >= kMinTcK || o.slices == 7)) {
+  if (who && (k >= kMinTcK || o.slices == 7)) {
     const bool same = !o.brow && zgemm_tc_same(opA, opB, m, n, A, lda, sA, B, ldb, sB);
-    bytes = std::min(zgemm_tc_work_bytes(o.slices, m, n, k, batch, same),
-                     std::max(zgemm_tc_work_bytes(o.slices, m, n, k, 1, same), kSliceBytes));
-    w = h->ensure_evict(wname, bytes);
+    const size_t one = zgemm_tc_work_bytes(o.slices, m, n, k, 1, same), limit = std::min(kSliceBytes, h->split_budget);
+    for (int nb = (int)std::min<size_t>(batch, std::max<size_t>(1, limit / one)); nb >= 1 && !w; nb /= 2) {
+      bytes = zgemm_tc_work_bytes(o.slices, m, n, k, nb, same);
+      w = h->ensure("zslices", bytes);
+    }
+    if (!w && o.slices == 7 && h->evict_other(who)) w = h->ensure("zslices", bytes = one);
+    if (!w && o.slices == 7) return fail(h, ISDF_ERR_OOM, "device allocation of zslices (%zu bytes) failed", one);
   }
   if (w)
     CK(zgemm_tc(h->st, opA, opB, m, n, k, alpha, A, lda, sA, B, ldb, sB, C, ldc, sC, batch, o, w, bytes,
@@ -585,14 +603,14 @@ int coulomb_tail(isdf_handle* h, const QHalf& qh, int neff, double2* Vxi, void* 
   ZOpt reps;
   reps.qmap = qlist;
   CK(cudaMemsetAsync(Lq, 0, sizeof(double2) * (size_t)nk * pp, h->st));
-  ZM(h->prec == ISDF_FP64_TC ? nullptr : "zwork", 'T', 'N', np, neff, neff, 1.0, W, np, pp, Lxi, np, pp, Lq, np, pp,
+  ZM(h->prec == ISDF_FP64_TC ? nullptr : "call", 'T', 'N', np, neff, neff, 1.0, W, np, pp, Lxi, np, pp, Lq, np, pp,
      qh.count, reps);
   CK(mirror_conj(h->st, Lq, pp, mir, nm));
   if (V_out) {
     // V^q = W^T V_xi conj(W)
     double2* tmp = Lxi;  // reuse
-    ZM("zwork", 'N', 'R', neff, np, neff, 1.0, Vxi, np, pp, W, np, pp, tmp, np, pp, qh.count, reps);
-    ZM("zwork", 'T', 'N', np, np, neff, 1.0, W, np, pp, tmp, np, pp, (double2*)V_out, np, pp, qh.count, reps);
+    ZM("call", 'N', 'R', neff, np, neff, 1.0, Vxi, np, pp, W, np, pp, tmp, np, pp, qh.count, reps);
+    ZM("call", 'T', 'N', np, np, neff, 1.0, W, np, pp, tmp, np, pp, (double2*)V_out, np, pp, qh.count, reps);
     CK(mirror_conj(h->st, (double2*)V_out, pp, mir, nm));
   }
   if (h->prec == ISDF_MIXED) {
@@ -811,10 +829,10 @@ int isdf_fit_zeta(isdf_handle* h, double solve_tol, int32_t* rank_out) {
   // these three products keep one fixed arithmetic there: FP64 FMA chains, and seven slices
   // for g.  The plain FP64 path moves by 1e-11 and takes the tensor cores throughout.
   const bool fp64 = h->prec == ISDF_FP64;
-  const char* zw = fp64 ? "grid_work_z" : nullptr;
+  const char* who = fp64 ? "fit" : nullptr;
   // Pi^q (Eq. 4): G^k_IJ = sum_mu conj(X^k_I mu) X^k_J mu, then the k-convolution
   ENSURE(Pi, double2, "Pi", (size_t)nk * np * np);
-  ZM(zw, 'R', 'T', np, np, nao, 1.0, X, nao, (int64_t)np * nao, X, nao, (int64_t)np * nao, Pi,
+  ZM(who, 'R', 'T', np, np, nao, 1.0, X, nao, (int64_t)np * nao, X, nao, (int64_t)np * nao, Pi,
            np, (int64_t)np * np, nk);
   CK(kdft_cols(h->st, Pi, (int64_t)np * np, km, +1, -1, 1, 1.0 / nk, fp64));
   // eta^q (Eq. 5): g^k_I(r) = sum_mu conj(X^k_I mu) Phi^k_mu(r), then the k-convolution.
@@ -822,7 +840,7 @@ int isdf_fit_zeta(isdf_handle* h, double solve_tol, int32_t* rank_out) {
   h->has_eta = false;  // until the new fit stands
   ZOpt g_opt;
   if (!fp64 && nao <= kZgemm7MaxK) g_opt.slices = 7;
-  ZM(fp64 || g_opt.slices == 7 ? "grid_work_z" : nullptr, 'R', 'N', np, ng, nao, 1.0, X, nao, (int64_t)np * nao, phi, ng,
+  ZM(fp64 || g_opt.slices == 7 ? "fit" : nullptr, 'R', 'N', np, ng, nao, 1.0, X, nao, (int64_t)np * nao, phi, ng,
      (int64_t)nao * ng, eta, ng, (int64_t)np * ng, nk, g_opt);
   // the k-convolution of Algorithm 1 over the grid columns: FP64 in the FP64 path,
   // float-float (~2^-44 relative, FP32 arithmetic) in the others
@@ -868,9 +886,9 @@ int isdf_fit_zeta(isdf_handle* h, double solve_tol, int32_t* rank_out) {
   tri_opt.sIdx = np;
   tri_opt.qmap = qlist;
   tri_opt.krank = rankPi;
-  ZM(zw, 'N', 'N', rx, ng, rx, 1.0, wwork, np, pp, eta, ng, pg, xi, ng, xg, qh.count, tri_opt);
+  ZM(who, 'N', 'N', rx, ng, rx, 1.0, wwork, np, pp, eta, ng, pg, xi, ng, xg, qh.count, tri_opt);
   // xi stands only if no wait of its product expired (FMA chains have none)
-  if (zw)
+  if (who)
     if (int e = tc_status(h, "xi of the fit")) return e;
   if (!qh.mirror.empty()) {
     const int2* mir = (const int2*)h->buf("q_mirror");
@@ -927,7 +945,7 @@ int isdf_coulomb_metric(isdf_handle* h, void* V_out) {
     CK(cudaMemcpyAsync(qlist, qh.list.data(), sizeof(int) * qh.list.size(), cudaMemcpyHostToDevice, h->st));
     ZOpt reps;
     reps.qmap = qlist;
-    ZM(h->prec == ISDF_FP64 ? "grid_work_z" : nullptr, 'R', 'T', rx, rx, ng, h->volume, xi, ng, xg, xi, ng, xg, Vxi, np, pp,
+    ZM(h->prec == ISDF_FP64 ? "fit" : nullptr, 'R', 'T', rx, rx, ng, h->volume, xi, ng, xg, xi, ng, xg, Vxi, np, pp,
        qh.count, reps);
   } else {
     // mixed: xi rows to float-float in place, the grid FFT in float-float, and
@@ -976,7 +994,7 @@ int isdf_coulomb_metric_eta(isdf_handle* h, void* V_out) {
                        cudaMemcpyDeviceToDevice, h->st));
     CK(grid_coulomb_fft(h->st, work + r.first * pg, np, r.first, r.second, h->cell, tw, gwork,
                         h->prec == ISDF_FP64));
-    ZM("grid_work_z", 'R', 'T', np, np, ng, h->volume, work + r.first * pg, ng, pg,
+    ZM("fit", 'R', 'T', np, np, ng, h->volume, work + r.first * pg, ng, pg,
              work + r.first * pg, ng, pg, Veta + r.first * pp, np, pp, r.second);
   }
   if (!qh.mirror.empty()) {
@@ -987,9 +1005,9 @@ int isdf_coulomb_metric_eta(isdf_handle* h, void* V_out) {
   // V_xi = conj(W) (V_eta W^T)
   double2* tmp = (double2*)h->ensure("W_work", sizeof(double2) * (size_t)nk * np * np);
   if (!tmp) return fail(h, ISDF_ERR_OOM, "workspace");
-  ZM("grid_work_z", 'N', 'T', np, np, np, 1.0, Veta, np, (int64_t)np * np, W, np, (int64_t)np * np, tmp, np,
+  ZM("fit", 'N', 'T', np, np, np, 1.0, Veta, np, (int64_t)np * np, W, np, (int64_t)np * np, tmp, np,
            (int64_t)np * np, nk);
-  ZM("grid_work_z", 'R', 'N', np, np, np, 1.0, W, np, (int64_t)np * np, tmp, np, (int64_t)np * np, Vxi, np,
+  ZM("fit", 'R', 'N', np, np, np, 1.0, W, np, (int64_t)np * np, tmp, np, (int64_t)np * np, Vxi, np,
            (int64_t)np * np, nk);
   return coulomb_tail(h, qh, np, Vxi, V_out);
 }
@@ -1077,7 +1095,7 @@ int isdf_fragment_eri(isdf_handle* h, int n_frag, const int32_t* n_orb, const vo
       if (f == 0) CK(scale_blocks(h->st, Lq, pp, nk, swd, Lw));
       {
         StageTimer stt(h, 3, frag_m_flops(nk, np, nf, nao, km));
-        ZM("tc_zwork", 'N', 'N', np, nf, nao, 1.0, X, nao, (int64_t)np * nao, Cf, nf, (int64_t)nao * nf, T,
+        ZM("frag_", 'N', 'N', np, nf, nao, 1.0, X, nao, (int64_t)np * nao, Cf, nf, (int64_t)nao * nf, T,
                  nf, (int64_t)np * nf, nk);
         CK(kdft_cols(h->st, T, (int64_t)np * nf, km, +1, +1, 0, 1.0, true));
         CK(pair_products(h->st, T, nk, np, nf, M));
@@ -1088,12 +1106,12 @@ int isdf_fragment_eri(isdf_handle* h, int n_frag, const int32_t* n_orb, const vo
         // nonzero columns of L^q
         StageTimer stt(h, 4, 8.0 * (double)n2 * np * sum_nv);
         for (const auto& r : runs)
-          ZM("tc_zwork", 'N', 'N', (int)n2, nj, np, 1.0, M + r.first * sq, np, sq, Lw + r.first * pp, np, pp,
+          ZM("frag_", 'N', 'N', (int)n2, nj, np, 1.0, M + r.first * sq, np, sq, Lw + r.first * pp, np, pp,
                    B + (int64_t)slot[r.first] * nj, (int64_t)nS * nj, nj, r.second);
       }
       {
         StageTimer stt(h, 5, 4.0 * (double)n2 * n2 * sum_nv);
-        ZM("tc_zwork", 'N', 'C', (int)n2, (int)n2, nS * nj, 1.0, B, (int64_t)nS * nj, 0, B, (int64_t)nS * nj, 0, E, n2, 0, 1);
+        ZM("frag_", 'N', 'C', (int)n2, (int)n2, nS * nj, 1.0, B, (int64_t)nS * nj, 0, B, (int64_t)nS * nj, 0, E, n2, 0, 1);
         if (h->q_sym) CK(eri_swapconj_sym(h->st, E, nf));
       }
       if (eri_out && eri_out[f]) CK(eri_permute(h->st, E, nf, 1.0 / nk, (double2*)eri_out[f]));
@@ -1240,7 +1258,7 @@ int isdf_fragment_eri(isdf_handle* h, int n_frag, const int32_t* n_orb, const vo
             double2* Tz = reinterpret_cast<double2*>(T);
             ZOpt t_opt;
             if (nao <= kZgemm7MaxK) t_opt.slices = 7;
-            ZM(t_opt.slices == 7 ? "tc_zwork" : nullptr, 'N', 'N', np, nf, nao, 1.0, Xz, nao, (int64_t)np * nao,
+            ZM(t_opt.slices == 7 ? "frag_" : nullptr, 'N', 'N', np, nf, nao, 1.0, Xz, nao, (int64_t)np * nao,
                (const double2*)C[f], nf, (int64_t)nao * nf, Tz, nf, (int64_t)np * nf, nk, t_opt);
             ffcomplex* Tff = reinterpret_cast<ffcomplex*>(Tz);
             CK(z2ff(h->st, Tz, Tff, (int64_t)nk * np * nf));
@@ -1410,9 +1428,9 @@ int isdf_ao_eri(isdf_handle* h, int n_quartet, const int32_t* quartets, void* ou
     CK(ao_pairs(h->st, X + k[0] * pa, X + k[1] * pa, np, nao, A));
     CK(ao_pairs(h->st, X + k[2] * pa, X + k[3] * pa, np, nao, Cc));
     // (mu nu|lam sig) = Nk A^T V^Q C with V^Q = L L^H: (L^T A)^T (L^H C)
-    ZM("zwork", 'T', 'N', nv, (int)nao2, np, 1.0, L, np, 0, A, nao2, 0, U, nao2, 0, 1);
-    ZM("zwork", 'C', 'N', nv, (int)nao2, np, 1.0, L, np, 0, Cc, nao2, 0, Wm, nao2, 0, 1);
-    ZM("zwork", 'T', 'N', (int)nao2, (int)nao2, nv, (double)nk, U, nao2, 0, Wm, nao2, 0, (double2*)out + (int64_t)n * nao2 * nao2, nao2, 0, 1);
+    ZM("call", 'T', 'N', nv, (int)nao2, np, 1.0, L, np, 0, A, nao2, 0, U, nao2, 0, 1);
+    ZM("call", 'C', 'N', nv, (int)nao2, np, 1.0, L, np, 0, Cc, nao2, 0, Wm, nao2, 0, 1);
+    ZM("call", 'T', 'N', (int)nao2, (int)nao2, nv, (double)nk, U, nao2, 0, Wm, nao2, 0, (double2*)out + (int64_t)n * nao2 * nao2, nao2, 0, 1);
   }
   return tc_status(h, "isdf_ao_eri");
 }
@@ -1442,14 +1460,14 @@ int isdf_sos_polarizability(isdf_handle* h, const void* C, int n_mo, int n_occ, 
   double2* chi = chi_out ? (double2*)chi_out : chi_w;
   CK(cudaMemcpyAsync(epsd, eps, sizeof(double) * (size_t)nk * n_mo, cudaMemcpyHostToDevice, h->st));
   // Y^k = X^k C^k (orbital values at the points, Eq. 14)
-  ZM("zwork", 'N', 'N', np, n_mo, nao, 1.0, X, nao, (int64_t)np * nao, (const double2*)C, n_mo,
+  ZM("call", 'N', 'N', np, n_mo, nao, 1.0, X, nao, (int64_t)np * nao, (const double2*)C, n_mo,
            (int64_t)nao * n_mo, Y, n_mo, (int64_t)np * n_mo, nk);
   // Go^k = Y_occ e^{+tau eps_i} Y_occ^H,  Gv^k = Y_vir e^{-tau eps_a} Y_vir^H (Eq. 15)
   CK(scale_cols(h->st, Y, nk, np, n_mo, 0, n_occ, epsd, +tau, Yo));
   CK(scale_cols(h->st, Y, nk, np, n_mo, n_occ, nvir, epsd, -tau, Yv));
-  ZM("zwork", 'N', 'C', np, np, n_occ, 1.0, Yo, n_occ, (int64_t)np * n_occ, Y, n_mo, (int64_t)np * n_mo,
+  ZM("call", 'N', 'C', np, np, n_occ, 1.0, Yo, n_occ, (int64_t)np * n_occ, Y, n_mo, (int64_t)np * n_mo,
            Go, np, pp, nk);
-  ZM("zwork", 'N', 'C', np, np, nvir, 1.0, Yv, nvir, (int64_t)np * nvir, Y + n_occ, n_mo, (int64_t)np * n_mo, Gv, np, pp, nk);
+  ZM("call", 'N', 'C', np, np, nvir, 1.0, Yv, nvir, (int64_t)np * nvir, Y + n_occ, n_mo, (int64_t)np * n_mo, Gv, np, pp, nk);
   // chi^Q_{IK} = sum_k Go^k_{KI} Gv^{k-Q}_{IK} (Eq. 13) by the convolution theorem, as
   // Algorithm 1 does for Pi^q: with hat(a)(R) = sum_k a(k) e^{+ik.R} and
   // check(b)(R) = sum_k b(k) e^{-ik.R},  chi = (1/Nk) DFT_-( hat(Go)^T o check(Gv) )
@@ -1460,9 +1478,9 @@ int isdf_sos_polarizability(isdf_handle* h, const void* C, int n_mo, int n_occ, 
   CK(kdft_cols(h->st, chi, pp, km, -1, -1, 0, 1.0 / nk, true));
   if (s_out) {
     // S = Nk^2 sum_Q tr[conj(V^Q) chi^Q conj(V^Q) (chi^{-Q})^T], V^Q = L^Q L^Q^H (Eq. 12)
-    ZM("zwork", 'N', 'C', np, np, l_cols(h), 1.0, Lq, np, pp, Lq, np, pp, Vq, np, pp, nk);
-    ZM("zwork", 'R', 'N', np, np, np, 1.0, Vq, np, pp, chi, np, pp, T1, np, pp, nk);
-    ZM("zwork", 'N', 'R', np, np, np, 1.0, T1, np, pp, Vq, np, pp, Go, np, pp, nk);  // Go reused
+    ZM("call", 'N', 'C', np, np, l_cols(h), 1.0, Lq, np, pp, Lq, np, pp, Vq, np, pp, nk);
+    ZM("call", 'R', 'N', np, np, np, 1.0, Vq, np, pp, chi, np, pp, T1, np, pp, nk);
+    ZM("call", 'N', 'R', np, np, np, 1.0, T1, np, pp, Vq, np, pp, Go, np, pp, nk);  // Go reused
     CK(sos_trace_parts(h->st, Go, chi, h->cell.kmesh, np, part));
     std::vector<double> hp(nk);
     CK(cudaMemcpyAsync(hp.data(), part, sizeof(double) * nk, cudaMemcpyDeviceToHost, h->st));
@@ -1487,12 +1505,12 @@ int isdf_exchange(isdf_handle* h, const void* P, void* K_out) {
   ENSURE(Vd, double2, "kx_V", (size_t)nk * np * np);
   ENSURE(t1, double2, "kx_t1", (size_t)nk * np * (nao > np ? nao : np));
   // rho^k = X^k P^k X^k^H
-  ZM("zwork", 'N', 'N', np, nao, nao, 1.0, X, nao, (int64_t)np * nao, (const double2*)P, nao,
+  ZM("call", 'N', 'N', np, nao, nao, 1.0, X, nao, (int64_t)np * nao, (const double2*)P, nao,
            (int64_t)nao * nao, t1, nao, (int64_t)np * nao, nk);
-  ZM("zwork", 'N', 'C', np, np, nao, 1.0, t1, nao, (int64_t)np * nao, X, nao, (int64_t)np * nao, rho, np,
+  ZM("call", 'N', 'C', np, np, nao, 1.0, t1, nao, (int64_t)np * nao, X, nao, (int64_t)np * nao, rho, np,
            (int64_t)np * np, nk);
   // V^q = L^q L^q^H
-  ZM("zwork", 'N', 'C', np, np, l_cols(h), 1.0, Lq, np, (int64_t)np * np, Lq, np, (int64_t)np * np, Vd, np,
+  ZM("call", 'N', 'C', np, np, l_cols(h), 1.0, Lq, np, (int64_t)np * np, Lq, np, (int64_t)np * np, Vd, np,
      (int64_t)np * np, nk);
   // Gamma^k = sum_k' (V^{k'-k})^T o rho^{k'}: DFT_- V, DFT_+ rho, transposed product, DFT_- / Nk
   CK(kdft_cols(h->st, Vd, (int64_t)np * np, km, -1, -1, 0, 1.0, true));
@@ -1500,9 +1518,9 @@ int isdf_exchange(isdf_handle* h, const void* P, void* K_out) {
   CK(hadamard_t(h->st, Vd, rho, np, nk, rho));
   CK(kdft_cols(h->st, rho, (int64_t)np * np, km, -1, -1, 0, 1.0 / nk, true));
   // K^k = -(1/Nk) X^k^H Gamma^k X^k
-  ZM("zwork", 'N', 'N', np, nao, np, 1.0, rho, np, (int64_t)np * np, X, nao, (int64_t)np * nao, t1, nao,
+  ZM("call", 'N', 'N', np, nao, np, 1.0, rho, np, (int64_t)np * np, X, nao, (int64_t)np * nao, t1, nao,
            (int64_t)np * nao, nk);
-  ZM("zwork", 'C', 'N', nao, nao, np, -1.0 / nk, X, nao, (int64_t)np * nao, t1, nao,
+  ZM("call", 'C', 'N', nao, nao, np, -1.0 / nk, X, nao, (int64_t)np * nao, t1, nao,
            (int64_t)np * nao, (double2*)K_out, nao, (int64_t)nao * nao, nk);
   return tc_status(h, "isdf_exchange");
 }
@@ -1573,7 +1591,7 @@ int isdf_get(isdf_handle* h, int what, void* out) {
       if (!h->has_xi) return fail(h, ISDF_ERR_STATE, "zeta not available (needs isdf_fit_zeta, before the metric)");
       // zeta = W^H xi with the rx stored rows of xi
       const int rx = h->xi_rows;
-      ZM("zwork", 'C', 'N', np, ng, rx, 1.0, (double2*)h->buf("W"), np, (int64_t)np * np, (double2*)h->buf("xi"),
+      ZM("call", 'C', 'N', np, ng, rx, 1.0, (double2*)h->buf("W"), np, (int64_t)np * np, (double2*)h->buf("xi"),
                ng, (int64_t)rx * ng, (double2*)out, ng, (int64_t)np * ng, nk);
       break;
     }

@@ -146,6 +146,88 @@ def test_a_call_does_not_report_the_wait_of_one_before(fake):
     g.close()
 
 
+def _one_entry(slices, m, n, k):
+    return (m + n) * ((k + 15) // 16 * 16) * slices * 4 + 256  # zgemm_tc_work_bytes of the fakes, one batch entry
+
+
+def test_slices_take_what_memory_there_is(fake):
+    """g of the FP64_TC fit has one fixed arithmetic: fewer k at a time, never another product."""
+    g = _handle(B.ISDF_FP64_TC)                       # n_p = 12, N_g = 120, N_AO = 4, Nk = 4
+    g.fit_zeta(1e-3)
+    calls = fake.fake_fma_calls(), fake.fake_tc_calls()
+    need = fake.fake_used()
+    assert fake.fake_last_work() > 3 * _one_entry(7, 12, 120, 4)
+    g.close()
+    g = _handle(B.ISDF_FP64_TC)
+    fake.fake_capacity(need - 2 * _one_entry(7, 12, 120, 4))
+    g.fit_zeta(1e-3)
+    assert (fake.fake_fma_calls(), fake.fake_tc_calls()) == (2 * calls[0], 2 * calls[1])
+    assert fake.fake_last_work() <= 2 * _one_entry(7, 12, 120, 4)
+    g.close()
+
+
+def test_a_product_of_fixed_arithmetic_without_memory_fails(fake):
+    g = _handle(B.ISDF_FP64_TC)
+    g.fit_zeta(1e-3)
+    full = fake.fake_used()
+    g.close()
+    g = _handle(B.ISDF_FP64_TC)
+    base = fake.fake_used()
+    # Pi and eta fit, one entry of slices does not
+    fake.fake_capacity(base + 16 * 4 * (12 * 12 + 12 * 120) + _one_entry(7, 12, 120, 4) - 1024)
+    assert base < full and _code(g.fit_zeta, 1e-3) == OOM
+    assert (fake.fake_tc_calls(), fake.fake_fma_calls()) == (1, 3)  # g of the first handle; Pi twice and xi once
+    assert _code(g.coulomb_metric) == STATE
+    g.close()
+
+
+def test_slices_keep_to_the_workspace_limit(fake):
+    g = _handle(B.ISDF_FP64_TC)
+    g.lib.isdf_set_workspace_limit(g.h, 1)
+    g.fit_zeta(1e-3)
+    assert fake.fake_last_work() == _one_entry(7, 12, 120, 4)
+    g.close()
+
+
+def test_slices_give_way_to_what_is_allocated_later(fake):
+    """What held without slices holds with them: the metric needs every byte."""
+    g = _wide()
+    fake.fake_rank(9)
+    g.fit_zeta(1e-3)
+    g.coulomb_metric()
+    g.close()
+    g = _wide()
+    g.fit_zeta(1e-3)
+    # V_xi is there; LtV, L and the small arrays of the metric follow
+    fake.fake_capacity(fake.fake_used() + 2 * 16 * 4 * 12 * 12)
+    g.coulomb_metric()
+    assert fake.fake_nulls() == 0
+    g.close()
+
+
+def test_slices_of_the_fp64_path_free_nothing_else(fake):
+    """Without memory for its slices an FP64 product runs as FMA chains and eta stays."""
+    g = _wide()
+    fake.fake_rank(9)
+    g.fit_zeta(1e-3)
+    g.coulomb_metric()
+    C = _Ptr(np.zeros((4, 8, 24), np.complex128))
+    g.fragment_eri([C], traces=False)
+    fma, used = fake.fake_fma_calls(), fake.fake_used()
+    g.close()
+    g = _wide()
+    g.fit_zeta(1e-3)
+    g.coulomb_metric()
+    # B = M L keeps one q at a time, E = B B^H nothing
+    fake.fake_capacity(used - 4 * _one_entry(8, 24 * 24, 12, 12) + (1 << 19))
+    base = fake.fake_fma_calls()
+    g.fragment_eri([C], traces=False)
+    assert fma == base and fake.fake_fma_calls() == base + 1
+    fake.fake_capacity(1 << 40)
+    g.coulomb_metric_eta()
+    g.close()
+
+
 class _Ptr:
     def __init__(self, a):
         self.a, self.shape = a, a.shape
