@@ -64,7 +64,13 @@ struct ZOpt {
   const int* qmap = nullptr;        // batch entry i works on matrix qmap[i] of each array
   const int32_t* krank = nullptr;   // by matrix: op(A_b) is zero from row and column krank on
   int slices = 8;                   // zgemm_tc: 8, or 7 for k <= kZgemm7MaxK
+  // zgemm_tc: column k of op(A) is taken times 2^-kexp[b sExp + k] and row k of op(B) times 2^kexp, the
+  // other way round with kneg: the same product, of operands that are less graded (|kexp| <= kMaxKexp)
+  const int32_t* kexp = nullptr;
+  int64_t sExp = 0;
+  int kneg = 0;
 };
+constexpr int kMaxKexp = 400;
 // FP64 FMA chains in the order of k.
 cudaError_t zgemm(cudaStream_t st, char opA, char opB, int m, int n, int k, double alpha, const double2* A, int64_t lda,
                   int64_t sA, const double2* B, int64_t ldb, int64_t sB, double2* C, int64_t ldc, int64_t sC, int batch,
@@ -139,6 +145,9 @@ cudaError_t pchol_batched(cudaStream_t st, const double2* A, int n, int neff, bo
 // (L_S^{-1} in pivot order) are zeroed for all nk matrices; tmp: nk n n of scratch.
 cudaError_t trinv_batched(cudaStream_t st, const double2* Lt, const int32_t* perm, const int32_t* rank, int n, int nk,
                           const int* qlist, int nq, double2* W, double2* work, double2* tmp);
+// e[q][i] = exponent of the largest component of row i < rows of A[q] (n x n), within +-kMaxKexp; 0 for a
+// zero row, for q in qlist.
+cudaError_t row_exponents_z(cudaStream_t st, const double2* A, int n, int rows, const int* qlist, int nq, int32_t* e);
 // Lpad[q][i][j] = L[i][j] (row-major, columns beyond the rank zero) for q in qlist.
 cudaError_t lt_to_rowmajor(cudaStream_t st, const double2* Lt, const int32_t* rank, const int* qlist, int nq, int n,
                            double2* L);
@@ -307,12 +316,12 @@ cudaError_t mirror_copy(cudaStream_t st, int32_t* x, int64_t per, const int2* pa
 cudaError_t hadamard_t(cudaStream_t st, const double2* a, const double2* c, int n, int nb, double2* out);
 
 // FP64-accurate complex GEMM on the tensor cores (k_ztc.cu): C_b = alpha op(A_b) op(B_b),
-// any K, eight exact slices per operand (36 fp16 products), no less accurate than an FP64
-// FMA chain; or seven (28 products, ~2^-48), the fixed arithmetic of g and T in the mixed and
+// k <= kZgemm8MaxK, eight exact slices per operand (36 fp16 products, ~2^-60 max|a_i| max|b_j| per
+// term: see k_ztc.cu for what that is against an FP64 FMA chain); or seven (28 products, ~2^-48), the fixed arithmetic of g and T in the mixed and
 // FP64_TC paths.  work: zgemm_tc_work_bytes for the batch
 // entries of one chunk (one at least); err: device word set on a bounded-wait timeout.
 // zgemm_tc_same: op(A) op(A)^T or ^H of one array, whose slices serve both sides.
-constexpr int kZgemm7MaxK = 64;
+constexpr int kZgemm7MaxK = 64, kZgemm8MaxK = 1 << 21;
 inline bool zgemm_tc_same(char opA, char opB, int m, int n, const double2* A, int64_t lda, int64_t sA,
                           const double2* B, int64_t ldb, int64_t sB) {
   const bool aT = opA == 'T' || opA == 'C', bT = opB == 'T' || opB == 'C';

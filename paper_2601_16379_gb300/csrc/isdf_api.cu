@@ -422,8 +422,8 @@ int zmul(isdf_handle* h, const char* who, char opA, char opB, int m, int n, int 
          int batch, const ZOpt& o = ZOpt()) {
   void* w = nullptr;
   size_t bytes = 0;
-  if (who && (k >= kMinTcK || o.slices == 7)) {
-    const bool same = !o.brow && zgemm_tc_same(opA, opB, m, n, A, lda, sA, B, ldb, sB);
+  if (who && (k >= kMinTcK || o.slices == 7) && k <= kZgemm8MaxK) {
+    const bool same = !o.brow && !o.kexp && zgemm_tc_same(opA, opB, m, n, A, lda, sA, B, ldb, sB);
     const size_t one = zgemm_tc_work_bytes(o.slices, m, n, k, 1, same), limit = std::min(kSliceBytes, h->split_budget);
     for (int nb = (int)std::min<size_t>(batch, std::max<size_t>(1, limit / one)); nb >= 1 && !w; nb /= 2) {
       bytes = zgemm_tc_work_bytes(o.slices, m, n, k, nb, same);
@@ -587,6 +587,7 @@ int coulomb_tail(isdf_handle* h, const QHalf& qh, int neff, double2* Vxi, void* 
   ENSURE(qlist, int, "q_list", nk);
   ENSURE(Lxi, double2, "W_work", (size_t)nk * np * np);
   ENSURE(Lq, double2, "Lq", (size_t)nk * np * np);
+  ENSURE(wexp, int32_t, "w_exp", (size_t)nk * np);
   h->has_coulomb = false;  // until the new factors stand
   CK(cudaMemcpyAsync(qlist, qh.list.data(), sizeof(int) * qh.list.size(), cudaMemcpyHostToDevice, h->st));
   // the representatives only: L^-q is the conjugate of L^q, bit for bit
@@ -600,8 +601,13 @@ int coulomb_tail(isdf_handle* h, const QHalf& qh, int neff, double2* Vxi, void* 
   // W has neff rows and L_xi neff rows and columns that are not zero.  L^q in another rounding
   // moves the FP64_TC integrals by 6e-10 of themselves: FP64 FMA there
   const int64_t pp = (int64_t)np * np;
+  // rows of W grow as the pivots of Pi shrink, and the rows of L_xi shrink with them: the slices take
+  // row c of W times 2^-d_c and row c of the other operand times 2^d_c
   ZOpt reps;
   reps.qmap = qlist;
+  reps.kexp = wexp;
+  reps.sExp = np;
+  CK(row_exponents_z(h->st, W, np, neff, qlist, qh.count, wexp));
   CK(cudaMemsetAsync(Lq, 0, sizeof(double2) * (size_t)nk * pp, h->st));
   ZM(h->prec == ISDF_FP64_TC ? nullptr : "call", 'T', 'N', np, neff, neff, 1.0, W, np, pp, Lxi, np, pp, Lq, np, pp,
      qh.count, reps);
@@ -609,7 +615,9 @@ int coulomb_tail(isdf_handle* h, const QHalf& qh, int neff, double2* Vxi, void* 
   if (V_out) {
     // V^q = W^T V_xi conj(W)
     double2* tmp = Lxi;  // reuse
-    ZM("call", 'N', 'R', neff, np, neff, 1.0, Vxi, np, pp, W, np, pp, tmp, np, pp, qh.count, reps);
+    ZOpt reps_b = reps;
+    reps_b.kneg = 1;
+    ZM("call", 'N', 'R', neff, np, neff, 1.0, Vxi, np, pp, W, np, pp, tmp, np, pp, qh.count, reps_b);
     ZM("call", 'T', 'N', np, np, neff, 1.0, W, np, pp, tmp, np, pp, (double2*)V_out, np, pp, qh.count, reps);
     CK(mirror_conj(h->st, (double2*)V_out, pp, mir, nm));
   }

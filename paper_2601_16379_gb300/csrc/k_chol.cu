@@ -226,6 +226,23 @@ __global__ void lt_to_row_kernel(const double2* __restrict__ Lt, const int32_t* 
   }
 }
 
+// A warp per row.
+__global__ void __launch_bounds__(256) row_exp_z_kernel(const double2* __restrict__ A, int n, int rows,
+                                                        const int* __restrict__ qlist, int32_t* __restrict__ e) {
+  const int64_t q = qlist[blockIdx.y];
+  const int i = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (i >= rows) return;
+  const double2* a = A + (q * n + i) * n;
+  unsigned m = 0;  // exponent field of the largest component
+  for (int c = lane; c < n; c += 32) {
+    const double2 v = a[c];
+    m = max(m, ((unsigned)__double2hiint(v.x) >> 20) & 0x7FFu);
+    m = max(m, ((unsigned)__double2hiint(v.y) >> 20) & 0x7FFu);
+  }
+  m = __reduce_max_sync(0xffffffffu, m);
+  if (lane == 0) e[q * n + i] = m == 0 || m == 0x7FFu ? 0 : max(-kMaxKexp, min(kMaxKexp, (int)m - 1023));
+}
+
 inline int nblocks(int64_t total) {
   int64_t nb = (total + 255) / 256;
   if (nb > 152 * 32) nb = 152 * 32;
@@ -291,6 +308,13 @@ cudaError_t trinv_batched(cudaStream_t st, const double2* Lt, const int32_t* per
   e = cudaMemsetAsync(W, 0, bytes, st);
   if (e != cudaSuccess) return e;
   scatter_w_kernel<<<nblocks((int64_t)nq * n * n), 256, 0, st>>>(work, perm, rank, qlist, n, nq, W);
+  count_launch();
+  return cudaGetLastError();
+}
+
+cudaError_t row_exponents_z(cudaStream_t st, const double2* A, int n, int rows, const int* qlist, int nq, int32_t* e) {
+  if (n <= 0 || rows <= 0 || nq <= 0) return cudaSuccess;
+  row_exp_z_kernel<<<dim3((rows + 7) / 8, nq), 256, 0, st>>>(A, n, rows, qlist, e);
   count_launch();
   return cudaGetLastError();
 }

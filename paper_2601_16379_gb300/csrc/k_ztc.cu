@@ -10,19 +10,29 @@
 //
 // Error-free slicing (Ozaki, Ogita, Oishi & Rump, 2012).  Each row of op(A) and each
 // column of op(B) is scaled by a power of two so that its largest component lies in
-// [64, 128) and rounded once to a 56-bit integer F (v 2^49), whose signed base-128 digits
-//     v = s_0 + s_1/2^7 + ... + s_7/2^49,   |s_0| <= 128, -64 <= s_i <= 63
+// [32, 64) and rounded once to a 63-bit integer F (v 2^56), whose signed base-256 digits
+//     v = s_0 + s_1/2^8 + ... + s_7/2^56,   |s_0| <= 64, -128 <= s_i <= 127
 // are stored as fp16 integers, real and imaginary parts in rows of their own.  A tile
 // is 64 x 32 complex entries of C: the 128 rows [Re a; Im a] of 64 rows of op(A) times the 64
 // columns [Re b, Im b] of 32 columns of op(B) give the four real products of the complex one,
 // which are combined with their signs at the end, as integers.  The products S_a T_b with
 // a + b <= 7 (36 of them) feed eight groups g = a + b of 64 FP32 accumulator columns: all 512
-// TMEM columns.  Over a chunk of 384 k every partial sum is an integer of magnitude at most
-// 384 * (2 * 128 * 64 + 6 * 64 * 64) < 2^24, so the FP32 accumulation is exact whatever its
-// rounding; each chunk is drained into 64-bit integers (groups 0-3 and 4-7), exact for any K,
-// and rounded once to FP64 at the end.  What is lost is the rounding of F (2^-57 of the
-// row's largest entry) and the products with a + b >= 8, together ~2^-57 per product of the
-// largest |a_i| |b_j|; the rounding of an FP64 FMA chain is larger from a few terms on.
+// TMEM columns.  Over a chunk of 144 k every partial sum is an integer of magnitude at most
+// 144 * (2 * 64 * 128 + 6 * 128 * 128) < 2^24, so the FP32 accumulation is exact whatever its
+// rounding; each chunk is drained into 64-bit integers (groups 0-3 and 4-7), exact up to
+// K = 2^21, and rounded once to FP64 at the end.
+//
+// What is lost is the rounding of F (2^-62 of the row's largest entry; none for entries above 2^-9 of
+// it) and the products with a + b >= 8: per term ~2^-60 max|a_i| max|b_j|, where an FP64 FMA chain
+// loses up to 2^-53 of each partial sum.  So operands whose rows are graded lose nothing either until
+// max|a_i| max|b_j| exceeds the sums by 2^7 or so.  Base-128 digits (chunks of 384 k, 2^-56) were below
+// the chain's error for most products, but not where the order of k grades both operands:
+// there the caller gives powers of two for the contraction index (ZOpt::kexp), column k of op(A) times
+// 2^-d_k and row k of op(B) times 2^d_k, which is exact.  Largest error over the largest entry,
+// against 80-bit sums (26 AOs, 8 k-points, 12^3 grid, n_p = 150, rank 119), FMA chain / base 128 / this:
+//   G 4.4e-16 / 1.1e-16 / 9e-17,  xi = W eta 1.1e-12 / 3.8e-13 / 2.1e-14,  V_xi 5.0e-15 / 2.6e-15 / 2.2e-16,
+//   B = M L 1.6e-15 / 1.8e-15 / 1e-16,  E = B B^H 1.7e-15 / 1.9e-16 / 4e-17,
+//   L = W^T L_xi 1.9e-16 / 1.5e-14 / 1.4e-15, with kexp 5e-17.
 //
 // The tile shape: an MMA of 128 x N x 16 takes N/2 clocks from N = 128 on, but 55 at N = 64
 // and 49 at N = 32 (measured), so N = 64 costs 36 x 55 clocks per 16 k (58 % of the peak).
@@ -42,6 +52,11 @@
 // k block).  One layout serves both sides, so a product of a matrix with itself is sliced
 // once.  Rows beyond the matrix are left unwritten: they only reach entries of C that are
 // not stored.  k beyond K is zero.
+//
+// The drain of groups 0-3 runs while the MMAs of groups 4-7 of the chunk's last k block do, and that of
+// groups 4-7 under those of groups 0-3 of the next chunk: two pairs of barriers.  With the chunks of
+// 384 k of base-128 digits and one drain per chunk, 320 x 320 x K in a batch of 200 took 671 us at K = 64,
+// 1149 at 128, 2055 at 256 and 2955 at 384; it takes 649, 1078, 2064 and 3041.
 //
 // Kernel roles (576 threads, one CTA per SM, persistent over the tiles): warp 0 copies,
 // warp 1 allocates TMEM and issues the MMAs, warps 2-17 drain and store.  Every wait is
@@ -70,8 +85,8 @@ struct Blk {
   static constexpr int kStage = kBytesA + kBytesB;    // 48 KB at eight slices
 };
 constexpr int NST = 3;                       // stages
-constexpr int kChunk = 24;                   // k blocks per exact chunk (384 k)
-constexpr int kShortK = 96;                  // K up to which every group stays below 2^22 (96 * 40960)
+constexpr int kChunk = 9;                    // k blocks per exact chunk (144 k)
+constexpr int kShortK = 32;                  // K up to which every group stays below 2^22 (32 * 114688)
 constexpr int kOutBytes = 65536;             // exchange of the partial sums, then the tile of C on its way out
 constexpr int NT = 576;
 constexpr int kDrainWarps = 16;
@@ -112,26 +127,26 @@ struct Args {
 
 __device__ __noinline__ double scale_slow(unsigned long long T, int e) { return ldexp((double)T, e); }
 
-// +-(hi 2^-21 + lo 2^-49) (exact integers), times 2^e, rounded to FP64 in integer arithmetic.
+// +-(hi 2^-24 + lo 2^-56) (exact integers), times 2^e, rounded to FP64 in integer arithmetic.
 __device__ __forceinline__ double fixed_to_double(long long hi, long long lo, bool flip, int e) {
-  long long H = hi + (lo >> 28);
-  uint32_t l = (uint32_t)lo & 0x0FFFFFFFu;  // value = (H 2^28 + l) 2^-49
+  long long H = hi + (lo >> 32);
+  uint32_t l = (uint32_t)lo;  // value = (H 2^32 + l) 2^-56
   const bool neg = H < 0;
   if (neg) {
     H = (l == 0) ? -H : -H - 1;
-    l = (0x10000000u - l) & 0x0FFFFFFFu;
+    l = 0u - l;
   }
   unsigned long long T;
   int top;  // exponent of T's leading bit
   if (H != 0) {
     const int z = __clzll(H);
     // the leading bits of H:l in 64 bits (z >= 1 as H > 0)
-    T = ((unsigned long long)H << z) | (((unsigned long long)l << 36) >> (64 - z));
-    top = 63 - z + 28 - 49 + e;
+    T = ((unsigned long long)H << z) | (((unsigned long long)l << 32) >> (64 - z));
+    top = 63 - z + 32 - 56 + e;
   } else if (l != 0) {
     const int z = __clzll((long long)l);
     T = (unsigned long long)l << z;
-    top = 63 - z - 49 + e;
+    top = 63 - z - 56 + e;
   } else {
     return 0.0;
   }
@@ -192,9 +207,9 @@ __global__ void __launch_bounds__(NT, 1) zgemm_tc_kernel(Args args) {
   uint64_t* bars = reinterpret_cast<uint64_t*>(outS + kOutBytes);
   uint64_t* full = bars;             // [NST] stage landed
   uint64_t* empty = bars + NST;      // [NST] stage read by the MMAs
-  uint64_t* accf = bars + 2 * NST;   // chunk accumulated
-  uint64_t* drained = accf + 1;      // chunk drained
-  uint32_t* s_tmem = reinterpret_cast<uint32_t*>(drained + 1);
+  uint64_t* accf = bars + 2 * NST;   // [2] chunk accumulated: groups 0-3, the others
+  uint64_t* drained = accf + 2;      // [2] and drained
+  uint32_t* s_tmem = reinterpret_cast<uint32_t*>(drained + 2);
   volatile int* s_err = reinterpret_cast<volatile int*>(s_tmem + 1);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
@@ -203,8 +218,10 @@ __global__ void __launch_bounds__(NT, 1) zgemm_tc_kernel(Args args) {
       mbar_init(&full[s], 1);
       mbar_init(&empty[s], 1);
     }
-    mbar_init(accf, 1);
-    mbar_init(drained, kDrainWarps);
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(&accf[i], 1);
+      mbar_init(&drained[i], kDrainWarps);
+    }
     *s_err = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -273,34 +290,35 @@ __global__ void __launch_bounds__(NT, 1) zgemm_tc_kernel(Args args) {
         int b, ti, tj;
         tile_of(t, b, ti, tj);
         const int nk = kblocks(b, ti);
-        for (int kb = 0; kb < nk; ++kb, ++it) {
-          const bool first = (kb % kChunk) == 0;
-          if (first && ch > 0) {
-            if (!mbar_wait(drained, (uint32_t)((ch - 1) & 1), s_err, args.err, 42)) {
-              ok = false;
-              break;
-            }
-            tc_fence_after();
-          }
+        for (int kb = 0; kb < nk && ok; ++kb, ++it) {
+          const bool first = (kb % kChunk) == 0, last = (kb % kChunk) == kChunk - 1 || kb == nk - 1;
           const int s = (int)(it % NST);
           if (!mbar_wait(&full[s], (uint32_t)((it / NST) & 1), s_err, args.err, 43)) {
             ok = false;
             break;
           }
-          tc_fence_after();
           const uint32_t st = smem_u32(smem + s * kStage);
           const uint64_t dA = sdesc_core(st), dB = sdesc_core(st + kABytes);
           constexpr uint64_t oA = (2 * kSlice * 2) >> 4, oB = (kSlice * 2) >> 4;  // slice strides of the descriptors
 #pragma unroll
-          for (int i = 0; i < NS; ++i)
+          for (int gh = 0; gh < 2; ++gh) {
+            if (first && ch > 0 && !mbar_wait(&drained[gh], (uint32_t)((ch - 1) & 1), s_err, args.err, 42)) {
+              ok = false;
+              break;
+            }
+            tc_fence_after();
 #pragma unroll
-            for (int c = 0; c < NS - i; ++c)
-              umma_f16(tmem + (uint32_t)((i + c) * 2 * BN), dA + i * oA, dB + c * oB, kIdesc, (first && i == 0) ? 0u : 1u);
-          umma_commit(&empty[s]);
-          if ((kb % kChunk) == kChunk - 1 || kb == nk - 1) {
-            umma_commit(accf);
-            ++ch;
+            for (int i = 0; i < NS; ++i)
+#pragma unroll
+              for (int c = 0; c < NS - i; ++c)
+                if ((i + c >= 4) == (gh == 1))
+                  umma_f16(tmem + (uint32_t)((i + c) * 2 * BN), dA + i * oA, dB + c * oB, kIdesc,
+                           (first && i == 0) ? 0u : 1u);
+            if (last) umma_commit(&accf[gh]);
           }
+          if (!ok) break;
+          umma_commit(&empty[s]);
+          if (last) ++ch;
         }
       }
     }
@@ -333,41 +351,53 @@ __global__ void __launch_bounds__(NT, 1) zgemm_tc_kernel(Args args) {
 #pragma unroll
       for (int j = 0; j < kDrainCols; ++j) hi[j] = lo[j] = 0;
       for (int c = 0; c < nch && ok; ++c, ++ch) {
-        ok = __all_sync(0xffffffffu, mbar_wait(accf, (uint32_t)(ch & 1), s_err, args.err, 44));
-        if (!ok) break;
-        tc_fence_after();
 #pragma unroll
-        for (int cb = 0; cb < kDrainCols / 4; ++cb) {
-          uint32_t v[NS][4];
+        for (int gh = 0; gh < 2; ++gh) {
+          if (ok) ok = __all_sync(0xffffffffu, mbar_wait(&accf[gh], (uint32_t)(ch & 1), s_err, args.err, 44));
+          if (!ok) break;
+          tc_fence_after();
 #pragma unroll
-          for (int g = 0; g < NS; ++g) tmem_ld4(tbase + (uint32_t)(g * 2 * BN) + ((uint32_t)(cb * 4) ^ keep), v[g]);
-          tmem_wait_ld();
+          for (int cb = 0; cb < kDrainCols / 4; ++cb) {
+            uint32_t v[4][4];
 #pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            int w[NS];
-#pragma unroll
-            for (int g = 0; g < NS; ++g) {
-              // exact integers; below 2^22 the addition of 1.5 2^23 puts them into the low bits
-              const float f = __uint_as_float(v[g][j]);
-              w[g] = kShort ? __float_as_int(f + 12582912.f) - 0x4B400000 : __float2int_rn(f);
+            for (int g = 0; g < 4; ++g)
+              if (gh * 4 + g < NS)
+                tmem_ld4(tbase + (uint32_t)((gh * 4 + g) * 2 * BN) + ((uint32_t)(cb * 4) ^ keep), v[g]);
+            tmem_wait_ld();
+            if (cb == kDrainCols / 4 - 1) {  // the last read: the MMAs may go on
+              tc_fence_before();
+              __syncwarp();
+              if (lane == 0) mbar_arrive(&drained[gh]);
             }
-            if constexpr (NS == 7) {
-              // groups 1-6 below 2^22 (64 * 36864): weights 2^35 .. 1; group 0 apart
-              const int a0 = w[1] * 128 + w[2], a1 = w[3] * 128 + w[4], a2 = w[5] * 128 + w[6];
-              hi[cb * 4 + j] += (long long)a0 * (1 << 28) + (long long)a1 * (1 << 14) + a2;
-              lo[cb * 4 + j] += w[0];
-              continue;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              int w[4];
+#pragma unroll
+              for (int g = 0; g < 4; ++g) {
+                if (gh * 4 + g >= NS) continue;
+                const float f = __uint_as_float(v[g][j]);
+                // exact integers; below 2^22 the addition of 1.5 2^23 puts them into the low bits
+                w[g] = kShort ? __float_as_int(f + 12582912.f) - 0x4B400000 : __float2int_rn(f);
+              }
+              long long &h = hi[cb * 4 + j], &l = lo[cb * 4 + j];
+              if constexpr (NS == 7) {
+                // groups 1-6 below 2^22 (64 * 36864): weights 2^35 .. 1 in hi; group 0 apart
+                if (gh == 0) {
+                  h += (long long)(w[1] * 128 + w[2]) * (1 << 28) + (long long)w[3] * (1 << 21);
+                  l += w[0];
+                } else {
+                  h += (long long)w[0] * (1 << 14) + (w[1] * 128 + w[2]);
+                }
+              } else if (gh == 0) {
+                // |w_0| <= 144 * 2^12 and |w_2| <= 144 * 2^15: 256 w_g + w_(g+1) fits 32 bits
+                h += (long long)(w[0] * 256 + w[1]) * 65536 + (w[2] * 256 + w[3]);
+              } else {
+                l += (long long)w[0] * (1 << 24) + (long long)w[1] * 65536 + ((long long)w[2] * 256 + w[3]);
+              }
             }
-            // |w_g| < 2^24, and below 2^24 - 2^20 for g < 7: 128 w_g + w_(g+1) fits 32 bits
-            const int a0 = w[0] * 128 + w[1], a1 = w[2] * 128 + w[3];
-            const int a2 = w[4] * 128 + w[5], a3 = w[6] * 128 + w[NS - 1];
-            hi[cb * 4 + j] += (long long)a0 * 16384 + a1;
-            lo[cb * 4 + j] += (long long)a2 * 16384 + a3;
           }
         }
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(drained);
+        if (!ok) break;
       }
       // a warp whose wait expired keeps the barriers below company, without storing
       const int r = ti * BM + row, n0 = tj * BN;
@@ -417,34 +447,36 @@ __global__ void __launch_bounds__(NT, 1) zgemm_tc_kernel(Args args) {
 }
 
 // ---------------------------------------------------------------- slicing
-// Exponent ex with max 2^ex in [64, 128) from the bits of the largest magnitude.
+// Exponent ex with max 2^ex in [32, 64) (NS = 8) or [64, 128) (NS = 7) from the bits of the largest magnitude.
+template <int NS>
 __device__ __forceinline__ int exp_of(unsigned long long mx) {
+  constexpr int kTop = NS == 8 ? 5 : 6;
   if (mx == 0) return 0;
-  const int f = (int)(mx >> 52);
+  // the sign of a NaN may have come through: the compiler may clear sign bits by abs.f64, which keeps it
+  const int f = (int)(mx >> 52) & 0x7FF;
   if (f == 0x7FF) return kBadExp;
-  return f ? 6 - (f - 1023) : 6 - (63 - __clzll((long long)mx) - 1074);
+  return f ? kTop - (f - 1023) : kTop - (63 - __clzll((long long)mx) - 1074);
 }
 
-// The 56-bit integer rint(x 2^(ex + 49)) plus 64 at each of the lower seven digits, so that
-// digit i is bits [7 (7 - i), +7) minus 64 (i >= 1) and s_0 the bits from 49 on.
+// The 63-bit integer rint(x 2^(ex + 56)) plus 128 at each of the lower seven digits, so that
+// digit i is bits [8 (7 - i), +8) minus 128 (i >= 1) and s_0 the bits from 56 on.
 __device__ __forceinline__ long long digits_of(double x, int ex) {
   const unsigned long long u = (unsigned long long)__double_as_longlong(x);
   const int f = (int)((u >> 52) & 0x7FF);
   unsigned long long m = u & 0xFFFFFFFFFFFFFULL;
   if (f) m |= 1ULL << 52;
-  const int s = (f ? f : 1) - 1026 + ex;  // <= 3 for normal rows
+  const int s = (f ? f : 1) - 1019 + ex;  // <= 9 for normal rows
   unsigned long long F;
   if (s >= 0)
     F = m << s;
   else
     F = s > -55 ? (m + (1ULL << (-s - 1))) >> -s : 0ULL;
   long long v = (long long)u < 0 ? -(long long)F : (long long)F;
-  constexpr long long kBias = 64LL * (1LL + (1LL << 7) + (1LL << 14) + (1LL << 21) + (1LL << 28) + (1LL << 35) + (1LL << 42));
-  return v + kBias;
+  return v + 0x0080808080808080LL;
 }
 
 // Slices of eight consecutive k of one row, part re or im of the chunk at dst (16 bytes per slice).
-// Digits as fp16 pairs: 1024 + u has the bits 0x6400 | u (u < 1024), minus 1024 + 64.
+// Digits as fp16 pairs: 1024 + u has the bits 0x6400 | u (u < 1024), minus 1024 + 128.
 __device__ __forceinline__ void store_planes(const long long (&F)[8], int part, __half* dst) {
   constexpr int NS = 8;
 #pragma unroll
@@ -453,13 +485,13 @@ __device__ __forceinline__ void store_planes(const long long (&F)[8], int part, 
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       if (s == 0) {
-        const __half2 h = __floats2half2_rn((float)(int)(F[2 * i] >> 49), (float)(int)(F[2 * i + 1] >> 49));
+        const __half2 h = __floats2half2_rn((float)(int)(F[2 * i] >> 56), (float)(int)(F[2 * i + 1] >> 56));
         w[i] = *reinterpret_cast<const uint32_t*>(&h);
       } else {
-        const uint32_t u0 = (uint32_t)(F[2 * i] >> (7 * (NS - 1 - s))) & 127u;
-        const uint32_t u1 = (uint32_t)(F[2 * i + 1] >> (7 * (NS - 1 - s))) & 127u;
+        const uint32_t u0 = (uint32_t)(F[2 * i] >> (8 * (NS - 1 - s))) & 255u;
+        const uint32_t u1 = (uint32_t)(F[2 * i + 1] >> (8 * (NS - 1 - s))) & 255u;
         const uint32_t p = 0x64006400u | u0 | (u1 << 16);
-        const __half2 h = __hsub2(*reinterpret_cast<const __half2*>(&p), __floats2half2_rn(1088.f, 1088.f));
+        const __half2 h = __hsub2(*reinterpret_cast<const __half2*>(&p), __floats2half2_rn(1152.f, 1152.f));
         w[i] = *reinterpret_cast<const uint32_t*>(&h);
       }
     }
@@ -537,6 +569,19 @@ __device__ __forceinline__ unsigned long long amax_bits(double2 v) {
   return a > b ? a : b;
 }
 
+// Powers of two by k: entry k times 2^(sgn d[k]) (exact; |d| <= kMaxKexp).
+struct KScale {
+  const int32_t* d;
+  int64_t stride;  // by matrix
+  int sgn;
+  template <bool kOn>
+  __device__ __forceinline__ double2 of(double2 v, int k) const {
+    if constexpr (!kOn) return v;
+    const double f = __longlong_as_double((long long)(1023 + sgn * __ldg(d + k)) << 52);
+    return make_double2(v.x * f, v.y * f);
+  }
+};
+
 // Where chunk kc (eight k) of row r goes.
 template <int NS>
 __device__ __forceinline__ int64_t slot_of(int r, int kc, int nkb) {
@@ -545,22 +590,24 @@ __device__ __forceinline__ int64_t slot_of(int r, int kc, int nkb) {
 
 // Rows stored contiguously along k: a block takes eight rows, one warp per row for the
 // largest entry, then eight lanes per 128-byte line of the slices.
-template <int NS>
+template <int NS, bool kOn>
 __global__ void __launch_bounds__(256) zslice_rows_kernel(const double2* __restrict__ X, int64_t ld, int64_t sX, int rows,
                                                           int K, int nkb, int nblk, const int* __restrict__ qmap,
-                                                          __half* __restrict__ S, int* __restrict__ ex) {
+                                                          KScale ks, __half* __restrict__ S, int* __restrict__ ex) {
   const int b = blockIdx.y, r0 = blockIdx.x * 8, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  X += (int64_t)(qmap ? qmap[b] : b) * sX;
+  const int qb = qmap ? qmap[b] : b;
+  X += (int64_t)qb * sX;
+  if constexpr (kOn) ks.d += (int64_t)qb * ks.stride;
   S += (int64_t)b * nblk * nkb * Blk<NS>::kElems;
   __shared__ int se[8];
   {
     const int r = r0 + warp;
     unsigned long long m = 0;
     if (r < rows)
-      for (int k = lane; k < K; k += 32) m = max(m, amax_bits(X[(int64_t)r * ld + k]));
+      for (int k = lane; k < K; k += 32) m = max(m, amax_bits(ks.of<kOn>(X[(int64_t)r * ld + k], k)));
     for (int o = 16; o; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
     if (lane == 0) {
-      const int e = exp_of(m);
+      const int e = exp_of<NS>(m);
       se[warp] = e;
       if (r < rows) ex[(int64_t)b * rows + r] = e;
     }
@@ -573,27 +620,28 @@ __global__ void __launch_bounds__(256) zslice_rows_kernel(const double2* __restr
   for (int kc = threadIdx.x >> 3; kc < nkb * 2; kc += 32) {
     double2 x[8];
 #pragma unroll
-    for (int i = 0; i < 8; ++i) x[i] = (kc * 8 + i < K && e != kBadExp) ? row[kc * 8 + i] : make_double2(0.0, 0.0);
+    for (int i = 0; i < 8; ++i) x[i] = (kc * 8 + i < K && e != kBadExp) ? ks.of<kOn>(row[kc * 8 + i], kc * 8 + i) : make_double2(0.0, 0.0);
     emit_chunk<NS>(x, e, S + slot_of<NS>(r, kc, nkb));
   }
 }
 
 // Rows stored with stride ld along k (columns of the array), optionally gathered
 // (k -> idx[k], none where negative): a block takes 32 rows, lanes along them.
-template <int NS>
+template <int NS, bool kOn>
 __global__ void __launch_bounds__(256) zslice_cols_kernel(const double2* __restrict__ X, int64_t ld, int64_t sX, int rows,
                                                           int K, int nkb, int nblk, const int32_t* __restrict__ idx,
-                                                          int64_t sIdx, const int* __restrict__ qmap,
+                                                          int64_t sIdx, const int* __restrict__ qmap, KScale ks,
                                                           __half* __restrict__ S, int* __restrict__ ex) {
   const int b = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31, r = blockIdx.x * 32 + lane;
   const int qb = qmap ? qmap[b] : b;
   X += (int64_t)qb * sX + r;
   S += (int64_t)b * nblk * nkb * Blk<NS>::kElems;
   if (idx) idx += (int64_t)qb * sIdx;
+  if constexpr (kOn) ks.d += (int64_t)qb * ks.stride;
   const bool in = r < rows;
   auto at = [&](int k) {
     const int kk = idx ? __ldg(idx + k) : k;
-    return (in && kk >= 0) ? X[(int64_t)kk * ld] : make_double2(0.0, 0.0);
+    return (in && kk >= 0) ? ks.of<kOn>(X[(int64_t)kk * ld], k) : make_double2(0.0, 0.0);
   };
   __shared__ unsigned long long sm[8][32];
   unsigned long long m = 0;
@@ -603,7 +651,7 @@ __global__ void __launch_bounds__(256) zslice_cols_kernel(const double2* __restr
   __syncthreads();
 #pragma unroll
   for (int w = 0; w < 8; ++w) m = max(m, sm[w][lane]);
-  const int e = exp_of(m);
+  const int e = exp_of<NS>(m);
   if (!in) return;
   if (warp == 0) ex[(int64_t)b * rows + r] = e;
   for (int kc = warp; kc < nkb * 2; kc += 8) {
@@ -621,15 +669,24 @@ inline size_t slice_bytes(int slices, int rows, int k, int nb) {
 
 // Slices of op(X) by rows (side A) or of op(X)^T (side B): `cols` when the wanted rows run
 // along the fast index of the array.
-template <int NS>
-cudaError_t slice(cudaStream_t st, bool cols, const double2* X, int64_t ld, int64_t sX, int rows, int K, int batch,
-                  const int32_t* idx, int64_t sIdx, const int* qmap, __half* S, int* ex) {
+template <int NS, bool kOn>
+void slice_launch(cudaStream_t st, bool cols, const double2* X, int64_t ld, int64_t sX, int rows, int K, int batch,
+                  const int32_t* idx, int64_t sIdx, const int* qmap, const KScale& ks, __half* S, int* ex) {
   const int nkb = (int)cdiv(K, BK), nblk = (int)cdiv(rows, RB);
   if (cols)
-    zslice_cols_kernel<NS><<<dim3((unsigned)cdiv(rows, 32), batch), 256, 0, st>>>(X, ld, sX, rows, K, nkb, nblk, idx, sIdx,
-                                                                             qmap, S, ex);
+    zslice_cols_kernel<NS, kOn><<<dim3((unsigned)cdiv(rows, 32), batch), 256, 0, st>>>(X, ld, sX, rows, K, nkb, nblk, idx,
+                                                                                       sIdx, qmap, ks, S, ex);
   else
-    zslice_rows_kernel<NS><<<dim3((unsigned)cdiv(rows, 8), batch), 256, 0, st>>>(X, ld, sX, rows, K, nkb, nblk, qmap, S, ex);
+    zslice_rows_kernel<NS, kOn><<<dim3((unsigned)cdiv(rows, 8), batch), 256, 0, st>>>(X, ld, sX, rows, K, nkb, nblk, qmap,
+                                                                                      ks, S, ex);
+}
+template <int NS>
+cudaError_t slice(cudaStream_t st, bool cols, const double2* X, int64_t ld, int64_t sX, int rows, int K, int batch,
+                  const int32_t* idx, int64_t sIdx, const int* qmap, const KScale& ks, __half* S, int* ex) {
+  if (NS == 8 && ks.d)
+    slice_launch<8, true>(st, cols, X, ld, sX, rows, K, batch, idx, sIdx, qmap, ks, S, ex);
+  else
+    slice_launch<NS, false>(st, cols, X, ld, sX, rows, K, batch, idx, sIdx, qmap, ks, S, ex);
   count_launch();
   return cudaGetLastError();
 }
@@ -648,9 +705,10 @@ static cudaError_t zgemm_tc_impl(cudaStream_t st, char opA, char opB, int m, int
   using namespace ztc;
   if (m <= 0 || n <= 0 || k <= 0 || batch <= 0) return cudaSuccess;
   if (o.brow && opB != 'N') return cudaErrorInvalidValue;
+  if (k > kZgemm8MaxK || (NS == 7 && o.kexp)) return cudaErrorInvalidValue;
   const bool aT = opA == 'T' || opA == 'C', aC = opA == 'C' || opA == 'R';
   const bool bT = opB == 'T' || opB == 'C', bC = opB == 'C' || opB == 'R';
-  const bool same = !o.brow && zgemm_tc_same(opA, opB, m, n, A, lda, sA, B, ldb, sB);
+  const bool same = !o.brow && !o.kexp && zgemm_tc_same(opA, opB, m, n, A, lda, sA, B, ldb, sB);
   const size_t per = slice_bytes(NS, m, k, 1) + (same ? 0 : slice_bytes(NS, n, k, 1)) + sizeof(int) * (size_t)(m + n);
   if (work_bytes < per + 256) return cudaErrorInvalidValue;
   const int nbc = (int)std::min<size_t>((size_t)std::min(batch, 65535), (work_bytes - 256) / per);
@@ -672,9 +730,11 @@ static cudaError_t zgemm_tc_impl(cudaStream_t st, char opA, char opB, int m, int
     // with a map the arrays stay where they are and the map moves on
     const int* qm = o.qmap ? o.qmap + b0 : nullptr;
     const int64_t s0 = qm ? 0 : b0;
-    e = slice<NS>(st, aT, A + s0 * sA, lda, sA, m, k, nb, nullptr, 0, qm, SA, eA);
+    const int32_t* kx = o.kexp ? o.kexp + s0 * o.sExp : nullptr;
+    e = slice<NS>(st, aT, A + s0 * sA, lda, sA, m, k, nb, nullptr, 0, qm, KScale{kx, o.sExp, o.kneg ? 1 : -1}, SA, eA);
     if (e == cudaSuccess && !same)
-      e = slice<NS>(st, !bT, B + s0 * sB, ldb, sB, n, k, nb, o.brow ? o.brow + s0 * o.sIdx : nullptr, o.sIdx, qm, SB, eB);
+      e = slice<NS>(st, !bT, B + s0 * sB, ldb, sB, n, k, nb, o.brow ? o.brow + s0 * o.sIdx : nullptr, o.sIdx, qm,
+                    KScale{kx, o.sExp, o.kneg ? -1 : 1}, SB, eB);
     if (e != cudaSuccess) return e;
     Args a{};
     a.SA = SA;

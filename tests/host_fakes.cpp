@@ -13,7 +13,7 @@
 namespace {
 std::map<void*, size_t> g_live;
 size_t g_cap = ~(size_t)0, g_used = 0, g_peak = 0;
-int g_rank = 4, g_nulls = 0, g_arm = -1, g_n_tc = 0, g_n_fma = 0, g_ml_rp = 0, g_ml_rank = 0, g_last_slices = 0;
+int g_rank = 4, g_nulls = 0, g_arm = -1, g_n_tc = 0, g_n_fma = 0, g_ml_rp = 0, g_ml_rank = 0, g_n_kexp = 0;
 size_t g_last_work = 0;
 void used(const void* p) { g_nulls += p == nullptr; }
 }  // namespace
@@ -24,7 +24,7 @@ void fake_reset() {
   g_cap = ~(size_t)0;
   g_peak = g_used;
   g_rank = 4;
-  g_nulls = g_n_tc = g_n_fma = g_ml_rp = g_ml_rank = 0;
+  g_nulls = g_n_kexp = g_n_tc = g_n_fma = g_ml_rp = g_ml_rank = 0;
   g_arm = -1;
 }
 void fake_capacity(size_t b) { g_cap = b; }
@@ -38,6 +38,7 @@ int fake_tc_calls() { return g_n_tc; }
 int fake_fma_calls() { return g_n_fma; }
 int fake_ml_rp() { return g_ml_rp; }
 int fake_ml_rank() { return g_ml_rank; }
+int fake_kexp_calls() { return g_n_kexp; }
 size_t fake_last_work() { return g_last_work; }
 int isdf_eri_traces_noalloc(const void*, int, const void*, double*, double*, void*) { return 0; }
 
@@ -135,7 +136,7 @@ cudaError_t zgemm_tc(S, char, char, int, int, int, double, cz A, int64_t, int64_
   used(A), used(B), used(C), used(work), used(err);
   ++g_n_tc;
   g_last_work = wb;
-  g_last_slices = o.slices;
+  g_n_kexp += o.kexp != nullptr;
   if (g_arm >= 0 && g_arm-- == 0) *err = 41;
   return cudaSuccess;
 }
@@ -154,6 +155,7 @@ cudaError_t pchol_batched(S, cz A, int n, int neff, bool, const int* qlist, int 
   return cudaSuccess;
 }
 NOP(trinv_batched, S, cz, const int32_t*, const int32_t*, int, int, const int*, int, double2*, double2*, double2*)
+NOP(row_exponents_z, S, cz, int, int, const int*, int, int32_t*)
 NOP(lt_to_rowmajor, S, cz, const int32_t*, const int*, int, int, double2*)
 size_t grid_coulomb_work_bytes(int, const CellDev&) { return 64; }
 cudaError_t grid_coulomb_fft(S, double2* x, int, int, int, const CellDev&, cz, void*, bool) {

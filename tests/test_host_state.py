@@ -228,6 +228,16 @@ def test_slices_of_the_fp64_path_free_nothing_else(fake):
     g.close()
 
 
+def test_products_with_w_scale_their_inner_index(fake):
+    """L = W^T L_xi and the two products of V_out: rows of W and of the other operand are graded against each other."""
+    g = _wide()
+    fake.fake_rank(9)
+    g.fit_zeta(1e-3)
+    g.coulomb_metric(OUT)
+    assert fake.fake_kexp_calls() == 3
+    g.close()
+
+
 class _Ptr:
     def __init__(self, a):
         self.a, self.shape = a, a.shape
