@@ -489,10 +489,10 @@ int finish_points(isdf_handle* h) {
 // smaller ones are stacked (ascending size) while the group's scratch -- pair
 // rows Z and M^q per row (padded to a tile boundary), and E per fragment -- stays
 // within what the largest fragment of the call needs alone (or kMinBytes).
-std::vector<std::vector<int>> fragment_groups(int n, const int32_t* n_orb, int nk, int nS, int np, double esz) {
+// per_row: bytes of Z, M and B per pair row.
+std::vector<std::vector<int>> fragment_groups(int n, const int32_t* n_orb, double per_row) {
   constexpr int64_t kWaves = 4, kSMs = 152;
   constexpr double kMinBytes = 4.0 * (1 << 30);
-  const double per_row = esz * (double)np * (4.0 * nk + 8.0 * nS);
   auto n2of = [&](int f) { return (int64_t)n_orb[f] * n_orb[f]; };
   int64_t n2max = 0;
   for (int f = 0; f < n; ++f) n2max = std::max(n2max, n2of(f));
@@ -1164,7 +1164,11 @@ int isdf_fragment_eri(isdf_handle* h, int n_frag, const int32_t* n_orb, const vo
     // their rows stacked (each block padded to a tile boundary) so that one launch
     // of each kernel covers the group and the tiles of all its diagonal blocks;
     // a group never needs more scratch than the largest fragment alone.
-    const std::vector<std::vector<int>> groups = fragment_groups(n_frag, n_orb, nk, nS, np, tc64 ? 2.0 : 1.0);
+    // mixed: M holds the gathered columns only (pitch pm) and B takes the place of Z, which M has
+    // used up by then; else M has all n_p columns and B overwrites it
+    const int pm = inv ? (rp + 3) / 4 * 4 : np;
+    const double per_row = std::max((double)zsz * nk * np, inv ? (double)msz * nS * nj : 0.0) + (double)msz * nS * pm;
+    const std::vector<std::vector<int>> groups = fragment_groups(n_frag, n_orb, per_row);
     for (const auto& grp : groups) {
       // rows of each fragment inside the stacked block; padding rows are zero
       std::vector<int64_t> row0(grp.size());
@@ -1174,9 +1178,6 @@ int isdf_fragment_eri(isdf_handle* h, int n_frag, const int32_t* n_orb, const vo
         row0[i] = rows;
         rows += (i + 1 < grp.size()) ? (n2f + 127) / 128 * 128 : n2f;
       }
-      // mixed: M holds the gathered columns only (pitch pm) and B has its own array; else B
-      // overwrites M
-      const int pm = inv ? (rp + 3) / 4 * 4 : np;
       const int64_t sqZ = rows * np, sq = rows * pm;  // position strides of Z and M
       const int64_t sqB = inv ? rows * nj : sq;
       int nfmax = 0;
@@ -1194,13 +1195,13 @@ int isdf_fragment_eri(isdf_handle* h, int n_frag, const int32_t* n_orb, const vo
       ENSURE(T, float2, "frag_T", (size_t)nk * np * nfmax * (tc64 ? 2 : 1));
       // real pair rows Z(R) of the time-reversal basis, and M^q (then B^q) of the
       // q of the sum, stored by their position in it
-      ENSURE(Zr, uint8_t, "frag_Zr", zsz * (size_t)nk * sqZ);
-      ENSURE(M, uint8_t, "frag_Mf", msz * (size_t)nS * (inv ? sq + sqB : sq));
+      ENSURE(Zr, uint8_t, "frag_Zr", std::max(zsz * (size_t)nk * sqZ, inv ? msz * (size_t)nS * sqB : 0));
+      ENSURE(M, uint8_t, "frag_Mf", msz * (size_t)nS * sq);
       float* Zr_f = reinterpret_cast<float*>(Zr);
       ffloat* Zr_ff = reinterpret_cast<ffloat*>(Zr);
       float2* M_f = reinterpret_cast<float2*>(M);
       ffcomplex* M_ff = reinterpret_cast<ffcomplex*>(M);
-      float2* B_f = inv ? M_f + (int64_t)nS * sq : M_f;
+      float2* B_f = inv ? reinterpret_cast<float2*>(Zr) : M_f;
       ENSURE(trpart, double2, "frag_traces_part", std::max<size_t>(2 * (size_t)n2max, syrk_tc_eri_part_count()));
       // tiles of every fragment's diagonal block, in the autotuned band order
       std::vector<int2>& tl = h->tiles_host;
@@ -1230,10 +1231,10 @@ int isdf_fragment_eri(isdf_handle* h, int n_frag, const int32_t* n_orb, const vo
         orb_off[i] = (int64_t)orb.size();
         orb.insert(orb.end(), o.begin(), o.end());
       }
-      // B^q = w_q^{1/2} M^q L^q overwrites M^q (row pitch nj on the tensor-core
-      // path, np through Bc on the SIMT path), qc q-points at a time; E' then
-      // takes the rows of B^q in chunks of qc positions (fp16 slices of 2 qc nj
-      // columns).  qc fits both slice buffers in the workspace limit.
+      // B^q = w_q^{1/2} M^q L^q: mixed in one launch over all q into the place of Z; FP64_TC over M^q,
+      // qc q-points at a time (row pitch nj on both); on the SIMT path over M^q through Bc (row pitch np).
+      // E' then takes the rows of B^q in chunks of qc positions (fp16 slices of 2 qc nj columns).
+      // qc fits the slices of B (and those of M in FP64_TC) in the workspace limit.
       auto syrk_split_bytes = [&](int64_t kc) {
         return tc64 ? syrk4_tc_split_bytes(rows, kc) : syrk_tc_split_bytes(rows, kc);
       };

@@ -238,6 +238,25 @@ def test_products_with_w_scale_their_inner_index(fake):
     g.close()
 
 
+@pytest.mark.parametrize("rank", [40, 80, 96])
+def test_b_of_mixed_fragments_takes_the_place_of_z(fake, rank):
+    """Z and M as wide as the points hold M and B of any rank; only at full rank B is the larger of Z and B, by the
+    q of the sum beyond half of the mesh (70 of 120 here)."""
+    kmesh, n_p, nf = (6, 4, 5), 96, 40
+    g = _handle(B.ISDF_MIXED, n_p=n_p, kmesh=kmesh, mesh=(5, 5, 5))
+    g.lib.isdf_set_workspace_limit(g.h, 1)
+    fake.fake_rank(rank)
+    g.fit_zeta(1e-3)
+    g.coulomb_metric()
+    base = fake.fake_used()
+    nk, n_s, rows = 120, 70, nf * nf
+    g.fragment_eri([_Ptr(np.zeros((nk, 4, nf), np.complex128))], traces=False)
+    z, m, b = 4 * nk * rows * n_p, 8 * n_s * rows * n_p, 8 * n_s * rows * rank
+    rest = 8 * nk * n_p * nf + 16 * rows * n_p        # T, one q of slices, maps and row maxima
+    assert fake.fake_peak() - base <= max(z, b) + m + rest
+    g.close()
+
+
 class _Ptr:
     def __init__(self, a):
         self.a, self.shape = a, a.shape
