@@ -53,6 +53,17 @@ inline void count_launch() {
   if (g_launch_counter) ++*g_launch_counter;
 }
 
+// Lets a kernel be launched with up to kMaxDynSmem bytes of dynamic shared memory.  The limit belongs to
+// the function, not to the launch: it is always set to the same value, so that a handle on another
+// thread never finds it below what its own launch needs.  (227 KB less the kernels' static arrays.)
+constexpr size_t kMaxDynSmem = 220 * 1024;
+template <typename F>
+cudaError_t allow_smem(F* kernel, size_t bytes) {
+  if (bytes <= 40 * 1024) return cudaSuccess;
+  if (bytes > kMaxDynSmem) return cudaErrorInvalidValue;
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxDynSmem);
+}
+
 // ------------------------------------------------------------------- kernels
 // Batched complex GEMM, row-major: C_b = alpha * op(A_b) op(B_b).
 // op: 'N' as is, 'T' transpose, 'C' conjugate transpose, 'R' conjugate only.

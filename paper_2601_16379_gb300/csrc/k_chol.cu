@@ -263,12 +263,9 @@ cudaError_t pchol_batched(cudaStream_t st, const double2* A, int n, int neff, bo
     const size_t per = (size_t)(neff + c - 1) / c;
     return kBp * sizeof(double2) + per * (2 * sizeof(double) + 1);
   };
-  size_t smem = smem_of(C);
-  if (smem > 220 * 1024) return cudaErrorInvalidValue;
-  if (smem > 40 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(pchol_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-  }
+  const size_t smem = smem_of(C);
+  cudaError_t e = allow_smem(pchol_kernel, smem);
+  if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3((unsigned)(nq * C));
   cfg.blockDim = dim3((unsigned)threads);
@@ -280,7 +277,7 @@ cudaError_t pchol_batched(cudaStream_t st, const double2* A, int n, int neff, bo
   at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  cudaError_t e = cudaLaunchKernelEx(&cfg, pchol_kernel, A, n, neff, live ? 1 : 0, qlist, tol, Lt, perm, rank);
+  e = cudaLaunchKernelEx(&cfg, pchol_kernel, A, n, neff, live ? 1 : 0, qlist, tol, Lt, perm, rank);
   count_launch();
   return e != cudaSuccess ? e : cudaGetLastError();
 }
@@ -298,10 +295,8 @@ cudaError_t trinv_batched(cudaStream_t st, const double2* Lt, const int32_t* per
   while (warps > 1 && (size_t)warps * n * sizeof(double2) > 64 * 1024) warps /= 2;
   const size_t smem = (size_t)warps * n * sizeof(double2);
   const bool in_smem = smem <= 200 * 1024;
-  if (in_smem && smem > 40 * 1024) {
-    e = cudaFuncSetAttribute(trinv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-  }
+  if (in_smem) e = allow_smem(trinv_kernel, smem);
+  if (e != cudaSuccess) return e;
   trinv_kernel<<<dim3((n + warps - 1) / warps, nq), warps * 32, in_smem ? smem : 0, st>>>(tmp, rank, qlist, n, in_smem, W,
                                                                                          work);
   count_launch();

@@ -606,11 +606,8 @@ cudaError_t kdft_cubic_launch(cudaStream_t st, TS* data, int64_t ncol, int mode,
   while (lct < 5 && ((int64_t)nk * sizeof(T) << (lct + 1)) <= 65536) ++lct;
   const int padk = kdft_cubic_pad(L, 1 << lct, (int)sizeof(T));
   const size_t smem = ((size_t)nk << lct) * sizeof(T) + (size_t)(nk / L) * padk * sizeof(T);
-  if (smem > 40 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(kdft_cubic_kernel<T, L, TS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
-    if (e != cudaSuccess) return e;
-  }
+  const cudaError_t e = allow_smem(kdft_cubic_kernel<T, L, TS>, smem);
+  if (e != cudaSuccess) return e;
   const int64_t nblk = (ncol + (1 << lct) - 1) >> lct;
   if (nblk > 2147483647LL) return cudaErrorInvalidValue;
   kdft_cubic_kernel<T, L, TS><<<(unsigned)nblk, 256, smem, st>>>(data, ncol, lct, padk, mode, t1, t2, scale);
@@ -626,11 +623,8 @@ cudaError_t kdft_real_cubic_launch(cudaStream_t st, const typename CT<T>::R* in,
   while (lct < 5 && ((int64_t)nk * sizeof(T) << (lct + 1)) <= 65536) ++lct;
   const int padk = kdft_cubic_pad(L, 1 << lct, (int)sizeof(T));
   const size_t smem = ((size_t)nk << lct) * sizeof(T) + (size_t)(nk / L) * padk * sizeof(T);
-  if (smem > 40 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(kdft_real_cubic_kernel<T, L>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
-    if (e != cudaSuccess) return e;
-  }
+  const cudaError_t e = allow_smem(kdft_real_cubic_kernel<T, L>, smem);
+  if (e != cudaSuccess) return e;
   const int64_t nblk = (ncol + (2 << lct) - 1) >> (lct + 1);  // 2 ct real columns per block
   if (nblk > 2147483647LL) return cudaErrorInvalidValue;
   // 16-byte vector loads when every row starts 16-byte aligned and a vector never
@@ -715,11 +709,8 @@ cudaError_t kdft_launch(cudaStream_t st, TS* data, int64_t ncol, KMesh km, int s
   if (ct < 1) ct = 1;
   if (ct > 32) ct = 32;
   size_t smem = (size_t)nk * ct * sizeof(T);
-  if (smem > 40 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(kdft_cols_kernel<T, TS, kRadix>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-  }
+  const cudaError_t e = allow_smem(kdft_cols_kernel<T, TS, kRadix>, smem);
+  if (e != cudaSuccess) return e;
   int64_t nblk = (ncol + ct - 1) / ct;
   if (nblk > 2147483647LL) return cudaErrorInvalidValue;
   kdft_cols_kernel<T, TS, kRadix><<<(unsigned)nblk, 256, smem, st>>>(data, ncol, km, ct, mode,
@@ -751,11 +742,8 @@ cudaError_t kdft_real_launch(cudaStream_t st, const typename CT<T>::R* in, T* ou
   if (ct < 1) ct = 1;
   if (ct > 32) ct = 32;
   const size_t smem = (size_t)nk * ct * sizeof(T);
-  if (smem > 40 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(kdft_real_cols_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
-    if (e != cudaSuccess) return e;
-  }
+  const cudaError_t e = allow_smem(kdft_real_cols_kernel<T>, smem);
+  if (e != cudaSuccess) return e;
   const int64_t nblk = (ncol + ct - 1) / ct;
   if (nblk > 2147483647LL) return cudaErrorInvalidValue;
   kdft_real_cols_kernel<T><<<(unsigned)nblk, 256, smem, st>>>(in, out, ncol, km, ct, qslot, tw, scale, keep);
@@ -1118,9 +1106,8 @@ cudaError_t grid_fft_launch(cudaStream_t st, T* x, int rows_per_q, int q0, int n
     const size_t s1 = ((size_t)np * (1 + two) + 256) * sizeof(T), s0 = ((size_t)n0 * 32 * (1 + two0) + 64) * sizeof(T);
     const int64_t planes = nrows * n0, chunks = nrows * ((np + 31) / 32);
     if (planes > 2147483647LL || chunks > 2147483647LL) return cudaErrorInvalidValue;
-    cudaError_t e = cudaFuncSetAttribute(grid_plane_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s1);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(grid_axis0_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s0);
+    cudaError_t e = allow_smem(grid_plane_kernel<T>, s1);
+    if (e == cudaSuccess) e = allow_smem(grid_axis0_kernel<T>, s0);
     if (e != cudaSuccess) return e;
     grid_plane_kernel<T><<<(unsigned)planes, 256, s1, st>>>(x, rows_per_q, q0, p, ph, dtw, P1, P2, two);
     count_launch();
@@ -1249,10 +1236,8 @@ cudaError_t pair_launch(cudaStream_t st, const T* t, int nk, int np, int nf, T* 
   if (nk > 65535) return cudaErrorInvalidValue;
   const size_t smem = (size_t)np * (kPairQ + 1) * sizeof(T);
   if (smem > 200 * 1024) return cudaErrorInvalidValue;
-  if (smem > 40 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(pair_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-  }
+  const cudaError_t e = allow_smem(pair_kernel<T>, smem);
+  if (e != cudaSuccess) return e;
   pair_kernel<T><<<dim3((nf + kPairP - 1) / kPairP, nk), 256, smem, st>>>(t, np, nf, Z);
   count_launch();
   return cudaGetLastError();
@@ -1265,10 +1250,8 @@ cudaError_t pair_real_launch(cudaStream_t st, const T* t, int nk, int np, int nf
   if (nk > 65535) return cudaErrorInvalidValue;
   const size_t smem = (size_t)np * (kPairQ + 1) * sizeof(T);
   if (smem > 200 * 1024) return cudaErrorInvalidValue;
-  if (smem > 40 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(pair_real_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-  }
+  const cudaError_t e = allow_smem(pair_real_kernel<T>, smem);
+  if (e != cudaSuccess) return e;
   pair_real_kernel<T><<<dim3((nf + kPairP - 1) / kPairP, nk), 256, smem, st>>>(t, np, nf, Zr, row0, rows);
   count_launch();
   return cudaGetLastError();
