@@ -39,3 +39,17 @@ def test_selection_out_of_rank(cuda, lib_built, kmesh, mesh, chol_tol):
         assert e.value.code == -4 and int(re.search(r"after (\d+) of", str(e.value)).group(1)) == found
     assert np.array_equal(g.build_points(found, 5, chol_tol), ref)
     g.close()
+
+
+def test_more_points_than_a_piece_of_the_factor(cuda, lib_built):
+    """600 points: the pivot's row of the factor is staged in pieces of 512.  The residuals keep 5e-13 of the
+    largest diagonal away from every tie window (rounding: ~1e-15), so that the indices are determined."""
+    from paper_2601_16379_gb300 import binding as B
+    sh = [W.Shell(a, l, (x,), (1.0,)) for a in (0, 1) for l, x in ((0, 0.6), (1, 0.9), (2, 1.4))]
+    cell = W.custom_cell(5.0, [[0.01, 0.02, 0.03], [0.37, 0.52, 0.21]], sh, (2, 2, 3), (16, 15, 17))
+    cell.lattice = np.diag([5.0, 5.3, 4.8])
+    ref, found = O.select_ips(O.bloch_ao(cell), 600, 11)
+    assert found == 600
+    g = B.Isdf(cell, B.ISDF_FP64)
+    assert np.array_equal(g.build_points(600, 11), ref)
+    g.close()
