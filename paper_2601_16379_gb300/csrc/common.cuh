@@ -139,7 +139,7 @@ cudaError_t ip_step(cudaStream_t st, const double2* phi, int nkao, int ng, int j
                     uint64_t seed, double tie_eps, double chol_tol, double* d0, int32_t* status);
 // The selection for orthorhombic cells from the per-axis factors of the Gram (all n_p steps);
 // ao_work: as left by ao_eval; terms: device [nterm][3] of (AO, primitive, primitive').
-bool ips_supported(const CellDev& c, int nterm);
+bool ips_supported(const CellDev& c, int nterm, int nao);
 size_t ips_work_bytes(const CellDev& c, int nterm);
 cudaError_t ips_select(cudaStream_t st, const CellDev& c, const BasisDev& b, const double* ao_work, const int* terms,
                        int nterm, int n_p, double* work, double* Lt, int32_t* piv, uint64_t seed, double tie_eps,

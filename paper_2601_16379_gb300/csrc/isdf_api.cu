@@ -765,7 +765,7 @@ int isdf_build_points(isdf_handle* h, int n_p, uint64_t seed, double chol_tol, i
   ENSURE(status, int32_t, "ip_status", 1);
   CK(cudaMemsetAsync(status, 0, sizeof(int32_t), h->st));
   CK(cudaMemsetAsync(piv, 0xff, sizeof(int32_t) * n_p, h->st));
-  if (ips_supported(h->cell, h->nterm)) {
+  if (ips_supported(h->cell, h->nterm, h->nao)) {
     ENSURE(work, double, "ip_work", ips_work_bytes(h->cell, h->nterm) / sizeof(double));
     CK(ips_select(h->st, h->cell, h->bdev, (const double*)h->buf("ao_work"), (const int*)h->buf("ip_terms"), h->nterm,
                   n_p, work, Lt, piv, seed, kTieEps, chol_tol, scal, status));

@@ -669,8 +669,16 @@ IpsLayout ips_layout(const CellDev& c, int nterm) {
 constexpr size_t kIpsMaxTable = (size_t)32 << 20;  // doubles (256 MB): beyond it, long contractions, Phi is read instead
 }  // namespace
 
-bool ips_supported(const CellDev& c, int nterm) {
-  return c.orthorhombic && nterm > 0 && nterm < (1 << 20) && ips_layout(c, nterm).table <= kIpsMaxTable;
+// Whether the separable selection is the faster one.  A step of it takes an FMA per term and grid point, a step
+// of the other a pass over Phi (Nk N_AO values per point) and three launches more, so that long contractions
+// (the square of the primitives of an AO each) on few k-points belong to the pass.  Nanoseconds per step, fitted to
+// runs with 30 to 120 AOs on grids of 16^3 to 40^3.  Separable against the pass over Phi, 120 AOs, 40^3 grid, 300
+// points: Nk = 1: 34 / 44 ms with 432 terms, 79 / 44 with 1488; Nk = 8: 81 / 102 with 1488, 116 / 103
+// with 2280; 30 AOs, 16^3, Nk = 1, 150 points: 3.3 / 4.4 with 570.
+bool ips_supported(const CellDev& c, int nterm, int nao) {
+  if (!c.orthorhombic || nterm <= 0 || nterm >= (1 << 20) || ips_layout(c, nterm).table > kIpsMaxTable) return false;
+  const double ng = (double)c.mesh[0] * c.mesh[1] * c.mesh[2], nk = (double)c.kmesh[0] * c.kmesh[1] * c.kmesh[2];
+  return nterm * std::max(19.0, 2.1e-3 * ng) <= 15000.0 + (0.75 + 3.4e-3 * nk * nao) * ng;
 }
 size_t ips_work_bytes(const CellDev& c, int nterm) { return ips_layout(c, nterm).total * sizeof(double); }
 

@@ -110,7 +110,7 @@ cudaError_t ao_eval(S, const CellDev&, const BasisDev&, double2* phi, double*) {
   used(phi);
   return cudaSuccess;
 }
-bool ips_supported(const CellDev&, int) { return true; }
+bool ips_supported(const CellDev&, int, int) { return true; }
 size_t ips_work_bytes(const CellDev&, int) { return 64; }
 NOP(ips_select, S, const CellDev&, const BasisDev&, const double*, const int*, int, int, double*, double*, int32_t*,
     uint64_t, double, double, double*, int32_t*)

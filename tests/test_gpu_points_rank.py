@@ -53,3 +53,17 @@ def test_more_points_than_a_piece_of_the_factor(cuda, lib_built):
     g = B.Isdf(cell, B.ISDF_FP64)
     assert np.array_equal(g.build_points(600, 11), ref)
     g.close()
+
+
+def test_long_contractions_at_gamma(cuda, lib_built):
+    """2000 terms at one k-point go by the pass over Phi: the same points as the oracle's."""
+    from paper_2601_16379_gb300 import binding as B
+    ex, cf = tuple(np.geomspace(0.4, 30.0, 10)), tuple(np.linspace(0.6, 0.1, 10))
+    sh = [W.Shell(a, l, ex, cf) for a in (0, 1) for l in (0, 1, 2)]
+    cell = W.custom_cell(5.0, [[0.01, 0.02, 0.03], [0.37, 0.52, 0.21]], sh, (1, 1, 1), (14, 13, 15))
+    cell.lattice = np.diag([5.0, 5.3, 4.8])
+    ref, found = O.select_ips(O.bloch_ao(cell), 40, 3)
+    assert found == 40
+    g = B.Isdf(cell, B.ISDF_FP64)
+    assert np.array_equal(g.build_points(40, 3), ref)
+    g.close()
