@@ -102,7 +102,8 @@ __global__ void __launch_bounds__(kSyrkThreads, 1)
   uint64_t* accf = bars + 2 * NST;      // [2] chunk accumulated (per buffer pair)
   uint64_t* acce = bars + 2 * NST + 2;  // [2] g0 buffer drained
   uint64_t* acce1 = bars + 2 * NST + 4; // [2] g1 buffer drained
-  uint32_t* s_tmem = reinterpret_cast<uint32_t*>(bars + 2 * NST + 6);
+  uint64_t* done = bars + 2 * NST + 6;  // settle_mmas
+  uint32_t* s_tmem = reinterpret_cast<uint32_t*>(done + 1);
   volatile int* s_err = reinterpret_cast<volatile int*>(s_tmem + 1);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -120,6 +121,7 @@ __global__ void __launch_bounds__(kSyrkThreads, 1)
       mbar_init(&acce[b], kDrainWarps);
       mbar_init(&acce1[b], kDrainWarps);
     }
+    mbar_init(done, 1);
     *s_err = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -134,6 +136,7 @@ __global__ void __launch_bounds__(kSyrkThreads, 1)
   tc_fence_after();
   const uint32_t tmem_base = *s_tmem;
 
+  int fills = 0;  // stages filled so far (thread 0)
   if (warp == 0) {
     if (lane == 0) {
       // stage layout: S1 rows of A, S2 rows of A, S1 rows of B, S2 rows of B
@@ -147,6 +150,7 @@ __global__ void __launch_bounds__(kSyrkThreads, 1)
         tma_load_2d(st + kA, &mS2, &full[s], x, tile.x * BM);
         tma_load_2d(st + 2 * kA, &mS1, &full[s], x, tile.y * BN);
         tma_load_2d(st + 2 * kA + kB, &mS2, &full[s], x, tile.y * BN);
+        ++fills;
       }
     }
   } else if (warp == 1) {
@@ -244,6 +248,11 @@ __global__ void __launch_bounds__(kSyrkThreads, 1)
   }
   tc_fence_before();
   __syncthreads();
+  if (*s_err) {  // a wait expired: wait for what is in flight
+    if (threadIdx.x == 0) settle_copies(full, NST, fills);
+    if (threadIdx.x == 32) settle_mmas(done);
+    __syncthreads();
+  }
   if (warp == 1) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(TMEM_COLS)
@@ -703,7 +712,8 @@ __global__ void __launch_bounds__(MTHREADS, 1)
   uint64_t* empty = bars + MSTAGES;      // [MSTAGES] read by the MMAs
   uint64_t* accf = bars + 2 * MSTAGES;   // pass accumulated
   uint64_t* drained = accf + 1;          // pass read out of TMEM
-  uint32_t* s_tmem = reinterpret_cast<uint32_t*>(drained + 1);
+  uint64_t* done = drained + 1;          // settle_mmas
+  uint32_t* s_tmem = reinterpret_cast<uint32_t*>(done + 1);
   volatile int* s_err = reinterpret_cast<volatile int*>(s_tmem + 1);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -716,6 +726,7 @@ __global__ void __launch_bounds__(MTHREADS, 1)
     }
     mbar_init(accf, 1);
     mbar_init(drained, MEPI);
+    mbar_init(done, 1);
     *s_err = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -732,10 +743,11 @@ __global__ void __launch_bounds__(MTHREADS, 1)
   // B' rows of pass p: 128, or 64 where at most 32 complex columns are left
   auto pass_n = [&](int p) { return args.nj_pad - p * (MPN / 2) > MPN / 4 ? MPN : MPN / 2; };
 
+  int64_t fills = 0;  // stages filled so far (thread 0)
   if (warp == 0) {
     if (lane == 0) {
       const CUtensorMap* mb[MSL] = {&mB1, &mB2, &mB3};
-      int64_t it = 0;
+      int64_t& it = fills;
       bool ok = true;
       for (int64_t u = blockIdx.x; u < args.units && ok; u += gridDim.x) {
         const int pos = (int)(u / args.mt);
@@ -942,6 +954,11 @@ __global__ void __launch_bounds__(MTHREADS, 1)
   }
   tc_fence_before();
   __syncthreads();
+  if (*s_err) {  // a wait expired: wait for what is in flight
+    if (threadIdx.x == 0) settle_copies(full, MSTAGES, fills);
+    if (threadIdx.x == 32) settle_mmas(done);
+    __syncthreads();
+  }
   if (warp == 1) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(kMlTmem)

@@ -119,7 +119,8 @@ __global__ void __launch_bounds__(NT4, 1)
   uint64_t* empty = bars + NST;          // [NST] stage consumed by the MMAs
   uint64_t* accf = bars + 2 * NST;       // chunk accumulated
   uint64_t* drained = bars + 2 * NST + 1;  // chunk drained (one arrive per drain warp)
-  uint32_t* s_tmem = reinterpret_cast<uint32_t*>(bars + 2 * NST + 2);
+  uint64_t* done = bars + 2 * NST + 2;  // settle_mmas
+  uint32_t* s_tmem = reinterpret_cast<uint32_t*>(done + 1);
   volatile int* s_err = reinterpret_cast<volatile int*>(s_tmem + 1);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -134,6 +135,7 @@ __global__ void __launch_bounds__(NT4, 1)
     }
     mbar_init(accf, 1);
     mbar_init(drained, (NT4 / 32) - 2);
+    mbar_init(done, 1);
     *s_err = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -148,6 +150,7 @@ __global__ void __launch_bounds__(NT4, 1)
   tc_fence_after();
   const uint32_t tmem_base = *s_tmem;
 
+  int fills = 0;  // stages filled so far (thread 0)
   if (warp == 0) {
     if (lane == 0) {
       const CUtensorMap* mp[NS4] = {&m1, &m2, &m3, &m4};
@@ -162,6 +165,7 @@ __global__ void __launch_bounds__(NT4, 1)
           tma_load_2d(st + i * kA, mp[i], &full[s], x, tile.x * BM);
           tma_load_2d(st + NS4 * kA + i * kB, mp[i], &full[s], x, tile.y * BN);
         }
+        ++fills;
       }
     }
   } else if (warp == 1) {
@@ -271,6 +275,11 @@ __global__ void __launch_bounds__(NT4, 1)
   }
   tc_fence_before();
   __syncthreads();
+  if (*s_err) {  // a wait expired: wait for what is in flight
+    if (threadIdx.x == 0) settle_copies(full, NST, fills);
+    if (threadIdx.x == 32) settle_mmas(done);
+    __syncthreads();
+  }
   if (warp == 1) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(TMEM_COLS)
@@ -360,7 +369,8 @@ __global__ void __launch_bounds__(NT5, 1)
   uint64_t* full = bars;               // [NST]
   uint64_t* empty = bars + NST;        // [NST]
   uint64_t* accf = bars + 2 * NST;     // accumulation finished
-  uint32_t* s_tmem = reinterpret_cast<uint32_t*>(bars + 2 * NST + 1);
+  uint64_t* done = bars + 2 * NST + 1;  // settle_mmas
+  uint32_t* s_tmem = reinterpret_cast<uint32_t*>(done + 1);
   volatile int* s_err = reinterpret_cast<volatile int*>(s_tmem + 1);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -376,6 +386,7 @@ __global__ void __launch_bounds__(NT5, 1)
       mbar_init(&empty[s], 1);
     }
     mbar_init(accf, 1);
+    mbar_init(done, 1);
     *s_err = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -390,6 +401,7 @@ __global__ void __launch_bounds__(NT5, 1)
   tc_fence_after();
   const uint32_t tmem_base = *s_tmem;
 
+  int fills = 0;  // stages filled so far (thread 0)
   if (warp == 0) {
     if (lane == 0) {
       const CUtensorMap* ma[NS5] = {&a1, &a2, &a3, &a4, &a5};
@@ -406,6 +418,7 @@ __global__ void __launch_bounds__(NT5, 1)
           tma_load_2d(st + i * kA, ma[i], &full[s], x, arow);
           tma_load_2d(st + NS5 * kA + i * kMB, mb[i], &full[s], x, brow);
         }
+        ++fills;
       }
     }
   } else if (warp == 1) {
@@ -495,6 +508,11 @@ __global__ void __launch_bounds__(NT5, 1)
   }
   tc_fence_before();
   __syncthreads();
+  if (*s_err) {  // a wait expired: wait for what is in flight
+    if (threadIdx.x == 0) settle_copies(full, NST, fills);
+    if (threadIdx.x == 32) settle_mmas(done);
+    __syncthreads();
+  }
   if (warp == 1) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(TMEM_COLS)

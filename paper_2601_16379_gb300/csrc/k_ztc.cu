@@ -209,7 +209,8 @@ __global__ void __launch_bounds__(NT, 1) zgemm_tc_kernel(Args args) {
   uint64_t* empty = bars + NST;      // [NST] stage read by the MMAs
   uint64_t* accf = bars + 2 * NST;   // [2] chunk accumulated: groups 0-3, the others
   uint64_t* drained = accf + 2;      // [2] and drained
-  uint32_t* s_tmem = reinterpret_cast<uint32_t*>(drained + 2);
+  uint64_t* done = drained + 2;      // settle_mmas
+  uint32_t* s_tmem = reinterpret_cast<uint32_t*>(done + 1);
   volatile int* s_err = reinterpret_cast<volatile int*>(s_tmem + 1);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
@@ -222,6 +223,7 @@ __global__ void __launch_bounds__(NT, 1) zgemm_tc_kernel(Args args) {
       mbar_init(&accf[i], 1);
       mbar_init(&drained[i], kDrainWarps);
     }
+    mbar_init(done, 1);
     *s_err = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -252,9 +254,10 @@ __global__ void __launch_bounds__(NT, 1) zgemm_tc_kernel(Args args) {
     return nk;
   };
 
+  int64_t fills = 0;  // stages filled so far (thread 0)
   if (warp == 0) {
     if (lane == 0) {
-      int64_t it = 0;  // stages filled so far
+      int64_t& it = fills;
       bool ok = true;
       for (int64_t t = blockIdx.x; t < args.ntiles && ok; t += gridDim.x) {
         int b, ti, tj;
@@ -440,6 +443,11 @@ __global__ void __launch_bounds__(NT, 1) zgemm_tc_kernel(Args args) {
   }
   tc_fence_before();
   __syncthreads();
+  if (*s_err) {  // a wait expired: wait for what is in flight
+    if (threadIdx.x == 0) settle_copies(full, NST, fills);
+    if (threadIdx.x == 32) settle_mmas(done);
+    __syncthreads();
+  }
   if (warp == 1) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmem) : "memory");

@@ -91,6 +91,23 @@ __device__ __forceinline__ void umma_commit(uint64_t* bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
                : "memory");
 }
+// Leaving after a wait has expired: the CTA's shared memory and TMEM go back only when nothing of its
+// own is in flight.  Up to kSettleNs each.
+constexpr unsigned long long kSettleNs = 1000000000ULL;
+__device__ __forceinline__ void mbar_settle(uint64_t* bar, uint32_t parity) {
+  const unsigned long long t0 = global_ns();
+  while (!mbar_try_wait(bar, parity) && global_ns() - t0 < kSettleNs) {
+  }
+}
+// The copies into the last of `fills` stage fills of a ring of nst (by the thread that issued them).
+__device__ __forceinline__ void settle_copies(uint64_t* full, int nst, int64_t fills) {
+  for (int64_t f = fills > nst ? fills - nst : 0; f < fills; ++f) mbar_settle(&full[f % nst], (uint32_t)((f / nst) & 1));
+}
+// The MMAs of the thread that issued them; done: a barrier of one arrival, not used otherwise.
+__device__ __forceinline__ void settle_mmas(uint64_t* done) {
+  umma_commit(done);
+  mbar_settle(done, 0);
+}
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
