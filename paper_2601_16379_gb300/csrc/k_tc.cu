@@ -1056,12 +1056,6 @@ __global__ void __launch_bounds__(256) lslice_kernel(const double2* __restrict__
   }
 }
 
-inline int nblk(int64_t total) {
-  int64_t nb = (total + 255) / 256;
-  if (nb > 152 * 32) nb = 152 * 32;
-  return nb < 1 ? 1 : (int)nb;
-}
-
 inline int64_t round_up(int64_t x, int64_t m) { return ((x + m - 1) / m) * m; }
 
 }  // namespace tc
