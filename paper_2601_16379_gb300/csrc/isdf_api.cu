@@ -2,9 +2,9 @@
 // fragment-ERI path (Section II of the paper; see include/isdf.h).
 //
 // Step -> kernels
-//   build_points   ao_eval (Eq. 1), ip_init/ip_step (Section II.A), gather_x
-//   fit_zeta       G^k = conj(X^k) X^k^T (zgemm), k-convolution |DFT|^2 -> Pi^q
-//                  (kdft_cols, Eq. 4 / Algorithm 1); g^k = conj(X^k) Phi^k (zgemm),
+//   build_points   ao_eval (Eq. 1), ips_select or ip_init/ip_step (Section II.A), gather_x
+//   fit_zeta       G^k = conj(X^k) X^k^T (zmul), k-convolution |DFT|^2 -> Pi^q
+//                  (kdft_cols, Eq. 4 / Algorithm 1); g^k = conj(X^k) Phi^k (zmul),
 //                  k-convolution -> eta^q (Eq. 5); pivoted Cholesky of Pi^q and
 //                  W = L_S^{-1} (Eq. 3); xi^q = W eta^q (zeta^q = W^H xi^q).
 //   coulomb_metric grid FFT of e^{-iq.r} xi^q with sqrt(4 pi/|q+G|^2) (Eq. 6),

@@ -10,7 +10,8 @@
 //           D(r,r') = Re sum_{k,mu} conj(Phi^k_mu(r)) Phi^k_mu(r') (D is real:
 //           the k and -k terms are conjugate).  One pivot per ip_step: argmax
 //           with ties, column generation, rank-one update.
-// ips_*     the same selection for orthorhombic cells, where D factorises as Phi does:
+// ips_*     the same selection for orthorhombic cells (where it is the faster form: ips_supported), in which D
+//           factorises as Phi does:
 //             D(r,r') = sum_mu sum_{p,p'} c_p c_p' prod_a A_a(g_a, g'_a),
 //             A_a(g, g') = sum_{m_a} conj(S_a^p(m_a, g)) S_a^p'(m_a, g')   (real),
 //           since the k-mesh is a product of its axes.  A column of D then costs N_AO

@@ -858,7 +858,7 @@ __global__ void __launch_bounds__(256) grid_axis_kernel(T* __restrict__ x, int64
 // axis 2, axis 1 -- and a second kernel axis 0 and the weight.  An axis of length L = P Q goes in two
 // steps of in-register transforms of at most 8 points; other lengths (a prime above 8 in them) by
 // the direct sum over that factor, four FMAs per product.  Measured with the k-transforms: fit and
-// metric of 125 k-points on an 18^3 grid 33.9 -> 18.1 ms, ragged quartets 20.5 -> 13.0.
+// metric of 27 k-points on a 24^3 grid 33.9 -> 18.1 ms, ragged quartets 20.5 -> 13.0.
 // In float-float (as accurate as the direct sum of L terms, and FP32-bound there): fit and metric of 64
 // k-points on a 32^3 grid 527 -> 463 ms.
 // FP64_TC keeps the direct sums: see isdf_fit_zeta.

@@ -102,7 +102,7 @@ __global__ void __launch_bounds__(kSyrkThreads, 1)
   uint64_t* accf = bars + 2 * NST;      // [2] chunk accumulated (per buffer pair)
   uint64_t* acce = bars + 2 * NST + 2;  // [2] g0 buffer drained
   uint64_t* acce1 = bars + 2 * NST + 4; // [2] g1 buffer drained
-  uint64_t* done = bars + 2 * NST + 6;  // settle_mmas
+  uint64_t* done = bars + 2 * NST + 6;  // settle
   uint32_t* s_tmem = reinterpret_cast<uint32_t*>(done + 1);
   volatile int* s_err = reinterpret_cast<volatile int*>(s_tmem + 1);
 
@@ -248,11 +248,7 @@ __global__ void __launch_bounds__(kSyrkThreads, 1)
   }
   tc_fence_before();
   __syncthreads();
-  if (*s_err) {  // a wait expired: wait for what is in flight
-    if (threadIdx.x == 0) settle_copies(full, NST, fills);
-    if (threadIdx.x == 32) settle_mmas(done);
-    __syncthreads();
-  }
+  if (*s_err) settle(full, NST, fills, done);  // a wait expired: wait for what is in flight
   if (warp == 1) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(TMEM_COLS)
@@ -712,7 +708,7 @@ __global__ void __launch_bounds__(MTHREADS, 1)
   uint64_t* empty = bars + MSTAGES;      // [MSTAGES] read by the MMAs
   uint64_t* accf = bars + 2 * MSTAGES;   // pass accumulated
   uint64_t* drained = accf + 1;          // pass read out of TMEM
-  uint64_t* done = drained + 1;          // settle_mmas
+  uint64_t* done = drained + 1;          // settle
   uint32_t* s_tmem = reinterpret_cast<uint32_t*>(done + 1);
   volatile int* s_err = reinterpret_cast<volatile int*>(s_tmem + 1);
 
@@ -954,11 +950,7 @@ __global__ void __launch_bounds__(MTHREADS, 1)
   }
   tc_fence_before();
   __syncthreads();
-  if (*s_err) {  // a wait expired: wait for what is in flight
-    if (threadIdx.x == 0) settle_copies(full, MSTAGES, fills);
-    if (threadIdx.x == 32) settle_mmas(done);
-    __syncthreads();
-  }
+  if (*s_err) settle(full, MSTAGES, fills, done);  // a wait expired: wait for what is in flight
   if (warp == 1) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(kMlTmem)

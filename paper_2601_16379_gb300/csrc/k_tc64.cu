@@ -119,7 +119,7 @@ __global__ void __launch_bounds__(NT4, 1)
   uint64_t* empty = bars + NST;          // [NST] stage consumed by the MMAs
   uint64_t* accf = bars + 2 * NST;       // chunk accumulated
   uint64_t* drained = bars + 2 * NST + 1;  // chunk drained (one arrive per drain warp)
-  uint64_t* done = bars + 2 * NST + 2;  // settle_mmas
+  uint64_t* done = bars + 2 * NST + 2;  // settle
   uint32_t* s_tmem = reinterpret_cast<uint32_t*>(done + 1);
   volatile int* s_err = reinterpret_cast<volatile int*>(s_tmem + 1);
 
@@ -275,11 +275,7 @@ __global__ void __launch_bounds__(NT4, 1)
   }
   tc_fence_before();
   __syncthreads();
-  if (*s_err) {  // a wait expired: wait for what is in flight
-    if (threadIdx.x == 0) settle_copies(full, NST, fills);
-    if (threadIdx.x == 32) settle_mmas(done);
-    __syncthreads();
-  }
+  if (*s_err) settle(full, NST, fills, done);  // a wait expired: wait for what is in flight
   if (warp == 1) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(TMEM_COLS)
@@ -369,7 +365,7 @@ __global__ void __launch_bounds__(NT5, 1)
   uint64_t* full = bars;               // [NST]
   uint64_t* empty = bars + NST;        // [NST]
   uint64_t* accf = bars + 2 * NST;     // accumulation finished
-  uint64_t* done = bars + 2 * NST + 1;  // settle_mmas
+  uint64_t* done = bars + 2 * NST + 1;  // settle
   uint32_t* s_tmem = reinterpret_cast<uint32_t*>(done + 1);
   volatile int* s_err = reinterpret_cast<volatile int*>(s_tmem + 1);
 
@@ -508,11 +504,7 @@ __global__ void __launch_bounds__(NT5, 1)
   }
   tc_fence_before();
   __syncthreads();
-  if (*s_err) {  // a wait expired: wait for what is in flight
-    if (threadIdx.x == 0) settle_copies(full, NST, fills);
-    if (threadIdx.x == 32) settle_mmas(done);
-    __syncthreads();
-  }
+  if (*s_err) settle(full, NST, fills, done);  // a wait expired: wait for what is in flight
   if (warp == 1) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(TMEM_COLS)

@@ -1,6 +1,7 @@
 // FP64-accurate batched complex GEMM on the tensor cores (tcgen05):
 //     C_b = alpha op(A_b) op(B_b),   op in {N, T, C, R}, complex128, row-major.
-// It carries every complex128 product of the library: the fit (Eqs. 3-5), the FP64
+// It carries the complex128 products of the library but those that the mixed and FP64_TC paths keep as FMA
+// chains (k_gemm.cu): the fit (Eqs. 3-5), the FP64
 // Coulomb metric (Eq. 6), the FP64 fragment contractions (Eq. 19), exchange (Eq. 10),
 // AO integrals (Eq. 9) and the polarisability (Eqs. 12-15).
 //
@@ -54,7 +55,8 @@
 // not stored.  k beyond K is zero.
 //
 // The drain of groups 0-3 runs while the MMAs of groups 4-7 of the chunk's last k block do, and that of
-// groups 4-7 under those of groups 0-3 of the next chunk: two pairs of barriers.  With the chunks of
+// groups 4-7 under those of groups 0-3 of the next chunk: two pairs of barriers (K <= 32 and seven slices: one
+// chunk and one drain, where a second wait per tile cost 4 to 11 % of the kernel).  With the chunks of
 // 384 k of base-128 digits and one drain per chunk, 320 x 320 x K in a batch of 200 took 671 us at K = 64,
 // 1149 at 128, 2055 at 256 and 2955 at 384; it takes 649, 1078, 2064 and 3041.
 //
@@ -202,6 +204,8 @@ __device__ __forceinline__ double seven_to_double(long long T1, int v0, bool fli
 template <int NS, bool kShort>
 __global__ void __launch_bounds__(NT, 1) zgemm_tc_kernel(Args args) {
   constexpr int kBlk = Blk<NS>::kElems, kABytes = Blk<NS>::kBytesA, kStage = Blk<NS>::kStage;
+  constexpr int kHalves = kShort ? 1 : 2;  // parts of a drain: all groups, or groups 0-3 and 4-7
+  constexpr int kGrp = kShort ? NS : 4;    // groups of a part
   extern __shared__ __align__(1024) uint8_t smem[];
   uint8_t* outS = smem + NST * kStage;
   uint64_t* bars = reinterpret_cast<uint64_t*>(outS + kOutBytes);
@@ -209,9 +213,10 @@ __global__ void __launch_bounds__(NT, 1) zgemm_tc_kernel(Args args) {
   uint64_t* empty = bars + NST;      // [NST] stage read by the MMAs
   uint64_t* accf = bars + 2 * NST;   // [2] chunk accumulated: groups 0-3, the others
   uint64_t* drained = accf + 2;      // [2] and drained
-  uint64_t* done = drained + 2;      // settle_mmas
+  uint64_t* done = drained + 2;      // settle
   uint32_t* s_tmem = reinterpret_cast<uint32_t*>(done + 1);
   volatile int* s_err = reinterpret_cast<volatile int*>(s_tmem + 1);
+  volatile int64_t* s_fills = reinterpret_cast<volatile int64_t*>(s_tmem + 2);  // stages filled by thread 0
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
   if (threadIdx.x == 0) {
@@ -254,10 +259,9 @@ __global__ void __launch_bounds__(NT, 1) zgemm_tc_kernel(Args args) {
     return nk;
   };
 
-  int64_t fills = 0;  // stages filled so far (thread 0)
   if (warp == 0) {
     if (lane == 0) {
-      int64_t& it = fills;
+      int64_t it = 0;  // stages filled so far
       bool ok = true;
       for (int64_t t = blockIdx.x; t < args.ntiles && ok; t += gridDim.x) {
         int b, ti, tj;
@@ -284,6 +288,7 @@ __global__ void __launch_bounds__(NT, 1) zgemm_tc_kernel(Args args) {
           }
         }
       }
+      *s_fills = it;
     }
   } else if (warp == 1) {
     if (lane == 0) {
@@ -304,7 +309,7 @@ __global__ void __launch_bounds__(NT, 1) zgemm_tc_kernel(Args args) {
           const uint64_t dA = sdesc_core(st), dB = sdesc_core(st + kABytes);
           constexpr uint64_t oA = (2 * kSlice * 2) >> 4, oB = (kSlice * 2) >> 4;  // slice strides of the descriptors
 #pragma unroll
-          for (int gh = 0; gh < 2; ++gh) {
+          for (int gh = 0; gh < kHalves; ++gh) {
             if (first && ch > 0 && !mbar_wait(&drained[gh], (uint32_t)((ch - 1) & 1), s_err, args.err, 42)) {
               ok = false;
               break;
@@ -314,7 +319,7 @@ __global__ void __launch_bounds__(NT, 1) zgemm_tc_kernel(Args args) {
             for (int i = 0; i < NS; ++i)
 #pragma unroll
               for (int c = 0; c < NS - i; ++c)
-                if ((i + c >= 4) == (gh == 1))
+                if (kShort || (i + c >= 4) == (gh == 1))
                   umma_f16(tmem + (uint32_t)((i + c) * 2 * BN), dA + i * oA, dB + c * oB, kIdesc,
                            (first && i == 0) ? 0u : 1u);
             if (last) umma_commit(&accf[gh]);
@@ -355,17 +360,16 @@ __global__ void __launch_bounds__(NT, 1) zgemm_tc_kernel(Args args) {
       for (int j = 0; j < kDrainCols; ++j) hi[j] = lo[j] = 0;
       for (int c = 0; c < nch && ok; ++c, ++ch) {
 #pragma unroll
-        for (int gh = 0; gh < 2; ++gh) {
+        for (int gh = 0; gh < kHalves; ++gh) {
           if (ok) ok = __all_sync(0xffffffffu, mbar_wait(&accf[gh], (uint32_t)(ch & 1), s_err, args.err, 44));
           if (!ok) break;
           tc_fence_after();
 #pragma unroll
           for (int cb = 0; cb < kDrainCols / 4; ++cb) {
-            uint32_t v[4][4];
+            uint32_t v[kGrp][4];
 #pragma unroll
-            for (int g = 0; g < 4; ++g)
-              if (gh * 4 + g < NS)
-                tmem_ld4(tbase + (uint32_t)((gh * 4 + g) * 2 * BN) + ((uint32_t)(cb * 4) ^ keep), v[g]);
+            for (int g = 0; g < kGrp; ++g)
+              tmem_ld4(tbase + (uint32_t)((gh * 4 + g) * 2 * BN) + ((uint32_t)(cb * 4) ^ keep), v[g]);
             tmem_wait_ld();
             if (cb == kDrainCols / 4 - 1) {  // the last read: the MMAs may go on
               tc_fence_before();
@@ -374,10 +378,9 @@ __global__ void __launch_bounds__(NT, 1) zgemm_tc_kernel(Args args) {
             }
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
-              int w[4];
+              int w[kGrp];
 #pragma unroll
-              for (int g = 0; g < 4; ++g) {
-                if (gh * 4 + g >= NS) continue;
+              for (int g = 0; g < kGrp; ++g) {
                 const float f = __uint_as_float(v[g][j]);
                 // exact integers; below 2^22 the addition of 1.5 2^23 puts them into the low bits
                 w[g] = kShort ? __float_as_int(f + 12582912.f) - 0x4B400000 : __float2int_rn(f);
@@ -385,17 +388,15 @@ __global__ void __launch_bounds__(NT, 1) zgemm_tc_kernel(Args args) {
               long long &h = hi[cb * 4 + j], &l = lo[cb * 4 + j];
               if constexpr (NS == 7) {
                 // groups 1-6 below 2^22 (64 * 36864): weights 2^35 .. 1 in hi; group 0 apart
-                if (gh == 0) {
-                  h += (long long)(w[1] * 128 + w[2]) * (1 << 28) + (long long)w[3] * (1 << 21);
-                  l += w[0];
-                } else {
-                  h += (long long)w[0] * (1 << 14) + (w[1] * 128 + w[2]);
-                }
-              } else if (gh == 0) {
-                // |w_0| <= 144 * 2^12 and |w_2| <= 144 * 2^15: 256 w_g + w_(g+1) fits 32 bits
-                h += (long long)(w[0] * 256 + w[1]) * 65536 + (w[2] * 256 + w[3]);
+                const int a0 = w[1] * 128 + w[2], a1 = w[3] * 128 + w[4], a2 = w[5] * 128 + w[6];
+                h += (long long)a0 * (1 << 28) + (long long)a1 * (1 << 14) + a2;
+                l += w[0];
               } else {
-                l += (long long)w[0] * (1 << 24) + (long long)w[1] * 65536 + ((long long)w[2] * 256 + w[3]);
+                // |w_0| <= 144 * 2^12 and |w_2| <= 144 * 2^15: 256 w_g + w_(g+1) fits 32 bits
+                constexpr int o = kShort ? 4 : 0;  // group 4 among the part's
+                if (gh == 0) h += (long long)(w[0] * 256 + w[1]) * 65536 + (w[2] * 256 + w[3]);
+                if (kShort || gh == 1)
+                  l += (long long)w[o] * (1 << 24) + (long long)w[o + 1] * 65536 + ((long long)w[o + 2] * 256 + w[o + 3]);
               }
             }
           }
@@ -443,11 +444,7 @@ __global__ void __launch_bounds__(NT, 1) zgemm_tc_kernel(Args args) {
   }
   tc_fence_before();
   __syncthreads();
-  if (*s_err) {  // a wait expired: wait for what is in flight
-    if (threadIdx.x == 0) settle_copies(full, NST, fills);
-    if (threadIdx.x == 32) settle_mmas(done);
-    __syncthreads();
-  }
+  if (*s_err) settle(full, NST, *s_fills, done);  // a wait expired: wait for what is in flight
   if (warp == 1) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmem) : "memory");

@@ -92,14 +92,17 @@ __device__ __forceinline__ void mbar_settle(uint64_t* bar, uint32_t parity) {
   while (!mbar_try_wait(bar, parity) && global_ns() - t0 < kSettleNs) {
   }
 }
-// The copies into the last of `fills` stage fills of a ring of nst (by the thread that issued them).
-__device__ __forceinline__ void settle_copies(uint64_t* full, int nst, int64_t fills) {
-  for (int64_t f = fills > nst ? fills - nst : 0; f < fills; ++f) mbar_settle(&full[f % nst], (uint32_t)((f / nst) & 1));
-}
-// The MMAs of the thread that issued them; done: a barrier of one arrival, not used otherwise.
-__device__ __forceinline__ void settle_mmas(uint64_t* done) {
-  umma_commit(done);
-  mbar_settle(done, 0);
+// By all threads of the CTA after the barrier behind their roles: thread 0 issued `fills` stage fills of a
+// ring of nst, thread 32 the MMAs; done: a barrier of one arrival, not used otherwise.  (A function of its own:
+// inlined, it cost the products' loops 1 %.)
+static __device__ __noinline__ void settle(uint64_t* full, int nst, int64_t fills, uint64_t* done) {
+  if (threadIdx.x == 0)
+    for (int64_t f = fills > nst ? fills - nst : 0; f < fills; ++f) mbar_settle(&full[f % nst], (uint32_t)((f / nst) & 1));
+  if (threadIdx.x == 32) {
+    umma_commit(done);
+    mbar_settle(done, 0);
+  }
+  __syncthreads();
 }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
