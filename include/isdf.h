@@ -58,8 +58,17 @@ typedef enum {
   ISDF_ERR_STATE = -6     /* calls made out of order                              */
 } isdf_status;
 
+/* FP64 accuracy below means: transforms, factorisations and sums in FP64, and complex128
+ * products either as FP64 FMA chains or on the tensor cores from eight exact integer
+ * slices of each operand, which lose ~2^-60 of the largest entries of a row and a
+ * column per term (an FMA chain: up to 2^-53 of each partial sum).
+ * ISDF_MIXED and ISDF_FP64_TC cut later operands to 28-30 bits, and the smallest pivots
+ * amplify the rounding of Pi, g and xi (in ISDF_FP64_TC also of V_xi and L) to 1e-8
+ * to 1e-7 of single integrals, as much as these modes' own error.  Those products
+ * therefore have one fixed arithmetic (FMA chains in the order of k; seven slices for
+ * g, and for T in ISDF_FP64_TC), which does not depend on memory or settings. */
 typedef enum {
-  ISDF_FP64 = 0,   /* every step in FP64                                          */
+  ISDF_FP64 = 0,   /* FP64 accuracy in every step                                  */
   ISDF_MIXED = 1,  /* FP64-class points and fit (Eqs. 3-5); V (Eq. 6) from a float-  */
                    /* float grid FFT and V_xi on the tensor cores with four exact   */
                    /* fp16 slices; the fragment pair tensor and ERI contractions   */
@@ -141,8 +150,8 @@ int isdf_coulomb_metric(isdf_handle* h, void* V_out);
  * truncated factor of Pi as isdf_fit_zeta: W^q = conj(Pi^+) V_eta conj(Pi^+)
  * (the conjugates express Eq. 8 in this library's index placement of Pi).
  * Produces the same V^q as isdf_coulomb_metric up to rounding, which here is
- * multiplied by cond(Pi^q) rather than its square root; computed in FP64 in
- * both precisions.  Replaces isdf_coulomb_metric (either may precede
+ * multiplied by cond(Pi^q) rather than its square root; computed with FP64
+ * accuracy in every precision.  Replaces isdf_coulomb_metric (either may precede
  * isdf_fragment_eri).  V_out as for isdf_coulomb_metric. */
 int isdf_coulomb_metric_eta(isdf_handle* h, void* V_out);
 
@@ -163,7 +172,8 @@ int isdf_coulomb_metric_eta(isdf_handle* h, void* V_out);
  * entries of eri_out may name the same buffer (each result then overwrites the
  * previous one).
  * Device memory: the handle keeps its scratch between calls; when an
- * allocation for a fragment fails, the grid-sized fit arrays (eta, xi) are
+ * allocation fails, the slices of the complex128 products are freed first; when
+ * one for a fragment still fails, the grid-sized fit arrays (eta, xi) are
  * freed and the allocation retried (isdf_get of eta or zeta and
  * isdf_coulomb_metric_eta then need a new isdf_fit_zeta); the fit frees the
  * fragment scratch in the same way. */
@@ -171,7 +181,7 @@ int isdf_fragment_eri(isdf_handle* h, int n_frag, const int32_t* n_orb,
                       const void* const* C, const void* const* gamma,
                       void* const* eri_out, double* ej_out, double* ek_out);
 
-/* k-point exchange matrix from the ISDF integrals (Eq. 10), FP64:
+/* k-point exchange matrix from the ISDF integrals (Eq. 10), FP64 accuracy (see isdf_precision):
  *   K^k_{mu nu} = -(1/Nk) sum_{k'} sum_{lam sig} P^{k'}_{lam sig} (mu k, lam k' | sig k', nu k)
  * computed as K^k = -(1/Nk) X^k^H Gamma^k X^k with
  *   rho^{k'} = X^{k'} P^{k'} X^{k'}^H  and  Gamma^k_IJ = sum_{k'} V^{k'-k}_JI rho^{k'}_IJ,
@@ -183,7 +193,7 @@ int isdf_fragment_eri(isdf_handle* h, int n_frag, const int32_t* n_orb,
 int isdf_exchange(isdf_handle* h, const void* P, void* K_out);
 
 /* Two-electron integrals of Bloch AOs for arbitrary k-quartets in the THC form
- * of Eq. 9, FP64, chemist's order:
+ * of Eq. 9, FP64 accuracy, chemist's order:
  *   (mu k1 nu k2 | lam k3 sig k4)
  *     = Nk sum_IJ conj(X^{k1}_{I mu}) X^{k2}_{I nu} V^{Q}_{IJ} conj(X^{k3}_{J lam}) X^{k4}_{J sig},
  *   Q = k1 - k2,
@@ -198,7 +208,7 @@ int isdf_exchange(isdf_handle* h, const void* P, void* K_out);
  * Needs the Coulomb metric (either route). */
 int isdf_ao_eri(isdf_handle* h, int n_quartet, const int32_t* quartets, void* out);
 
-/* k-SOS-MP2 building blocks at one imaginary time tau >= 0 (Eqs. 11-15), FP64.
+/* k-SOS-MP2 building blocks at one imaginary time tau >= 0 (Eqs. 11-15), FP64 accuracy.
  * With orbital values at the points Y^k = X^k C^k and energies measured from a
  * chemical potential inside the gap:
  *   Go^k(tau) = Y_occ e^{+tau eps_i} Y_occ^H,   Gv^k(tau) = Y_vir e^{-tau eps_a} Y_vir^H,
