@@ -250,7 +250,8 @@ int isdf_set_time_reversal(isdf_handle* h, int enable);
  * Every mode: also the limit (with 512 MiB) for the integer slices of the
  * complex128 tensor-core products, which go in chunks of batch entries (one at
  * least; the same bits for any limit).  Where the device has no memory for the
- * slices of one entry, products of the FP64 path run on the FP64 pipe instead;
+ * slices of one entry, the fit arrays (in a fragment call) or the fragment scratch
+ * are freed if that makes room; else products of the FP64 path run on the FP64 pipe and
  * those whose arithmetic the other modes fix return ISDF_ERR_OOM.
  * Returns ISDF_ERR_ARG for 0. */
 int isdf_set_workspace_limit(isdf_handle* h, uint64_t bytes);

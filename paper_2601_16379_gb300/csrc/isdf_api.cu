@@ -169,18 +169,25 @@ struct isdf_handle {
   static bool in_fit_group(const std::string& n) {
     return n == "eta" || n == "xi" || n == "grid_work" || n == "grid_work_v";
   }
+  static bool in_other_group(const std::string& n, const char* name) {
+    return in_frag_group(name) ? in_fit_group(n) : in_frag_group(n);
+  }
   bool evict_other(const char* name) {
-    const std::string n(name);
     bool freed = false;
-    const bool frag = in_frag_group(n);
-    for (auto& b : bufs) {
-      const bool other = frag ? in_fit_group(b.first) : in_frag_group(b.first);
-      if (other && b.second.p) {
+    for (auto& b : bufs)
+      if (in_other_group(b.first, name) && b.second.p) {
         drop(b);
         freed = true;
       }
-    }
     return freed;
+  }
+  // Whether `bytes` would fit once the other group is free.
+  bool fits_without_other(const char* name, size_t bytes) const {
+    size_t free_bytes = 0, total = 0;
+    if (cudaMemGetInfo(&free_bytes, &total) != cudaSuccess) return false;
+    for (const auto& b : bufs)
+      if (in_other_group(b.first, name)) free_bytes += b.second.bytes;
+    return free_bytes >= bytes;
   }
   // The slices of a complex128 product (zmul) are dead as soon as it is enqueued: they give way
   // to whatever else does not fit.
@@ -405,10 +412,9 @@ int upload_basis(isdf_handle* h) {
 // in the buffer "zslices" (see isdf_handle::drop_slices) for as many batch entries at a time as fit
 // kSliceBytes, the workspace limit and the free memory, one at least; on the FP64 pipe
 // with `who` NULL and where the inner dimension is too short to pay for the slicing.
-// Where not even one entry's slices can be had: eight slices stand for FP64 FMA chains, which take their
-// place as the form without a workspace (nothing else is freed for them); seven slices are the fixed
-// arithmetic of their products (see isdf_fit_zeta), for which the group other than that of `who` is freed,
-// else the call fails.  A bounded wait that expires sets the handle's error word, read by tc_status at the next
+// Where not even one entry's slices can be had, the group other than that of `who` is freed if that makes room.
+// If not, eight slices stand for FP64 FMA chains, which take their place as the form without a workspace;
+// seven slices are the fixed arithmetic of their products (see isdf_fit_zeta) and the call fails.  A bounded wait that expires sets the handle's error word, read by tc_status at the next
 // synchronisation point.
 //
 // kMinTcK: a 64 x 64 tile of the SIMT kernel takes 4.3 us per unit of K however few tiles there
@@ -425,11 +431,14 @@ int zmul(isdf_handle* h, const char* who, char opA, char opB, int m, int n, int 
   if (who && (k >= kMinTcK || o.slices == 7) && k <= kZgemm8MaxK) {
     const bool same = !o.brow && !o.kexp && zgemm_tc_same(opA, opB, m, n, A, lda, sA, B, ldb, sB);
     const size_t one = zgemm_tc_work_bytes(o.slices, m, n, k, 1, same), limit = std::min(kSliceBytes, h->split_budget);
-    for (int nb = (int)std::min<size_t>(batch, std::max<size_t>(1, limit / one)); nb >= 1 && !w; nb /= 2) {
-      bytes = zgemm_tc_work_bytes(o.slices, m, n, k, nb, same);
-      w = h->ensure("zslices", bytes);
-    }
-    if (!w && o.slices == 7 && h->evict_other(who)) w = h->ensure("zslices", bytes = one);
+    auto ask = [&]() {
+      for (int nb = (int)std::min<size_t>(batch, std::max<size_t>(1, limit / one)); nb >= 1 && !w; nb /= 2) {
+        bytes = zgemm_tc_work_bytes(o.slices, m, n, k, nb, same);
+        w = h->ensure("zslices", bytes);
+      }
+    };
+    ask();
+    if (!w && h->fits_without_other(who, one) && h->evict_other(who)) ask();
     if (!w && o.slices == 7) return fail(h, ISDF_ERR_OOM, "device allocation of zslices (%zu bytes) failed", one);
   }
   if (w)

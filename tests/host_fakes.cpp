@@ -61,6 +61,11 @@ cudaError_t cudaFree(void* p) {
   g_live.erase(it);
   return cudaSuccess;
 }
+cudaError_t cudaMemGetInfo(size_t* f, size_t* t) {
+  *t = g_cap;
+  *f = g_cap > g_used ? g_cap - g_used : 0;
+  return cudaSuccess;
+}
 cudaError_t cudaMemcpy(void* d, const void* s, size_t n, cudaMemcpyKind) {
   used(d), used(s);
   if (d && s && n < ((size_t)64 << 20)) memcpy(d, s, n);

@@ -205,8 +205,10 @@ def test_slices_give_way_to_what_is_allocated_later(fake):
     g.close()
 
 
-def test_slices_of_the_fp64_path_free_nothing_else(fake):
-    """Without memory for its slices an FP64 product runs as FMA chains and eta stays."""
+@pytest.mark.parametrize("room", [True, False])
+def test_slices_free_the_other_group_only_if_that_is_enough(fake, room):
+    """E = B B^H of an FP64 fragment without memory for its slices: with eta and xi gone they fit (room), and the
+    documented price is a new fit; else the product runs as FMA chains and eta stays."""
     g = _wide()
     fake.fake_rank(9)
     g.fit_zeta(1e-3)
@@ -218,13 +220,17 @@ def test_slices_of_the_fp64_path_free_nothing_else(fake):
     g = _wide()
     g.fit_zeta(1e-3)
     g.coulomb_metric()
-    # B = M L keeps one q at a time, E = B B^H nothing
-    fake.fake_capacity(used - 4 * _one_entry(8, 24 * 24, 12, 12) + (1 << 19))
+    # B = M L keeps one q at a time; E needs 864 KB, eta and xi hold 154
+    free = 840 if room else 600
+    fake.fake_capacity(used - 4 * _one_entry(8, 24 * 24, 12, 12) + (free << 10))
     base = fake.fake_fma_calls()
     g.fragment_eri([C], traces=False)
-    assert fma == base and fake.fake_fma_calls() == base + 1
+    assert fma == base and fake.fake_fma_calls() == base + (0 if room else 1)
     fake.fake_capacity(1 << 40)
-    g.coulomb_metric_eta()
+    if room:
+        assert _code(g.coulomb_metric_eta) == STATE
+    else:
+        g.coulomb_metric_eta()
     g.close()
 
 
