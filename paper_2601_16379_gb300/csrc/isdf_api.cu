@@ -904,9 +904,6 @@ int isdf_fit_zeta(isdf_handle* h, double solve_tol, int32_t* rank_out) {
   tri_opt.qmap = qlist;
   tri_opt.krank = rankPi;
   ZM(who, 'N', 'N', rx, ng, rx, 1.0, wwork, np, pp, eta, ng, pg, xi, ng, xg, qh.count, tri_opt);
-  // xi stands only if no wait of its product expired (FMA chains have none)
-  if (who)
-    if (int e = tc_status(h, "xi of the fit")) return e;
   if (!qh.mirror.empty()) {
     const int2* mir = (const int2*)h->buf("q_mirror");
     CK(mirror_conj(h->st, W, pp, mir, (int)qh.mirror.size()));
@@ -917,6 +914,9 @@ int isdf_fit_zeta(isdf_handle* h, double solve_tol, int32_t* rank_out) {
   for (const auto& r : qh.runs)
     for (int q = r.first; q < r.first + r.second; ++q) tri_flops += (double)h->ranks[q] * h->ranks[q];
   stt.flops = 8.0 * nk * (double)np * ng * nao + 4.0 * tri_flops * ng;
+  // the fit stands only if no wait of xi's product expired (FMA chains have none)
+  if (who)
+    if (int e = tc_status(h, "xi of the fit")) return e;
   h->has_fit = true;
   h->has_xi = true;
   h->has_eta = true;
